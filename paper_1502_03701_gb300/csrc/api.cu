@@ -70,6 +70,7 @@ static void free_handle(stab_handle h) {
   for (int a = 0; a < 3; ++a) {
     dfree(h, h->ax[a].tab[0]);
     dfree(h, h->ax[a].tabf[0]);
+    dfree(h, h->ax[a].ptab[0]);
     dfree(h, h->d_dmat[a]);
     dfree(h, h->d_dmat_low[a]);
   }

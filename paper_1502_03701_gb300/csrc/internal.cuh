@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/stab.h"
+#include "pairs.cuh"
 
 #define STAB_MAX_DIM 3
 #define STAB_MAX_JOBS 16
@@ -21,6 +22,18 @@
 // elimination for bounded lines, the two first-order factors of the
 // circulant matrix for periodic lines.
 // ---------------------------------------------------------------------------
+// Constants of the pair-arithmetic line pass (pair_lines.cuh) per derivative
+// kind: the root r of the factorised interior rows, the stencil ratio rho,
+// 1/(1 - r^2), 1/(1 - r^n) (periodic lines), the closure rows' amplitude
+// matrix (wa, wb) and right-hand sides (cl, c0) of a bounded line, the
+// distance past which r^k no longer reaches the result (reach) or only its
+// low part (near).
+constexpr int kPairMaxC = 64;  // points per chunk
+struct PairKind {
+  ffn r, rho, kap, invn, wa, wb, cl[4], c0[3];
+  int reach, near;
+};
+
 struct AxisTables {
   int n;
   int periodic;
@@ -31,7 +44,33 @@ struct AxisTables {
   float* tabf[2];       // device FP32 copies [l'(n), m(n)] per kind (far warm-up)
   double* tab[2];       // device, per kind: [l'(n), dinv(n), m(n)]: Thomas factors of the sweep on the
                         // right-hand side scaled by dinv (l'_t = l_t d_{t-1} / d_t)
+  PairKind pk[2];       // pair-arithmetic pass
+  ffn* ptab[2];         // device: its powers of r and chunk factors
+  double pscale[2];     // its outputs are the derivatives divided by this
 };
+
+// Division by an invariant divisor with a multiply and a shift (Granlund and
+// Montgomery, "Division by invariant integers using multiplication", 1994):
+// p = 31 + ceil(log2 d), m = ceil(2^p / d), x / d = umulhi(x, m) >> (p - 32)
+// for 0 <= x < 2^31.
+struct FastDiv {
+  unsigned d, m;
+  int s;
+};
+inline FastDiv make_fastdiv(unsigned d) {
+  FastDiv f{d, 0u, 0};
+  if (d > 1) {
+    int l = 0;
+    while ((1ull << l) < d) ++l;
+    const int p = 31 + l;
+    f.m = (unsigned)(((1ull << p) + d - 1) / d);
+    f.s = p - 32;
+  }
+  return f;
+}
+__device__ __forceinline__ unsigned fdiv(unsigned x, const FastDiv& f) {
+  return f.d == 1 ? x : (__umulhi(x, f.m) >> f.s);
+}
 
 struct LineJob {
   const double2* in;
@@ -127,7 +166,7 @@ struct StabHandle {
   double* d_btab_low = nullptr;  // base tables with the reduced operator's derivatives
   double* d_coef;        // per-row tangent coefficients of the pointwise map (y-only base)
   double* d_coef_f;      // the same with the y metric folded in (inputs: eta-derivatives)
-  struct ffn* d_coef_p;  // d_coef_f as FP32 pairs (hi, lo), read by the pointwise kernel
+  ffn* d_coef_p;         // d_coef_f as FP32 pairs (hi, lo), read by the pointwise kernel
   float* d_btab_f;       // FP32 copy of the base tables (for the O(eps) remainder)
   bool force_dn_path;    // use the full FP64 difference-number pointwise kernel
   void* cublas = nullptr;  // cuBLAS handle of the tensor-core block factorisation (created on first use)
@@ -274,7 +313,7 @@ cudaError_t batch_stage(stab_jv_batch_s* B, const BatchImage& im);
 // copied to the device once) and the launches that read them.  gates[i]
 // (nullable) skips instance i's work while *gates[i] != 0.
 struct JvBatchPlan {
-  BatchSection norm, temp, line[3][4], point[2];
+  BatchSection norm, temp, line[3], point[2][2];
   std::vector<double*> zero_eps;  // epsilon slots of the exact-tangent instances
 };
 cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* const* v, double2* const* out,

@@ -23,7 +23,7 @@
 
 #include "internal.cuh"
 
-#include "pairs.cuh"
+#include "pair_lines.cuh"
 #include "pointwise.cuh"
 
 using pw::bt_count;
@@ -42,29 +42,6 @@ namespace {
 // warm-up of K points, after which the influence of the unknown start value
 // has decayed below 2^-56), then backward.
 // ---------------------------------------------------------------------------
-// Division by an invariant divisor with a multiply and a shift (Granlund and
-// Montgomery, "Division by invariant integers using multiplication", 1994):
-// p = 31 + ceil(log2 d), m = ceil(2^p / d), x / d = umulhi(x, m) >> (p - 32)
-// for 0 <= x < 2^31.
-struct FastDiv {
-  unsigned d, m;
-  int s;
-};
-inline FastDiv make_fastdiv(unsigned d) {
-  FastDiv f{d, 0u, 0};
-  if (d > 1) {
-    int l = 0;
-    while ((1ull << l) < d) ++l;
-    const int p = 31 + l;
-    f.m = (unsigned)(((1ull << p) + d - 1) / d);
-    f.s = p - 32;
-  }
-  return f;
-}
-__device__ __forceinline__ unsigned fdiv(unsigned x, const FastDiv& f) {
-  return f.d == 1 ? x : (__umulhi(x, f.m) >> f.s);
-}
-
 struct PassParams {
   LineJob job[STAB_MAX_JOBS];
   int njobs;
@@ -625,6 +602,7 @@ struct PointParams {
   double2 shift;
   pw::Phys phys;
   const int* gate;  // as PassParams::gate
+  float sc1[4], sc2[4];  // scales of the pair passes' first and second derivatives per axis
   FastDiv divnx, divny;  // division by nx and ny (points < 2^31)
 };
 
@@ -744,102 +722,156 @@ __global__ void k_coeffs(const PointParams P, double* coef) {
 
 
 
-// Inputs: raw line-pass outputs (eta-derivatives in y); the coefficients have
-// the y metric folded in (k_coeffs_fold) and are stored as FP32 pairs.  The
-// tangent part C_j w is formed with exact FP32 two-products of the pairs and
-// two-sum accumulation (~2^-47 relative per term), the O(eps) remainder in
-// FP32 from the inputs' high parts and FP32 base tables: no FP64 products.
+// The coefficients that can differ from zero for a base flow that depends on y
+// only (its x and z derivatives vanish): row a (0 = p, 1..D = u_i, D+1 = s),
+// input q in the order of pw::WIn.
 template <int D>
+__host__ __device__ constexpr bool coef_used(int a, int q) {
+  const int Y = 1, fp = 0, fv = 1 + Y, fs = D + 1, fT = D + 2;
+  const bool prow = a == 0, srow = a == D + 1;
+  if (q < D + 3) return q == fp || q == fv || q == fT || (q == fs && !srow);
+  q -= D + 3;
+  if (q < D * (D + 3)) {  // d f / dx_ax
+    const int ax = q / (D + 3), f = q % (D + 3);
+    // dissipation and dilatation (rows p and s): div u, and the shears that the base flow has
+    if (prow || srow)
+      return f == (prow ? fp : fs) || (f == fT && ax == Y) ||
+             (f >= 1 && f <= D && (f - 1 == ax || ax == Y || f == fv));
+    const int b = a - 1;  // momentum
+    if (f == a || (f == fp && ax == b)) return true;
+    if (b == Y) return f == fT || (f >= 1 && f <= D && f - 1 == ax);
+    return (f == fv && ax == b) || (f == fT && (ax == Y || ax == b));
+  }
+  q -= D * (D + 3);
+  if (q < D * (D + 1)) return q % (D + 1) == D ? (prow || srow) : q % (D + 1) == a - 1;
+  q -= D * (D + 1);
+  return q / D == a - 1 && q / D != q % D;
+}
+
+// Inputs: line-pass outputs (pairs, in units of the passes' scales); the
+// coefficients have the y metric and those scales folded in (k_coeffs_fold)
+// and are stored as FP32 pairs.  One thread per real value: it streams over
+// the inputs, adds each to the rows that it reaches (85 of the 225 products in
+// 3-D, 40 of 100 in 2-D) by exact FP32 two-products and two-sum accumulation, and
+// (EPS) evaluates the O(eps) remainder in FP32 from the inputs' high parts and
+// FP32 base tables: no FP64 products.
+template <int D, bool EPS>
 __device__ __forceinline__ void point_fast_body(const PointParams& P, const ffn* __restrict__ coefp,
                                                 const float* __restrict__ btab_f, unsigned bidx, unsigned nb) {
   constexpr int NW = pw::nw_inputs(D);
-  constexpr int o2 = (D + 3) + D * (D + 3), om = o2 + D * (D + 1);
-  const double e = *P.eps;
+  constexpr int o1 = D + 3, o2 = o1 + D * (D + 3), om = o2 + D * (D + 1);
+  const double e = EPS ? *P.eps : 0.0;
   const bool visc = P.phys.visc;
-  for (long long pt = (long long)bidx * blockDim.x + threadIdx.x; pt < P.npts; pt += (long long)nb * blockDim.x) {
-    const int j = row_of(P, pt);
-    const bool bc_row = (j == 0 || j == P.ny - 1);
-    const unsigned fl = bc_row ? P.bcflags[(j == P.ny - 1 ? (long long)P.nx * P.nz : 0)] : 0u;
+  const double* v = (const double*)P.v;
+  const float2* S = (const float2*)P.scratch;
+  const long long nreal = 2 * P.npts;
+  for (long long i = (long long)bidx * blockDim.x + threadIdx.x; i < nreal; i += (long long)nb * blockDim.x) {
+    const int j = row_of(P, i >> 1);
     const float2* Cp = (const float2*)(coefp + (long long)j * (D + 2) * NW);
-    auto S = [&](int slot) { return P.scratch[(long long)slot * P.npts + pt]; };
-#pragma unroll 1
-    for (int part = 0; part < 2; ++part) {
-      auto pick = [&](double2 z) { return part ? z.y : z.x; };
-      double w[NW];
+    ffn acc[D + 2];
+    float hi[EPS ? NW : 1];
 #pragma unroll
-      for (int f = 0; f < D + 2; ++f) w[f] = pick(P.v[(long long)f * P.npts + pt]);
-      w[D + 2] = visc ? pick(S(P.s_Tw)) : 0.0;
+    for (int a = 0; a < D + 2; ++a) acc[a] = ffn{0.0f, 0.0f};
+    if (EPS) {
+#pragma unroll
+      for (int q = 0; q < NW; ++q) hi[q] = 0.0f;
+    }
+    auto put = [&](int q, ffn w) {
+      if (EPS) hi[q] = w.hi;
+#pragma unroll
+      for (int a = 0; a < D + 2; ++a)
+        if (coef_used<D>(a, q)) {
+          const float2 c = __ldg(Cp + a * NW + q);
+          acc[a] = ff2_fma_u(ffn{c.x, c.y}, w, acc[a]);
+        }
+    };
+    auto slot = [&](int s) { const float2 w = S[(long long)s * nreal + i]; return ffn{w.x, w.y}; };
+#pragma unroll
+    for (int f = 0; f < D + 2; ++f) put(f, ff2_split(v[(long long)f * nreal + i]));
+#pragma unroll
+    for (int ax = 0; ax < D; ++ax)
+#pragma unroll
+      for (int f = 0; f < D + 2; ++f) put(o1 + ax * (D + 3) + f, slot(P.s_d1[ax][f]));
+    if (visc) {
+      put(D + 2, ff2_split(((const double*)P.scratch)[(long long)P.s_Tw * nreal + i]));
+#pragma unroll
+      for (int ax = 0; ax < D; ++ax) put(o1 + ax * (D + 3) + D + 2, slot(P.s_d1[ax][D + 2]));
 #pragma unroll
       for (int ax = 0; ax < D; ++ax)
 #pragma unroll
-        for (int f = 0; f < D + 3; ++f) w[D + 3 + ax * (D + 3) + f] = (f < D + 2 || visc) ? pick(S(P.s_d1[ax][f])) : 0.0;
-#pragma unroll
-      for (int ax = 0; ax < D; ++ax)
-#pragma unroll
-        for (int g = 0; g < D + 1; ++g) w[o2 + ax * (D + 1) + g] = visc ? pick(S(P.s_d2[ax][g])) : 0.0;
+        for (int g = 0; g < D + 1; ++g) put(o2 + ax * (D + 1) + g, slot(P.s_d2[ax][g]));
 #pragma unroll
       for (int a = 0; a < D; ++a)
 #pragma unroll
-        for (int c = 0; c < D; ++c) w[om + a * D + c] = (visc && a != c) ? pick(S(P.s_mix[a][c])) : 0.0;
-      ffn wp[NW];
+        for (int c = 0; c < D; ++c)
+          if (a != c) put(om + a * D + c, slot(P.s_mix[a][c]));
+    }
+    double res[D + 2];
 #pragma unroll
-      for (int q = 0; q < NW; ++q) wp[q] = ff_split(w[q]);
-      double res[D + 2];
+    for (int a = 0; a < D + 2; ++a) res[a] = ff2_to_d(acc[a]);
+    if (EPS && e != 0.0) {  // O(eps) remainder of the quotient, FP32, physical (metric-applied) inputs
+      const bool bc_row = (j == 0 || j == P.ny - 1);
+      const unsigned fl = bc_row ? P.bcflags[(j == P.ny - 1 ? (long long)P.nx * P.nz : 0)] : 0u;
+      const float ey = (float)P.eta_y[j], eyy = (float)P.eta_yy[j];
+      pw::WIn<D, float> Wf;
 #pragma unroll
-      for (int a = 0; a < D + 2; ++a) {
-        ffn acc{0.0f, 0.0f};
+      for (int q = 0; q < NW; ++q) set_input<D, float>(Wf, q, hi[q]);
 #pragma unroll
-        for (int q = 0; q < NW; ++q) {
-          const float2 c = __ldg(Cp + a * NW + q);
-          ff_acc_prod(acc, ffn{c.x, c.y}, wp[q]);
-        }
-        res[a] = ff_to_d(acc);
-      }
-      if (e != 0.0) {  // O(eps) remainder of the quotient, FP32, physical (metric-applied) inputs
-        const float ey = ff_split(P.eta_y[j]).hi, eyy = ff_split(P.eta_yy[j]).hi;
-        pw::WIn<D, float> Wf;
+      for (int ax = 0; ax < D; ++ax) {
+        const float s1 = P.sc1[ax], s2 = P.sc2[ax];
 #pragma unroll
-        for (int q = 0; q < NW; ++q) set_input<D, float>(Wf, q, wp[q].hi);
+        for (int f = 0; f < D + 3; ++f) Wf.d1[ax][f] *= s1;
 #pragma unroll
-        for (int f = 0; f < D + 3; ++f) Wf.d1[1][f] *= ey;
+        for (int g = 0; g < D + 1; ++g) Wf.d2[ax][g] *= s2;
 #pragma unroll
-        for (int g = 0; g < D + 1; ++g)
-          Wf.d2[1][g] = fmaf(Wf.d2[1][g], ey * ey, wp[D + 3 + (D + 3) + (g < D ? 1 + g : D + 2)].hi * eyy);
-#pragma unroll
-        for (int a = 0; a < D; ++a)
-#pragma unroll
-          for (int c = 0; c < D; ++c)
-            if (a == 1 || c == 1) Wf.mix[a][c] *= ey;
-        auto Bf = [&](int slot) { return btab_f[(long long)slot * P.nbase + j]; };
-        pw::DN3 o[D + 2];
-        pw::rhs_num<D, pw::DN3>(P.phys, Bf, Wf, e, bc_row, fl, o);
-#pragma unroll
-        for (int a = 0; a < D + 2; ++a) res[a] += f2d_exact(o[a].w2);
+        for (int c = 0; c < D; ++c) Wf.mix[ax][c] *= s1 * P.sc1[c];
       }
 #pragma unroll
+      for (int g = 0; g < D + 1; ++g) Wf.d2[1][g] = fmaf(Wf.d2[1][g], ey * ey, Wf.d1[1][g < D ? 1 + g : D + 2] * eyy);
+#pragma unroll
+      for (int f = 0; f < D + 3; ++f) Wf.d1[1][f] *= ey;
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+          if (a == 1 || c == 1) Wf.mix[a][c] *= ey;
+      auto Bf = [&](int slot) { return btab_f[(long long)slot * P.nbase + j]; };
+      pw::DN3 o[D + 2];
+      pw::rhs_num<D, pw::DN3>(P.phys, Bf, Wf, e, bc_row, fl, o);
+#pragma unroll
+      for (int a = 0; a < D + 2; ++a) res[a] += f2d_exact(o[a].w2);
+    }
+    double* out = (double*)P.out;
+    if (P.shift.x != 0.0 || P.shift.y != 0.0) {
+      const double sy = (i & 1) ? P.shift.y : -P.shift.y;  // the other component's factor
+#pragma unroll
       for (int a = 0; a < D + 2; ++a) {
-        const long long o = (long long)a * P.npts + pt;
-        double2 vv = P.v[o];
-        double sv = part ? (P.shift.x * vv.y + P.shift.y * vv.x) : (P.shift.x * vv.x - P.shift.y * vv.y);
-        double r = res[a] - sv;
-        if (part) P.out[o].y = r; else P.out[o].x = r;
+        const long long o = (long long)a * nreal + i;
+        res[a] -= fma(P.shift.x, v[o], sy * v[o ^ 1]);
       }
     }
+#pragma unroll
+    for (int a = 0; a < D + 2; ++a) out[(long long)a * nreal + i] = res[a];
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(128, D == 2 ? 4 : 3) k_point_fast(const PointParams P, const ffn* __restrict__ coefp,
-                                                   const float* __restrict__ btab_f) {
+template <int D, bool EPS>
+__global__ void __launch_bounds__(128, EPS ? (D == 2 ? 4 : 3) : 6)
+    k_point_fast(const __grid_constant__ PointParams P, const ffn* __restrict__ coefp, const float* __restrict__ btab_f) {
   if (P.gate && *P.gate) return;
-  point_fast_body<D>(P, coefp, btab_f, blockIdx.x, gridDim.x);
+  point_fast_body<D, EPS>(P, coefp, btab_f, blockIdx.x, gridDim.x);
 }
 
-// Fold the y metric into the per-row coefficients so that the pointwise kernel
-// can use the line passes' eta-derivatives directly:
-//   f_y = f_eta ey,  f_yy = f_etaeta ey^2 + f_eta eyy,  mixed with y: x ey.
+// Fold the y metric and the line passes' scales into the per-row coefficients
+// so that the pointwise kernel can use the passes' outputs directly:
+//   f_y = f_eta ey,  f_yy = f_etaeta ey^2 + f_eta eyy,  mixed with y: x ey;
+//   then x S1 of the axis (first), S2 (second), the product of both axes' S1 (mixed).
+struct PassScales {
+  double s1[3], s2[3];
+};
 template <int D>
-__global__ void k_coeffs_fold(const double* coef, const double* eta_y, const double* eta_yy, int ny, double* out) {
+__global__ void k_coeffs_fold(const double* coef, const double* eta_y, const double* eta_yy, int ny, PassScales sc,
+                              double* out) {
   constexpr int NW = pw::nw_inputs(D);
   constexpr int o1 = D + 3, o2 = (D + 3) + D * (D + 3), om = o2 + D * (D + 1);
   const int j = blockIdx.x, a = threadIdx.x;
@@ -857,13 +889,18 @@ __global__ void k_coeffs_fold(const double* coef, const double* eta_y, const dou
   for (int i = 0; i < D; ++i)
     for (int k = 0; k < D; ++k)
       if (i != k && (i == 1 || k == 1)) f[om + i * D + k] = c[om + i * D + k] * ey;
+  for (int i = 0; i < D; ++i) {
+    for (int k = 0; k < D + 3; ++k) f[o1 + i * (D + 3) + k] *= sc.s1[i];
+    for (int k = 0; k < D + 1; ++k) f[o2 + i * (D + 1) + k] *= sc.s2[i];
+    for (int k = 0; k < D; ++k) f[om + i * D + k] *= sc.s1[i] * sc.s1[k];
+  }
   double* o = out + ((long long)j * (D + 2) + a) * NW;
   for (int q = 0; q < NW; ++q) o[q] = f[q];
 }
 
 __global__ void k_split_pairs(const double* in, ffn* out, long long count) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
-    out[i] = ff_split(in[i]);
+    out[i] = ff2_split(in[i]);
 }
 
 __global__ void k_to_float_tab(const double* in, float* out, long long count) {
@@ -1034,7 +1071,7 @@ struct PointItem {
   const ffn* coefp;
   const float* btab_f;
 };
-static_assert(sizeof(PassParams) % 8 == 0 && sizeof(TempItem) % 8 == 0 && sizeof(PointItem) % 8 == 0,
+static_assert(sizeof(TempItem) % 8 == 0 && sizeof(PointItem) % 8 == 0,
               "items are copied to shared memory in 8-byte words");
 
 // largest i with start[i] <= b (start[0] = 0, increasing)
@@ -1073,8 +1110,8 @@ __global__ void k_temperature_fast_batch(const TempItem* __restrict__ items, con
   temperature_fast_body(sI.P, sI.Tw, blockIdx.x - s0, (unsigned)__ldg(start + i + 1) - s0);
 }
 
-template <int D>
-__global__ void __launch_bounds__(128, D == 2 ? 4 : 3)
+template <int D, bool EPS>
+__global__ void __launch_bounds__(128, EPS ? (D == 2 ? 4 : 3) : 6)
     k_point_fast_batch(const PointItem* __restrict__ items, const int* __restrict__ start, int count) {
   __shared__ PointItem sI;
   const int i = batch_item(start, count, blockIdx.x);
@@ -1082,32 +1119,17 @@ __global__ void __launch_bounds__(128, D == 2 ? 4 : 3)
   __syncthreads();
   if (sI.P.gate && *sI.P.gate) return;
   const unsigned s0 = (unsigned)__ldg(start + i);
-  point_fast_body<D>(sI.P, sI.coefp, sI.btab_f, blockIdx.x - s0, (unsigned)__ldg(start + i + 1) - s0);
+  point_fast_body<D, EPS>(sI.P, sI.coefp, sI.btab_f, blockIdx.x - s0, (unsigned)__ldg(start + i + 1) - s0);
 }
 
-// line passes: item = (instance, axis, chunk of at most STAB_MAX_JOBS jobs);
-// its blocks are (line block, job) with the line block fastest
-template <bool FF>
-__global__ void k_line_pass_batch(const PassParams* __restrict__ items, const int* __restrict__ start, int count) {
-  __shared__ PassParams sP;
+// line passes: item = (instance, axis), its blocks as in the single launch
+__global__ void __launch_bounds__(pl::kMaxThreads, 2)
+    k_pair_pass_batch(const pl::PairPass* __restrict__ items, const int* __restrict__ start, int count) {
+  __shared__ pl::PairPass sP;
   const int i = batch_item(start, count, blockIdx.x);
-  copy_to_shared(&sP, items + i, sizeof(PassParams));
+  copy_to_shared(&sP, items + i, sizeof(pl::PairPass));
   __syncthreads();
-  const unsigned local = blockIdx.x - (unsigned)__ldg(start + i);
-  const unsigned nbx = (unsigned)((sP.nlines + sP.L - 1) / sP.L);
-  line_pass_body<FF>(sP, local % nbx, local / nbx);
-}
-
-template <bool FF>
-__global__ void __launch_bounds__(kCompactMaxThreads)
-    k_line_pass_compact_batch(const PassParams* __restrict__ items, const int* __restrict__ start, int count) {
-  __shared__ PassParams sP;
-  const int i = batch_item(start, count, blockIdx.x);
-  copy_to_shared(&sP, items + i, sizeof(PassParams));
-  __syncthreads();
-  const unsigned local = blockIdx.x - (unsigned)__ldg(start + i);
-  const unsigned nbx = (unsigned)((sP.nlines + sP.L - 1) / sP.L);
-  line_pass_compact_body<FF>(sP, local % nbx, local / nbx);
+  pl::pair_pass_body(sP, blockIdx.x - (unsigned)__ldg(start + i));
 }
 
 }  // namespace
@@ -1168,6 +1190,57 @@ static void fill_axis_tables(AxisTables& A, std::vector<double>& host) {
   }
 }
 
+static ffn host_pair(double d) {
+  const float hi = (float)d;
+  return ffn{hi, (float)(d - (double)hi)};
+}
+
+// Constants and tables of the pair-arithmetic pass (pair_lines.cuh) for the
+// scheme alpha x_{t-1} + x_t + alpha x_{t+1} = c1 (f_{t+1} -+ f_{t-1}) + ..,
+// factorised as c (1 - r S^-1)(1 - r S).  Closure rows of a bounded line:
+// x_0 + a0 x_1 = R0, beta x_0 + x_1 + beta x_2 = R1, which with
+// x_t = p_t + A r^(t-1) + B r^(n-2-t) give a A + b B = R1 - beta R0 -
+// (1 - beta a0) p_1 - beta p_2 and its mirror image.
+static void fill_pair_tables(AxisTables& A, std::vector<ffn>& host) {
+  const int n = A.n;
+  host.assign((size_t)2 * pl::kTab, ffn{0.0f, 0.0f});
+  for (int kind = 0; kind < 2; ++kind) {
+    const double al = kind == 0 ? 1.0 / 3.0 : 2.0 / 11.0;
+    const double r = (-1.0 + std::sqrt(1.0 - 4.0 * al * al)) / (2.0 * al);
+    const double c = -al / r, lr = -std::log2(-r);
+    const double ih = 1.0 / A.h;
+    A.pscale[kind] = kind == 0 ? (7.0 / 9.0) * ih / c : (27.0 / 22.0) * ih * ih / c;
+    PairKind& K = A.pk[kind];
+    K = PairKind{};
+    K.r = host_pair(r);
+    K.rho = host_pair(kind == 0 ? 1.0 / 28.0 : 1.0 / 18.0);
+    K.kap = host_pair(1.0 / (1.0 - r * r));
+    K.invn = host_pair(1.0 / (1.0 - std::pow(r, n)));
+    K.reach = (int)std::ceil(54.0 / lr) + 1;
+    K.near = (int)std::ceil(26.0 / lr) + 1;
+    const double beta = kind == 0 ? 0.25 : 0.1, a0 = kind == 0 ? 2.0 : 11.0;
+    const double a = (1.0 - beta * a0) + beta * r;
+    const double b = (1.0 - beta * a0) * std::pow(r, n - 3) + beta * std::pow(r, n - 4);
+    K.wa = host_pair(a / (a * a - b * b));
+    K.wb = host_pair(-b / (a * a - b * b));
+    // kind 0: u = f_2 - f_0, v = f_1 - f_0: R0 = k (u/2 + 2 v), R1 = k (3/4) u;
+    // kind 1: u, v the second differences at rows 1, 2: R0 = k (13 u - v), R1 = k (6/5) u
+    const double k = kind == 0 ? 9.0 * c / 7.0 : 22.0 * c / 27.0;
+    const double r0u = kind == 0 ? 0.5 : 13.0, r0v = kind == 0 ? 2.0 : -1.0, r1u = kind == 0 ? 0.75 : 1.2;
+    K.cl[0] = host_pair(k * (r1u - beta * r0u));
+    K.cl[1] = host_pair(-k * beta * r0v);
+    K.cl[2] = host_pair(-(1.0 - beta * a0));
+    K.cl[3] = host_pair(-beta);
+    K.c0[0] = host_pair(k * r0u);
+    K.c0[1] = host_pair(k * r0v);
+    K.c0[2] = host_pair(-a0);
+    ffn* T = host.data() + (size_t)kind * pl::kTab;
+    for (int i = 0; i < pl::kTabPow; ++i) T[i] = host_pair(std::pow(r, i - 2));
+    for (int len = 0; len <= kPairMaxC; ++len)
+      T[pl::kTabPow + len] = host_pair(r * (1.0 - std::pow(r, 2 * len)) / (1.0 - r * r));
+  }
+}
+
 static void make_slots(StabHandle* h) {
   Slots& S = h->slots;
   const int D = h->dim;
@@ -1193,6 +1266,8 @@ static void make_slots(StabHandle* h) {
 
 // Parameters and launch shape of one axis's line pass for njobs jobs (the job
 // list itself is filled by the caller, STAB_MAX_JOBS per launch).
+static void axis_jobs(StabHandle* h, int ax, const double2* const* src, std::vector<LineJob>& jobs);
+
 static cudaError_t pass_shape(StabHandle* h, int axis, const PassParams& base_params, size_t njobs,
                               long long contiguous_lines, PassParams& P, int& threads, size_t& smem) {
   P = base_params;
@@ -1279,6 +1354,96 @@ static cudaError_t pass_shape(StabHandle* h, int axis, const PassParams& base_pa
   threads = ((threads + 31) / 32) * 32;
   smem = (size_t)smem_line * L + kLineSmemExtra;
   return cudaSuccess;
+}
+
+// Parameters and launch shape of one axis's pair-arithmetic pass (jobs filled
+// in by the caller).  Chunks of 32 points cost the fewest corrections per
+// point; shorter ones and fewer lines per CTA spread small grids over the SMs.
+static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, pl::PairPass& P, int& threads, size_t& smem,
+                              long long& blocks) {
+  const AxisTables& A = h->ax[axis];
+  const int n = A.n;
+  P = pl::PairPass{};
+  P.k[0] = A.pk[0];
+  P.k[1] = A.pk[1];
+  P.tab[0] = A.ptab[0];
+  P.tab[1] = A.ptab[1];
+  P.gate = h->gate;
+  P.nlines = h->npts / n;
+  P.stride = axis == 0 ? 1 : axis == 1 ? h->nx : (long long)h->nx * h->ny;
+  P.njobs = njobs;
+  P.axis = axis;
+  P.n = n;
+  P.nx = h->nx;
+  P.ny = h->ny;
+  P.bounded = !A.periodic;
+  const LineCfg cfg = h->line_cfg[axis];
+  auto smem_of = [&](int L, int nch) {
+    const int RL = 2 * L, RLp = RL % 4 == 0 ? RL + 2 : RL;
+    return (size_t)n * RLp * 8 + ((size_t)2 * RL * nch + 2 * RL + pl::kTab) * 8;
+  };
+  const long long want = 152LL * 1024;  // threads that fill the SMs
+  int C = cfg.C;
+  if (C <= 0) {
+    C = 32;
+    if (2 * P.nlines * njobs * ((n + 31) / 32) < want) C = 16;
+  }
+  if (C > kPairMaxC) C = kPairMaxC;
+  const int nch = (n + C - 1) / C;
+  int L = cfg.L;
+  if (L <= 0) {
+    L = 16;
+    while (L > 2 && (smem_of(L, nch) > 72 * 1024 || 2 * L * nch > 256 ||
+                     (P.nlines + L - 1) / L * njobs < 2 * 152))
+      L /= 2;
+  }
+  L = (int)std::min<long long>(L, std::max<long long>(1, P.nlines));
+  while (L > 1 && (2 * L * nch > pl::kMaxThreads || smem_of(L, nch) > pl::kSmemMax)) --L;
+  if (2 * L * nch > pl::kMaxThreads || smem_of(L, nch) > pl::kSmemMax) return cudaErrorInvalidValue;
+  P.L = L;
+  P.RL = 2 * L;
+  P.RLp = P.RL % 4 == 0 ? P.RL + 2 : P.RL;
+  P.nch = nch;
+  P.q = n / nch;
+  P.rem = n % nch;
+  P.divjobs = make_fastdiv((unsigned)njobs);
+  P.divRL = make_fastdiv((unsigned)P.RL);
+  P.divL = make_fastdiv((unsigned)L);
+  P.divn = make_fastdiv((unsigned)n);
+  P.divnx = make_fastdiv((unsigned)h->nx);
+  threads = ((P.RL * nch + 31) / 32) * 32;
+  smem = smem_of(L, nch);
+  blocks = (P.nlines + L - 1) / L * njobs;
+  return blocks > 0x7FFFFFFFLL ? cudaErrorInvalidValue : cudaSuccess;
+}
+
+// The pass of axis ax for the fields src (as axis_jobs): one job per derivative.
+static cudaError_t pair_pass(StabHandle* h, int ax, const double2* const* src, pl::PairPass& P, int& threads,
+                             size_t& smem, long long& blocks) {
+  std::vector<LineJob> jobs;
+  axis_jobs(h, ax, src, jobs);
+  const size_t raw = h->visc ? h->dim + 3 : h->dim + 2;  // the jobs after the fields' take pass outputs
+  std::vector<pl::PairJob> pj;
+  for (size_t q = 0; q < jobs.size(); ++q) {
+    const int pin = q >= raw;
+    if (jobs[q].out1) pj.push_back(pl::PairJob{(const double*)jobs[q].in, (float2*)jobs[q].out1, 0, pin});
+    if (jobs[q].out2) pj.push_back(pl::PairJob{(const double*)jobs[q].in, (float2*)jobs[q].out2, 1, pin});
+  }
+  if (pj.empty() || pj.size() > STAB_MAX_JOBS) return cudaErrorInvalidValue;
+  const cudaError_t e = pair_shape(h, ax, (int)pj.size(), P, threads, smem, blocks);
+  std::copy(pj.begin(), pj.end(), P.job);
+  return e;
+}
+
+static cudaError_t run_pair_pass(StabHandle* h, int ax, const double2* const* src) {
+  pl::PairPass P;
+  int threads = 0;
+  size_t smem = 0;
+  long long blocks = 0;
+  const cudaError_t e = pair_pass(h, ax, src, P, threads, smem, blocks);
+  if (e != cudaSuccess) return e;
+  pl::k_pair_pass<<<(unsigned)blocks, threads, smem, h->stream>>>(P);
+  return cudaGetLastError();
 }
 
 static cudaError_t run_pass(StabHandle* h, int axis, const PassParams& base_params, const std::vector<LineJob>& jobs,
@@ -1417,8 +1582,9 @@ cudaError_t jv_reduced_base_table(StabHandle* h, double* btab) {
 }
 
 // all derivative passes for field sources src[f] (f = 0..D+2): y, then z,
-// then x (the mixed derivatives need the y and z passes)
-static cudaError_t run_derivatives(StabHandle* h, const double2* const* src, int ff) {
+// then x (the mixed derivatives need the y and z passes); fast: in pair
+// arithmetic (pairs in the slots), else in FP64 (ff: pair right-hand sides)
+static cudaError_t run_derivatives(StabHandle* h, const double2* const* src, int ff, bool fast) {
   PassParams P{};
   P.gate = h->gate;
   P.ff = ff;
@@ -1427,10 +1593,15 @@ static cudaError_t run_derivatives(StabHandle* h, const double2* const* src, int
   for (int q = 0; q < 3; ++q) {
     const int ax = order[q];
     if (ax >= h->dim) continue;
-    std::vector<LineJob> jobs;
-    axis_jobs(h, ax, src, jobs);
     const int ts = phase_begin(h, phase[q]);
-    cudaError_t err = run_pass(h, ax, P, jobs);
+    cudaError_t err;
+    if (fast) {
+      err = run_pair_pass(h, ax, src);
+    } else {
+      std::vector<LineJob> jobs;
+      axis_jobs(h, ax, src, jobs);
+      err = run_pass(h, ax, P, jobs);
+    }
     if (err != cudaSuccess) return err;
     phase_end(h, ts);
   }
@@ -1505,7 +1676,11 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
     LineCfg best{};
     double best_ms = 1e300;
     const int n = h->ax[ax].n;
+    // with a y-only base flow the pair-arithmetic pass runs, which has no kinds variants
+    const bool fast = h->homog && h->d_coef && !h->force_dn_path;
+    auto pass = [&]() { return fast ? run_pair_pass(h, ax, src) : run_pass(h, ax, P, jobs); };
     for (int kp : {1, 2, 3}) {
+      if (fast && kp != 3) continue;
       for (int C : {16, 32, 64}) {
         if (C > 16 && C >= 2 * n) continue;
         for (int L : {1, 2, 4, 8, 16, 32}) {
@@ -1516,7 +1691,7 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
           if (tpl * L > (kp == 3 ? kCompactMaxThreads : 1024) || planes * 8 * LS * L + kLineSmemExtra > kLineSmemMax)
             continue;
           h->line_cfg[ax] = LineCfg{C, L, kp};
-          if (run_pass(h, ax, P, jobs) != cudaSuccess) {  // a shape this device cannot launch: skip it
+          if (pass() != cudaSuccess) {  // a shape this device cannot launch: skip it
             cudaGetLastError();
             continue;
           }
@@ -1524,7 +1699,7 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
           float best_t = 1e30f;
           for (int r = 0; r < 5 && err == cudaSuccess; ++r) {
             cudaEventRecord(e0, h->stream);
-            for (int q = 0; q < 3 && err == cudaSuccess; ++q) err = run_pass(h, ax, P, jobs);
+            for (int q = 0; q < 3 && err == cudaSuccess; ++q) err = pass();
             cudaEventRecord(e1, h->stream);
             cudaEventSynchronize(e1);
             float t = 0.f;
@@ -1633,6 +1808,10 @@ static PointParams point_params(StabHandle* h, const double2* v) {
   P.bcflags = h->d_bcflags;
   P.eps = h->d_eps;
   P.phys = phys_of(h);
+  for (int a = 0; a < h->dim; ++a) {
+    P.sc1[a] = (float)h->ax[a].pscale[0];
+    P.sc2[a] = (float)h->ax[a].pscale[1];
+  }
   return P;
 }
 
@@ -1650,8 +1829,10 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
   const int D = h->dim;
   cudaError_t err;
   // set once per handle (current device), never during a stream capture
-  const void* line_kernels[4] = {(const void*)k_line_pass<false>, (const void*)k_line_pass<true>,
-                                 (const void*)k_line_pass_compact<false>, (const void*)k_line_pass_compact<true>};
+  const void* line_kernels[5] = {(const void*)k_line_pass<false>, (const void*)k_line_pass<true>,
+                                 (const void*)k_line_pass_compact<false>, (const void*)k_line_pass_compact<true>,
+                                 (const void*)pl::k_pair_pass};
+  static_assert(kLineSmemMax == pl::kSmemMax, "one opt-in size for the line kernels");
   for (const void* k : line_kernels)
     if ((err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmemMax)) != cudaSuccess)
       return err;
@@ -1665,6 +1846,7 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
     A.h = ax == 0 ? h->lx / h->nx : ax == 1 ? 1.0 / (h->ny - 1) : (D == 3 ? h->lz / h->nz : 1.0);
     A.tab[0] = A.tab[1] = nullptr;
     A.tabf[0] = A.tabf[1] = nullptr;
+    A.ptab[0] = A.ptab[1] = nullptr;
     if (ax >= D) continue;
     std::vector<double> host;
     fill_axis_tables(A, host);
@@ -1682,6 +1864,12 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
     float* df;
     if ((err = dalloc(h, &df, hf.size() * sizeof(float))) != cudaSuccess) return err;
     if ((err = cudaMemcpyAsync(df, hf.data(), hf.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream)) != cudaSuccess)
+      return err;
+    std::vector<ffn> hp;
+    fill_pair_tables(A, hp);
+    if ((err = dalloc(h, &A.ptab[0], hp.size() * sizeof(ffn))) != cudaSuccess) return err;
+    A.ptab[1] = A.ptab[0] + pl::kTab;
+    if ((err = cudaMemcpyAsync(A.ptab[0], hp.data(), hp.size() * sizeof(ffn), cudaMemcpyHostToDevice, h->stream)) != cudaSuccess)
       return err;
     if ((err = cudaStreamSynchronize(h->stream)) != cudaSuccess) return err;  // host vectors go out of scope
     A.tabf[0] = df;
@@ -1746,7 +1934,7 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
   const double2* src[6];
   for (int f = 0; f < D + 2; ++f) src[f] = bv + (long long)f * h->npts;
   src[D + 2] = bT;
-  if ((err = run_derivatives(h, src, 0)) != cudaSuccess) return err;  // base tables: FP64 right-hand sides
+  if ((err = run_derivatives(h, src, 0, false)) != cudaSuccess) return err;  // base tables: FP64 right-hand sides
   PackParams K = pack_params(h, h->d_btab);
   k_pack_base<<<grid_for(h->nbase, thr), thr, 0, h->stream>>>(K);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
@@ -1758,8 +1946,13 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
     else k_coeffs<3><<<h->ny, 64, 0, h->stream>>>(PP, h->d_coef);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     if ((err = dalloc(h, &h->d_coef_f, (size_t)h->ny * (D + 2) * nw * sizeof(double))) != cudaSuccess) return err;
-    if (D == 2) k_coeffs_fold<2><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, h->d_coef_f);
-    else k_coeffs_fold<3><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, h->d_coef_f);
+    PassScales sc{};
+    for (int a = 0; a < D; ++a) {
+      sc.s1[a] = h->ax[a].pscale[0];
+      sc.s2[a] = h->ax[a].pscale[1];
+    }
+    if (D == 2) k_coeffs_fold<2><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, sc, h->d_coef_f);
+    else k_coeffs_fold<3><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, sc, h->d_coef_f);
     const long long ncf = (long long)h->ny * (D + 2) * nw;
     if ((err = dalloc(h, &h->d_coef_p, ncf * sizeof(ffn))) != cudaSuccess) return err;
     k_split_pairs<<<64, 256, 0, h->stream>>>(h->d_coef_f, h->d_coef_p, ncf);
@@ -1814,11 +2007,14 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   const double2* src[6];
   for (int f = 0; f < D + 2; ++f) src[f] = v + (long long)f * h->npts;
   src[D + 2] = Tw;
-  if ((err = run_derivatives(h, src, h->stencil_ff)) != cudaSuccess) return err;
+  if ((err = run_derivatives(h, src, h->stencil_ff, fast)) != cudaSuccess) return err;
   const int tp = phase_begin(h, STAB_PHASE_POINTWISE);
   if (fast) {
-    if (D == 2) k_point_fast<2><<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
-    else k_point_fast<3><<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
+    const int g = grid_for(2 * h->npts, thr);
+    if (D == 2 && eps_mode == 2) k_point_fast<2, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
+    else if (D == 2) k_point_fast<2, true><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
+    else if (eps_mode == 2) k_point_fast<3, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
+    else k_point_fast<3, true><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
   } else {
     if (D == 2) k_point<2><<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P);
     else k_point<3><<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P);
@@ -1895,13 +2091,7 @@ cudaError_t batch_order_end(stab_jv_batch_s* B) {
 }
 
 static cudaError_t jv_batch_attributes() {
-  const void* ks[4] = {(const void*)k_line_pass_batch<false>, (const void*)k_line_pass_batch<true>,
-                       (const void*)k_line_pass_compact_batch<false>, (const void*)k_line_pass_compact_batch<true>};
-  for (const void* k : ks) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmemMax);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return cudaFuncSetAttribute(k_pair_pass_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl::kSmemMax);
 }
 
 // Parameter-image sections of one batched J v (every phase, one section per
@@ -1917,9 +2107,9 @@ cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
   // 2. temperature differences (viscous instances)
   std::vector<TempItem> temps;
   std::vector<int> temp_blocks;
-  // 4. pointwise assembly, per dimension
-  std::vector<PointItem> points[2];
-  std::vector<int> point_blocks[2];
+  // 4. pointwise assembly, per dimension and J v form (tangent, epsilon-quotient)
+  std::vector<PointItem> points[2][2];
+  std::vector<int> point_blocks[2][2];
   plan.zero_eps.clear();
   for (int i = 0; i < count; ++i) {
     StabHandle* h = hs[i];
@@ -1951,20 +2141,20 @@ cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
       temps.push_back(TempItem{P, Tw});
       temp_blocks.push_back(grid_for(h->npts, 128));
     }
-    points[h->dim - 2].push_back(PointItem{P, h->d_coef_p, h->d_btab_f});
-    point_blocks[h->dim - 2].push_back(grid_for(h->npts, 128));
+    const int form = h->opts.eps_mode != 2;
+    points[h->dim - 2][form].push_back(PointItem{P, h->d_coef_p, h->d_btab_f});
+    point_blocks[h->dim - 2][form].push_back(grid_for(2 * h->npts, 128));
   }
   plan.norm = im.section(norms, norm_blocks, 256, 0);
   plan.temp = im.section(temps, temp_blocks, 128, 0);
-  // 3. line passes y, z, x; per axis one section per kernel variant (main /
-  // compact, FP64 / pair right-hand sides)
+  // 3. line passes y, z, x: one section per axis
   static const int order[3] = {1, 2, 0};
   for (int q = 0; q < 3; ++q) {
     const int ax = order[q];
-    std::vector<PassParams> items[4];
-    std::vector<int> blocks[4];
-    int threads[4] = {0, 0, 0, 0};
-    size_t smem[4] = {0, 0, 0, 0};
+    std::vector<pl::PairPass> items;
+    std::vector<int> blocks;
+    int threads = 0;
+    size_t smem = 0;
     for (int i = 0; i < count; ++i) {
       StabHandle* h = hs[i];
       if (ax >= h->dim) continue;
@@ -1972,32 +2162,22 @@ cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
       const double2* src[6];
       for (int f = 0; f < D + 2; ++f) src[f] = v[i] + (long long)f * h->npts;
       src[D + 2] = h->d_scratch + (long long)h->slots.Tw * h->npts;
-      std::vector<LineJob> jobs;
-      axis_jobs(h, ax, src, jobs);
-      if (jobs.empty()) continue;
-      PassParams base{};
-      base.ff = h->stencil_ff;
-      base.gate = gates ? gates[i] : nullptr;
-      PassParams P;
+      pl::PairPass P;
       int thr = 0;
       size_t sm = 0;
-      const cudaError_t e = pass_shape(h, ax, base, jobs.size(), -1, P, thr, sm);
+      long long nb = 0;
+      const cudaError_t e = pair_pass(h, ax, src, P, thr, sm, nb);
       if (e != cudaSuccess) return e;
-      const int var = (P.KP == 3 ? 2 : 0) + (P.ff ? 1 : 0);
-      const long long nbx = (P.nlines + P.L - 1) / P.L;
-      if (nbx * STAB_MAX_JOBS > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
-      for (size_t j0 = 0; j0 < jobs.size(); j0 += STAB_MAX_JOBS) {
-        P.njobs = (int)std::min<size_t>(STAB_MAX_JOBS, jobs.size() - j0);
-        for (int k = 0; k < P.njobs; ++k) P.job[k] = jobs[j0 + k];
-        items[var].push_back(P);
-        blocks[var].push_back((int)(nbx * P.njobs));
-      }
-      threads[var] = std::max(threads[var], thr);
-      smem[var] = std::max(smem[var], sm);
+      P.gate = gates ? gates[i] : nullptr;
+      items.push_back(P);
+      blocks.push_back((int)nb);
+      threads = std::max(threads, thr);
+      smem = std::max(smem, sm);
     }
-    for (int k = 0; k < 4; ++k) plan.line[q][k] = im.section(items[k], blocks[k], threads[k], smem[k]);
+    plan.line[q] = im.section(items, blocks, threads, smem);
   }
-  for (int d = 0; d < 2; ++d) plan.point[d] = im.section(points[d], point_blocks[d], 128, 0);
+  for (int d = 0; d < 2; ++d)
+    for (int f = 0; f < 2; ++f) plan.point[d][f] = im.section(points[d][f], point_blocks[d][f], 128, 0);
   return im.overflow ? cudaErrorInvalidValue : cudaSuccess;
 }
 
@@ -2011,22 +2191,18 @@ cudaError_t jv_batch_launch(const JvBatchPlan& plan, const unsigned char* d, cud
   if (plan.temp.count)
     k_temperature_fast_batch<<<plan.temp.blocks, 128, 0, st>>>((const TempItem*)items_of(plan.temp),
                                                                start_of(plan.temp), plan.temp.count);
-  for (int q = 0; q < 3; ++q)
-    for (int k = 0; k < 4; ++k) {
-      const BatchSection& s = plan.line[q][k];
-      if (!s.count) continue;
-      const PassParams* it = (const PassParams*)items_of(s);
-      if (k == 0) k_line_pass_batch<false><<<s.blocks, s.threads, s.smem, st>>>(it, start_of(s), s.count);
-      else if (k == 1) k_line_pass_batch<true><<<s.blocks, s.threads, s.smem, st>>>(it, start_of(s), s.count);
-      else if (k == 2) k_line_pass_compact_batch<false><<<s.blocks, s.threads, s.smem, st>>>(it, start_of(s), s.count);
-      else k_line_pass_compact_batch<true><<<s.blocks, s.threads, s.smem, st>>>(it, start_of(s), s.count);
-    }
-  if (plan.point[0].count)
-    k_point_fast_batch<2><<<plan.point[0].blocks, 128, 0, st>>>((const PointItem*)items_of(plan.point[0]),
-                                                               start_of(plan.point[0]), plan.point[0].count);
-  if (plan.point[1].count)
-    k_point_fast_batch<3><<<plan.point[1].blocks, 128, 0, st>>>((const PointItem*)items_of(plan.point[1]),
-                                                               start_of(plan.point[1]), plan.point[1].count);
+  for (int q = 0; q < 3; ++q) {
+    const BatchSection& s = plan.line[q];
+    if (s.count)
+      k_pair_pass_batch<<<s.blocks, s.threads, s.smem, st>>>((const pl::PairPass*)items_of(s), start_of(s), s.count);
+  }
+  auto point = [&](const BatchSection& s, auto kernel) {
+    if (s.count) kernel<<<s.blocks, 128, 0, st>>>((const PointItem*)items_of(s), start_of(s), s.count);
+  };
+  point(plan.point[0][0], k_point_fast_batch<2, false>);
+  point(plan.point[0][1], k_point_fast_batch<2, true>);
+  point(plan.point[1][0], k_point_fast_batch<3, false>);
+  point(plan.point[1][1], k_point_fast_batch<3, true>);
   return cudaGetLastError();
 }
 

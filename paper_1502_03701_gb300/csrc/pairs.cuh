@@ -105,3 +105,59 @@ __device__ __forceinline__ ffn ff_warp_sum(ffn x) {
   }
   return x;
 }
+
+// ---------------------------------------------------------------------------
+// Pair arithmetic of the derivative passes (rounding intrinsics, so that the
+// compiler fuses nothing across the error terms).
+// ---------------------------------------------------------------------------
+// d to the nearest pair: hi is d rounded to 24 bits, lo the rest (29 bits,
+// signed) rounded to 24, so |d - hi - lo| <= 2^-49 |d|.  Integer operations
+// but one conversion: the FP64 pipe is not used.  |d| below 2^-126 gives zero,
+// lo is kept from 2^-74 up; from 2^127 up and for NaN, hi is Inf or NaN.
+__device__ __forceinline__ ffn ff2_split(double d) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  const unsigned e = (h >> 20) & 0x7FFu;
+  const unsigned long long t = (((unsigned long long)h << 32) | l) + 0x10000000ull;  // half a unit of hi
+  const unsigned sign = h & 0x80000000u;
+  // exponent rebased by 896 modulo 512: exact for results in [1, 254]
+  unsigned hb = sign | (((unsigned)(t >> 29) - (384u << 23)) & 0x7FFFFFFFu);
+  float lo = __int2float_rn((int)(l << 3) >> 3) * __uint_as_float(sign | ((unsigned)max((int)e - 948, 0) << 23));
+  if (e - 897u >= 253u) {  // zero, tiny, huge, Inf or NaN
+    hb = e < 897u ? sign : (sign | (e == 0x7FFu && ((h & 0xFFFFFu) | l) ? 0x7FC00000u : 0x7F800000u));
+    lo = 0.0f;
+  }
+  return ffn{__uint_as_float(hb), lo};
+}
+__device__ __forceinline__ ffn ff2_norm(ffn a) {
+  const float t = __fadd_rn(a.hi, a.lo);
+  return ffn{t, __fsub_rn(a.lo, __fsub_rn(t, a.hi))};
+}
+__device__ __forceinline__ float ff2_two_sum(float a, float b, float& err) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
+// a + b; _u: low part not folded back into the high part
+__device__ __forceinline__ ffn ff2_add_u(ffn a, ffn b) {
+  float e;
+  const float s = ff2_two_sum(a.hi, b.hi, e);
+  return ffn{s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
+}
+__device__ __forceinline__ ffn ff2_add(ffn a, ffn b) { return ff2_norm(ff2_add_u(a, b)); }
+// w + c x: exact product of the high parts, cross terms, two-sum
+__device__ __forceinline__ ffn ff2_fma_u(ffn c, ffn x, ffn w) {
+  const float p = __fmul_rn(c.hi, x.hi);
+  float e = __fmaf_rn(c.hi, x.hi, -p), t;
+  e = __fmaf_rn(c.hi, x.lo, e);
+  e = __fmaf_rn(c.lo, x.hi, e);
+  const float s = ff2_two_sum(w.hi, p, t);
+  return ffn{s, __fadd_rn(__fadd_rn(t, w.lo), e)};
+}
+__device__ __forceinline__ ffn ff2_fma(ffn c, ffn x, ffn w) { return ff2_norm(ff2_fma_u(c, x, w)); }
+// hi + lo in FP64 with integer conversions and one add; Inf and NaN are kept
+__device__ __forceinline__ double ff2_to_d(ffn a) {
+  const unsigned u = __float_as_uint(a.hi);
+  const double d = f2d_exact(a.hi) + f2d_exact(a.lo);
+  if ((u & 0x7F800000u) != 0x7F800000u) return d;
+  return __hiloint2double((int)((u & 0x80000000u) | 0x7FF00000u | ((u & 0x7FFFFFu) ? 0x80000u : 0u)), 0);
+}

@@ -69,42 +69,48 @@ __device__ __forceinline__ DN sqrt_t(DN x, double sqa, double inva, double e) {
 struct DN3 {
   float a, w1, w2;
 };
+// Rounding intrinsics and explicit FMAs throughout: every kernel that
+// inlines this code rounds alike (the batched and the single launches agree
+// bit for bit).
+__device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ DN3 dn3(float a, float w1, float w2) { return DN3{a, w1, w2}; }
-__device__ __forceinline__ DN3 operator+(DN3 x, DN3 y) { return dn3(x.a + y.a, x.w1 + y.w1, x.w2 + y.w2); }
-__device__ __forceinline__ DN3 operator-(DN3 x, DN3 y) { return dn3(x.a - y.a, x.w1 - y.w1, x.w2 - y.w2); }
+__device__ __forceinline__ DN3 operator+(DN3 x, DN3 y) { return dn3(fadd(x.a, y.a), fadd(x.w1, y.w1), fadd(x.w2, y.w2)); }
+__device__ __forceinline__ DN3 operator-(DN3 x, DN3 y) { return dn3(fsub(x.a, y.a), fsub(x.w1, y.w1), fsub(x.w2, y.w2)); }
 __device__ __forceinline__ DN3 operator-(DN3 x) { return dn3(-x.a, -x.w1, -x.w2); }
 __device__ __forceinline__ DN3 operator*(double c, DN3 x) {
   float cf = (float)c;
-  return dn3(cf * x.a, cf * x.w1, cf * x.w2);
+  return dn3(fmul(cf, x.a), fmul(cf, x.w1), fmul(cf, x.w2));
 }
-__device__ __forceinline__ DN3 add(DN3 x, double c) { return dn3(x.a + (float)c, x.w1, x.w2); }
+__device__ __forceinline__ DN3 add(DN3 x, double c) { return dn3(fadd(x.a, (float)c), x.w1, x.w2); }
 __device__ __forceinline__ DN3 mul(DN3 x, DN3 y, double ed) {
   const float e = (float)ed;
-  float w1 = fmaf(x.a, y.w1, x.w1 * y.a);
-  float w2 = fmaf(x.a, y.w2, fmaf(x.w2, y.a, e * (x.w1 + x.w2) * (y.w1 + y.w2)));
-  return dn3(x.a * y.a, w1, w2);
+  float w1 = fmaf(x.a, y.w1, fmul(x.w1, y.a));
+  float w2 = fmaf(x.a, y.w2, fmaf(x.w2, y.a, fmul(fmul(e, fadd(x.w1, x.w2)), fadd(y.w1, y.w2))));
+  return dn3(fmul(x.a, y.a), w1, w2);
 }
 // x/(1+x) and (1/(1+x) - 1) = -x/(1+x)
 __device__ __forceinline__ float xinv1pf(float x) {
-  if (fabsf(x) < 1e-3f) return x * fmaf(x, fmaf(x, 1.0f - x, -1.0f), 1.0f);
-  return x / (1.0f + x);
+  if (fabsf(x) < 1e-3f) return fmul(x, fmaf(x, fmaf(x, fsub(1.0f, x), -1.0f), 1.0f));
+  return x / fadd(1.0f, x);
 }
 __device__ __forceinline__ DN3 rcp_t(DN3 x, double inva_d, double ed) {
-  const float inva = (float)inva_d, i2 = inva * inva;
-  const float w = x.w1 + x.w2;
-  const float X = (float)ed * w * inva;
-  return dn3(inva, -x.w1 * i2, fmaf(-x.w2, i2, w * i2 * xinv1pf(X)));
+  const float inva = (float)inva_d, i2 = fmul(inva, inva);
+  const float w = fadd(x.w1, x.w2);
+  const float X = fmul(fmul((float)ed, w), inva);
+  return dn3(inva, fmul(-x.w1, i2), fmaf(-x.w2, i2, fmul(fmul(w, i2), xinv1pf(X))));
 }
 // (sqrt(1+x) - 1)/x - 1/2 = x (-1/8 + x/16 - 5x^2/128 + ...)
 __device__ __forceinline__ float sqrt_corr(float x) {
-  if (fabsf(x) < 1e-3f) return x * fmaf(x, fmaf(x, -5.0f / 128.0f, 1.0f / 16.0f), -1.0f / 8.0f);
-  return (sqrtf(1.0f + x) - 1.0f) / x - 0.5f;
+  if (fabsf(x) < 1e-3f) return fmul(x, fmaf(x, fmaf(x, -5.0f / 128.0f, 1.0f / 16.0f), -1.0f / 8.0f));
+  return fsub(fsub(sqrtf(fadd(1.0f, x)), 1.0f) / x, 0.5f);
 }
 __device__ __forceinline__ DN3 sqrt_t(DN3 x, double sqa_d, double inva_d, double ed) {
-  const float sqa = (float)sqa_d, inva = (float)inva_d, k = sqa * inva;
-  const float w = x.w1 + x.w2;
-  const float X = (float)ed * w * inva;
-  return dn3(sqa, 0.5f * k * x.w1, fmaf(0.5f * k, x.w2, w * k * sqrt_corr(X)));
+  const float sqa = (float)sqa_d, inva = (float)inva_d, k = fmul(sqa, inva);
+  const float w = fadd(x.w1, x.w2);
+  const float X = fmul(fmul((float)ed, w), inva);
+  return dn3(sqa, fmul(fmul(0.5f, k), x.w1), fmaf(fmul(0.5f, k), x.w2, fmul(fmul(w, k), sqrt_corr(X))));
 }
 
 // ---------------------------------------------------------------------------
@@ -129,12 +135,12 @@ __device__ __forceinline__ double closure_T_w(const ClosureK& C, double T0, doub
 
 // e^z - 1 - z over z, and ln(1+z) - z over z, for the FP32 remainder
 __device__ __forceinline__ float expm1_m1_over_f(float z) {
-  if (fabsf(z) < 1e-3f) return z * fmaf(z, fmaf(z, 1.0f / 24.0f, 1.0f / 6.0f), 0.5f);
-  return expm1f(z) / z - 1.0f;
+  if (fabsf(z) < 1e-3f) return fmul(z, fmaf(z, fmaf(z, 1.0f / 24.0f, 1.0f / 6.0f), 0.5f));
+  return fsub(expm1f(z) / z, 1.0f);
 }
 __device__ __forceinline__ float log1p_m1_over_f(float z) {
-  if (fabsf(z) < 1e-3f) return z * fmaf(z, fmaf(z, -0.25f, 1.0f / 3.0f), -0.5f);
-  return log1pf(z) / z - 1.0f;
+  if (fabsf(z) < 1e-3f) return fmul(z, fmaf(z, fmaf(z, -0.25f, 1.0f / 3.0f), -0.5f));
+  return fsub(log1pf(z) / z, 1.0f);
 }
 
 // Closure functions by number type: rho from the inputs (p, s).
@@ -143,11 +149,11 @@ __device__ __forceinline__ DN make_rho(const ClosureK& C, double rho0, double ip
 }
 __device__ __forceinline__ DN3 make_rho(const ClosureK& C, double rho0, double ip0, DN3 p, DN3 s, double ed) {
   const float e = (float)ed, r0 = (float)rho0;
-  const float q = p.w1 * (float)ip0;
-  const float X1 = fmaf((float)C.ig, q, -s.w1 * (float)C.icp);
-  const float X2 = (float)C.ig * q * log1p_m1_over_f(e * q);
-  const float X = X1 + X2;
-  return dn3(r0, r0 * X1, r0 * fmaf(X, expm1_m1_over_f(e * X), X2));
+  const float q = fmul(p.w1, (float)ip0);
+  const float X1 = fmaf((float)C.ig, q, fmul(-s.w1, (float)C.icp));
+  const float X2 = fmul(fmul((float)C.ig, q), log1p_m1_over_f(fmul(e, q)));
+  const float X = fadd(X1, X2);
+  return dn3(r0, fmul(r0, X1), fmul(r0, fmaf(X, expm1_m1_over_f(fmul(e, X)), X2)));
 }
 
 // ---------------------------------------------------------------------------

@@ -66,6 +66,7 @@ static void free_handle(stab_handle h) {
   dfree(h, h->d_coef_f);
   dfree(h, h->d_coef_p);
   dfree(h, h->d_btab_f);
+  dfree(h, h->d_tcoef);
   dfree(h, h->d_btab_low);
   for (int a = 0; a < 3; ++a) {
     dfree(h, h->ax[a].tab[0]);

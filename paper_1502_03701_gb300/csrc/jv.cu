@@ -601,7 +601,9 @@ struct PointParams {
   double2* out;
   double2 shift;
   pw::Phys phys;
+  pw::PhysT<float> physf;
   const int* gate;  // as PassParams::gate
+  const double* tcoef;  // [2][ny]: T_w = tcoef[0] p_w + tcoef[1] s_w to first order (y-only base)
   float sc1[4], sc2[4];  // scales of the pair passes' first and second derivatives per axis
   FastDiv divnx, divny;  // division by nx and ny (points < 2^31)
 };
@@ -757,7 +759,7 @@ __host__ __device__ constexpr bool coef_used(int a, int q) {
 // FP32 base tables: no FP64 products.
 template <int D, bool EPS>
 __device__ __forceinline__ void point_fast_body(const PointParams& P, const ffn* __restrict__ coefp,
-                                                const float* __restrict__ btab_f, unsigned bidx, unsigned nb) {
+                                                const float* __restrict__ btab_f, unsigned bidx) {
   constexpr int NW = pw::nw_inputs(D);
   constexpr int o1 = D + 3, o2 = o1 + D * (D + 3), om = o2 + D * (D + 1);
   const double e = EPS ? *P.eps : 0.0;
@@ -765,46 +767,43 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const ffn*
   const double* v = (const double*)P.v;
   const float2* S = (const float2*)P.scratch;
   const long long nreal = 2 * P.npts;
-  for (long long i = (long long)bidx * blockDim.x + threadIdx.x; i < nreal; i += (long long)nb * blockDim.x) {
+  const long long i = (long long)bidx * blockDim.x + threadIdx.x;  // no loop: its invariant addresses would take
+  if (i < nreal) {                                                 // the registers that the loads in flight need
     const int j = row_of(P, i >> 1);
     const float2* Cp = (const float2*)(coefp + (long long)j * (D + 2) * NW);
+    // all inputs first, so that their loads are in flight together
+    double vd[D + 3];
+    float2 in[NW];
+#pragma unroll
+    for (int f = 0; f < D + 2; ++f) vd[f] = v[(long long)f * nreal + i];
+    vd[D + 2] = visc ? ((const double*)P.scratch)[(long long)P.s_Tw * nreal + i] : 0.0;
+    auto slot = [&](int s) { return S[(long long)s * nreal + i]; };
+    const float2 zero = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int ax = 0; ax < D; ++ax) {
+#pragma unroll
+      for (int f = 0; f < D + 2; ++f) in[o1 + ax * (D + 3) + f] = slot(P.s_d1[ax][f]);
+      in[o1 + ax * (D + 3) + D + 2] = visc ? slot(P.s_d1[ax][D + 2]) : zero;
+#pragma unroll
+      for (int g = 0; g < D + 1; ++g) in[o2 + ax * (D + 1) + g] = visc ? slot(P.s_d2[ax][g]) : zero;
+#pragma unroll
+      for (int c = 0; c < D; ++c) in[om + ax * D + c] = visc && c != ax ? slot(P.s_mix[ax][c]) : zero;
+    }
     ffn acc[D + 2];
-    float hi[EPS ? NW : 1];
 #pragma unroll
     for (int a = 0; a < D + 2; ++a) acc[a] = ffn{0.0f, 0.0f};
-    if (EPS) {
 #pragma unroll
-      for (int q = 0; q < NW; ++q) hi[q] = 0.0f;
-    }
-    auto put = [&](int q, ffn w) {
-      if (EPS) hi[q] = w.hi;
+    for (int q = 0; q < NW; ++q) {
+      if (q < D + 3) {
+        const ffn w = ff2_split(vd[q]);
+        in[q] = make_float2(w.hi, w.lo);
+      }
 #pragma unroll
       for (int a = 0; a < D + 2; ++a)
         if (coef_used<D>(a, q)) {
           const float2 c = __ldg(Cp + a * NW + q);
-          acc[a] = ff2_fma_u(ffn{c.x, c.y}, w, acc[a]);
+          acc[a] = ff2_fma_u(ffn{c.x, c.y}, ffn{in[q].x, in[q].y}, acc[a]);
         }
-    };
-    auto slot = [&](int s) { const float2 w = S[(long long)s * nreal + i]; return ffn{w.x, w.y}; };
-#pragma unroll
-    for (int f = 0; f < D + 2; ++f) put(f, ff2_split(v[(long long)f * nreal + i]));
-#pragma unroll
-    for (int ax = 0; ax < D; ++ax)
-#pragma unroll
-      for (int f = 0; f < D + 2; ++f) put(o1 + ax * (D + 3) + f, slot(P.s_d1[ax][f]));
-    if (visc) {
-      put(D + 2, ff2_split(((const double*)P.scratch)[(long long)P.s_Tw * nreal + i]));
-#pragma unroll
-      for (int ax = 0; ax < D; ++ax) put(o1 + ax * (D + 3) + D + 2, slot(P.s_d1[ax][D + 2]));
-#pragma unroll
-      for (int ax = 0; ax < D; ++ax)
-#pragma unroll
-        for (int g = 0; g < D + 1; ++g) put(o2 + ax * (D + 1) + g, slot(P.s_d2[ax][g]));
-#pragma unroll
-      for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int c = 0; c < D; ++c)
-          if (a != c) put(om + a * D + c, slot(P.s_mix[a][c]));
     }
     double res[D + 2];
 #pragma unroll
@@ -815,7 +814,7 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const ffn*
       const float ey = (float)P.eta_y[j], eyy = (float)P.eta_yy[j];
       pw::WIn<D, float> Wf;
 #pragma unroll
-      for (int q = 0; q < NW; ++q) set_input<D, float>(Wf, q, hi[q]);
+      for (int q = 0; q < NW; ++q) set_input<D, float>(Wf, q, in[q].x);
 #pragma unroll
       for (int ax = 0; ax < D; ++ax) {
         const float s1 = P.sc1[ax], s2 = P.sc2[ax];
@@ -837,7 +836,7 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const ffn*
           if (a == 1 || c == 1) Wf.mix[a][c] *= ey;
       auto Bf = [&](int slot) { return btab_f[(long long)slot * P.nbase + j]; };
       pw::DN3 o[D + 2];
-      pw::rhs_num<D, pw::DN3>(P.phys, Bf, Wf, e, bc_row, fl, o);
+      pw::rhs_num<D, pw::DN3>(P.physf, Bf, Wf, (float)e, bc_row, fl, o);
 #pragma unroll
       for (int a = 0; a < D + 2; ++a) res[a] += f2d_exact(o[a].w2);
     }
@@ -856,10 +855,10 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const ffn*
 }
 
 template <int D, bool EPS>
-__global__ void __launch_bounds__(128, EPS ? (D == 2 ? 4 : 3) : 6)
+__global__ void __launch_bounds__(128, D == 3 ? 3 : 4)
     k_point_fast(const __grid_constant__ PointParams P, const ffn* __restrict__ coefp, const float* __restrict__ btab_f) {
   if (P.gate && *P.gate) return;
-  point_fast_body<D, EPS>(P, coefp, btab_f, blockIdx.x, gridDim.x);
+  point_fast_body<D, EPS>(P, coefp, btab_f, blockIdx.x);
 }
 
 // Fold the y metric and the line passes' scales into the per-row coefficients
@@ -908,38 +907,44 @@ __global__ void k_to_float_tab(const double* in, float* out, long long count) {
     out[i] = (float)in[i];
 }
 
-// T's scaled difference split the same way: FP64 first order + FP32 rest
-__device__ __forceinline__ void temperature_fast_body(const PointParams& P, double2* Tw, unsigned bidx, unsigned nb) {
+// T's scaled difference split the same way: FP64 first order (two operations
+// per real value, with per-row factors) + FP32 rest.  One thread per real value.
+template <bool EPS>
+__device__ __forceinline__ void temperature_fast_body(const PointParams& P, double* Tw, unsigned bidx, unsigned nb) {
   const int D = P.nz > 1 ? 3 : 2;
-  const double e = *P.eps;
-  const float ef = (float)e;
-  const pw::ClosureK C = P.phys.C;
-  for (long long pt = (long long)bidx * blockDim.x + threadIdx.x; pt < P.npts; pt += (long long)nb * blockDim.x) {
-    const int j = row_of(P, pt);
-    const double ip0 = P.btab[pw::bt_extra(D, pw::X_IP) * P.nbase + j];
-    const double T0 = P.btab[pw::bt_val(D, D + 2) * P.nbase + j];
-    const double2 wp = P.v[pt], ws = P.v[(long long)(D + 1) * P.npts + pt];
-    double t[2];
-#pragma unroll
-    for (int part = 0; part < 2; ++part) {
-      const double q = (part ? wp.y : wp.x) * ip0, s = part ? ws.y : ws.x;
-      const double X1 = fma(C.omig, q, s * C.icp);
-      double r = T0 * X1;
-      if (e != 0.0) {
-        const float qf = (float)q;
-        const float X2 = (float)C.omig * qf * pw::log1p_m1_over_f(ef * qf);
-        const float X = (float)X1 + X2;
-        r += (double)((float)T0 * fmaf(X, pw::expm1_m1_over_f(ef * X), X2));
-      }
-      t[part] = r;
+  const float ef = EPS ? (float)*P.eps : 0.0f;
+  const pw::ClosureT<float> C = P.physf.C;
+  const double* v = (const double*)P.v;
+  const long long nreal = 2 * P.npts;
+  for (long long i = (long long)bidx * blockDim.x + threadIdx.x; i < nreal; i += (long long)nb * blockDim.x) {
+    const int j = row_of(P, i >> 1);
+    const double wp = v[i], ws = v[(long long)(D + 1) * nreal + i];
+    double r = fma(__ldg(P.tcoef + j), wp, __ldg(P.tcoef + P.ny + j) * ws);
+    if (EPS && ef != 0.0f) {
+      const float T0 = ff2_split(P.btab[pw::bt_val(D, D + 2) * P.nbase + j]).hi;
+      const float ip0 = ff2_split(P.btab[pw::bt_extra(D, pw::X_IP) * P.nbase + j]).hi;
+      const float q = __fmul_rn(ff2_split(wp).hi, ip0), s = ff2_split(ws).hi;
+      const float X2 = __fmul_rn(__fmul_rn(C.omig, q), pw::log1p_m1_over_f(__fmul_rn(ef, q)));
+      const float X = __fadd_rn(fmaf(C.omig, q, __fmul_rn(s, C.icp)), X2);
+      r += f2d_exact(__fmul_rn(T0, fmaf(X, pw::expm1_m1_over_f(__fmul_rn(ef, X)), X2)));
     }
-    Tw[pt] = make_double2(t[0], t[1]);
+    Tw[i] = r;
   }
 }
 
-__global__ void k_temperature_fast(const PointParams P, double2* Tw) {
+template <bool EPS>
+__global__ void k_temperature_fast(const __grid_constant__ PointParams P, double* Tw) {
   if (P.gate && *P.gate) return;
-  temperature_fast_body(P, Tw, blockIdx.x, gridDim.x);
+  temperature_fast_body<EPS>(P, Tw, blockIdx.x, gridDim.x);
+}
+
+// the per-row factors of T's first-order difference: T0 (1 - 1/gamma) / p0 and T0 / cp
+__global__ void k_tcoef(const double* btab, int D, int ny, pw::ClosureK C, double* out) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < ny; j += gridDim.x * blockDim.x) {
+    const double T0 = btab[(long long)pw::bt_val(D, D + 2) * ny + j];
+    out[j] = T0 * (C.omig * btab[(long long)pw::bt_extra(D, pw::X_IP) * ny + j]);
+    out[ny + j] = T0 * C.icp;
+  }
 }
 
 // base state as complex fields + base temperature (imaginary parts zero)
@@ -1064,7 +1069,7 @@ struct NormItem {
 };
 struct TempItem {
   PointParams P;
-  double2* Tw;
+  double* Tw;
 };
 struct PointItem {
   PointParams P;
@@ -1100,6 +1105,7 @@ __global__ void k_norm2_batch(const NormItem* __restrict__ items, const int* __r
              blockIdx.x - (unsigned)__ldg(start + i), nb);
 }
 
+template <bool EPS>
 __global__ void k_temperature_fast_batch(const TempItem* __restrict__ items, const int* __restrict__ start, int count) {
   __shared__ TempItem sI;
   const int i = batch_item(start, count, blockIdx.x);
@@ -1107,19 +1113,18 @@ __global__ void k_temperature_fast_batch(const TempItem* __restrict__ items, con
   __syncthreads();
   if (sI.P.gate && *sI.P.gate) return;
   const unsigned s0 = (unsigned)__ldg(start + i);
-  temperature_fast_body(sI.P, sI.Tw, blockIdx.x - s0, (unsigned)__ldg(start + i + 1) - s0);
+  temperature_fast_body<EPS>(sI.P, sI.Tw, blockIdx.x - s0, (unsigned)__ldg(start + i + 1) - s0);
 }
 
 template <int D, bool EPS>
-__global__ void __launch_bounds__(128, EPS ? (D == 2 ? 4 : 3) : 6)
+__global__ void __launch_bounds__(128, D == 3 ? 3 : 4)
     k_point_fast_batch(const PointItem* __restrict__ items, const int* __restrict__ start, int count) {
   __shared__ PointItem sI;
   const int i = batch_item(start, count, blockIdx.x);
   copy_to_shared(&sI, items + i, sizeof(PointItem));
   __syncthreads();
   if (sI.P.gate && *sI.P.gate) return;
-  const unsigned s0 = (unsigned)__ldg(start + i);
-  point_fast_body<D, EPS>(sI.P, sI.coefp, sI.btab_f, blockIdx.x - s0, (unsigned)__ldg(start + i + 1) - s0);
+  point_fast_body<D, EPS>(sI.P, sI.coefp, sI.btab_f, blockIdx.x - (unsigned)__ldg(start + i));
 }
 
 // line passes: item = (instance, axis), its blocks as in the single launch
@@ -1137,21 +1142,24 @@ __global__ void __launch_bounds__(pl::kMaxThreads, 2)
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-pw::Phys phys_of(const StabHandle* h) {
-  pw::Phys p;
-  p.gamma = h->gamma;
-  p.R = h->R;
-  p.cp = h->cp;
-  p.Pr = h->Pr;
-  p.S = h->S;
-  p.Re = h->Re;
-  p.bulk = h->bulk;
-  p.C.ig = 1.0 / h->gamma;
-  p.C.omig = 1.0 - 1.0 / h->gamma;
-  p.C.icp = 1.0 / h->cp;
+template <class F>
+static pw::PhysT<F> phys_as(const StabHandle* h) {
+  pw::PhysT<F> p;
+  p.gamma = (F)h->gamma;
+  p.R = (F)h->R;
+  p.S = (F)h->S;
+  p.bulk = (F)h->bulk;
+  p.mu0 = (F)((1.0 + h->S) / h->Re);
+  p.kl = (F)(h->cp / h->Pr);
+  p.gm1 = (F)(h->gamma - 1.0);
+  p.bulk23 = (F)(h->bulk - 2.0 / 3.0);
+  p.C.ig = (F)(1.0 / h->gamma);
+  p.C.omig = (F)(1.0 - 1.0 / h->gamma);
+  p.C.icp = (F)(1.0 / h->cp);
   p.visc = h->visc;
   return p;
 }
+pw::Phys phys_of(const StabHandle* h) { return phys_as<double>(h); }
 
 static void fill_axis_tables(AxisTables& A, std::vector<double>& host) {
   const int n = A.n;
@@ -1380,7 +1388,7 @@ static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, pl::PairPass& 
   const LineCfg cfg = h->line_cfg[axis];
   auto smem_of = [&](int L, int nch) {
     const int RL = 2 * L, RLp = RL % 4 == 0 ? RL + 2 : RL;
-    return (size_t)n * RLp * 8 + ((size_t)2 * RL * nch + 2 * RL + pl::kTab) * 8;
+    return (size_t)n * RLp * 8 + ((size_t)2 * RL * nch + 8 * RL + pl::kTab) * 8;
   };
   const long long want = 152LL * 1024;  // threads that fill the SMs
   int C = cfg.C;
@@ -1406,15 +1414,18 @@ static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, pl::PairPass& 
   P.nch = nch;
   P.q = n / nch;
   P.rem = n % nch;
-  P.divjobs = make_fastdiv((unsigned)njobs);
+  const long long nblk = (P.nlines + L - 1) / L;
+  if (nblk * njobs > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
+  P.nblk = (int)nblk;
+  P.divblk = make_fastdiv((unsigned)nblk);
   P.divRL = make_fastdiv((unsigned)P.RL);
   P.divL = make_fastdiv((unsigned)L);
   P.divn = make_fastdiv((unsigned)n);
   P.divnx = make_fastdiv((unsigned)h->nx);
   threads = ((P.RL * nch + 31) / 32) * 32;
   smem = smem_of(L, nch);
-  blocks = (P.nlines + L - 1) / L * njobs;
-  return blocks > 0x7FFFFFFFLL ? cudaErrorInvalidValue : cudaSuccess;
+  blocks = nblk * njobs;
+  return cudaSuccess;
 }
 
 // The pass of axis ax for the fields src (as axis_jobs): one job per derivative.
@@ -1808,6 +1819,8 @@ static PointParams point_params(StabHandle* h, const double2* v) {
   P.bcflags = h->d_bcflags;
   P.eps = h->d_eps;
   P.phys = phys_of(h);
+  P.physf = phys_as<float>(h);
+  P.tcoef = h->d_tcoef;
   for (int a = 0; a < h->dim; ++a) {
     P.sc1[a] = (float)h->ax[a].pscale[0];
     P.sc2[a] = (float)h->ax[a].pscale[1];
@@ -1942,6 +1955,8 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
     const int nw = pw::nw_inputs(D);
     if ((err = dalloc(h, &h->d_coef, (size_t)h->ny * (D + 2) * nw * sizeof(double))) != cudaSuccess) return err;
     PointParams PP = point_params(h, nullptr);
+    if ((err = dalloc(h, &h->d_tcoef, (size_t)2 * h->ny * sizeof(double))) != cudaSuccess) return err;
+    k_tcoef<<<(h->ny + 127) / 128, 128, 0, h->stream>>>(h->d_btab, D, h->ny, phys_of(h).C, h->d_tcoef);
     if (D == 2) k_coeffs<2><<<h->ny, 32, 0, h->stream>>>(PP, h->d_coef);
     else k_coeffs<3><<<h->ny, 64, 0, h->stream>>>(PP, h->d_coef);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
@@ -1999,7 +2014,9 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   const bool fast = h->homog && h->d_coef && !h->force_dn_path;
   if (h->visc) {
     const int ts = phase_begin(h, STAB_PHASE_TEMPERATURE);
-    if (fast) k_temperature_fast<<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P, Tw);
+    const int g = grid_for(2 * h->npts, thr);
+    if (fast && eps_mode == 2) k_temperature_fast<false><<<g, thr, 0, h->stream>>>(P, (double*)Tw);
+    else if (fast) k_temperature_fast<true><<<g, thr, 0, h->stream>>>(P, (double*)Tw);
     else k_temperature<<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P, Tw);
     phase_end(h, ts);
   }
@@ -2010,7 +2027,7 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   if ((err = run_derivatives(h, src, h->stencil_ff, fast)) != cudaSuccess) return err;
   const int tp = phase_begin(h, STAB_PHASE_POINTWISE);
   if (fast) {
-    const int g = grid_for(2 * h->npts, thr);
+    const unsigned g = (unsigned)((2 * h->npts + thr - 1) / thr);
     if (D == 2 && eps_mode == 2) k_point_fast<2, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
     else if (D == 2) k_point_fast<2, true><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
     else if (eps_mode == 2) k_point_fast<3, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
@@ -2105,8 +2122,8 @@ cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
   std::vector<NormItem> norms;
   std::vector<int> norm_blocks;
   // 2. temperature differences (viscous instances)
-  std::vector<TempItem> temps;
-  std::vector<int> temp_blocks;
+  std::vector<TempItem> temps[2];
+  std::vector<int> temp_blocks[2];
   // 4. pointwise assembly, per dimension and J v form (tangent, epsilon-quotient)
   std::vector<PointItem> points[2][2];
   std::vector<int> point_blocks[2][2];
@@ -2136,17 +2153,16 @@ cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
     P.gate = gate;
     P.out = out[i];
     P.shift = shifts ? shifts[i] : make_double2(0.0, 0.0);
-    double2* Tw = h->d_scratch + (long long)h->slots.Tw * h->npts;
-    if (h->visc) {
-      temps.push_back(TempItem{P, Tw});
-      temp_blocks.push_back(grid_for(h->npts, 128));
-    }
     const int form = h->opts.eps_mode != 2;
+    if (h->visc) {
+      temps[form].push_back(TempItem{P, (double*)(h->d_scratch + (long long)h->slots.Tw * h->npts)});
+      temp_blocks[form].push_back(grid_for(2 * h->npts, 128));
+    }
     points[h->dim - 2][form].push_back(PointItem{P, h->d_coef_p, h->d_btab_f});
-    point_blocks[h->dim - 2][form].push_back(grid_for(2 * h->npts, 128));
+    point_blocks[h->dim - 2][form].push_back((int)((2 * h->npts + 127) / 128));
   }
   plan.norm = im.section(norms, norm_blocks, 256, 0);
-  plan.temp = im.section(temps, temp_blocks, 128, 0);
+  for (int f = 0; f < 2; ++f) plan.temp[f] = im.section(temps[f], temp_blocks[f], 128, 0);
   // 3. line passes y, z, x: one section per axis
   static const int order[3] = {1, 2, 0};
   for (int q = 0; q < 3; ++q) {
@@ -2188,9 +2204,11 @@ cudaError_t jv_batch_launch(const JvBatchPlan& plan, const unsigned char* d, cud
   if (plan.norm.count)
     k_norm2_batch<<<plan.norm.blocks, 256, 0, st>>>((const NormItem*)items_of(plan.norm), start_of(plan.norm),
                                                     plan.norm.count);
-  if (plan.temp.count)
-    k_temperature_fast_batch<<<plan.temp.blocks, 128, 0, st>>>((const TempItem*)items_of(plan.temp),
-                                                               start_of(plan.temp), plan.temp.count);
+  auto temperature = [&](const BatchSection& s, auto kernel) {
+    if (s.count) kernel<<<s.blocks, 128, 0, st>>>((const TempItem*)items_of(s), start_of(s), s.count);
+  };
+  temperature(plan.temp[0], k_temperature_fast_batch<false>);
+  temperature(plan.temp[1], k_temperature_fast_batch<true>);
   for (int q = 0; q < 3; ++q) {
     const BatchSection& s = plan.line[q];
     if (s.count)

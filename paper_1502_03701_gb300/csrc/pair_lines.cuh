@@ -48,10 +48,11 @@ struct PairPass {
   long long nlines;  // complex lines
   long long stride;  // points between consecutive points of a line
   int njobs, axis, n, nx, ny;
+  int nblk;          // line blocks
   int L, RL, RLp;    // complex lines per CTA, real lines (2 L), shared-memory pitch in reals
   int nch, q, rem;   // chunks per line: the first rem have q + 1 points, the others q
-  int bounded, pad;
-  FastDiv divjobs, divRL, divL, divn, divnx;
+  int bounded;
+  FastDiv divblk, divRL, divL, divn, divnx;
 };
 static_assert(sizeof(PairPass) % 8 == 0, "items are copied to shared memory in 8-byte words");
 
@@ -103,30 +104,30 @@ __device__ __forceinline__ void solve_chunks(const PairPass& P, double* F, float
   auto neg = [](ffn a) { return ffn{-a.hi, -a.lo}; };
   // the neighbours' points, and the wall rows' right-hand sides, before any point is overwritten
   double fm2 = 0, fm1 = 0, fp0 = 0, fp1 = 0;
-  ffn uL{0, 0}, vL{0, 0}, uR{0, 0}, vR{0, 0};
-  const bool left = bounded && act && c == 0, right = bounded && act && c == nch - 1;
+  // side 0: rows 0 and 1 in the first chunk; side 1: rows n - 1 and n - 2 in the last one
+  auto wall = [&](int side) { return bounded && act && c == (side ? nch - 1 : 0); };
   if (act) {
     fm2 = at(t0 - 2);
     fm1 = at(t0 - 1);
     fp0 = at(t1);
     fp1 = at(t1 + 1);
-    if (left) {
-      if (KIND == 0) { uL = dif(at(2), at(0)); vL = dif(at(1), at(0)); }
-      else {
-        const ffn g0 = dif(at(1), at(0)), g1 = dif(at(2), at(1)), g2 = dif(at(3), at(2));
-        uL = ff2_add(g1, neg(g0));
-        vL = ff2_add(g2, neg(g1));
-      }
-    }
-    if (right) {
-      if (KIND == 0) { uR = dif(at(n - 1), at(n - 3)); vR = dif(at(n - 1), at(n - 2)); }
-      else {
-        const ffn g0 = dif(at(n - 1), at(n - 2)), g1 = dif(at(n - 2), at(n - 3)), g2 = dif(at(n - 3), at(n - 4));
-        uR = ff2_add(g0, neg(g1));
-        vR = ff2_add(g1, neg(g2));
-      }
-    }
   }
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side)
+    if (wall(side)) {
+      ffn u, v;
+      if (KIND == 0) {
+        const int i = side ? n - 2 : 1, k = side ? n - 2 : 0;
+        u = dif(at(i + 1), at(i - 1));
+        v = dif(at(k + 1), at(k));
+      } else {
+        auto second = [&](int i) { return ff2_add(dif(at(i + 1), at(i)), neg(dif(at(i), at(i - 1)))); };
+        u = second(side ? n - 2 : 1);
+        v = second(side ? n - 3 : 2);
+      }
+      W[(2 + side) * RL + r] = f2(u);
+      W[(4 + side) * RL + r] = f2(v);
+    }
   __syncthreads();
   // forward sweep from zero, in place: g_t = w_t + r g_{t-1}, w_t = d_t + rho (d_{t-1} + d_{t+1}),
   // d_t = f_{t+1} - f_{t-1} (first) or f_{t+1} - 2 f_t + f_{t-1} (second derivative)
@@ -164,10 +165,8 @@ __device__ __forceinline__ void solve_chunks(const PairPass& P, double* F, float
       fa = fb;
       fb = fc;
     };
-#pragma unroll 4
-    for (int k = 0; k < len - 2; ++k) step(k, col[(k + 2) * RLp]);
-    step(len - 2, fp0);
-    step(len - 1, fp1);
+#pragma unroll 2
+    for (int k = 0; k < len; ++k) step(k, k + 2 < len ? col[(k + 2) * RLp] : k + 2 == len ? fp0 : fp1);
     E[c * RL + r] = f2(g);
   }
   __syncthreads();
@@ -213,45 +212,41 @@ __device__ __forceinline__ void solve_chunks(const PairPass& P, double* F, float
     A = ff2_fma(K.kap, G, ffn{0, 0});
     B = ff2_fma(neg(pw(len + 1)), A, xn);
   }
-  ffn pL{0, 0}, pR{0, 0};
   if (bounded) {
-    auto value = [&](int k) { return ff2_fma(pw(len - k), B, ff2_fma(pw(k + 1), A, got(k))); };
-    auto wall = [&](ffn u, ffn v, ffn p1, ffn p2) {
-      return ff2_fma(K.cl[3], p2, ff2_fma(K.cl[2], p1, ff2_fma(K.cl[1], v, ff2_fma(K.cl[0], u, ffn{0, 0}))));
-    };
-    if (left) {
-      pL = value(1);
-      W[r] = f2(wall(uL, vL, pL, value(2)));
-    }
-    if (right) {
-      pR = value(len - 2);
-      W[RL + r] = f2(wall(uR, vR, pR, value(len - 3)));
-    }
+    auto load = [](const float2* p) { const float2 x = *p; return ffn{x.x, x.y}; };
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side)
+      if (wall(side)) {
+        auto value = [&](int k) { return ff2_fma(pw(len - k), B, ff2_fma(pw(k + 1), A, got(k))); };
+        const ffn p1 = value(side ? len - 2 : 1);
+        ffn s = ff2_fma(K.cl[3], value(side ? len - 3 : 2), ffn{0, 0});
+        s = ff2_fma(K.cl[2], p1, s);
+        s = ff2_fma(K.cl[1], load(W + (4 + side) * RL + r), s);
+        W[side * RL + r] = f2(ff2_fma(K.cl[0], load(W + (2 + side) * RL + r), s));
+        W[(6 + side) * RL + r] = f2(p1);
+      }
     __syncthreads();
     if (act) {
-      const float2 l2 = W[r], r2 = W[RL + r];
-      const ffn wl{l2.x, l2.y}, wr{r2.x, r2.y};
+      const ffn wl = load(W + r), wr = load(W + RL + r);
       const ffn Aw = ff2_fma(K.wb, wr, ff2_fma(K.wa, wl, ffn{0, 0}));
       const ffn Bw = ff2_fma(K.wb, wl, ff2_fma(K.wa, wr, ffn{0, 0}));
       if (t0 - 2 < K.reach) A = ff2_fma(pw(t0 - 2), Aw, A);
       if (n - t1 - 2 < K.reach) B = ff2_fma(pw(n - t1 - 2), Bw, B);
-      const ffn far = n - 3 < K.reach ? pw(n - 3) : ffn{0, 0};
-      // the wall rows: x_0 = R_0 - a_0 x_1
-      if (left) {
-        const ffn x1 = ff2_fma(far, Bw, ff2_add(pL, Aw));
-        pL = ff2_fma(K.c0[2], x1, ff2_fma(K.c0[1], vL, ff2_fma(K.c0[0], uL, ffn{0, 0})));
-      }
-      if (right) {
-        const ffn x1 = ff2_fma(far, Aw, ff2_add(pR, Bw));
-        pR = ff2_fma(K.c0[2], x1, ff2_fma(K.c0[1], vR, ff2_fma(K.c0[0], uR, ffn{0, 0})));
-      }
+#pragma unroll 1
+      for (int side = 0; side < 2; ++side)
+        if (wall(side)) {  // the wall rows: x_0 = R_0 - a_0 x_1
+          ffn x1 = ff2_add(load(W + (6 + side) * RL + r), side ? Bw : Aw);
+          if (n - 3 < K.reach) x1 = ff2_fma(pw(n - 3), side ? Aw : Bw, x1);
+          ffn x0 = ff2_fma(K.c0[1], load(W + (4 + side) * RL + r), ff2_fma(K.c0[2], x1, ffn{0, 0}));
+          W[(6 + side) * RL + r] = f2(ff2_fma(K.c0[0], load(W + (2 + side) * RL + r), x0));
+        }
     }
   }
   // x_t = local + A r^(k+1) + B r^(len-k); past `near` points a term only reaches the low part
   if (act) {
     const int near = K.near;
     const long long gs = 2 * P.stride;
-#pragma unroll 2
+#pragma unroll 1
     for (int k = 0; k < len; ++k) {
       ffn y = got(k);
       const ffn pa = pw(k + 1), pb = pw(len - k);
@@ -260,27 +255,28 @@ __device__ __forceinline__ void solve_chunks(const PairPass& P, double* F, float
       if (len - k < near) y = ff2_fma_u(pb, B, y);
       else y.lo = __fmaf_rn(pb.hi, B.hi, y.lo);
       y = ff2_norm(y);
-      if (left && k == 0) y = pL;
-      if (right && k == len - 1) y = pR;
       if (gout) gout[k * gs] = f2(y);
       else pairs(k) = f2(y);
     }
+    if (wall(0)) gout[0] = W[6 * RL + r];
+    if (wall(1)) gout[(len - 1) * gs] = W[7 * RL + r];
   }
 }
 
-// CTA bid: job bid % njobs of line block bid / njobs (the jobs of one line
-// block run side by side, so a field's second read hits the L2 cache).
+// CTA bid: line block bid % nblk of job bid / nblk.  CTAs that run at the same
+// time then mostly run the same derivative kind (the instruction cache holds one
+// variant), and a field's second read, by the next job, still hits the L2 cache.
 __device__ __forceinline__ void pair_pass_body(const PairPass& P, unsigned bid) {
   if (P.gate && *P.gate) return;
   extern __shared__ __align__(16) double pl_smem[];
-  const unsigned lb = fdiv(bid, P.divjobs);
-  const PairJob J = P.job[bid - lb * P.njobs];
+  const unsigned jb = fdiv(bid, P.divblk), lb = bid - jb * P.nblk;
+  const PairJob J = P.job[jb];
   const int n = P.n, L = P.L, RL = P.RL, RLp = P.RLp, tid = threadIdx.x;
   double* F = pl_smem;
   float2* E = (float2*)(F + (size_t)n * RLp);
   float2* X = E + RL * P.nch;
   float2* W = X + RL * P.nch;
-  float2* tab = W + 2 * RL;
+  float2* tab = W + 8 * RL;
   const long long l0 = (long long)lb * L;
   // stage the lines: [t][line][re, im]
   for (int idx = tid; idx < n * L; idx += blockDim.x) {
@@ -304,13 +300,9 @@ __device__ __forceinline__ void pair_pass_body(const PairPass& P, unsigned bid) 
     const int t0 = c * P.q + min(c, P.rem);
     gout = J.out + 2 * (line_start(P, l0 + (r >> 1)) + (long long)t0 * P.stride) + (r & 1);
   }
-  if (J.pair_in) {
-    if (J.kind == 0) solve_chunks<0, true>(P, F, E, X, W, tab, act, c, r, gout);
-    else solve_chunks<1, true>(P, F, E, X, W, tab, act, c, r, gout);
-  } else {
-    if (J.kind == 0) solve_chunks<0, false>(P, F, E, X, W, tab, act, c, r, gout);
-    else solve_chunks<1, false>(P, F, E, X, W, tab, act, c, r, gout);
-  }
+  if (J.pair_in) solve_chunks<0, true>(P, F, E, X, W, tab, act, c, r, gout);  // mixed derivatives: first only
+  else if (J.kind == 0) solve_chunks<0, false>(P, F, E, X, W, tab, act, c, r, gout);
+  else solve_chunks<1, false>(P, F, E, X, W, tab, act, c, r, gout);
   if (P.axis != 0) return;
   __syncthreads();
   for (int idx = tid; idx < n * L; idx += blockDim.x) {

@@ -84,8 +84,7 @@ __device__ __forceinline__ DN3 operator*(double c, DN3 x) {
   return dn3(fmul(cf, x.a), fmul(cf, x.w1), fmul(cf, x.w2));
 }
 __device__ __forceinline__ DN3 add(DN3 x, double c) { return dn3(fadd(x.a, (float)c), x.w1, x.w2); }
-__device__ __forceinline__ DN3 mul(DN3 x, DN3 y, double ed) {
-  const float e = (float)ed;
+__device__ __forceinline__ DN3 mul(DN3 x, DN3 y, float e) {
   float w1 = fmaf(x.a, y.w1, fmul(x.w1, y.a));
   float w2 = fmaf(x.a, y.w2, fmaf(x.w2, y.a, fmul(fmul(e, fadd(x.w1, x.w2)), fadd(y.w1, y.w2))));
   return dn3(fmul(x.a, y.a), w1, w2);
@@ -95,10 +94,10 @@ __device__ __forceinline__ float xinv1pf(float x) {
   if (fabsf(x) < 1e-3f) return fmul(x, fmaf(x, fmaf(x, fsub(1.0f, x), -1.0f), 1.0f));
   return x / fadd(1.0f, x);
 }
-__device__ __forceinline__ DN3 rcp_t(DN3 x, double inva_d, double ed) {
-  const float inva = (float)inva_d, i2 = fmul(inva, inva);
+__device__ __forceinline__ DN3 rcp_t(DN3 x, float inva, float e) {
+  const float i2 = fmul(inva, inva);
   const float w = fadd(x.w1, x.w2);
-  const float X = fmul(fmul((float)ed, w), inva);
+  const float X = fmul(fmul(e, w), inva);
   return dn3(inva, fmul(-x.w1, i2), fmaf(-x.w2, i2, fmul(fmul(w, i2), xinv1pf(X))));
 }
 // (sqrt(1+x) - 1)/x - 1/2 = x (-1/8 + x/16 - 5x^2/128 + ...)
@@ -106,10 +105,10 @@ __device__ __forceinline__ float sqrt_corr(float x) {
   if (fabsf(x) < 1e-3f) return fmul(x, fmaf(x, fmaf(x, -5.0f / 128.0f, 1.0f / 16.0f), -1.0f / 8.0f));
   return fsub(fsub(sqrtf(fadd(1.0f, x)), 1.0f) / x, 0.5f);
 }
-__device__ __forceinline__ DN3 sqrt_t(DN3 x, double sqa_d, double inva_d, double ed) {
-  const float sqa = (float)sqa_d, inva = (float)inva_d, k = fmul(sqa, inva);
+__device__ __forceinline__ DN3 sqrt_t(DN3 x, float sqa, float inva, float e) {
+  const float k = fmul(sqa, inva);
   const float w = fadd(x.w1, x.w2);
-  const float X = fmul(fmul((float)ed, w), inva);
+  const float X = fmul(fmul(e, w), inva);
   return dn3(sqa, fmul(fmul(0.5f, k), x.w1), fmaf(fmul(0.5f, k), x.w2, fmul(fmul(w, k), sqrt_corr(X))));
 }
 
@@ -117,9 +116,11 @@ __device__ __forceinline__ DN3 sqrt_t(DN3 x, double sqa_d, double inva_d, double
 // Closure: rho(p, s) = (p/p_ref)^{1/gamma} e^{-s/c_p}, T = (p/p_ref)^{(gamma-1)/gamma} e^{s/c_p}
 //   rho(q0 + e w)/rho0 = exp(x_rho),  x_rho = (1/gamma) ln(1 + e wp/p0) - e ws/c_p
 // ---------------------------------------------------------------------------
-struct ClosureK {
-  double ig, omig, icp;  // 1/gamma, 1 - 1/gamma, 1/c_p
+template <class R>
+struct ClosureT {
+  R ig, omig, icp;  // 1/gamma, 1 - 1/gamma, 1/c_p
 };
+typedef ClosureT<double> ClosureK;
 __device__ __forceinline__ double closure_lq(double wp, double ip0, double e) {
   double q = wp * ip0;
   return q * log1p_over(e * q);
@@ -147,11 +148,10 @@ __device__ __forceinline__ float log1p_m1_over_f(float z) {
 __device__ __forceinline__ DN make_rho(const ClosureK& C, double rho0, double ip0, DN p, DN s, double e) {
   return dn(rho0, closure_rho_w(C, rho0, closure_lq(p.w, ip0, e), s.w, e));
 }
-__device__ __forceinline__ DN3 make_rho(const ClosureK& C, double rho0, double ip0, DN3 p, DN3 s, double ed) {
-  const float e = (float)ed, r0 = (float)rho0;
-  const float q = fmul(p.w1, (float)ip0);
-  const float X1 = fmaf((float)C.ig, q, fmul(-s.w1, (float)C.icp));
-  const float X2 = fmul(fmul((float)C.ig, q), log1p_m1_over_f(fmul(e, q)));
+__device__ __forceinline__ DN3 make_rho(const ClosureT<float>& C, float r0, float ip0, DN3 p, DN3 s, float e) {
+  const float q = fmul(p.w1, ip0);
+  const float X1 = fmaf(C.ig, q, fmul(-s.w1, C.icp));
+  const float X2 = fmul(fmul(C.ig, q), log1p_m1_over_f(fmul(e, q)));
   const float X = fadd(X1, X2);
   return dn3(r0, fmul(r0, X1), fmul(r0, fmaf(X, expm1_m1_over_f(fmul(e, X)), X2)));
 }
@@ -171,11 +171,20 @@ __host__ __device__ __forceinline__ int bt_extra(int D, int x) {
 }
 __host__ __device__ __forceinline__ int bt_count(int D) { return bt_extra(D, X_COUNT); }
 
-struct Phys {
-  double gamma, R, cp, Pr, S, Re, bulk;
-  ClosureK C;
+// Flow constants, in the precision of the evaluation (the FP32 remainder takes
+// FP32 copies: conversions and divisions by FP64 constants in every thread
+// kept the FP64 pipe 72 % busy in the pointwise kernel).
+template <class F>
+struct PhysT {
+  F gamma, R, S, bulk;
+  F mu0;     // (1 + S) / Re
+  F kl;      // cp / Pr
+  F gm1;     // gamma - 1
+  F bulk23;  // bulk - 2/3
+  ClosureT<F> C;
   int visc;
 };
+typedef PhysT<double> Phys;
 
 // Scaled perturbation at one point for one real direction.  Fields f:
 // 0 = p, 1..D = u_i, D+1 = s, D+2 = T; d2 fields g: 0..D-1 = u_i, D = T.
@@ -210,8 +219,9 @@ struct NumOps<DN3> {
 // non-reflective flags of a y-boundary row (bit0 drop X+, bit1 drop X-,
 // bit2 drop y-convection), bc_row: the point lies on one.
 template <int D, class Num, class BaseFn>
-__device__ __forceinline__ void rhs_num(const Phys& P, const BaseFn& B, const WIn<D, typename NumOps<Num>::V>& W,
-                                        double e, bool bc_row, unsigned bcfl, Num* out) {
+__device__ __forceinline__ void rhs_num(const PhysT<typename NumOps<Num>::V>& P, const BaseFn& B,
+                                        const WIn<D, typename NumOps<Num>::V>& W, typename NumOps<Num>::V e, bool bc_row,
+                                        unsigned bcfl, Num* out) {
   typedef NumOps<Num> O;
   const int Y = 1;
   Num p = O::make(B(bt_val(D, 0)), W.v[0]);
@@ -248,16 +258,15 @@ __device__ __forceinline__ void rhs_num(const Phys& P, const BaseFn& B, const WI
     Num sqT = sqrt_t(T, B(bt_extra(D, X_SQT)), iT0, e);
     const auto iTS0 = B(bt_extra(D, X_ITS));
     Num rTS = rcp_t(add(T, P.S), iTS0, e);
-    Num mu = ((1.0 + P.S) / P.Re) * mul(mul(T, sqT, e), rTS, e);
+    Num mu = P.mu0 * mul(mul(T, sqT, e), rTS, e);
     Num dmu = mul(mu, 1.5 * rcp_t(T, iT0, e) - rTS, e);
-    const double kl = P.cp / P.Pr;
     Num lapT = O::zero(), gT2 = O::zero();
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       lapT = lapT + O::make(B(bt_d2(D, a, D)), W.d2[a][D]);
       gT2 = gT2 + mul(dT[a], dT[a], e);
     }
-    Num heat = kl * (mul(mu, lapT, e) + mul(dmu, gT2, e));
+    Num heat = P.kl * (mul(mu, lapT, e) + mul(dmu, gT2, e));
     Num SS = O::zero();
 #pragma unroll
     for (int a = 0; a < D; ++a)
@@ -280,7 +289,7 @@ __device__ __forceinline__ void rhs_num(const Phys& P, const BaseFn& B, const WI
         cross = cross + mul(dT[c], du[a][c] + du[c][a], e);
       }
       vis[a] = mul(mu, lap + (1.0 / 3.0) * ddiv, e) + P.bulk * mul(mu, ddiv, e) + mul(dmu, cross, e) +
-               mul(mul((P.bulk - 2.0 / 3.0) * dmu, dT[a], e), div, e);
+               mul(mul(P.bulk23 * dmu, dT[a], e), div, e);
     }
   }
 
@@ -306,7 +315,7 @@ __device__ __forceinline__ void rhs_num(const Phys& P, const BaseFn& B, const WI
 #pragma unroll
   for (int a = 0; a < D; ++a)
     if (a != Y) pt = pt - (mul(u[a], dp[a], e) + P.gamma * mul(p, du[a][a], e));
-  pt = pt + (P.gamma - 1.0) * src;
+  pt = pt + P.gm1 * src;
   out[0] = pt;
 #pragma unroll
   for (int c = 0; c < D; ++c) {

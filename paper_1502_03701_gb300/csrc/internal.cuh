@@ -166,7 +166,7 @@ struct StabHandle {
   double* d_btab_low = nullptr;  // base tables with the reduced operator's derivatives
   double* d_coef;        // per-row tangent coefficients of the pointwise map (y-only base)
   double* d_coef_f;      // the same with the y metric folded in (inputs: eta-derivatives)
-  ffn* d_coef_p;         // d_coef_f as FP32 pairs (hi, lo), read by the pointwise kernel
+  float4* d_coef_p;      // d_coef_f as FP32 pairs (hi, lo), read by the pointwise kernel
   double* d_tcoef = nullptr;  // per-row factors of T's first-order difference (y-only base)
   float* d_btab_f;       // FP32 copy of the base tables (for the O(eps) remainder)
   bool force_dn_path;    // use the full FP64 difference-number pointwise kernel
@@ -314,7 +314,7 @@ cudaError_t batch_stage(stab_jv_batch_s* B, const BatchImage& im);
 // copied to the device once) and the launches that read them.  gates[i]
 // (nullable) skips instance i's work while *gates[i] != 0.
 struct JvBatchPlan {
-  BatchSection norm, temp[2], line[3], point[2][2];
+  BatchSection norm, temp[2], line[3][2], point[2][2];
   std::vector<double*> zero_eps;  // epsilon slots of the exact-tangent instances
 };
 cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* const* v, double2* const* out,

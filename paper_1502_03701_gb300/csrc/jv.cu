@@ -750,113 +750,182 @@ __host__ __device__ constexpr bool coef_used(int a, int q) {
   return q / D == a - 1 && q / D != q % D;
 }
 
+template <int D>
+__host__ __device__ constexpr int coefs_used() {
+  int c = 0;
+  for (int q = 0; q < pw::nw_inputs(D); ++q)
+    for (int a = 0; a < D + 2; ++a) c += coef_used<D>(a, q);
+  return c;
+}
+static_assert(coefs_used<2>() == 51 && coefs_used<3>() == 85, "products per point of the pointwise map");
+
 // Inputs: line-pass outputs (pairs, in units of the passes' scales); the
 // coefficients have the y metric and those scales folded in (k_coeffs_fold)
-// and are stored as FP32 pairs.  One thread per real value: it streams over
-// the inputs, adds each to the rows that it reaches (85 of the 225 products in
-// 3-D, 40 of 100 in 2-D) by exact FP32 two-products and two-sum accumulation, and
-// (EPS) evaluates the O(eps) remainder in FP32 from the inputs' high parts and
-// FP32 base tables: no FP64 products.
-template <int D, bool EPS>
-__device__ __forceinline__ void point_fast_body(const PointParams& P, const ffn* __restrict__ coefp,
-                                                const float* __restrict__ btab_f, unsigned bidx) {
-  constexpr int NW = pw::nw_inputs(D);
-  constexpr int o1 = D + 3, o2 = o1 + D * (D + 3), om = o2 + D * (D + 1);
-  const double e = EPS ? *P.eps : 0.0;
-  const bool visc = P.phys.visc;
-  const double* v = (const double*)P.v;
-  const float2* S = (const float2*)P.scratch;
-  const long long nreal = 2 * P.npts;
-  const long long i = (long long)bidx * blockDim.x + threadIdx.x;  // no loop: its invariant addresses would take
-  if (i < nreal) {                                                 // the registers that the loads in flight need
-    const int j = row_of(P, i >> 1);
-    const float2* Cp = (const float2*)(coefp + (long long)j * (D + 2) * NW);
-    // all inputs first, so that their loads are in flight together
-    double vd[D + 3];
-    float2 in[NW];
-#pragma unroll
-    for (int f = 0; f < D + 2; ++f) vd[f] = v[(long long)f * nreal + i];
-    vd[D + 2] = visc ? ((const double*)P.scratch)[(long long)P.s_Tw * nreal + i] : 0.0;
-    auto slot = [&](int s) { return S[(long long)s * nreal + i]; };
-    const float2 zero = make_float2(0.0f, 0.0f);
-#pragma unroll
+// and are stored as FP32 pairs, both halves duplicated for the packed
+// instructions, the used ones of a row one after the other (k_pack_coefs).
+// One thread per point streams over the inputs, both components side by side,
+// and adds each to the rows that it reaches (85 of the 225 products in 3-D, 51
+// of 100 in 2-D) by exact FP32 two-products and two-sum accumulation; EPS adds
+// the O(eps) remainder, evaluated in FP32 from the inputs' high parts.  No
+// FP64 instruction is issued: the FP64 pipe's rate (1/64 of FP32) made the
+// conversions and the shift the kernel's bound before.
+// The remainder on a non-reflective boundary row (general form, one component
+// at a time); out of line, so that the rows inside do not carry its registers.
+template <int D>
+__device__ __noinline__ void wall_remainder(const pw::PhysT<float>& phys, const float* __restrict__ btab_f, long long nbase,
+                                            int j, unsigned fl, const pw::WIn<D, float2>& W, float ef, float2* w2) {
+  auto Bf = [&](int s) { return btab_f[(long long)s * nbase + j]; };
+#pragma unroll 1
+  for (int part = 0; part < 2; ++part) {
+    auto pick = [&](float2 t) { return part ? t.y : t.x; };
+    pw::WIn<D, float> Wf;
+    for (int f = 0; f < D + 3; ++f) Wf.v[f] = pick(W.v[f]);
     for (int ax = 0; ax < D; ++ax) {
-#pragma unroll
-      for (int f = 0; f < D + 2; ++f) in[o1 + ax * (D + 3) + f] = slot(P.s_d1[ax][f]);
-      in[o1 + ax * (D + 3) + D + 2] = visc ? slot(P.s_d1[ax][D + 2]) : zero;
-#pragma unroll
-      for (int g = 0; g < D + 1; ++g) in[o2 + ax * (D + 1) + g] = visc ? slot(P.s_d2[ax][g]) : zero;
-#pragma unroll
-      for (int c = 0; c < D; ++c) in[om + ax * D + c] = visc && c != ax ? slot(P.s_mix[ax][c]) : zero;
+      for (int f = 0; f < D + 3; ++f) Wf.d1[ax][f] = pick(W.d1[ax][f]);
+      for (int g = 0; g < D + 1; ++g) Wf.d2[ax][g] = pick(W.d2[ax][g]);
+      for (int c = 0; c < D; ++c) Wf.mix[ax][c] = pick(W.mix[ax][c]);
     }
-    ffn acc[D + 2];
-#pragma unroll
-    for (int a = 0; a < D + 2; ++a) acc[a] = ffn{0.0f, 0.0f};
-#pragma unroll
-    for (int q = 0; q < NW; ++q) {
-      if (q < D + 3) {
-        const ffn w = ff2_split(vd[q]);
-        in[q] = make_float2(w.hi, w.lo);
-      }
-#pragma unroll
-      for (int a = 0; a < D + 2; ++a)
-        if (coef_used<D>(a, q)) {
-          const float2 c = __ldg(Cp + a * NW + q);
-          acc[a] = ff2_fma_u(ffn{c.x, c.y}, ffn{in[q].x, in[q].y}, acc[a]);
-        }
-    }
-    double res[D + 2];
-#pragma unroll
-    for (int a = 0; a < D + 2; ++a) res[a] = ff2_to_d(acc[a]);
-    if (EPS && e != 0.0) {  // O(eps) remainder of the quotient, FP32, physical (metric-applied) inputs
-      const bool bc_row = (j == 0 || j == P.ny - 1);
-      const unsigned fl = bc_row ? P.bcflags[(j == P.ny - 1 ? (long long)P.nx * P.nz : 0)] : 0u;
-      const float ey = (float)P.eta_y[j], eyy = (float)P.eta_yy[j];
-      pw::WIn<D, float> Wf;
-#pragma unroll
-      for (int q = 0; q < NW; ++q) set_input<D, float>(Wf, q, in[q].x);
-#pragma unroll
-      for (int ax = 0; ax < D; ++ax) {
-        const float s1 = P.sc1[ax], s2 = P.sc2[ax];
-#pragma unroll
-        for (int f = 0; f < D + 3; ++f) Wf.d1[ax][f] *= s1;
-#pragma unroll
-        for (int g = 0; g < D + 1; ++g) Wf.d2[ax][g] *= s2;
-#pragma unroll
-        for (int c = 0; c < D; ++c) Wf.mix[ax][c] *= s1 * P.sc1[c];
-      }
-#pragma unroll
-      for (int g = 0; g < D + 1; ++g) Wf.d2[1][g] = fmaf(Wf.d2[1][g], ey * ey, Wf.d1[1][g < D ? 1 + g : D + 2] * eyy);
-#pragma unroll
-      for (int f = 0; f < D + 3; ++f) Wf.d1[1][f] *= ey;
-#pragma unroll
-      for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int c = 0; c < D; ++c)
-          if (a == 1 || c == 1) Wf.mix[a][c] *= ey;
-      auto Bf = [&](int slot) { return btab_f[(long long)slot * P.nbase + j]; };
-      pw::DN3 o[D + 2];
-      pw::rhs_num<D, pw::DN3>(P.physf, Bf, Wf, (float)e, bc_row, fl, o);
-#pragma unroll
-      for (int a = 0; a < D + 2; ++a) res[a] += f2d_exact(o[a].w2);
-    }
-    double* out = (double*)P.out;
-    if (P.shift.x != 0.0 || P.shift.y != 0.0) {
-      const double sy = (i & 1) ? P.shift.y : -P.shift.y;  // the other component's factor
-#pragma unroll
-      for (int a = 0; a < D + 2; ++a) {
-        const long long o = (long long)a * nreal + i;
-        res[a] -= fma(P.shift.x, v[o], sy * v[o ^ 1]);
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < D + 2; ++a) out[(long long)a * nreal + i] = res[a];
+    pw::DN3 o[D + 2];
+    pw::rhs_num<D, pw::DN3>(phys, Bf, Wf, ef, true, fl, o);
+    for (int a = 0; a < D + 2; ++a)
+      if (part) w2[a].y = o[a].w2; else w2[a].x = o[a].w2;
   }
 }
 
 template <int D, bool EPS>
+__device__ __forceinline__ void point_fast_body(const PointParams& P, const float4* __restrict__ coefp,
+                                                const float* __restrict__ btab_f, unsigned bidx) {
+  constexpr int NW = pw::nw_inputs(D);
+  constexpr int o1 = D + 3, o2 = o1 + D * (D + 3), om = o2 + D * (D + 1);
+  const long long i = (long long)bidx * blockDim.x + threadIdx.x;  // no loop: its invariant addresses would take
+  if (i >= P.npts) return;                                         // the registers that the loads in flight need
+  const double e = EPS ? *P.eps : 0.0;
+  const bool visc = P.phys.visc;
+  const float4* S = (const float4*)P.scratch;
+  const int j = row_of(P, i);
+  const float4* Cp = coefp + (long long)j * coefs_used<D>();
+  ffn2 acc[D + 2], vp[D + 2];
+  pw::WIn<D, float2> W;  // EPS: the remainder's inputs
+#pragma unroll
+  for (int a = 0; a < D + 2; ++a) acc[a] = ff2_zero2();
+  int u = 0;  // running index of the row's coefficients (a constant once unrolled)
+  auto put = [&](int q, ffn2 w) {
+#pragma unroll
+    for (int a = 0; a < D + 2; ++a)
+      if (coef_used<D>(a, q)) acc[a] = ff2_fma(ff2_unpack(__ldg(Cp + u++)), w, acc[a]);
+  };
+  auto slot = [&](int s) { return S[(long long)s * P.npts + i]; };
+  const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  // Inputs in groups (v and T; per axis the first, then the second derivatives; the mixed ones), each
+  // loaded two groups ahead of its use.
+  constexpr int kGroups = 2 * D + 1, kMost = D + 3;
+  float4 buf[3][kMost];
+  auto fetch = [&](int g) {
+    float4* in = buf[g % 3];
+    if (g < D) {
+#pragma unroll
+      for (int f = 0; f < D + 3; ++f) in[f] = f < D + 2 || visc ? slot(P.s_d1[g][f]) : zero;
+    } else if (g < 2 * D) {
+#pragma unroll
+      for (int f = 0; f < D + 1; ++f) in[f] = visc ? slot(P.s_d2[g - D][f]) : zero;
+    } else if (g == 2 * D) {
+      int k = 0;
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+          if (a != c) in[k++] = visc ? slot(P.s_mix[a][c]) : zero;
+    }
+  };
+  double2 vd[D + 3];
+#pragma unroll
+  for (int f = 0; f < D + 2; ++f) vd[f] = P.v[(long long)f * P.npts + i];
+  vd[D + 2] = visc ? P.scratch[(long long)P.s_Tw * P.npts + i] : make_double2(0.0, 0.0);
+  fetch(0);
+  fetch(1);
+#pragma unroll
+  for (int f = 0; f < D + 3; ++f) {
+    const ffn2 w = ff2_split(vd[f]);
+    if (f < D + 2) vp[f] = w;
+    if (EPS) W.v[f] = w.hi;
+    put(f, w);
+  }
+#pragma unroll
+  for (int g = 0; g < kGroups; ++g) {
+    if (g + 2 < kGroups) fetch(g + 2);
+    const float4* in = buf[g % 3];
+    if (g < D) {
+#pragma unroll
+      for (int f = 0; f < D + 3; ++f) put(o1 + g * (D + 3) + f, ff2_from_slot(in[f]));
+    } else if (g < 2 * D) {
+#pragma unroll
+      for (int f = 0; f < D + 1; ++f) put(o2 + (g - D) * (D + 1) + f, ff2_from_slot(in[f]));
+    } else {
+      int k = 0;
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+          if (a != c) put(om + a * D + c, ff2_from_slot(in[k++]));
+    }
+  }
+  if (P.shift.x != 0.0 || P.shift.y != 0.0) {  // - shift v: (-sx, -sx) v + (sy, -sy) (im v, re v)
+    const ffn sx = ff2_split(-P.shift.x), sy = ff2_split(P.shift.y);
+    const ffn2 cx = ff2_dup(sx), cy{make_float2(sy.hi, -sy.hi), make_float2(sy.lo, -sy.lo)};
+#pragma unroll
+    for (int a = 0; a < D + 2; ++a) {
+      const ffn2 sw{make_float2(vp[a].hi.y, vp[a].hi.x), make_float2(vp[a].lo.y, vp[a].lo.x)};
+      acc[a] = ff2_fma(cy, sw, ff2_fma(cx, vp[a], acc[a]));
+    }
+  }
+  if (EPS && e != 0.0) {  // O(eps) remainder of the quotient, FP32, physical (metric-applied) inputs
+    const float ey = ff2_split(P.eta_y[j]).hi, eyy = ff2_split(P.eta_yy[j]).hi, ef = ff2_split(e).hi;
+    // read the high parts again (they are in the caches) rather than hold 84 registers through the sums above
+    asm volatile("" ::: "memory");
+    auto high = [&](int s) { const float4 w = slot(s); return make_float2(w.x, w.z); };
+    const float2 z2 = v2(0.0f);
+#pragma unroll
+    for (int ax = 0; ax < D; ++ax) {
+#pragma unroll
+      for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = f < D + 2 || visc ? high(P.s_d1[ax][f]) : z2;
+#pragma unroll
+      for (int g = 0; g < D + 1; ++g) W.d2[ax][g] = visc ? high(P.s_d2[ax][g]) : z2;
+#pragma unroll
+      for (int c = 0; c < D; ++c) W.mix[ax][c] = visc && c != ax ? high(P.s_mix[ax][c]) : z2;
+    }
+#pragma unroll
+    for (int ax = 0; ax < D; ++ax) {
+      const float s1 = P.sc1[ax], s2 = P.sc2[ax];
+      const float f1 = ax == 1 ? __fmul_rn(s1, ey) : s1;
+#pragma unroll
+      for (int g = 0; g < D + 1; ++g) {
+        W.d2[ax][g] = v2_mul(W.d2[ax][g], v2(ax == 1 ? __fmul_rn(s2, __fmul_rn(ey, ey)) : s2));
+        if (ax == 1) W.d2[1][g] = v2_fma(W.d1[1][g < D ? 1 + g : D + 2], v2(__fmul_rn(s1, eyy)), W.d2[1][g]);
+      }
+#pragma unroll
+      for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = v2_mul(W.d1[ax][f], v2(f1));
+#pragma unroll
+      for (int c = 0; c < D; ++c)
+        if (c != ax) W.mix[ax][c] = v2_mul(W.mix[ax][c], v2(__fmul_rn(f1, c == 1 ? __fmul_rn(P.sc1[c], ey) : P.sc1[c])));
+    }
+    auto Bf = [&](int s) { return btab_f[(long long)s * P.nbase + j]; };
+    float2 w2[D + 2];
+    if (j != 0 && j != P.ny - 1) {
+      pw::remainder_y_base<D>(P.physf, Bf, W, ef, w2);
+    } else {
+      const pw::WIn<D, float2> Wc = W;
+      wall_remainder<D>(P.physf, btab_f, P.nbase, j, P.bcflags[j == 0 ? 0 : (long long)P.nx * P.nz], Wc, ef, w2);
+    }
+#pragma unroll
+    for (int a = 0; a < D + 2; ++a) acc[a].lo = v2_add(acc[a].lo, w2[a]);
+  }
+#pragma unroll
+  for (int a = 0; a < D + 2; ++a) P.out[(long long)a * P.npts + i] = ff2_to_d(ff2_norm(acc[a]));
+}
+
+template <int D, bool EPS>
 __global__ void __launch_bounds__(128, D == 3 ? 3 : 4)
-    k_point_fast(const __grid_constant__ PointParams P, const ffn* __restrict__ coefp, const float* __restrict__ btab_f) {
+    k_point_fast(const __grid_constant__ PointParams P, const float4* __restrict__ coefp, const float* __restrict__ btab_f) {
   if (P.gate && *P.gate) return;
   point_fast_body<D, EPS>(P, coefp, btab_f, blockIdx.x);
 }
@@ -897,9 +966,17 @@ __global__ void k_coeffs_fold(const double* coef, const double* eta_y, const dou
   for (int q = 0; q < NW; ++q) o[q] = f[q];
 }
 
-__global__ void k_split_pairs(const double* in, ffn* out, long long count) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
-    out[i] = ff2_split(in[i]);
+// The used coefficients of every row, in the order of the pointwise kernel's
+// streaming (input by input), as duplicated FP32 pairs.
+template <int D>
+__global__ void k_pack_coefs(const double* in, int ny, float4* out) {
+  constexpr int NW = pw::nw_inputs(D);
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < ny; j += gridDim.x * blockDim.x) {
+    float4* o = out + (long long)j * coefs_used<D>();
+    for (int q = 0; q < NW; ++q)
+      for (int a = 0; a < D + 2; ++a)
+        if (coef_used<D>(a, q)) *o++ = ff2_pack(ff2_dup(ff2_split(in[((long long)j * (D + 2) + a) * NW + q])));
+  }
 }
 
 __global__ void k_to_float_tab(const double* in, float* out, long long count) {
@@ -1073,7 +1150,7 @@ struct TempItem {
 };
 struct PointItem {
   PointParams P;
-  const ffn* coefp;
+  const float4* coefp;
   const float* btab_f;
 };
 static_assert(sizeof(TempItem) % 8 == 0 && sizeof(PointItem) % 8 == 0,
@@ -1128,13 +1205,14 @@ __global__ void __launch_bounds__(128, D == 3 ? 3 : 4)
 }
 
 // line passes: item = (instance, axis), its blocks as in the single launch
-__global__ void __launch_bounds__(pl::kMaxThreads, 2)
+template <int LANES>
+__global__ void __launch_bounds__(pl::kMaxThreads, LANES == 2 ? 1 : 2)
     k_pair_pass_batch(const pl::PairPass* __restrict__ items, const int* __restrict__ start, int count) {
   __shared__ pl::PairPass sP;
   const int i = batch_item(start, count, blockIdx.x);
   copy_to_shared(&sP, items + i, sizeof(pl::PairPass));
   __syncthreads();
-  pl::pair_pass_body(sP, blockIdx.x - (unsigned)__ldg(start + i));
+  pl::pair_pass_body<LANES>(sP, blockIdx.x - (unsigned)__ldg(start + i));
 }
 
 }  // namespace
@@ -1365,10 +1443,10 @@ static cudaError_t pass_shape(StabHandle* h, int axis, const PassParams& base_pa
 }
 
 // Parameters and launch shape of one axis's pair-arithmetic pass (jobs filled
-// in by the caller).  Chunks of 32 points cost the fewest corrections per
+// in by the caller; batch: for a launch over several instances).  Chunks of 32 points cost the fewest corrections per
 // point; shorter ones and fewer lines per CTA spread small grids over the SMs.
-static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, pl::PairPass& P, int& threads, size_t& smem,
-                              long long& blocks) {
+static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, bool batch, pl::PairPass& P, int& threads,
+                              size_t& smem, long long& blocks) {
   const AxisTables& A = h->ax[axis];
   const int n = A.n;
   P = pl::PairPass{};
@@ -1386,62 +1464,65 @@ static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, pl::PairPass& 
   P.ny = h->ny;
   P.bounded = !A.periodic;
   const LineCfg cfg = h->line_cfg[axis];
+  // both components in a thread when that leaves every SM enough threads
+  const long long chunks16 = P.nlines * njobs * ((n + 15) / 16);
+  P.lanes = chunks16 >= 152LL * 1024 ? 2 : 1;
+  const int per = 2 / P.lanes;  // threads per complex line and chunk
   auto smem_of = [&](int L, int nch) {
-    const int RL = 2 * L, RLp = RL % 4 == 0 ? RL + 2 : RL;
-    return (size_t)n * RLp * 8 + ((size_t)2 * RL * nch + 8 * RL + pl::kTab) * 8;
+    return ((size_t)n * (L | 1) + ((size_t)2 * L * nch + 8 * L) + (P.lanes == 2 ? pl::kTab : (pl::kTab + 1) / 2)) *
+           sizeof(float4);
   };
-  const long long want = 152LL * 1024;  // threads that fill the SMs
   int C = cfg.C;
-  if (C <= 0) {
-    C = 32;
-    if (2 * P.nlines * njobs * ((n + 31) / 32) < want) C = 16;
-  }
+  if (C <= 0) C = P.lanes == 1 && chunks16 >= 152LL * 512 ? 32 : 16;
   if (C > kPairMaxC) C = kPairMaxC;
   const int nch = (n + C - 1) / C;
   int L = cfg.L;
-  if (L <= 0) {
-    L = 16;
-    while (L > 2 && (smem_of(L, nch) > 72 * 1024 || 2 * L * nch > 256 ||
-                     (P.nlines + L - 1) / L * njobs < 2 * 152))
+  if (batch) {  // one launch for uneven instances: CTAs of about 128 threads for all of them
+    L = std::max(1, 128 / (per * nch));
+    while (L > 1 && smem_of(L, nch) > 48 * 1024) --L;
+  } else if (L <= 0) {
+    L = 32;
+    while (L > 2 && (smem_of(L, nch) > 48 * 1024 || per * L * nch > 256 || (P.nlines + L - 1) / L * njobs < 3 * 152))
       L /= 2;
   }
   L = (int)std::min<long long>(L, std::max<long long>(1, P.nlines));
-  while (L > 1 && (2 * L * nch > pl::kMaxThreads || smem_of(L, nch) > pl::kSmemMax)) --L;
-  if (2 * L * nch > pl::kMaxThreads || smem_of(L, nch) > pl::kSmemMax) return cudaErrorInvalidValue;
+  while (L > 1 && (per * L * nch > pl::kMaxThreads || smem_of(L, nch) > pl::kSmemMax)) --L;
+  if (per * L * nch > pl::kMaxThreads || smem_of(L, nch) > pl::kSmemMax) return cudaErrorInvalidValue;
   P.L = L;
-  P.RL = 2 * L;
-  P.RLp = P.RL % 4 == 0 ? P.RL + 2 : P.RL;
+  P.Lp = L | 1;
+  P.U = per * P.L;
+  P.Up = per * P.Lp;
   P.nch = nch;
   P.q = n / nch;
   P.rem = n % nch;
+  P.divU = make_fastdiv((unsigned)P.U);
   const long long nblk = (P.nlines + L - 1) / L;
   if (nblk * njobs > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
   P.nblk = (int)nblk;
   P.divblk = make_fastdiv((unsigned)nblk);
-  P.divRL = make_fastdiv((unsigned)P.RL);
   P.divL = make_fastdiv((unsigned)L);
   P.divn = make_fastdiv((unsigned)n);
   P.divnx = make_fastdiv((unsigned)h->nx);
-  threads = ((P.RL * nch + 31) / 32) * 32;
+  threads = ((P.U * nch + 31) / 32) * 32;
   smem = smem_of(L, nch);
   blocks = nblk * njobs;
   return cudaSuccess;
 }
 
 // The pass of axis ax for the fields src (as axis_jobs): one job per derivative.
-static cudaError_t pair_pass(StabHandle* h, int ax, const double2* const* src, pl::PairPass& P, int& threads,
-                             size_t& smem, long long& blocks) {
+static cudaError_t pair_pass(StabHandle* h, int ax, const double2* const* src, bool batch, pl::PairPass& P,
+                             int& threads, size_t& smem, long long& blocks) {
   std::vector<LineJob> jobs;
   axis_jobs(h, ax, src, jobs);
   const size_t raw = h->visc ? h->dim + 3 : h->dim + 2;  // the jobs after the fields' take pass outputs
   std::vector<pl::PairJob> pj;
   for (size_t q = 0; q < jobs.size(); ++q) {
     const int pin = q >= raw;
-    if (jobs[q].out1) pj.push_back(pl::PairJob{(const double*)jobs[q].in, (float2*)jobs[q].out1, 0, pin});
-    if (jobs[q].out2) pj.push_back(pl::PairJob{(const double*)jobs[q].in, (float2*)jobs[q].out2, 1, pin});
+    if (jobs[q].out1) pj.push_back(pl::PairJob{jobs[q].in, (float4*)jobs[q].out1, 0, pin});
+    if (jobs[q].out2) pj.push_back(pl::PairJob{jobs[q].in, (float4*)jobs[q].out2, 1, pin});
   }
   if (pj.empty() || pj.size() > STAB_MAX_JOBS) return cudaErrorInvalidValue;
-  const cudaError_t e = pair_shape(h, ax, (int)pj.size(), P, threads, smem, blocks);
+  const cudaError_t e = pair_shape(h, ax, (int)pj.size(), batch, P, threads, smem, blocks);
   std::copy(pj.begin(), pj.end(), P.job);
   return e;
 }
@@ -1451,9 +1532,10 @@ static cudaError_t run_pair_pass(StabHandle* h, int ax, const double2* const* sr
   int threads = 0;
   size_t smem = 0;
   long long blocks = 0;
-  const cudaError_t e = pair_pass(h, ax, src, P, threads, smem, blocks);
+  const cudaError_t e = pair_pass(h, ax, src, false, P, threads, smem, blocks);
   if (e != cudaSuccess) return e;
-  pl::k_pair_pass<<<(unsigned)blocks, threads, smem, h->stream>>>(P);
+  if (P.lanes == 2) pl::k_pair_pass<2><<<(unsigned)blocks, threads, smem, h->stream>>>(P);
+  else pl::k_pair_pass<1><<<(unsigned)blocks, threads, smem, h->stream>>>(P);
   return cudaGetLastError();
 }
 
@@ -1842,9 +1924,9 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
   const int D = h->dim;
   cudaError_t err;
   // set once per handle (current device), never during a stream capture
-  const void* line_kernels[5] = {(const void*)k_line_pass<false>, (const void*)k_line_pass<true>,
+  const void* line_kernels[6] = {(const void*)k_line_pass<false>, (const void*)k_line_pass<true>,
                                  (const void*)k_line_pass_compact<false>, (const void*)k_line_pass_compact<true>,
-                                 (const void*)pl::k_pair_pass};
+                                 (const void*)pl::k_pair_pass<1>, (const void*)pl::k_pair_pass<2>};
   static_assert(kLineSmemMax == pl::kSmemMax, "one opt-in size for the line kernels");
   for (const void* k : line_kernels)
     if ((err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmemMax)) != cudaSuccess)
@@ -1968,9 +2050,10 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
     }
     if (D == 2) k_coeffs_fold<2><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, sc, h->d_coef_f);
     else k_coeffs_fold<3><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, sc, h->d_coef_f);
-    const long long ncf = (long long)h->ny * (D + 2) * nw;
-    if ((err = dalloc(h, &h->d_coef_p, ncf * sizeof(ffn))) != cudaSuccess) return err;
-    k_split_pairs<<<64, 256, 0, h->stream>>>(h->d_coef_f, h->d_coef_p, ncf);
+    const size_t ncf = (size_t)h->ny * (D == 2 ? coefs_used<2>() : coefs_used<3>());
+    if ((err = dalloc(h, &h->d_coef_p, ncf * sizeof(float4))) != cudaSuccess) return err;
+    if (D == 2) k_pack_coefs<2><<<(h->ny + 31) / 32, 32, 0, h->stream>>>(h->d_coef_f, h->ny, h->d_coef_p);
+    else k_pack_coefs<3><<<(h->ny + 31) / 32, 32, 0, h->stream>>>(h->d_coef_f, h->ny, h->d_coef_p);
     const long long nbt = (long long)bt_count(D) * h->nbase;
     if ((err = dalloc(h, &h->d_btab_f, nbt * sizeof(float))) != cudaSuccess) return err;
     k_to_float_tab<<<64, 256, 0, h->stream>>>(h->d_btab, h->d_btab_f, nbt);
@@ -2027,7 +2110,7 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   if ((err = run_derivatives(h, src, h->stencil_ff, fast)) != cudaSuccess) return err;
   const int tp = phase_begin(h, STAB_PHASE_POINTWISE);
   if (fast) {
-    const unsigned g = (unsigned)((2 * h->npts + thr - 1) / thr);
+    const unsigned g = (unsigned)((h->npts + thr - 1) / thr);
     if (D == 2 && eps_mode == 2) k_point_fast<2, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
     else if (D == 2) k_point_fast<2, true><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
     else if (eps_mode == 2) k_point_fast<3, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
@@ -2108,7 +2191,10 @@ cudaError_t batch_order_end(stab_jv_batch_s* B) {
 }
 
 static cudaError_t jv_batch_attributes() {
-  return cudaFuncSetAttribute(k_pair_pass_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl::kSmemMax);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_pair_pass_batch<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl::kSmemMax);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_pair_pass_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl::kSmemMax);
 }
 
 // Parameter-image sections of one batched J v (every phase, one section per
@@ -2159,18 +2245,18 @@ cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
       temp_blocks[form].push_back(grid_for(2 * h->npts, 128));
     }
     points[h->dim - 2][form].push_back(PointItem{P, h->d_coef_p, h->d_btab_f});
-    point_blocks[h->dim - 2][form].push_back((int)((2 * h->npts + 127) / 128));
+    point_blocks[h->dim - 2][form].push_back((int)((h->npts + 127) / 128));
   }
   plan.norm = im.section(norms, norm_blocks, 256, 0);
   for (int f = 0; f < 2; ++f) plan.temp[f] = im.section(temps[f], temp_blocks[f], 128, 0);
-  // 3. line passes y, z, x: one section per axis
+  // 3. line passes y, z, x: per axis one section per kernel variant (components per thread)
   static const int order[3] = {1, 2, 0};
   for (int q = 0; q < 3; ++q) {
     const int ax = order[q];
-    std::vector<pl::PairPass> items;
-    std::vector<int> blocks;
-    int threads = 0;
-    size_t smem = 0;
+    std::vector<pl::PairPass> items[2];
+    std::vector<int> blocks[2];
+    int threads[2] = {0, 0};
+    size_t smem[2] = {0, 0};
     for (int i = 0; i < count; ++i) {
       StabHandle* h = hs[i];
       if (ax >= h->dim) continue;
@@ -2182,15 +2268,16 @@ cudaError_t jv_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
       int thr = 0;
       size_t sm = 0;
       long long nb = 0;
-      const cudaError_t e = pair_pass(h, ax, src, P, thr, sm, nb);
+      const cudaError_t e = pair_pass(h, ax, src, true, P, thr, sm, nb);
       if (e != cudaSuccess) return e;
       P.gate = gates ? gates[i] : nullptr;
-      items.push_back(P);
-      blocks.push_back((int)nb);
-      threads = std::max(threads, thr);
-      smem = std::max(smem, sm);
+      const int k = P.lanes - 1;
+      items[k].push_back(P);
+      blocks[k].push_back((int)nb);
+      threads[k] = std::max(threads[k], thr);
+      smem[k] = std::max(smem[k], sm);
     }
-    plan.line[q] = im.section(items, blocks, threads, smem);
+    for (int k = 0; k < 2; ++k) plan.line[q][k] = im.section(items[k], blocks[k], threads[k], smem[k]);
   }
   for (int d = 0; d < 2; ++d)
     for (int f = 0; f < 2; ++f) plan.point[d][f] = im.section(points[d][f], point_blocks[d][f], 128, 0);
@@ -2210,9 +2297,12 @@ cudaError_t jv_batch_launch(const JvBatchPlan& plan, const unsigned char* d, cud
   temperature(plan.temp[0], k_temperature_fast_batch<false>);
   temperature(plan.temp[1], k_temperature_fast_batch<true>);
   for (int q = 0; q < 3; ++q) {
-    const BatchSection& s = plan.line[q];
-    if (s.count)
-      k_pair_pass_batch<<<s.blocks, s.threads, s.smem, st>>>((const pl::PairPass*)items_of(s), start_of(s), s.count);
+    const BatchSection& s1 = plan.line[q][0];
+    const BatchSection& s2 = plan.line[q][1];
+    if (s1.count)
+      k_pair_pass_batch<1><<<s1.blocks, s1.threads, s1.smem, st>>>((const pl::PairPass*)items_of(s1), start_of(s1), s1.count);
+    if (s2.count)
+      k_pair_pass_batch<2><<<s2.blocks, s2.threads, s2.smem, st>>>((const pl::PairPass*)items_of(s2), start_of(s2), s2.count);
   }
   auto point = [&](const BatchSection& s, auto kernel) {
     if (s.count) kernel<<<s.blocks, 128, 0, st>>>((const PointItem*)items_of(s), start_of(s), s.count);

@@ -110,23 +110,20 @@ __device__ __forceinline__ ffn ff_warp_sum(ffn x) {
 // Pair arithmetic of the derivative passes (rounding intrinsics, so that the
 // compiler fuses nothing across the error terms).
 // ---------------------------------------------------------------------------
-// d to the nearest pair: hi is d rounded to 24 bits, lo the rest (29 bits,
-// signed) rounded to 24, so |d - hi - lo| <= 2^-49 |d|.  Integer operations
-// but one conversion: the FP64 pipe is not used.  |d| below 2^-126 gives zero,
-// lo is kept from 2^-74 up; from 2^127 up and for NaN, hi is Inf or NaN.
+// d to the nearest pair: hi is d rounded to 24 bits (half away from zero), lo
+// the rest (29 bits, signed) rounded to 24, so |d - hi - lo| <= 2^-49 |d|.
+// Integer operations but one conversion: the FP64 pipe is not used.  |d| below
+// 2^-126 gives zero (to 2^-146), lo is kept from 2^-74 up; from 2^127 up and
+// for Inf and NaN, hi is Inf or NaN.
 __device__ __forceinline__ ffn ff2_split(double d) {
   const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
-  const unsigned e = (h >> 20) & 0x7FFu;
-  const unsigned long long t = (((unsigned long long)h << 32) | l) + 0x10000000ull;  // half a unit of hi
-  const unsigned sign = h & 0x80000000u;
-  // exponent rebased by 896 modulo 512: exact for results in [1, 254]
-  unsigned hb = sign | (((unsigned)(t >> 29) - (384u << 23)) & 0x7FFFFFFFu);
-  float lo = __int2float_rn((int)(l << 3) >> 3) * __uint_as_float(sign | ((unsigned)max((int)e - 948, 0) << 23));
-  if (e - 897u >= 253u) {  // zero, tiny, huge, Inf or NaN
-    hb = e < 897u ? sign : (sign | (e == 0x7FFu && ((h & 0xFFFFFu) | l) ? 0x7FC00000u : 0x7F800000u));
-    lo = 0.0f;
-  }
-  return ffn{__uint_as_float(hb), lo};
+  const unsigned a = h & 0x7FFFFFFFu, tl = l + 0x10000000u;  // plus half a unit of hi
+  // exponent rebased by 896, clamped to the FP32 range
+  const int th = min(max((int)(a + (tl < l ? 1u : 0u)) - (896 << 20), 0), 255 << 20);
+  const float hi = __uint_as_float(__funnelshift_l(tl, (unsigned)th, 3) | (h & 0x80000000u));
+  // the low 29 bits as a signed integer, in units of 2^(e - 52)
+  const unsigned sc = ((unsigned)max((int)a - (948 << 20), 0) << 3) & 0x7F800000u;
+  return ffn{hi, __fmul_rn(__int2float_rn((int)(l << 3) >> 3), __uint_as_float(sc | (h & 0x80000000u)))};
 }
 __device__ __forceinline__ ffn ff2_norm(ffn a) {
   const float t = __fadd_rn(a.hi, a.lo);
@@ -154,10 +151,79 @@ __device__ __forceinline__ ffn ff2_fma_u(ffn c, ffn x, ffn w) {
   return ffn{s, __fadd_rn(__fadd_rn(t, w.lo), e)};
 }
 __device__ __forceinline__ ffn ff2_fma(ffn c, ffn x, ffn w) { return ff2_norm(ff2_fma_u(c, x, w)); }
-// hi + lo in FP64 with integer conversions and one add; Inf and NaN are kept
+// hi + lo in FP64 (normalised pair), correctly rounded to 53 bits but for one
+// unit, with integer operations: lo is rounded to units of hi's 52-bit
+// mantissa and added to hi's bit pattern.  A power of two with lo of the other
+// sign (the unit halves below it) takes an FP64 add; Inf and NaN are kept.
 __device__ __forceinline__ double ff2_to_d(ffn a) {
-  const unsigned u = __float_as_uint(a.hi);
-  const double d = f2d_exact(a.hi) + f2d_exact(a.lo);
-  if ((u & 0x7F800000u) != 0x7F800000u) return d;
-  return __hiloint2double((int)((u & 0x80000000u) | 0x7FF00000u | ((u & 0x7FFFFFu) ? 0x80000u : 0u)), 0);
+  const unsigned u = __float_as_uint(a.hi), ex = (u >> 23) & 0xFFu, m = u & 0x7FFFFFu;
+  if (ex <= 52u || ex >= 200u || m == 0u) {  // tiny, huge, zero, Inf, NaN or a power of two
+    if (ex != 0xFFu) return f2d_exact(a.hi) + f2d_exact(a.lo);
+    return __hiloint2double((int)((u & 0x80000000u) | 0x7FF00000u | (m ? 0x80000u : 0u)), 0);
+  }
+  // lo / 2^(e - 52) with hi's sign taken off; |.| <= 2^28
+  const float sc = __uint_as_float((u & 0x80000000u) | ((306u - ex) << 23));
+  const int li = __float2int_rn(__fmul_rn(a.lo, sc));
+  const unsigned long long b = ((unsigned long long)((u & 0x80000000u) | ((ex + 896u) << 20) | (m >> 3)) << 32) |
+                               (unsigned long long)(m << 29);
+  return __longlong_as_double((long long)(b + (unsigned long long)(long long)li));
 }
+
+// ---------------------------------------------------------------------------
+// Two pairs side by side (the real and imaginary components), on the packed
+// FP32 instructions of sm_100: one issue slot for two operations.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 v2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 v2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 v2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 v2_sub(float2 a, float2 b) { return __fadd2_rn(a, v2_neg(b)); }
+__device__ __forceinline__ float2 v2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 v2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float v2_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+struct ffn2 {
+  float2 hi, lo;
+};
+__device__ __forceinline__ ffn2 ff2_dup(ffn a) { return ffn2{v2(a.hi), v2(a.lo)}; }
+__device__ __forceinline__ ffn2 ff2_zero2() { return ffn2{v2(0.0f), v2(0.0f)}; }
+__device__ __forceinline__ ffn2 ff2_neg(ffn2 a) { return ffn2{v2_neg(a.hi), v2_neg(a.lo)}; }
+// in 16 (8) bytes, highs first; a slot of the derivative scratch holds (re.hi, re.lo, im.hi, im.lo)
+__device__ __forceinline__ float4 ff2_pack(ffn2 a) { return make_float4(a.hi.x, a.hi.y, a.lo.x, a.lo.y); }
+__device__ __forceinline__ ffn2 ff2_unpack(float4 a) { return ffn2{make_float2(a.x, a.y), make_float2(a.z, a.w)}; }
+__device__ __forceinline__ float4 ff2_to_slot(ffn2 a) { return make_float4(a.hi.x, a.lo.x, a.hi.y, a.lo.y); }
+__device__ __forceinline__ ffn2 ff2_from_slot(float4 a) { return ffn2{make_float2(a.x, a.z), make_float2(a.y, a.w)}; }
+__device__ __forceinline__ float2 ff2_pack(ffn a) { return make_float2(a.hi, a.lo); }
+__device__ __forceinline__ ffn ff2_unpack(float2 a) { return ffn{a.x, a.y}; }
+__device__ __forceinline__ float2 ff2_to_slot(ffn a) { return make_float2(a.hi, a.lo); }
+__device__ __forceinline__ ffn ff2_from_slot(float2 a) { return ffn{a.x, a.y}; }
+__device__ __forceinline__ ffn ff2_neg(ffn a) { return ffn{-a.hi, -a.lo}; }
+__device__ __forceinline__ ffn2 ff2_split(double2 d) {
+  const ffn a = ff2_split(d.x), b = ff2_split(d.y);
+  return ffn2{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)};
+}
+__device__ __forceinline__ double2 ff2_to_d(ffn2 a) {
+  return make_double2(ff2_to_d(ffn{a.hi.x, a.lo.x}), ff2_to_d(ffn{a.hi.y, a.lo.y}));
+}
+__device__ __forceinline__ ffn2 ff2_norm(ffn2 a) {
+  const float2 t = v2_add(a.hi, a.lo);
+  return ffn2{t, v2_sub(a.lo, v2_sub(t, a.hi))};
+}
+__device__ __forceinline__ float2 ff2_two_sum(float2 a, float2 b, float2& err) {
+  const float2 s = v2_add(a, b), bb = v2_sub(s, a);
+  err = v2_add(v2_sub(a, v2_sub(s, bb)), v2_sub(b, bb));
+  return s;
+}
+__device__ __forceinline__ ffn2 ff2_add_u(ffn2 a, ffn2 b) {
+  float2 e;
+  const float2 s = ff2_two_sum(a.hi, b.hi, e);
+  return ffn2{s, v2_add(e, v2_add(a.lo, b.lo))};
+}
+__device__ __forceinline__ ffn2 ff2_add(ffn2 a, ffn2 b) { return ff2_norm(ff2_add_u(a, b)); }
+__device__ __forceinline__ ffn2 ff2_fma_u(ffn2 c, ffn2 x, ffn2 w) {
+  const float2 p = v2_mul(c.hi, x.hi);
+  float2 e = v2_fma(c.hi, x.hi, v2_neg(p)), t;
+  e = v2_fma(c.hi, x.lo, e);
+  e = v2_fma(c.lo, x.hi, e);
+  const float2 s = ff2_two_sum(w.hi, p, t);
+  return ffn2{s, v2_add(v2_add(t, w.lo), e)};
+}
+__device__ __forceinline__ ffn2 ff2_fma(ffn2 c, ffn2 x, ffn2 w) { return ff2_norm(ff2_fma_u(c, x, w)); }

@@ -338,7 +338,7 @@ cudaError_t pc_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
                           const int* const* gates, BatchImage& im, PcBatchPlan& plan);
 cudaError_t pc_batch_launch(const PcBatchPlan& plan, const unsigned char* d, cudaStream_t st);
 struct CgsBatchPlan {
-  BatchSection S, N;
+  BatchSection C[2], S, N;
   size_t sm = 0;
 };
 // Order the batch's stream after the work queued so far on every handle's own
@@ -348,6 +348,7 @@ struct CgsBatchPlan {
 cudaError_t batch_order_begin(stab_jv_batch_s* B);
 cudaError_t batch_order_end(stab_jv_batch_s* B);
 struct CgsJob {  // one instance of a batched CGS2 (scratch as for kry_cgs2)
+  StabHandle* h;
   const double2* V;
   int k;
   long long n;

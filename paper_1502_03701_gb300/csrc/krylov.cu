@@ -6,6 +6,8 @@
 #include "internal.cuh"
 #include "pairs.cuh"
 
+#include <algorithm>
+
 namespace {
 
 constexpr int kThreads = 256;
@@ -376,6 +378,363 @@ __global__ void k_norm_final(const double* partial, int nb, double* out, const i
   norm_final_body(partial, nb, out);
 }
 
+// ---------------------------------------------------------------------------
+// Gram-Schmidt passes for up to kColMax basis vectors: V^H w (dots), w -= V h
+// (update), or both with one read of V.
+//
+// What bounds them: the basis is read from HBM once per pass, 16 bytes and
+// about 60 FP32 issue slots per entry (FP64 runs at 1/64 of the FP32 rate, so
+// products are exact FP32 two-products of split pairs on the packed FP32
+// instructions).  A CTA of 16 warps takes 32 RG rows at a time: the warps of a
+// row group (CW of them, up to four columns each) hold the group's part of V in
+// registers as pairs, add up w's correction, exchange it through shared memory
+// and take the new w's products with the same registers, so the second pass of
+// CGS2 reads V once and splits it once.  The next rows' loads are in flight
+// meanwhile.  Sums over blocks: the last block to finish adds the blocks'
+// partial sums in block order (reproducible) and resets the counter.
+// ---------------------------------------------------------------------------
+constexpr int kColThreads = 512, kColWarps = kColThreads / 32, kCpw = 4, kColMax = kColWarps * kCpw;
+
+// column warps per row group: the smallest power of two with kCpw CW >= k
+__host__ __device__ inline int col_warps(int k) {
+  int cw = 1;
+  while (cw * kCpw < k) cw *= 2;
+  return cw;
+}
+// one row per thread from 384 rows per SM up
+__host__ __device__ inline bool by_rows(long long n) { return n >= 152LL * 384; }
+int col_blocks(long long n, int k) {
+  if (by_rows(n)) return 152;
+  const long long rows = 32LL * (kColWarps / col_warps(k));
+  const long long b = (n + rows - 1) / rows;
+  return (int)(b < 152 ? (b < 1 ? 1 : b) : 152);
+}
+
+struct ColArgs {
+  const double2* V;
+  double2* w;
+  const double2* h;     // update: coefficients (null: none)
+  double2* partial;     // dots: nb x k block sums (null: none)
+  double* npart;        // |w|^2 block sums (null: none)
+  double2* out_h;       // dots: the reduced sums
+  double2* sum_h;       // added to as well when set (h1 + h2)
+  double* out_norm;     // ||w|| (of the updated w)
+  double* ref_norm;     // decide: ||w|| before the update; *skip = out >= eta ref
+  int* skip;
+  unsigned* counter;    // zero on entry, zero on exit
+  long long n;
+  int k, nb;
+};
+
+struct ColShared {
+  float4 H[kColMax][2];       // coefficients as duplicated pairs, re and im
+  union {
+    struct {
+      float4 red[kColWarps][32];  // column split: a warp's share of the correction per row, pairs re, im
+      float4 wn[kColWarps][32][2];  // the group's updated w as duplicated pairs, re and im
+    };
+    struct {
+      float4 wr[kColThreads], wi[kColThreads];  // row split: the chunk's w as duplicated pairs
+    };
+  };
+  double2 dots[kColWarps][kCpw];
+  double nrm[kColWarps];
+  int last;
+};
+
+// hi, lo of a complex value as one packed pair (re, im), and one component duplicated
+__device__ __forceinline__ ffn2 dup_part(ffn2 a, bool im) {
+  return im ? ffn2{v2(a.hi.y), v2(a.lo.y)} : ffn2{v2(a.hi.x), v2(a.lo.x)};
+}
+__device__ __forceinline__ ffn2 swap_parts(ffn2 a) {
+  return ffn2{make_float2(a.hi.y, a.hi.x), make_float2(a.lo.y, a.lo.x)};
+}
+
+template <bool UPDATE, bool DOTS, bool NORM>
+__device__ __forceinline__ void finish_pass(const ColArgs& A, unsigned bidx, ColShared& S, ffn2* d1, ffn2* d2,
+                                            double nrm) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int k = A.k, CW = col_warps(k), RG = kColWarps / CW;
+  const int cw = wid % CW;
+  // block sums
+  if (DOTS) {
+#pragma unroll
+    for (int q = 0; q < kCpw; ++q) {
+      if (cw + q * CW >= k) continue;  // warp-uniform
+      ffn2 t = swap_parts(d2[q]);      // (im, re) of d2
+      ffn2 a = d1[q];
+      a.hi.y = -a.hi.y;
+      a.lo.y = -a.lo.y;
+      t = ff2_add(a, t);  // (d1.re + d2.im, d2.re - d1.im)
+      for (int o = 16; o > 0; o >>= 1) {
+        const ffn2 u{make_float2(__shfl_xor_sync(0xffffffffu, t.hi.x, o), __shfl_xor_sync(0xffffffffu, t.hi.y, o)),
+                     make_float2(__shfl_xor_sync(0xffffffffu, t.lo.x, o), __shfl_xor_sync(0xffffffffu, t.lo.y, o))};
+        t = ff2_add(t, u);
+      }
+      if (lane == 0) S.dots[wid][q] = ff2_to_d(t);
+    }
+  }
+  if (NORM) {
+    nrm = warp_sum(nrm);
+    if (lane == 0) S.nrm[wid] = nrm;
+  }
+  __syncthreads();
+  if (DOTS && threadIdx.x < k) {
+    const int j = threadIdx.x, c = j % CW, q = j / CW;
+    double sr = 0.0, si = 0.0;
+    for (int g = 0; g < RG; ++g) {
+      sr += S.dots[g * CW + c][q].x;
+      si += S.dots[g * CW + c][q].y;
+    }
+    A.partial[(long long)bidx * k + j] = make_double2(sr, si);
+  }
+  if (NORM && threadIdx.x == kColThreads - 1) {
+    double t = 0.0;
+    for (int g = 0; g < kColWarps; ++g) t += S.nrm[g];
+    A.npart[bidx] = t;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) S.last = atomicAdd(A.counter, 1u) == (unsigned)A.nb - 1;
+  __syncthreads();
+  if (!S.last) return;
+  __threadfence();
+  if (DOTS) {
+    for (int j = wid; j < k; j += kColWarps) {
+      double sr = 0.0, si = 0.0;
+#pragma unroll 5
+      for (int b = lane; b < A.nb; b += 32) {
+        const double2 p = __ldcg(A.partial + (long long)b * k + j);
+        sr += p.x;
+        si += p.y;
+      }
+      sr = warp_sum(sr);
+      si = warp_sum(si);
+      if (lane == 0) {
+        A.out_h[j] = make_double2(sr, si);
+        if (A.sum_h) A.sum_h[j] = make_double2(A.sum_h[j].x + sr, A.sum_h[j].y + si);
+      }
+    }
+  }
+  if (NORM && wid == kColWarps - 1) {
+    double t = 0.0;
+#pragma unroll 5
+    for (int b = lane; b < A.nb; b += 32) t += __ldcg(A.npart + b);
+    t = sqrt(warp_sum(t));
+    if (lane == 0) {
+      *A.out_norm = t;
+      if (A.skip) *A.skip = t >= 0.70710678118654752 * *A.ref_norm;  // NaN: reorthogonalise (and let the norm report it)
+    }
+  }
+  if (UPDATE && !DOTS && A.sum_h)
+    for (int j = threadIdx.x; j < k; j += kColThreads)
+      A.sum_h[j] = make_double2(A.sum_h[j].x + A.h[j].x, A.sum_h[j].y + A.h[j].y);
+  if (threadIdx.x == 0) *A.counter = 0u;
+}
+
+template <bool UPDATE, bool DOTS, bool NORM>
+__device__ __forceinline__ void col_pass(const ColArgs& A, unsigned bidx, ColShared& S) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int k = A.k, CW = col_warps(k), RG = kColWarps / CW;
+  const int grp = wid / CW, cw = wid - grp * CW;
+  const long long n = A.n;
+  if (UPDATE) {
+    for (int j = threadIdx.x; j < k; j += kColThreads) {
+      const ffn2 p = ff2_split(A.h[j]);
+      S.H[j][0] = ff2_pack(dup_part(p, false));
+      S.H[j][1] = ff2_pack(dup_part(p, true));
+    }
+    __syncthreads();
+  }
+  // conj(V_j) w = d1.re + d2.im, d2.re - d1.im with d1 += V_j re(w), d2 += V_j im(w)
+  ffn2 d1[kCpw], d2[kCpw];
+#pragma unroll
+  for (int q = 0; q < kCpw; ++q) d1[q] = d2[q] = ff2_zero2();
+  double nrm = 0.0;
+  const long long step = 32LL * RG * A.nb;
+  long long row = 32LL * ((long long)bidx * RG + grp) + lane;
+  double2 nv[kCpw], nw = make_double2(0.0, 0.0);
+  auto fetch = [&](long long r) {
+#pragma unroll
+    for (int q = 0; q < kCpw; ++q) {
+      const int j = cw + q * CW;
+      nv[q] = j < k && r < n ? A.V[(long long)j * n + r] : make_double2(0.0, 0.0);
+    }
+    if (!UPDATE || cw == 0) nw = r < n ? A.w[r] : make_double2(0.0, 0.0);
+  };
+  fetch(row);
+  for (long long r0 = 32LL * bidx * RG; r0 < n; r0 += step, row += step) {  // block-uniform
+    ffn2 v[kCpw];
+    const double2 wold = nw;
+#pragma unroll
+    for (int q = 0; q < kCpw; ++q) v[q] = ff2_split(nv[q]);
+    fetch(row + step);
+    ffn2 wr, wi;
+    if (UPDATE) {
+      // V h = a1 + i a2 with a1 += V re(h), a2 += V im(h)
+      ffn2 a1 = ff2_zero2(), a2 = ff2_zero2();
+#pragma unroll
+      for (int q = 0; q < kCpw; ++q) {
+        const int j = cw + q * CW;
+        if (j < k) {
+          a1 = ff2_fma_u(ff2_unpack(S.H[j][0]), v[q], a1);
+          a2 = ff2_fma_u(ff2_unpack(S.H[j][1]), v[q], a2);
+        }
+      }
+      ffn2 s2 = swap_parts(a2);  // i a2 = (-im, re)
+      s2.hi.x = -s2.hi.x;
+      s2.lo.x = -s2.lo.x;
+      const ffn2 mine = ff2_add(a1, s2);
+      if (CW > 1) {
+        S.red[wid][lane] = ff2_pack(mine);
+        __syncthreads();
+      }
+      if (cw == 0) {
+        ffn2 t = mine;
+        for (int c = 1; c < CW; ++c) t = ff2_add(t, ff2_unpack(S.red[wid + c][lane]));
+        const double2 wnew = make_double2(wold.x - ff2_to_d(ffn{t.hi.x, t.lo.x}), wold.y - ff2_to_d(ffn{t.hi.y, t.lo.y}));
+        if (row < n) A.w[row] = wnew;
+        if (NORM) nrm = fma(wnew.x, wnew.x, fma(wnew.y, wnew.y, nrm));
+        if (DOTS) {
+          const ffn2 p = ff2_split(wnew);
+          wr = dup_part(p, false);
+          wi = dup_part(p, true);
+          if (CW > 1) {
+            S.wn[grp][lane][0] = ff2_pack(wr);
+            S.wn[grp][lane][1] = ff2_pack(wi);
+          }
+        }
+      }
+      if (CW > 1) {
+        __syncthreads();
+        if (DOTS && cw != 0) {
+          wr = ff2_unpack(S.wn[grp][lane][0]);
+          wi = ff2_unpack(S.wn[grp][lane][1]);
+        }
+      }
+    } else {
+      const ffn2 p = ff2_split(wold);
+      wr = dup_part(p, false);
+      wi = dup_part(p, true);
+      if (NORM && cw == 0) nrm = fma(wold.x, wold.x, fma(wold.y, wold.y, nrm));
+    }
+    if (DOTS) {
+#pragma unroll
+      for (int q = 0; q < kCpw; ++q)
+        if (cw + q * CW < k) {
+          d1[q] = ff2_norm(ff2_fma_u(wr, v[q], d1[q]));
+          d2[q] = ff2_norm(ff2_fma_u(wi, v[q], d2[q]));
+        }
+    }
+  }
+  finish_pass<UPDATE, DOTS, NORM>(A, bidx, S, d1, d2, nrm);
+}
+
+// The same passes with one row per thread in the update (no exchange between
+// warps) and the products column by column afterwards: the chunk of V that the
+// update has just read (512 rows; 68 MB over all SMs at k = 55) comes back from
+// L2.  Needs enough rows to fill the threads.  With the column split, the
+// exchange of 16 warps' shares per 32 rows left 60 % of the issue slots empty at
+// k = 55 (312 us for update + products of 524,288 unknowns).
+template <bool UPDATE, bool DOTS, bool NORM>
+__device__ __forceinline__ void row_pass(const ColArgs& A, unsigned bidx, ColShared& S) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int k = A.k, CW = col_warps(k), RG = kColWarps / CW;
+  const int grp = wid / CW, cw = wid - grp * CW;
+  const long long n = A.n;
+  if (UPDATE) {
+    for (int j = threadIdx.x; j < k; j += kColThreads) {
+      const ffn2 p = ff2_split(A.h[j]);
+      S.H[j][0] = ff2_pack(dup_part(p, false));
+      S.H[j][1] = ff2_pack(dup_part(p, true));
+    }
+    __syncthreads();
+  }
+  ffn2 d1[kCpw], d2[kCpw];
+#pragma unroll
+  for (int q = 0; q < kCpw; ++q) d1[q] = d2[q] = ff2_zero2();
+  double nrm = 0.0;
+  const long long rows = ((n + A.nb - 1) / A.nb + 31) / 32 * 32;
+  const long long r0 = rows * bidx, r1 = r0 + rows < n ? r0 + rows : n;
+  for (long long c0 = r0; c0 < r1; c0 += kColThreads) {
+    const long long row = c0 + threadIdx.x;
+    double2 w = make_double2(0.0, 0.0);
+    if (row < r1) {
+      w = A.w[row];
+      if (UPDATE) {
+        const double2* Vr = A.V + row;
+        ffn2 a1 = ff2_zero2(), a2 = ff2_zero2();
+        constexpr int G = 8;  // loads in flight per thread
+        for (int j0 = 0; j0 < k; j0 += G) {
+          double2 v[G];
+#pragma unroll
+          for (int q = 0; q < G; ++q)
+            if (j0 + q < k) v[q] = Vr[(long long)(j0 + q) * n];
+#pragma unroll
+          for (int q = 0; q < G; ++q) {
+            if (j0 + q >= k) break;
+            const ffn2 p = ff2_split(v[q]);
+            a1 = ff2_fma_u(ff2_unpack(S.H[j0 + q][0]), p, a1);
+            a2 = ff2_fma_u(ff2_unpack(S.H[j0 + q][1]), p, a2);
+          }
+          a1 = ff2_norm(a1);
+          a2 = ff2_norm(a2);
+        }
+        ffn2 s2 = swap_parts(a2);  // i a2 = (-im, re)
+        s2.hi.x = -s2.hi.x;
+        s2.lo.x = -s2.lo.x;
+        const double2 c = ff2_to_d(ff2_add(a1, s2));
+        w = make_double2(w.x - c.x, w.y - c.y);
+        A.w[row] = w;
+      }
+      if (NORM) nrm = fma(w.x, w.x, fma(w.y, w.y, nrm));
+    }
+    if (DOTS) {
+      const ffn2 p = ff2_split(w);
+      S.wr[threadIdx.x] = ff2_pack(dup_part(p, false));
+      S.wi[threadIdx.x] = ff2_pack(dup_part(p, true));
+      __syncthreads();
+      const int per = kColThreads / RG;  // rows of this warp's group
+      const int left = (int)(r1 - c0 < kColThreads ? r1 - c0 : kColThreads);
+#pragma unroll 2
+      for (int i = grp * per; i < grp * per + per && i < left; i += 32) {
+        const ffn2 wr = ff2_unpack(S.wr[i + lane]), wi = ff2_unpack(S.wi[i + lane]);
+        const bool in = i + lane < left;
+        double2 v[kCpw];
+#pragma unroll
+        for (int q = 0; q < kCpw; ++q) {
+          const int j = cw + q * CW;
+          v[q] = in && j < k ? A.V[(long long)j * n + c0 + i + lane] : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int q = 0; q < kCpw; ++q)
+          if (cw + q * CW < k) {
+            const ffn2 p = ff2_split(v[q]);
+            d1[q] = ff2_norm(ff2_fma_u(wr, p, d1[q]));
+            d2[q] = ff2_norm(ff2_fma_u(wi, p, d2[q]));
+          }
+      }
+      __syncthreads();
+    }
+  }
+  finish_pass<UPDATE, DOTS, NORM>(A, bidx, S, d1, d2, nrm);
+}
+
+template <bool UPDATE, bool DOTS, bool NORM, bool ROWS>
+__global__ void __launch_bounds__(kColThreads) k_col_pass(const __grid_constant__ ColArgs A, const int* gate,
+                                                         const int* skip) {
+  if ((gate && *gate) || (skip && *skip)) return;
+  __shared__ ColShared S;
+  if (ROWS) row_pass<UPDATE, DOTS, NORM>(A, blockIdx.x, S);
+  else col_pass<UPDATE, DOTS, NORM>(A, blockIdx.x, S);
+}
+
+template <bool UPDATE, bool DOTS, bool NORM>
+void launch_col_pass(cudaStream_t st, const ColArgs& A, const int* gate, const int* skip) {
+  if (by_rows(A.n)) k_col_pass<UPDATE, DOTS, NORM, true><<<A.nb, kColThreads, 0, st>>>(A, gate, skip);
+  else k_col_pass<UPDATE, DOTS, NORM, false><<<A.nb, kColThreads, 0, st>>>(A, gate, skip);
+}
+
 // Batched CGS2 over several handles (stab_jv_batch_orthogonalize): item i
 // owns the flat blocks [start[i], start[i+1]) (its own block count nb, so its
 // row ranges and reduction order are those of its single launch).
@@ -388,10 +747,31 @@ struct CgsItem {
   double* np;
   double* d_norm;
   const int* gate;  // per-instance gate of a batched solver (nullable)
+  unsigned* counter;
   long long n;
   int k, nb;
 };
 static_assert(sizeof(CgsItem) % 8 == 0, "items are read as 8-byte words");
+
+// the three passes of CGS2 for k <= kColMax: h1 = V^H w; w -= V h1 and
+// h2 = V^H w, h = h1 + h2; w -= V h2 and ||w||
+__host__ __device__ inline ColArgs cgs2_pass(int pass, const double2* V, int k, long long n, double2* w, double2* p1,
+                                             double2* d_h, double* np, double* d_norm, unsigned* counter, int nb) {
+  ColArgs A{};
+  A.V = V;
+  A.w = w;
+  A.k = k;
+  A.n = n;
+  A.nb = nb;
+  A.counter = counter;
+  A.h = pass == 0 ? nullptr : d_h + (pass == 1 ? 0 : k);
+  A.partial = pass < 2 ? p1 : nullptr;
+  A.out_h = d_h + (pass == 1 ? k : 0);
+  A.sum_h = pass == 1 ? d_h : nullptr;
+  A.npart = np;
+  A.out_norm = d_norm;
+  return A;
+}
 
 __device__ __forceinline__ int cgs_item(const int* __restrict__ start, int count, unsigned b) {
   int lo = 0, hi = count - 1;  // largest i with start[i] <= b
@@ -401,6 +781,19 @@ __device__ __forceinline__ int cgs_item(const int* __restrict__ start, int count
     else hi = mid - 1;
   }
   return lo;
+}
+
+template <int PASS, bool ROWS>
+__global__ void __launch_bounds__(kColThreads) k_col_pass_batch(const CgsItem* __restrict__ items,
+                                                               const int* __restrict__ start, int count) {
+  __shared__ ColShared S;
+  const int i = cgs_item(start, count, blockIdx.x);
+  const CgsItem it = items[i];
+  if (it.gate && *it.gate) return;
+  const ColArgs A = cgs2_pass(PASS, it.V, it.k, it.n, it.w, it.p1, it.d_h, it.np, it.d_norm, it.counter, it.nb);
+  const unsigned b = blockIdx.x - (unsigned)__ldg(start + i);
+  if (ROWS) row_pass<PASS != 0, PASS != 2, PASS == 2>(A, b, S);
+  else col_pass<PASS != 0, PASS != 2, PASS == 2>(A, b, S);
 }
 
 __global__ void __launch_bounds__(kThreads) k_cgs2_a_batch(const CgsItem* __restrict__ items,
@@ -639,6 +1032,12 @@ int cgs_blocks(long long n) {
   return (int)(b < 1 ? 1 : b);
 }
 
+// block count that the partial-sum buffers are laid out for: either kind of pass
+int part_blocks(long long n) {
+  const long long c = (n + 31) / 32;
+  return std::max(cgs_blocks(n), (int)(c < 152 ? c : 152));
+}
+
 int red_blocks(long long n) {
   long long b = (n + kThreads - 1) / kThreads;
   if (b > 152 * 4) b = 152 * 4;
@@ -652,6 +1051,9 @@ int grid_n(long long n) {
 }
 
 }  // namespace
+
+// completion counter of the Gram-Schmidt passes (zeroed at set-up, left at zero by every pass)
+static unsigned* col_counter(StabHandle* h) { return (unsigned*)(h->d_red + h->red_blocks + 16); }
 
 cudaError_t kry_dot(StabHandle* h, const double2* V, int k, long long n, const double2* w, double2* d_h,
                             double2* partial, int accumulate) {
@@ -679,13 +1081,21 @@ cudaError_t kry_gemv_add(StabHandle* h, const double2* V, int k, long long n, co
 // the norm partials); d_h holds 2k complex.
 cudaError_t kry_cgs2(StabHandle* h, const double2* V, int k, long long n, double2* w, double2* d_h, double* d_norm,
                      double2* partial) {
-  const int nb = cgs_blocks(n);
+  const int nb = cgs_blocks(n), pb = part_blocks(n);
   double2* p1 = partial;
-  double2* p2 = partial + (size_t)nb * (k > 0 ? k : 1);
-  double* np = (double*)(p2 + (size_t)nb * (k > 0 ? k : 1));
+  double2* p2 = partial + (size_t)pb * (k > 0 ? k : 1);
+  double* np = (double*)(p2 + (size_t)pb * (k > 0 ? k : 1));
   const int ts = phase_begin(h, STAB_PHASE_CGS2);
   cudaError_t e;
-  if (k > 0) {
+  if (k > 0 && k <= kColMax) {
+    const int cb = col_blocks(n, k);
+    unsigned* counter = col_counter(h);
+    auto args = [&](int pass) { return cgs2_pass(pass, V, k, n, w, p1, d_h, np, d_norm, counter, cb); };
+    launch_col_pass<false, true, false>(h->stream, args(0), h->gate, nullptr);
+    launch_col_pass<true, true, false>(h->stream, args(1), h->gate, nullptr);
+    launch_col_pass<true, false, true>(h->stream, args(2), h->gate, nullptr);
+    e = cudaGetLastError();
+  } else if (k > 0) {
     const size_t sm = (size_t)k * (sizeof(double2) + 2 * sizeof(ffn));
     k_cgs2_a<<<nb, kThreads, 0, h->stream>>>(V, k, n, w, p1, h->gate);
     k_cgs2_b<<<nb, kThreads, sm, h->stream>>>(V, k, n, w, p1, p2, d_h, h->gate);
@@ -722,7 +1132,7 @@ cudaError_t kry_update_basis(StabHandle* h, double2* V, int m, int kk, long long
 }
 
 int kry_dgks_partial_elems(long long n, int k) {
-  const int nb = cgs_blocks(n);
+  const int nb = part_blocks(n);
   return 2 * nb * (k > 0 ? k : 1) + (3 * nb + 1) / 2 + 2;
 }
 
@@ -732,13 +1142,43 @@ cudaError_t kry_dgks(StabHandle* h, const double2* V, int k, long long n, double
                      double2* partial) {
   if (k <= 0) return kry_cgs2(h, V, k, n, w, d_h, d_norm, partial);
   const int ts = phase_begin(h, STAB_PHASE_CGS2);
-  const int nb = cgs_blocks(n);
+  const int nb = cgs_blocks(n), pb = part_blocks(n);
   double2* p1 = partial;
-  double2* p2 = partial + (size_t)nb * k;
-  double* np0 = (double*)(p2 + (size_t)nb * k);
-  double* np1 = np0 + nb;
-  double* np2 = np1 + nb;
-  int* skip = (int*)(np2 + nb);
+  double2* p2 = partial + (size_t)pb * k;
+  double* np0 = (double*)(p2 + (size_t)pb * k);
+  double* np1 = np0 + pb;
+  double* np2 = np1 + pb;
+  int* skip = (int*)(np2 + pb);
+  if (k <= kColMax) {
+    // the update takes the second pass's products along (no extra read of V); the second update runs
+    // only when the first one cancelled
+    const int cb = col_blocks(n, k);
+    ColArgs A{};
+    A.V = V;
+    A.w = w;
+    A.k = k;
+    A.n = n;
+    A.nb = cb;
+    A.counter = col_counter(h);
+    A.partial = p1;
+    A.npart = np0;
+    A.out_h = d_h;
+    A.out_norm = np2;  // ||w|| before
+    launch_col_pass<false, true, true>(h->stream, A, h->gate, nullptr);
+    A.h = d_h;
+    A.out_h = d_h + k;
+    A.out_norm = d_norm;
+    A.ref_norm = np2;
+    A.skip = skip;
+    launch_col_pass<true, true, true>(h->stream, A, h->gate, nullptr);
+    A.h = d_h + k;
+    A.partial = nullptr;
+    A.skip = nullptr;
+    A.sum_h = d_h;
+    launch_col_pass<true, false, true>(h->stream, A, h->gate, skip);
+    phase_end(h, ts);
+    return cudaGetLastError();
+  }
   const size_t sm = (size_t)k * (sizeof(double2) + 2 * sizeof(ffn));
   constexpr double eta = 0.70710678118654752;
   k_dgks_dots<double2><<<nb, kThreads, 0, h->stream>>>(V, k, n, w, p1, np0, h->gate, nullptr);
@@ -802,7 +1242,7 @@ cudaError_t kry_init_attributes() {
 }
 
 int kry_partial_elems(long long n, int k) {
-  const int nb = cgs_blocks(n);
+  const int nb = part_blocks(n);
   return 2 * nb * (k > 0 ? k : 1) + (nb + 1) / 2 + 1;
 }
 
@@ -829,29 +1269,36 @@ cudaError_t kry_cgs2_stream(cudaStream_t st, const double2* V, int k, long long 
 
 // Parameter image of a batched CGS2 (job i gated by J.gate) and its launches.
 cudaError_t cgs2_batch_plan(const std::vector<CgsJob>& jobs, BatchImage& im, CgsBatchPlan& plan) {
-  std::vector<CgsItem> items;
-  std::vector<int> blocks, ones;
+  std::vector<CgsItem> items, cols[2];  // k > kColMax; k <= kColMax by columns, by rows
+  std::vector<int> blocks, ones, col_bl[2];
   size_t sm = 0;
   for (const CgsJob& J : jobs) {
     if (J.k < 1) return cudaErrorInvalidValue;
-    const int nb = cgs_blocks(J.n);
+    const int pb = part_blocks(J.n);
     CgsItem it{};
     it.V = J.V;
     it.w = J.w;
     it.p1 = J.partial;
-    it.p2 = J.partial + (size_t)nb * J.k;
-    it.np = (double*)(it.p2 + (size_t)nb * J.k);
+    it.p2 = J.partial + (size_t)pb * J.k;
+    it.np = (double*)(it.p2 + (size_t)pb * J.k);
     it.d_h = J.d_h;
     it.d_norm = J.d_norm;
     it.gate = J.gate;
+    it.counter = col_counter(J.h);
     it.n = J.n;
     it.k = J.k;
-    it.nb = nb;
+    it.nb = J.k <= kColMax ? col_blocks(J.n, J.k) : cgs_blocks(J.n);
+    if (J.k <= kColMax) {
+      cols[by_rows(J.n)].push_back(it);
+      col_bl[by_rows(J.n)].push_back(it.nb);
+      continue;
+    }
     items.push_back(it);
-    blocks.push_back(nb);
+    blocks.push_back(it.nb);
     ones.push_back(1);
     sm = std::max(sm, (size_t)J.k * (sizeof(double2) + 2 * sizeof(ffn)));
   }
+  for (int r = 0; r < 2; ++r) plan.C[r] = im.section(cols[r], col_bl[r], kColThreads, 0);
   plan.S = im.section(items, blocks, kThreads, sm);
   plan.N = im.section(items, ones, 32, 0);
   plan.sm = sm;
@@ -859,13 +1306,25 @@ cudaError_t cgs2_batch_plan(const std::vector<CgsJob>& jobs, BatchImage& im, Cgs
 }
 
 cudaError_t cgs2_batch_launch(const CgsBatchPlan& plan, const unsigned char* d, cudaStream_t st) {
-  if (!plan.S.count) return cudaSuccess;
-  const CgsItem* it = (const CgsItem*)(d + plan.S.items);
-  const int* sp = (const int*)(d + plan.S.start);
-  k_cgs2_a_batch<<<plan.S.blocks, kThreads, 0, st>>>(it, sp, plan.S.count);
-  k_cgs2_b_batch<<<plan.S.blocks, kThreads, plan.sm, st>>>(it, sp, plan.S.count);
-  k_cgs2_c_batch<<<plan.S.blocks, kThreads, plan.sm, st>>>(it, sp, plan.S.count);
-  k_norm_final_batch<<<plan.N.count, 32, 0, st>>>((const CgsItem*)(d + plan.N.items), plan.N.count);
+  auto pass = [&](auto by_col, auto by_row) {
+    if (plan.C[0].count)
+      by_col<<<plan.C[0].blocks, kColThreads, 0, st>>>((const CgsItem*)(d + plan.C[0].items),
+                                                       (const int*)(d + plan.C[0].start), plan.C[0].count);
+    if (plan.C[1].count)
+      by_row<<<plan.C[1].blocks, kColThreads, 0, st>>>((const CgsItem*)(d + plan.C[1].items),
+                                                       (const int*)(d + plan.C[1].start), plan.C[1].count);
+  };
+  pass(k_col_pass_batch<0, false>, k_col_pass_batch<0, true>);
+  pass(k_col_pass_batch<1, false>, k_col_pass_batch<1, true>);
+  pass(k_col_pass_batch<2, false>, k_col_pass_batch<2, true>);
+  if (plan.S.count) {
+    const CgsItem* it = (const CgsItem*)(d + plan.S.items);
+    const int* sp = (const int*)(d + plan.S.start);
+    k_cgs2_a_batch<<<plan.S.blocks, kThreads, 0, st>>>(it, sp, plan.S.count);
+    k_cgs2_b_batch<<<plan.S.blocks, kThreads, plan.sm, st>>>(it, sp, plan.S.count);
+    k_cgs2_c_batch<<<plan.S.blocks, kThreads, plan.sm, st>>>(it, sp, plan.S.count);
+    k_norm_final_batch<<<plan.N.count, 32, 0, st>>>((const CgsItem*)(d + plan.N.items), plan.N.count);
+  }
   return cudaGetLastError();
 }
 

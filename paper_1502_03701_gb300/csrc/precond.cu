@@ -365,6 +365,8 @@ struct BtApplyParams {
   double2* z;
   const void* F;
   int m, nlev, tx, ty, tz, ntx, nty, nx, ny;
+  int staged;    // k_bt_rhs: the level's matrix goes through shared memory
+  FastDiv divc;  // 16-byte chunks per matrix row
   long long npts;
   const int* gate;
 };
@@ -385,43 +387,39 @@ __device__ __forceinline__ int bt_group(int m) {
   return G;
 }
 
-// w_l = S_l^{-1} q_l for every level of every tile, into z (grid: tiles x levels).
-// KP > 0: each thread's row fragment (at most KP entries) is loaded in one
-// unrolled batch, so all its loads are in flight together.
-template <class R, bool Q32, int KP>
-__global__ void __launch_bounds__(256) k_bt_rhs(const BtApplyParams P) {
-  if (P.gate && *P.gate) return;
-  extern __shared__ unsigned char smraw[];
-  C2<R>* t = (C2<R>*)smraw;
-  const int m = P.m, l = blockIdx.y;
-  const long long tile = blockIdx.x, mm = (long long)m * m;
-  const C2<R>* S = (const C2<R>*)P.F + (tile * P.nlev + l) * 3 * mm + mm;
-  for (int r = threadIdx.x; r < m; r += blockDim.x) {
-    const long long d = bt_dof(P, tile, l, r);
-    if (Q32) { const float2 v = P.q32[d]; t[r] = C2<R>{(R)v.x, (R)v.y}; }
-    else { const double2 v = P.q[d]; t[r] = C2<R>{(R)v.x, (R)v.y}; }
+// Shared-memory pitch (in complex values) of a staged level matrix: 16-byte
+// aligned rows, and the rows that half a warp reads together (16 / G of them, G
+// consecutive entries each) in different banks.
+template <class R>
+__host__ __device__ constexpr int bt_pitch(int m, int G) {
+  const int per = 128 / (int)sizeof(C2<R>);  // values per 32 banks
+  const int step = G < 2 ? 2 : G;
+  return (m + per - 1) / per * per + step;
+}
+
+// Queue the copy of an m x m row-major matrix into shared memory (cp.async,
+// 16 bytes at a time: every request is a run of whole sectors; the products
+// themselves read 8 rows x 32 bytes per request, which kept the L1 tag stage busy
+// for about 1,000 cycles per level when they went to global memory).
+template <class R>
+__device__ __forceinline__ void bt_stage(C2<R>* dst, int pitch, const C2<R>* src, int m, const FastDiv& divc) {
+  constexpr int per = 16 / (int)sizeof(C2<R>);
+  const int chunks = m / per;  // per row
+  for (int i = threadIdx.x; i < m * chunks; i += blockDim.x) {
+    const int r = (int)fdiv(i, divc), c = i - r * chunks;
+    const unsigned s = (unsigned)__cvta_generic_to_shared(dst + r * pitch + c * per);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src + (long long)r * m + c * per) : "memory");
   }
-  __syncthreads();
-  const int G = bt_group(m);
-  const int row = threadIdx.x / G, g = threadIdx.x % G;
+}
+
+// (M x)_row over this thread's entries g, g + G, ..., then over the row's G threads
+template <class R>
+__device__ __forceinline__ C2<R> bt_product(const C2<R>* Mrow, const C2<R>* x, int m, int g, int G, bool act) {
   R sx = 0, sy = 0;
-  if (KP > 0) {
-    C2<R> a[KP > 0 ? KP : 1];
-#pragma unroll
-    for (int j = 0; j < KP; ++j) {
-      const int k = g + j * G;
-      a[j] = (row < m && k < m) ? S[(long long)row * m + k] : C2<R>{0, 0};
-    }
-#pragma unroll
-    for (int j = 0; j < KP; ++j) {
-      const int k = g + j * G;
-      const C2<R> b = k < m ? t[k] : C2<R>{0, 0};
-      sx += a[j].x * b.x - a[j].y * b.y;
-      sy += a[j].x * b.y + a[j].y * b.x;
-    }
-  } else if (row < m) {
+  if (act) {
+#pragma unroll 4
     for (int k = g; k < m; k += G) {
-      const C2<R> a = S[(long long)row * m + k], b = t[k];
+      const C2<R> a = Mrow[k], b = x[k];
       sx += a.x * b.x - a.y * b.y;
       sy += a.x * b.y + a.y * b.x;
     }
@@ -430,110 +428,147 @@ __global__ void __launch_bounds__(256) k_bt_rhs(const BtApplyParams P) {
     sx += __shfl_xor_sync(0xffffffffu, sx, o);
     sy += __shfl_xor_sync(0xffffffffu, sy, o);
   }
-  if (row < m && g == 0) P.z[bt_dof(P, tile, l, row)] = make_double2((double)sx, (double)sy);
+  return C2<R>{sx, sy};
+}
+
+// w_l = S_l^{-1} q_l for every level of every tile, into z (grid: tiles x levels).
+template <class R, bool Q32>
+__global__ void __launch_bounds__(256) k_bt_rhs(const __grid_constant__ BtApplyParams P) {
+  if (P.gate && *P.gate) return;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int m = P.m, l = blockIdx.y;
+  const int G = bt_group(m), lg = __ffs(G) - 1, row = threadIdx.x >> lg, g = threadIdx.x & (G - 1);
+  const int pitch = bt_pitch<R>(m, G);
+  C2<R>* Ms = (C2<R>*)smraw;
+  C2<R>* t = Ms + (P.staged ? m * pitch : 0);
+  const long long tile = blockIdx.x, mm = (long long)m * m;
+  const C2<R>* S = (const C2<R>*)P.F + (tile * P.nlev + l) * 3 * mm + mm;
+  if (P.staged) {
+    bt_stage<R>(Ms, pitch, S, m, P.divc);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  for (int r = threadIdx.x; r < m; r += blockDim.x) {
+    const long long d = bt_dof(P, tile, l, r);
+    if (Q32) { const float2 v = P.q32[d]; t[r] = C2<R>{(R)v.x, (R)v.y}; }
+    else { const double2 v = P.q[d]; t[r] = C2<R>{(R)v.x, (R)v.y}; }
+  }
+  const bool act = row < m;
+  double2* z = P.z + (act && g == 0 ? bt_dof(P, tile, l, row) : 0);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  const C2<R>* Mr = P.staged ? Ms + row * pitch : S + (long long)row * m;
+  const C2<R> s = bt_product<R>(Mr, t, m, g, G, act);
+  if (act && g == 0) *z = make_double2((double)s.x, (double)s.y);
 }
 
 // The level recurrences of one tile (one CTA per tile), z holding w on entry:
-// forward y_l = w_l - P_l y_{l-1}, backward x_l = y_l - X_l x_{l+1}.  Each row's
-// product is split over G threads; with KP > 0 every thread holds its
-// fragment (at most KP entries) of the next level's matrix and the next w in
-// registers, loaded while the current level is reduced, so the dependency
-// chain carries no global-memory latency.
-template <class R, int KP>
-__global__ void __launch_bounds__(256) k_bt_sweep(const BtApplyParams P) {
+// forward y_l = w_l - P_l y_{l-1}, backward x_l = y_l - X_l x_{l+1}.  The chain is a
+// level's product, a shuffle sum and a barrier; the levels' matrices stream
+// through a ring of STAGES shared-memory buffers, STAGES - 1 levels ahead, and a
+// thread's right-hand sides one ring ahead in registers.  A row's unknowns of
+// consecutive levels are 2 nx apart, so their address is formed once (eight
+// integer divisions that used to run three times per level).  128 x 256 layer in
+// 8 x 64 tiles (64 tiles, 32 levels of 64 unknowns): 139 us before.
+template <class R, int STAGES>
+__global__ void __launch_bounds__(256) k_bt_sweep(const __grid_constant__ BtApplyParams P) {
   if (P.gate && *P.gate) return;
-  extern __shared__ unsigned char smraw[];
-  C2<R>* va = (C2<R>*)smraw;
-  C2<R>* vb = va + P.m;
+  extern __shared__ __align__(16) unsigned char smraw[];
   const int m = P.m, nlev = P.nlev;
+  const int G = bt_group(m), lg = __ffs(G) - 1, row = threadIdx.x >> lg, g = threadIdx.x & (G - 1);
+  const int pitch = bt_pitch<R>(m, G);
+  const bool act = row < m, lead = act && g == 0;
   const long long tile = blockIdx.x, mm = (long long)m * m;
   const C2<R>* Ft = (const C2<R>*)P.F + tile * nlev * 3 * mm;
-  const int G = bt_group(m);
-  const int row = threadIdx.x / G, g = threadIdx.x % G;
-  const bool act = row < m, lead = act && g == 0;
-  C2<R> cur[KP > 0 ? KP : 1], nxt[KP > 0 ? KP : 1];
-  auto fetch = [&](C2<R>* frag, const C2<R>* M) {
-#pragma unroll
-    for (int j = 0; j < KP; ++j) {
-      const int k = g + j * G;
-      frag[j] = (act && k < m) ? M[(long long)row * m + k] : C2<R>{0, 0};
-    }
-  };
-  // (M x)_row from registers (KP > 0) or from memory, complete in every lane of the row's group
-  auto mv = [&](const C2<R>* frag, const C2<R>* M, const C2<R>* x) {
-    R sx = 0, sy = 0;
-    if (KP > 0) {
-#pragma unroll
-      for (int j = 0; j < KP; ++j) {
-        const int k = g + j * G;
-        const C2<R> b = k < m ? x[k] : C2<R>{0, 0};
-        sx += frag[j].x * b.x - frag[j].y * b.y;
-        sy += frag[j].x * b.y + frag[j].y * b.x;
+  constexpr bool kStaged = STAGES > 0;
+  constexpr int kAhead = kStaged ? STAGES - 1 : 1;
+  C2<R>* ring = (C2<R>*)smraw;
+  C2<R>* yp = ring + (size_t)STAGES * m * pitch;
+  C2<R>* yc = yp + m;
+  double2* z = P.z + (act ? bt_dof(P, tile, 0, row) : 0);
+  const long long dz = 2LL * P.nx;
+  // one direction: level i of count is first + dir i, its matrix at M + 3 mm l
+  auto sweep = [&](const C2<R>* M, int first, int dir, int count) {
+    double2 rhs[kAhead];
+    auto fetch = [&](int i) {
+      const int l = first + dir * i;
+      if (kStaged) {
+        if (i < count) bt_stage<R>(ring + (size_t)(i % (kStaged ? STAGES : 1)) * m * pitch, pitch, M + 3 * mm * l, m, P.divc);
+        asm volatile("cp.async.commit_group;" ::: "memory");
       }
-    } else if (act) {
-      for (int k = g; k < m; k += G) {
-        const C2<R> a = M[(long long)row * m + k], b = x[k];
-        sx += a.x * b.x - a.y * b.y;
-        sy += a.x * b.y + a.y * b.x;
+      return lead && i < count ? z[l * dz] : make_double2(0.0, 0.0);
+    };
+#pragma unroll
+    for (int d = 0; d < kAhead; ++d) rhs[d] = fetch(d);
+    for (int i0 = 0; i0 < count; i0 += kAhead) {
+#pragma unroll
+      for (int d = 0; d < kAhead; ++d) {
+        const int i = i0 + d;
+        if (i >= count) break;
+        if (kStaged) asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
+        __syncthreads();  // this level's matrix and the previous level's y; the previous buffer is free
+        const double2 w = rhs[d];
+        rhs[d] = fetch(i + kAhead);
+        const int l = first + dir * i;
+        const C2<R>* Mr = kStaged ? ring + ((size_t)(i % (kStaged ? STAGES : 1)) * m + row) * pitch
+                                  : M + 3 * mm * l + (long long)(act ? row : 0) * m;
+        const C2<R> s = bt_product<R>(Mr, yp, m, g, G, act);
+        if (lead) {
+          const C2<R> y = {(R)w.x - s.x, (R)w.y - s.y};
+          yc[row] = y;
+          z[l * dz] = make_double2((double)y.x, (double)y.y);
+        }
+        C2<R>* tmp = yp; yp = yc; yc = tmp;
       }
     }
-    for (int o = G >> 1; o > 0; o >>= 1) {
-      sx += __shfl_xor_sync(0xffffffffu, sx, o);
-      sy += __shfl_xor_sync(0xffffffffu, sy, o);
-    }
-    return C2<R>{sx, sy};
+    if (kStaged) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // the ring and y are free / complete
   };
   // forward: y_0 = w_0
-  C2<R>* yp = va;
-  C2<R>* yc = vb;
-  double2 wn = make_double2(0.0, 0.0);
   if (lead) {
-    const double2 w = P.z[bt_dof(P, tile, 0, row)];
+    const double2 w = z[0];
     yp[row] = C2<R>{(R)w.x, (R)w.y};
-    if (nlev > 1) wn = P.z[bt_dof(P, tile, 1, row)];
   }
-  if (KP > 0 && nlev > 1) fetch(nxt, Ft + 3 * mm);
-  __syncthreads();
-  for (int l = 1; l < nlev; ++l) {
-    const C2<R>* Pl = Ft + (long long)l * 3 * mm;
-    const double2 w = wn;
-    if (KP > 0) {
-#pragma unroll
-      for (int j = 0; j < KP; ++j) cur[j] = nxt[j];
-      if (l + 1 < nlev) fetch(nxt, Pl + 3 * mm);
-    }
-    if (lead && l + 1 < nlev) wn = P.z[bt_dof(P, tile, l + 1, row)];
-    const C2<R> s = mv(cur, Pl, yp);
-    if (lead) {
-      const C2<R> y = {(R)w.x - s.x, (R)w.y - s.y};
-      yc[row] = y;
-      P.z[bt_dof(P, tile, l, row)] = make_double2((double)y.x, (double)y.y);
-    }
-    __syncthreads();
-    C2<R>* tmp = yp; yp = yc; yc = tmp;
-  }
+  sweep(Ft, 1, 1, nlev - 1);
   // backward: x_{nlev-1} = y_{nlev-1} (in yp)
-  if (KP > 0 && nlev > 1) fetch(nxt, Ft + (long long)(nlev - 2) * 3 * mm + 2 * mm);
-  double2 yn = make_double2(0.0, 0.0);
-  if (lead && nlev > 1) yn = P.z[bt_dof(P, tile, nlev - 2, row)];
-  for (int l = nlev - 2; l >= 0; --l) {
-    const C2<R>* Xl = Ft + (long long)l * 3 * mm + 2 * mm;
-    const double2 y = yn;
-    if (KP > 0) {
-#pragma unroll
-      for (int j = 0; j < KP; ++j) cur[j] = nxt[j];
-      if (l > 0) fetch(nxt, Xl - 3 * mm);
-    }
-    if (lead && l > 0) yn = P.z[bt_dof(P, tile, l - 1, row)];
-    const C2<R> s = mv(cur, Xl, yp);
-    if (lead) {
-      const C2<R> x = {(R)y.x - s.x, (R)y.y - s.y};
-      yc[row] = x;
-      P.z[bt_dof(P, tile, l, row)] = make_double2((double)x.x, (double)x.y);
-    }
-    __syncthreads();
-    C2<R>* tmp = yp; yp = yc; yc = tmp;
+  sweep(Ft + 2 * mm, nlev - 2, -1, nlev - 1);
+}
+
+constexpr size_t kBtSmem = 200 * 1024;
+
+template <class R>
+cudaError_t launch_bt_apply(const BtApplyParams& B0, long long ntiles, cudaStream_t st) {
+  BtApplyParams B = B0;
+  int G = 1;
+  while (G < 32 && 2 * G * B.m <= 256) G *= 2;
+  const size_t level = (size_t)B.m * bt_pitch<R>(B.m, G) * sizeof(C2<R>), vec = (size_t)B.m * sizeof(C2<R>);
+  B.divc = make_fastdiv((unsigned)(B.m * sizeof(C2<R>) / 16));
+  const dim3 grid((unsigned)ntiles, (unsigned)B.nlev);
+  // a level per CTA, two CTAs per SM at least
+  B.staged = level + vec <= kBtSmem / 2;
+  const size_t rsm = (B.staged ? level : 0) + vec;
+  if (B.q32) k_bt_rhs<R, true><<<grid, 256, rsm, st>>>(B);
+  else k_bt_rhs<R, false><<<grid, 256, rsm, st>>>(B);
+  // ring: five buffers where every tile has an SM of its own, three where two tiles share one
+  const bool alone = ntiles <= 152;
+  auto sweep = [&](auto kernel, int stages) {
+    kernel<<<(unsigned)ntiles, 256, stages * level + 2 * vec, st>>>(B);
+  };
+  if (alone && 5 * level + 2 * vec <= kBtSmem) sweep(k_bt_sweep<R, 5>, 5);
+  else if (3 * level + 2 * vec <= kBtSmem) sweep(k_bt_sweep<R, 3>, 3);
+  else sweep(k_bt_sweep<R, 0>, 0);
+  return cudaGetLastError();
+}
+
+// shared-memory opt-in of the apply kernels (set at the build, never during a stream capture)
+template <class R>
+cudaError_t bt_attributes() {
+  const void* ks[5] = {(const void*)k_bt_rhs<R, true>, (const void*)k_bt_rhs<R, false>, (const void*)k_bt_sweep<R, 5>,
+                       (const void*)k_bt_sweep<R, 3>, (const void*)k_bt_sweep<R, 0>};
+  for (const void* k : ks) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBtSmem);
+    if (e != cudaSuccess) return e;
   }
+  return cudaSuccess;
 }
 
 struct ApplyParams {
@@ -1138,6 +1173,7 @@ cudaError_t pc_build_reduced(StabHandle* h, const Geo& g, double2 sigma) {
   cudaError_t e;
   if ((e = ensure_reduced(h)) != cudaSuccess) return e;
   const int prec = h->opts.precond_prec == 64 ? 64 : 32;
+  if ((e = prec == 64 ? bt_attributes<double>() : bt_attributes<float>()) != cudaSuccess) return e;
   const size_t esz = prec == 64 ? sizeof(double2) : sizeof(float2);
   const size_t per = (size_t)bg.nlev * 3 * bg.m * bg.m;  // complex values per tile
   if (!h->d_pinv || h->ntiles != g.ntiles || h->bsize != -(long long)bg.m * bg.nlev || h->pprec != prec) {
@@ -1276,35 +1312,9 @@ cudaError_t pc_apply(StabHandle* h, const double2* q, double2* z, const float2* 
     B.m = bg.m; B.nlev = bg.nlev; B.tx = g.tx; B.ty = g.ty; B.tz = g.tz; B.ntx = g.ntx; B.nty = g.nty;
     B.nx = h->nx; B.ny = h->ny; B.npts = h->npts; B.gate = h->gate;
     const int ts = phase_begin(h, STAB_PHASE_PRECOND_APPLY);
-    const dim3 grid_rhs((unsigned)g.ntiles, (unsigned)bg.nlev);
-    const unsigned nt = (unsigned)g.ntiles;
-    // threads per row of the 256-thread products, and the row fragment length
-    int G = 1;
-    while (G < 32 && 2 * G * bg.m <= 256) G *= 2;
-    const int frag = (bg.m + G - 1) / G;
-    if (h->pprec == 64) {
-      const size_t sm = 2 * bg.m * sizeof(double2);
-      if (frag <= 8) {
-        if (q32) k_bt_rhs<double, true, 8><<<grid_rhs, 256, sm, h->stream>>>(B);
-        else k_bt_rhs<double, false, 8><<<grid_rhs, 256, sm, h->stream>>>(B);
-        k_bt_sweep<double, 8><<<nt, 256, sm, h->stream>>>(B);
-      } else {
-        if (q32) k_bt_rhs<double, true, 0><<<grid_rhs, 256, sm, h->stream>>>(B);
-        else k_bt_rhs<double, false, 0><<<grid_rhs, 256, sm, h->stream>>>(B);
-        k_bt_sweep<double, 0><<<nt, 256, sm, h->stream>>>(B);
-      }
-    } else {
-      const size_t sm = 2 * bg.m * sizeof(float2);
-      if (frag <= 16) {
-        if (q32) k_bt_rhs<float, true, 16><<<grid_rhs, 256, sm, h->stream>>>(B);
-        else k_bt_rhs<float, false, 16><<<grid_rhs, 256, sm, h->stream>>>(B);
-        k_bt_sweep<float, 16><<<nt, 256, sm, h->stream>>>(B);
-      } else {
-        if (q32) k_bt_rhs<float, true, 0><<<grid_rhs, 256, sm, h->stream>>>(B);
-        else k_bt_rhs<float, false, 0><<<grid_rhs, 256, sm, h->stream>>>(B);
-        k_bt_sweep<float, 0><<<nt, 256, sm, h->stream>>>(B);
-      }
-    }
+    const cudaError_t e = h->pprec == 64 ? launch_bt_apply<double>(B, g.ntiles, h->stream)
+                                         : launch_bt_apply<float>(B, g.ntiles, h->stream);
+    if (e != cudaSuccess) return e;
     phase_end(h, ts);
     return cudaGetLastError();
   }

@@ -1766,12 +1766,15 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
     cudaEventCreate(&e1);
     PassParams P{};
     P.ff = h->stencil_ff;
-    LineCfg best{};
-    double best_ms = 1e300;
     const int n = h->ax[ax].n;
     // with a y-only base flow the pair-arithmetic pass runs, which has no kinds variants
     const bool fast = h->homog && h->d_coef && !h->force_dn_path;
     auto pass = [&]() { return fast ? run_pair_pass(h, ax, src) : run_pass(h, ax, P, jobs); };
+    struct Candidate {
+      LineCfg cfg;
+      float ms;
+    };
+    std::vector<Candidate> cand;
     for (int kp : {1, 2, 3}) {
       if (fast && kp != 3) continue;
       for (int C : {16, 32, 64}) {
@@ -1788,27 +1791,31 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
             cudaGetLastError();
             continue;
           }
-          // three back-to-back launches per sample (less launch and clock noise), best of five samples
-          float best_t = 1e30f;
-          for (int r = 0; r < 5 && err == cudaSuccess; ++r) {
-            cudaEventRecord(e0, h->stream);
-            for (int q = 0; q < 3 && err == cudaSuccess; ++q) err = pass();
-            cudaEventRecord(e1, h->stream);
-            cudaEventSynchronize(e1);
-            float t = 0.f;
-            cudaEventElapsedTime(&t, e0, e1);
-            best_t = std::min(best_t, t / 3.0f);
-          }
-          if (err != cudaSuccess) break;
-          if (best_t < best_ms) { best_ms = best_t; best = LineCfg{C, L, kp}; }
+          cand.push_back(Candidate{LineCfg{C, L, kp}, 1e30f});
         }
+      }
+    }
+    // five rounds over all candidates (a clock that is still rising then favours none of them), three
+    // back-to-back launches per sample (less launch noise), best sample of each
+    for (int r = 0; r < 5 && err == cudaSuccess; ++r)
+      for (Candidate& c : cand) {
+        h->line_cfg[ax] = c.cfg;
+        cudaEventRecord(e0, h->stream);
+        for (int q = 0; q < 3 && err == cudaSuccess; ++q) err = pass();
+        cudaEventRecord(e1, h->stream);
+        cudaEventSynchronize(e1);
+        float t = 0.f;
+        cudaEventElapsedTime(&t, e0, e1);
+        c.ms = std::min(c.ms, t / 3.0f);
         if (err != cudaSuccess) break;
       }
-      if (err != cudaSuccess) break;
-    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (err != cudaSuccess) break;
+    LineCfg best{};
+    double best_ms = 1e300;
+    for (const Candidate& c : cand)
+      if (c.ms < best_ms) { best_ms = c.ms; best = c.cfg; }
     h->line_cfg[ax] = best;
     if (ms_out) ms_out[ax] = best_ms;
     std::lock_guard<std::mutex> lk(g_tune_mu);

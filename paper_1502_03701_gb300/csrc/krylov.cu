@@ -86,7 +86,10 @@ __global__ void __launch_bounds__(kThreads) k_gemv(const double2* __restrict__ V
 // x = x / *d_norm  (into out if given); gate as in the J v kernels
 __global__ void k_scale_inv(double2* x, long long n, const double* d_norm, double2* out, const int* gate) {
   if (gate && *gate) return;
-  const double s = 1.0 / *d_norm;
+  __shared__ double s_inv;  // one division per block: FP64 divisions in every thread took most of the time
+  if (threadIdx.x == 0) s_inv = 1.0 / *d_norm;
+  __syncthreads();
+  const double s = s_inv;
   double2* o = out ? out : x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     double2 v = x[i];
@@ -458,21 +461,27 @@ __device__ __forceinline__ void finish_pass(const ColArgs& A, unsigned bidx, Col
   const int cw = wid % CW;
   // block sums
   if (DOTS) {
+    // the four columns' sums over the lanes together: the first two steps halve the columns that a
+    // lane carries, so six exchanges serve all of them; lanes 0, 8, 16, 24 end with columns 0..3
+    ffn2 t[kCpw];
 #pragma unroll
     for (int q = 0; q < kCpw; ++q) {
-      if (cw + q * CW >= k) continue;  // warp-uniform
-      ffn2 t = swap_parts(d2[q]);      // (im, re) of d2
       ffn2 a = d1[q];
       a.hi.y = -a.hi.y;
       a.lo.y = -a.lo.y;
-      t = ff2_add(a, t);  // (d1.re + d2.im, d2.re - d1.im)
-      for (int o = 16; o > 0; o >>= 1) {
-        const ffn2 u{make_float2(__shfl_xor_sync(0xffffffffu, t.hi.x, o), __shfl_xor_sync(0xffffffffu, t.hi.y, o)),
-                     make_float2(__shfl_xor_sync(0xffffffffu, t.lo.x, o), __shfl_xor_sync(0xffffffffu, t.lo.y, o))};
-        t = ff2_add(t, u);
-      }
-      if (lane == 0) S.dots[wid][q] = ff2_to_d(t);
+      t[q] = ff2_add(a, swap_parts(d2[q]));  // (d1.re + d2.im, d2.re - d1.im)
     }
+    auto other = [](ffn2 x, int o) {
+      return ffn2{make_float2(__shfl_xor_sync(0xffffffffu, x.hi.x, o), __shfl_xor_sync(0xffffffffu, x.hi.y, o)),
+                  make_float2(__shfl_xor_sync(0xffffffffu, x.lo.x, o), __shfl_xor_sync(0xffffffffu, x.lo.y, o))};
+    };
+    auto choose = [](bool c, ffn2 x, ffn2 y) { return c ? x : y; };
+    const bool up = lane & 16, mid = lane & 8;
+    const ffn2 u0 = ff2_add(choose(up, t[2], t[0]), other(choose(up, t[0], t[2]), 16));
+    const ffn2 u1 = ff2_add(choose(up, t[3], t[1]), other(choose(up, t[1], t[3]), 16));
+    ffn2 v = ff2_add(choose(mid, u1, u0), other(choose(mid, u0, u1), 8));
+    for (int o = 4; o > 0; o >>= 1) v = ff2_add(v, other(v, o));
+    if ((lane & 7) == 0) S.dots[wid][lane >> 3] = ff2_to_d(v);
   }
   if (NORM) {
     nrm = warp_sum(nrm);
@@ -563,6 +572,7 @@ __device__ __forceinline__ void col_pass(const ColArgs& A, unsigned bidx, ColSha
     if (!UPDATE || cw == 0) nw = r < n ? A.w[r] : make_double2(0.0, 0.0);
   };
   fetch(row);
+  int rounds = 0;
   for (long long r0 = 32LL * bidx * RG; r0 < n; r0 += step, row += step) {  // block-uniform
     ffn2 v[kCpw];
     const double2 wold = nw;
@@ -622,9 +632,16 @@ __device__ __forceinline__ void col_pass(const ColArgs& A, unsigned bidx, ColSha
 #pragma unroll
       for (int q = 0; q < kCpw; ++q)
         if (cw + q * CW < k) {
-          d1[q] = ff2_norm(ff2_fma_u(wr, v[q], d1[q]));
-          d2[q] = ff2_norm(ff2_fma_u(wi, v[q], d2[q]));
+          d1[q] = ff2_fma_u(wr, v[q], d1[q]);
+          d2[q] = ff2_fma_u(wi, v[q], d2[q]);
         }
+      if ((++rounds & 3) == 0) {
+#pragma unroll
+        for (int q = 0; q < kCpw; ++q) {
+          d1[q] = ff2_norm(d1[q]);
+          d2[q] = ff2_norm(d2[q]);
+        }
+      }
     }
   }
   finish_pass<UPDATE, DOTS, NORM>(A, bidx, S, d1, d2, nrm);
@@ -664,12 +681,18 @@ __device__ __forceinline__ void row_pass(const ColArgs& A, unsigned bidx, ColSha
       if (UPDATE) {
         const double2* Vr = A.V + row;
         ffn2 a1 = ff2_zero2(), a2 = ff2_zero2();
-        constexpr int G = 8;  // loads in flight per thread
-        for (int j0 = 0; j0 < k; j0 += G) {
-          double2 v[G];
+        constexpr int G = 4;  // columns per step, the next step's in flight
+        double2 v[G], nx[G];
+        auto fetch = [&](int j0) {
 #pragma unroll
           for (int q = 0; q < G; ++q)
-            if (j0 + q < k) v[q] = Vr[(long long)(j0 + q) * n];
+            if (j0 + q < k) nx[q] = Vr[(long long)(j0 + q) * n];
+        };
+        fetch(0);
+        for (int j0 = 0; j0 < k; j0 += G) {
+#pragma unroll
+          for (int q = 0; q < G; ++q) v[q] = nx[q];
+          fetch(j0 + G);
 #pragma unroll
           for (int q = 0; q < G; ++q) {
             if (j0 + q >= k) break;
@@ -696,23 +719,35 @@ __device__ __forceinline__ void row_pass(const ColArgs& A, unsigned bidx, ColSha
       __syncthreads();
       const int per = kColThreads / RG;  // rows of this warp's group
       const int left = (int)(r1 - c0 < kColThreads ? r1 - c0 : kColThreads);
-#pragma unroll 2
-      for (int i = grp * per; i < grp * per + per && i < left; i += 32) {
-        const ffn2 wr = ff2_unpack(S.wr[i + lane]), wi = ff2_unpack(S.wi[i + lane]);
-        const bool in = i + lane < left;
-        double2 v[kCpw];
+      const int i1 = grp * per + per < left ? grp * per + per : left;
+      double2 v[kCpw], nx[kCpw];
+      auto fetch = [&](int i) {
 #pragma unroll
         for (int q = 0; q < kCpw; ++q) {
           const int j = cw + q * CW;
-          v[q] = in && j < k ? A.V[(long long)j * n + c0 + i + lane] : make_double2(0.0, 0.0);
+          nx[q] = i + lane < i1 && j < k ? A.V[(long long)j * n + c0 + i + lane] : make_double2(0.0, 0.0);
         }
+      };
+      fetch(grp * per);
+      for (int i = grp * per; i < i1; i += 32) {
+#pragma unroll
+        for (int q = 0; q < kCpw; ++q) v[q] = nx[q];
+        fetch(i + 32);
+        const ffn2 wr = ff2_unpack(S.wr[i + lane]), wi = ff2_unpack(S.wi[i + lane]);
 #pragma unroll
         for (int q = 0; q < kCpw; ++q)
           if (cw + q * CW < k) {
             const ffn2 p = ff2_split(v[q]);
-            d1[q] = ff2_norm(ff2_fma_u(wr, p, d1[q]));
-            d2[q] = ff2_norm(ff2_fma_u(wi, p, d2[q]));
+            d1[q] = ff2_fma_u(wr, p, d1[q]);
+            d2[q] = ff2_fma_u(wi, p, d2[q]);
           }
+        if ((i & 96) == 96) {
+#pragma unroll
+          for (int q = 0; q < kCpw; ++q) {
+            d1[q] = ff2_norm(d1[q]);
+            d2[q] = ff2_norm(d2[q]);
+          }
+        }
       }
       __syncthreads();
     }

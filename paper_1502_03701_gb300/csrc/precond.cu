@@ -366,16 +366,16 @@ struct BtApplyParams {
   const void* F;
   int m, nlev, tx, ty, tz, ntx, nty, nx, ny;
   int staged;    // k_bt_rhs: the level's matrix goes through shared memory
-  FastDiv divc;  // 16-byte chunks per matrix row
+  FastDiv divNP, divtx, divntx, divnty;  // points per level, tile width, tiles in x and y
   long long npts;
   const int* gate;
 };
 
-__device__ __forceinline__ long long bt_dof(const BtApplyParams& P, long long tile, int l, int r) {
-  const int NP = 2 * P.tx * P.tz;
-  const int tX = (int)(tile % P.ntx), tY = (int)((tile / P.ntx) % P.nty), tZ = (int)(tile / ((long long)P.ntx * P.nty));
-  const int a = r / NP, pp = r % NP;
-  const int x = tX * P.tx + pp % P.tx, y = tY * P.ty + 2 * l + (pp / P.tx) % 2, z = tZ * P.tz + pp / (2 * P.tx);
+__device__ __forceinline__ long long bt_dof(const BtApplyParams& P, unsigned tile, int l, unsigned r) {
+  const unsigned NP = 2 * P.tx * P.tz;
+  const unsigned tYZ = fdiv(tile, P.divntx), tX = tile - tYZ * P.ntx, tZ = fdiv(tYZ, P.divnty), tY = tYZ - tZ * P.nty;
+  const unsigned a = fdiv(r, P.divNP), pp = r - a * NP, py = fdiv(pp, P.divtx);
+  const unsigned x = tX * P.tx + (pp - py * P.tx), y = tY * P.ty + 2 * l + (py & 1), z = tZ * P.tz + (py >> 1);
   return (long long)a * P.npts + ((long long)z * P.ny + y) * P.nx + x;
 }
 
@@ -400,17 +400,31 @@ __host__ __device__ constexpr int bt_pitch(int m, int G) {
 // Queue the copy of an m x m row-major matrix into shared memory (cp.async,
 // 16 bytes at a time: every request is a run of whole sectors; the products
 // themselves read 8 rows x 32 bytes per request, which kept the L1 tag stage busy
-// for about 1,000 cycles per level when they went to global memory).
+// for about 1,000 cycles per level when they went to global memory).  A thread
+// keeps its column and steps over the rows.
 template <class R>
-__device__ __forceinline__ void bt_stage(C2<R>* dst, int pitch, const C2<R>* src, int m, const FastDiv& divc) {
-  constexpr int per = 16 / (int)sizeof(C2<R>);
-  const int chunks = m / per;  // per row
-  for (int i = threadIdx.x; i < m * chunks; i += blockDim.x) {
-    const int r = (int)fdiv(i, divc), c = i - r * chunks;
-    const unsigned s = (unsigned)__cvta_generic_to_shared(dst + r * pitch + c * per);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src + (long long)r * m + c * per) : "memory");
+struct BtStage {
+  int r0, rows, dst, src;  // first row, rows per step, element offsets of the first chunk
+  bool on;
+  __device__ __forceinline__ BtStage(int m, int pitch) {
+    constexpr int per = 16 / (int)sizeof(C2<R>);
+    const int chunks = m / per;  // per row, <= 256
+    rows = (int)blockDim.x / chunks;
+    r0 = (int)threadIdx.x / chunks;
+    const int c = ((int)threadIdx.x - r0 * chunks) * per;
+    on = r0 < rows;
+    dst = r0 * pitch + c;
+    src = r0 * m + c;
   }
-}
+  __device__ __forceinline__ void copy(C2<R>* to, int pitch, const C2<R>* from, int m) const {
+    if (!on) return;
+    unsigned s = (unsigned)__cvta_generic_to_shared(to + dst);
+    const C2<R>* g = from + src;
+    const unsigned ds = (unsigned)(rows * pitch * (int)sizeof(C2<R>));
+    for (int r = r0; r < m; r += rows, s += ds, g += rows * m)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(g) : "memory");
+  }
+};
 
 // (M x)_row over this thread's entries g, g + G, ..., then over the row's G threads
 template <class R>
@@ -444,7 +458,7 @@ __global__ void __launch_bounds__(256) k_bt_rhs(const __grid_constant__ BtApplyP
   const long long tile = blockIdx.x, mm = (long long)m * m;
   const C2<R>* S = (const C2<R>*)P.F + (tile * P.nlev + l) * 3 * mm + mm;
   if (P.staged) {
-    bt_stage<R>(Ms, pitch, S, m, P.divc);
+    BtStage<R>(m, pitch).copy(Ms, pitch, S, m);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
   for (int r = threadIdx.x; r < m; r += blockDim.x) {
@@ -486,13 +500,14 @@ __global__ void __launch_bounds__(256) k_bt_sweep(const __grid_constant__ BtAppl
   C2<R>* yc = yp + m;
   double2* z = P.z + (act ? bt_dof(P, tile, 0, row) : 0);
   const long long dz = 2LL * P.nx;
+  const BtStage<R> stage(m, pitch);
   // one direction: level i of count is first + dir i, its matrix at M + 3 mm l
   auto sweep = [&](const C2<R>* M, int first, int dir, int count) {
     double2 rhs[kAhead];
     auto fetch = [&](int i) {
       const int l = first + dir * i;
       if (kStaged) {
-        if (i < count) bt_stage<R>(ring + (size_t)(i % (kStaged ? STAGES : 1)) * m * pitch, pitch, M + 3 * mm * l, m, P.divc);
+        if (i < count) stage.copy(ring + (i % (kStaged ? STAGES : 1)) * m * pitch, pitch, M + 3 * mm * l, m);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
       return lead && i < count ? z[l * dz] : make_double2(0.0, 0.0);
@@ -541,7 +556,6 @@ cudaError_t launch_bt_apply(const BtApplyParams& B0, long long ntiles, cudaStrea
   int G = 1;
   while (G < 32 && 2 * G * B.m <= 256) G *= 2;
   const size_t level = (size_t)B.m * bt_pitch<R>(B.m, G) * sizeof(C2<R>), vec = (size_t)B.m * sizeof(C2<R>);
-  B.divc = make_fastdiv((unsigned)(B.m * sizeof(C2<R>) / 16));
   const dim3 grid((unsigned)ntiles, (unsigned)B.nlev);
   // a level per CTA, two CTAs per SM at least
   B.staged = level + vec <= kBtSmem / 2;
@@ -719,12 +733,25 @@ __device__ __forceinline__ void apply_rows_body(const ApplyParams& P, long long 
     const C2<R>* row = M + (long long)r * P.bsz;
     R ar = 0, ai = 0;
     if (vec) {
+      // eight 16-byte loads in flight per lane (one at a time, the 64 MB of a 32 x 64 layer's inverses
+      // came from L2 at 2.5 TB/s), added in column order
       const float4* row4 = (const float4*)row;
-      for (int c2 = lane; c2 < P.bsz / 2; c2 += 32) {
-        const float4 m = __ldg(row4 + c2);
-        const C2<R> x0 = qs[2 * c2], x1 = qs[2 * c2 + 1];
-        ar += m.x * x0.x - m.y * x0.y + m.z * x1.x - m.w * x1.y;
-        ai += m.x * x0.y + m.y * x0.x + m.z * x1.y + m.w * x1.x;
+      constexpr int G = 8;
+      const int half = P.bsz / 2;
+      for (int c0 = lane; c0 < half; c0 += 32 * G) {
+        float4 mm[G];
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+          if (c0 + 32 * q < half) mm[q] = __ldg(row4 + c0 + 32 * q);
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+          const int c2 = c0 + 32 * q;
+          if (c2 >= half) break;
+          const float4 m = mm[q];
+          const C2<R> x0 = qs[2 * c2], x1 = qs[2 * c2 + 1];
+          ar += m.x * x0.x - m.y * x0.y + m.z * x1.x - m.w * x1.y;
+          ai += m.x * x0.y + m.y * x0.x + m.z * x1.y + m.w * x1.x;
+        }
       }
     } else {
       for (int c = lane; c < P.bsz; c += 32) {
@@ -1311,6 +1338,10 @@ cudaError_t pc_apply(StabHandle* h, const double2* q, double2* z, const float2* 
     B.q = q; B.q32 = q32; B.z = z; B.F = h->d_pinv;
     B.m = bg.m; B.nlev = bg.nlev; B.tx = g.tx; B.ty = g.ty; B.tz = g.tz; B.ntx = g.ntx; B.nty = g.nty;
     B.nx = h->nx; B.ny = h->ny; B.npts = h->npts; B.gate = h->gate;
+    B.divNP = make_fastdiv((unsigned)(2 * g.tx * g.tz));
+    B.divtx = make_fastdiv((unsigned)g.tx);
+    B.divntx = make_fastdiv((unsigned)g.ntx);
+    B.divnty = make_fastdiv((unsigned)g.nty);
     const int ts = phase_begin(h, STAB_PHASE_PRECOND_APPLY);
     const cudaError_t e = h->pprec == 64 ? launch_bt_apply<double>(B, g.ntiles, h->stream)
                                          : launch_bt_apply<float>(B, g.ntiles, h->stream);

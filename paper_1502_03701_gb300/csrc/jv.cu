@@ -1475,6 +1475,9 @@ static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, bool batch, pl
   int C = cfg.C;
   if (C <= 0) C = P.lanes == 1 && chunks16 >= 152LL * 512 ? 32 : 16;
   if (C > kPairMaxC) C = kPairMaxC;
+  // fewer than two warps per SM: a pass is one warp's latency, so chunks of half the length (the x pass of a
+  // 32 x 64 layer 10.7 -> 9.3 us, its J v 45 -> 40 us)
+  if (P.lanes == 1 && 2 * P.nlines * njobs * ((n + C - 1) / C) < 152LL * 64) C /= 2;
   const int nch = (n + C - 1) / C;
   int L = cfg.L;
   if (batch) {  // one launch for uneven instances: CTAs of about 128 threads for all of them

@@ -183,7 +183,7 @@ extern "C" stab_status stab_create(stab_handle* out, const double* base_flow, in
   e = dalloc(h, &h->d_q0, h->n * sizeof(double));
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_q0, q0.data(), h->n * sizeof(double), cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess) e = jv_setup(h, q0.data());
-  if (e == cudaSuccess) e = kry_init_attributes();
+  if (e == cudaSuccess) e = kry_init_attributes(h);
   if (e != cudaSuccess) {
     g_create_err = std::string("stab_create: ") + cudaGetErrorString(e);
     stab_status st = e == cudaErrorMemoryAllocation ? STAB_ERR_OOM : STAB_ERR_CUDA;

@@ -174,6 +174,7 @@ struct StabHandle {
   // statistics
   stab_stats stats;
   PhaseTimer timer;
+  bool cluster_ok = false;  // the device schedules clusters of 16 CTAs (gram_schmidt.cuh)
   LineCfg line_cfg[3];  // per axis, from stab_autotune
   // graph capture of the GMRES cycle (solver.cu): while gate is set, the
   // gated kernels launched by jv_apply, pc_apply, kry_cgs2 and kry_scale
@@ -237,7 +238,8 @@ cudaError_t kry_scale32(StabHandle* h, float2* x, long long n, const double* d_n
 cudaError_t kry_to_f64(StabHandle* h, const float2* in, long long n, double2* out);
 cudaError_t kry_gemv32(StabHandle* h, const float2* V, int k, const int* kdev, long long n, const double2* y,
                        double2* out);
-cudaError_t kry_init_attributes();
+cudaError_t kry_init_attributes(StabHandle* h);
+bool kry_one_cluster(const StabHandle* h, long long n, int k);
 cudaError_t kry_cgs2_stream(cudaStream_t st, const double2* V, int k, long long n, double2* w, double2* d_h,
                             double* d_norm, double2* partial, double* norm_partial, int norm_blocks);
 cudaError_t launch_norm2_stream(cudaStream_t st, const double2* v, long long n, double* partial, int nb,
@@ -338,7 +340,7 @@ cudaError_t pc_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
                           const int* const* gates, BatchImage& im, PcBatchPlan& plan);
 cudaError_t pc_batch_launch(const PcBatchPlan& plan, const unsigned char* d, cudaStream_t st);
 struct CgsBatchPlan {
-  BatchSection C[2], S, N;
+  BatchSection U[2], C[2], S, N;
   size_t sm = 0;
 };
 // Order the batch's stream after the work queued so far on every handle's own

@@ -4,18 +4,15 @@
 // Vectors are complex128 (double2); a basis V of k vectors stores column j at
 // V + j*n.
 #include "internal.cuh"
-#include "pairs.cuh"
+#include "gram_schmidt.cuh"
 
 #include <algorithm>
+
+using namespace gs;
 
 namespace {
 
 constexpr int kThreads = 256;
-
-__device__ __forceinline__ double warp_sum(double x) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
 
 // partial[b * k + j] = sum over this block's rows of conj(V_j[i]) w[i]
 __global__ void __launch_bounds__(kThreads) k_dot_partial(const double2* __restrict__ V, int k, long long n,
@@ -381,380 +378,6 @@ __global__ void k_norm_final(const double* partial, int nb, double* out, const i
   norm_final_body(partial, nb, out);
 }
 
-// ---------------------------------------------------------------------------
-// Gram-Schmidt passes for up to kColMax basis vectors: V^H w (dots), w -= V h
-// (update), or both with one read of V.
-//
-// What bounds them: the basis is read from HBM once per pass, 16 bytes and
-// about 60 FP32 issue slots per entry (FP64 runs at 1/64 of the FP32 rate, so
-// products are exact FP32 two-products of split pairs on the packed FP32
-// instructions).  A CTA of 16 warps takes 32 RG rows at a time: the warps of a
-// row group (CW of them, up to four columns each) hold the group's part of V in
-// registers as pairs, add up w's correction, exchange it through shared memory
-// and take the new w's products with the same registers, so the second pass of
-// CGS2 reads V once and splits it once.  The next rows' loads are in flight
-// meanwhile.  Sums over blocks: the last block to finish adds the blocks'
-// partial sums in block order (reproducible) and resets the counter.
-// ---------------------------------------------------------------------------
-constexpr int kColThreads = 512, kColWarps = kColThreads / 32, kCpw = 4, kColMax = kColWarps * kCpw;
-
-// column warps per row group: the smallest power of two with kCpw CW >= k
-__host__ __device__ inline int col_warps(int k) {
-  int cw = 1;
-  while (cw * kCpw < k) cw *= 2;
-  return cw;
-}
-// one row per thread from 384 rows per SM up
-__host__ __device__ inline bool by_rows(long long n) { return n >= 152LL * 384; }
-int col_blocks(long long n, int k) {
-  if (by_rows(n)) return 152;
-  const long long rows = 32LL * (kColWarps / col_warps(k));
-  const long long b = (n + rows - 1) / rows;
-  return (int)(b < 152 ? (b < 1 ? 1 : b) : 152);
-}
-
-struct ColArgs {
-  const double2* V;
-  double2* w;
-  const double2* h;     // update: coefficients (null: none)
-  double2* partial;     // dots: nb x k block sums (null: none)
-  double* npart;        // |w|^2 block sums (null: none)
-  double2* out_h;       // dots: the reduced sums
-  double2* sum_h;       // added to as well when set (h1 + h2)
-  double* out_norm;     // ||w|| (of the updated w)
-  double* ref_norm;     // decide: ||w|| before the update; *skip = out >= eta ref
-  int* skip;
-  unsigned* counter;    // zero on entry, zero on exit
-  long long n;
-  int k, nb;
-};
-
-struct ColShared {
-  float4 H[kColMax][2];       // coefficients as duplicated pairs, re and im
-  union {
-    struct {
-      float4 red[kColWarps][32];  // column split: a warp's share of the correction per row, pairs re, im
-      float4 wn[kColWarps][32][2];  // the group's updated w as duplicated pairs, re and im
-    };
-    struct {
-      float4 wr[kColThreads], wi[kColThreads];  // row split: the chunk's w as duplicated pairs
-    };
-  };
-  double2 dots[kColWarps][kCpw];
-  double nrm[kColWarps];
-  int last;
-};
-
-// hi, lo of a complex value as one packed pair (re, im), and one component duplicated
-__device__ __forceinline__ ffn2 dup_part(ffn2 a, bool im) {
-  return im ? ffn2{v2(a.hi.y), v2(a.lo.y)} : ffn2{v2(a.hi.x), v2(a.lo.x)};
-}
-__device__ __forceinline__ ffn2 swap_parts(ffn2 a) {
-  return ffn2{make_float2(a.hi.y, a.hi.x), make_float2(a.lo.y, a.lo.x)};
-}
-
-template <bool UPDATE, bool DOTS, bool NORM>
-__device__ __forceinline__ void finish_pass(const ColArgs& A, unsigned bidx, ColShared& S, ffn2* d1, ffn2* d2,
-                                            double nrm) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int k = A.k, CW = col_warps(k), RG = kColWarps / CW;
-  const int cw = wid % CW;
-  // block sums
-  if (DOTS) {
-    // the four columns' sums over the lanes together: the first two steps halve the columns that a
-    // lane carries, so six exchanges serve all of them; lanes 0, 8, 16, 24 end with columns 0..3
-    ffn2 t[kCpw];
-#pragma unroll
-    for (int q = 0; q < kCpw; ++q) {
-      ffn2 a = d1[q];
-      a.hi.y = -a.hi.y;
-      a.lo.y = -a.lo.y;
-      t[q] = ff2_add(a, swap_parts(d2[q]));  // (d1.re + d2.im, d2.re - d1.im)
-    }
-    auto other = [](ffn2 x, int o) {
-      return ffn2{make_float2(__shfl_xor_sync(0xffffffffu, x.hi.x, o), __shfl_xor_sync(0xffffffffu, x.hi.y, o)),
-                  make_float2(__shfl_xor_sync(0xffffffffu, x.lo.x, o), __shfl_xor_sync(0xffffffffu, x.lo.y, o))};
-    };
-    auto choose = [](bool c, ffn2 x, ffn2 y) { return c ? x : y; };
-    const bool up = lane & 16, mid = lane & 8;
-    const ffn2 u0 = ff2_add(choose(up, t[2], t[0]), other(choose(up, t[0], t[2]), 16));
-    const ffn2 u1 = ff2_add(choose(up, t[3], t[1]), other(choose(up, t[1], t[3]), 16));
-    ffn2 v = ff2_add(choose(mid, u1, u0), other(choose(mid, u0, u1), 8));
-    for (int o = 4; o > 0; o >>= 1) v = ff2_add(v, other(v, o));
-    if ((lane & 7) == 0) S.dots[wid][lane >> 3] = ff2_to_d(v);
-  }
-  if (NORM) {
-    nrm = warp_sum(nrm);
-    if (lane == 0) S.nrm[wid] = nrm;
-  }
-  __syncthreads();
-  if (DOTS && threadIdx.x < k) {
-    const int j = threadIdx.x, c = j % CW, q = j / CW;
-    double sr = 0.0, si = 0.0;
-    for (int g = 0; g < RG; ++g) {
-      sr += S.dots[g * CW + c][q].x;
-      si += S.dots[g * CW + c][q].y;
-    }
-    A.partial[(long long)bidx * k + j] = make_double2(sr, si);
-  }
-  if (NORM && threadIdx.x == kColThreads - 1) {
-    double t = 0.0;
-    for (int g = 0; g < kColWarps; ++g) t += S.nrm[g];
-    A.npart[bidx] = t;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) S.last = atomicAdd(A.counter, 1u) == (unsigned)A.nb - 1;
-  __syncthreads();
-  if (!S.last) return;
-  __threadfence();
-  if (DOTS) {
-    for (int j = wid; j < k; j += kColWarps) {
-      double sr = 0.0, si = 0.0;
-#pragma unroll 5
-      for (int b = lane; b < A.nb; b += 32) {
-        const double2 p = __ldcg(A.partial + (long long)b * k + j);
-        sr += p.x;
-        si += p.y;
-      }
-      sr = warp_sum(sr);
-      si = warp_sum(si);
-      if (lane == 0) {
-        A.out_h[j] = make_double2(sr, si);
-        if (A.sum_h) A.sum_h[j] = make_double2(A.sum_h[j].x + sr, A.sum_h[j].y + si);
-      }
-    }
-  }
-  if (NORM && wid == kColWarps - 1) {
-    double t = 0.0;
-#pragma unroll 5
-    for (int b = lane; b < A.nb; b += 32) t += __ldcg(A.npart + b);
-    t = sqrt(warp_sum(t));
-    if (lane == 0) {
-      *A.out_norm = t;
-      if (A.skip) *A.skip = t >= 0.70710678118654752 * *A.ref_norm;  // NaN: reorthogonalise (and let the norm report it)
-    }
-  }
-  if (UPDATE && !DOTS && A.sum_h)
-    for (int j = threadIdx.x; j < k; j += kColThreads)
-      A.sum_h[j] = make_double2(A.sum_h[j].x + A.h[j].x, A.sum_h[j].y + A.h[j].y);
-  if (threadIdx.x == 0) *A.counter = 0u;
-}
-
-template <bool UPDATE, bool DOTS, bool NORM>
-__device__ __forceinline__ void col_pass(const ColArgs& A, unsigned bidx, ColShared& S) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int k = A.k, CW = col_warps(k), RG = kColWarps / CW;
-  const int grp = wid / CW, cw = wid - grp * CW;
-  const long long n = A.n;
-  if (UPDATE) {
-    for (int j = threadIdx.x; j < k; j += kColThreads) {
-      const ffn2 p = ff2_split(A.h[j]);
-      S.H[j][0] = ff2_pack(dup_part(p, false));
-      S.H[j][1] = ff2_pack(dup_part(p, true));
-    }
-    __syncthreads();
-  }
-  // conj(V_j) w = d1.re + d2.im, d2.re - d1.im with d1 += V_j re(w), d2 += V_j im(w)
-  ffn2 d1[kCpw], d2[kCpw];
-#pragma unroll
-  for (int q = 0; q < kCpw; ++q) d1[q] = d2[q] = ff2_zero2();
-  double nrm = 0.0;
-  const long long step = 32LL * RG * A.nb;
-  long long row = 32LL * ((long long)bidx * RG + grp) + lane;
-  double2 nv[kCpw], nw = make_double2(0.0, 0.0);
-  auto fetch = [&](long long r) {
-#pragma unroll
-    for (int q = 0; q < kCpw; ++q) {
-      const int j = cw + q * CW;
-      nv[q] = j < k && r < n ? A.V[(long long)j * n + r] : make_double2(0.0, 0.0);
-    }
-    if (!UPDATE || cw == 0) nw = r < n ? A.w[r] : make_double2(0.0, 0.0);
-  };
-  fetch(row);
-  int rounds = 0;
-  for (long long r0 = 32LL * bidx * RG; r0 < n; r0 += step, row += step) {  // block-uniform
-    ffn2 v[kCpw];
-    const double2 wold = nw;
-#pragma unroll
-    for (int q = 0; q < kCpw; ++q) v[q] = ff2_split(nv[q]);
-    fetch(row + step);
-    ffn2 wr, wi;
-    if (UPDATE) {
-      // V h = a1 + i a2 with a1 += V re(h), a2 += V im(h)
-      ffn2 a1 = ff2_zero2(), a2 = ff2_zero2();
-#pragma unroll
-      for (int q = 0; q < kCpw; ++q) {
-        const int j = cw + q * CW;
-        if (j < k) {
-          a1 = ff2_fma_u(ff2_unpack(S.H[j][0]), v[q], a1);
-          a2 = ff2_fma_u(ff2_unpack(S.H[j][1]), v[q], a2);
-        }
-      }
-      ffn2 s2 = swap_parts(a2);  // i a2 = (-im, re)
-      s2.hi.x = -s2.hi.x;
-      s2.lo.x = -s2.lo.x;
-      const ffn2 mine = ff2_add(a1, s2);
-      if (CW > 1) {
-        S.red[wid][lane] = ff2_pack(mine);
-        __syncthreads();
-      }
-      if (cw == 0) {
-        ffn2 t = mine;
-        for (int c = 1; c < CW; ++c) t = ff2_add(t, ff2_unpack(S.red[wid + c][lane]));
-        const double2 wnew = make_double2(wold.x - ff2_to_d(ffn{t.hi.x, t.lo.x}), wold.y - ff2_to_d(ffn{t.hi.y, t.lo.y}));
-        if (row < n) A.w[row] = wnew;
-        if (NORM) nrm = fma(wnew.x, wnew.x, fma(wnew.y, wnew.y, nrm));
-        if (DOTS) {
-          const ffn2 p = ff2_split(wnew);
-          wr = dup_part(p, false);
-          wi = dup_part(p, true);
-          if (CW > 1) {
-            S.wn[grp][lane][0] = ff2_pack(wr);
-            S.wn[grp][lane][1] = ff2_pack(wi);
-          }
-        }
-      }
-      if (CW > 1) {
-        __syncthreads();
-        if (DOTS && cw != 0) {
-          wr = ff2_unpack(S.wn[grp][lane][0]);
-          wi = ff2_unpack(S.wn[grp][lane][1]);
-        }
-      }
-    } else {
-      const ffn2 p = ff2_split(wold);
-      wr = dup_part(p, false);
-      wi = dup_part(p, true);
-      if (NORM && cw == 0) nrm = fma(wold.x, wold.x, fma(wold.y, wold.y, nrm));
-    }
-    if (DOTS) {
-#pragma unroll
-      for (int q = 0; q < kCpw; ++q)
-        if (cw + q * CW < k) {
-          d1[q] = ff2_fma_u(wr, v[q], d1[q]);
-          d2[q] = ff2_fma_u(wi, v[q], d2[q]);
-        }
-      if ((++rounds & 3) == 0) {
-#pragma unroll
-        for (int q = 0; q < kCpw; ++q) {
-          d1[q] = ff2_norm(d1[q]);
-          d2[q] = ff2_norm(d2[q]);
-        }
-      }
-    }
-  }
-  finish_pass<UPDATE, DOTS, NORM>(A, bidx, S, d1, d2, nrm);
-}
-
-// The same passes with one row per thread in the update (no exchange between
-// warps) and the products column by column afterwards: the chunk of V that the
-// update has just read (512 rows; 68 MB over all SMs at k = 55) comes back from
-// L2.  Needs enough rows to fill the threads.  With the column split, the
-// exchange of 16 warps' shares per 32 rows left 60 % of the issue slots empty at
-// k = 55 (312 us for update + products of 524,288 unknowns).
-template <bool UPDATE, bool DOTS, bool NORM>
-__device__ __forceinline__ void row_pass(const ColArgs& A, unsigned bidx, ColShared& S) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int k = A.k, CW = col_warps(k), RG = kColWarps / CW;
-  const int grp = wid / CW, cw = wid - grp * CW;
-  const long long n = A.n;
-  if (UPDATE) {
-    for (int j = threadIdx.x; j < k; j += kColThreads) {
-      const ffn2 p = ff2_split(A.h[j]);
-      S.H[j][0] = ff2_pack(dup_part(p, false));
-      S.H[j][1] = ff2_pack(dup_part(p, true));
-    }
-    __syncthreads();
-  }
-  ffn2 d1[kCpw], d2[kCpw];
-#pragma unroll
-  for (int q = 0; q < kCpw; ++q) d1[q] = d2[q] = ff2_zero2();
-  double nrm = 0.0;
-  const long long rows = ((n + A.nb - 1) / A.nb + 31) / 32 * 32;
-  const long long r0 = rows * bidx, r1 = r0 + rows < n ? r0 + rows : n;
-  for (long long c0 = r0; c0 < r1; c0 += kColThreads) {
-    const long long row = c0 + threadIdx.x;
-    double2 w = make_double2(0.0, 0.0);
-    if (row < r1) {
-      w = A.w[row];
-      if (UPDATE) {
-        const double2* Vr = A.V + row;
-        ffn2 a1 = ff2_zero2(), a2 = ff2_zero2();
-        constexpr int G = 4;  // columns per step, the next step's in flight
-        double2 v[G], nx[G];
-        auto fetch = [&](int j0) {
-#pragma unroll
-          for (int q = 0; q < G; ++q)
-            if (j0 + q < k) nx[q] = Vr[(long long)(j0 + q) * n];
-        };
-        fetch(0);
-        for (int j0 = 0; j0 < k; j0 += G) {
-#pragma unroll
-          for (int q = 0; q < G; ++q) v[q] = nx[q];
-          fetch(j0 + G);
-#pragma unroll
-          for (int q = 0; q < G; ++q) {
-            if (j0 + q >= k) break;
-            const ffn2 p = ff2_split(v[q]);
-            a1 = ff2_fma_u(ff2_unpack(S.H[j0 + q][0]), p, a1);
-            a2 = ff2_fma_u(ff2_unpack(S.H[j0 + q][1]), p, a2);
-          }
-          a1 = ff2_norm(a1);
-          a2 = ff2_norm(a2);
-        }
-        ffn2 s2 = swap_parts(a2);  // i a2 = (-im, re)
-        s2.hi.x = -s2.hi.x;
-        s2.lo.x = -s2.lo.x;
-        const double2 c = ff2_to_d(ff2_add(a1, s2));
-        w = make_double2(w.x - c.x, w.y - c.y);
-        A.w[row] = w;
-      }
-      if (NORM) nrm = fma(w.x, w.x, fma(w.y, w.y, nrm));
-    }
-    if (DOTS) {
-      const ffn2 p = ff2_split(w);
-      S.wr[threadIdx.x] = ff2_pack(dup_part(p, false));
-      S.wi[threadIdx.x] = ff2_pack(dup_part(p, true));
-      __syncthreads();
-      const int per = kColThreads / RG;  // rows of this warp's group
-      const int left = (int)(r1 - c0 < kColThreads ? r1 - c0 : kColThreads);
-      const int i1 = grp * per + per < left ? grp * per + per : left;
-      double2 v[kCpw], nx[kCpw];
-      auto fetch = [&](int i) {
-#pragma unroll
-        for (int q = 0; q < kCpw; ++q) {
-          const int j = cw + q * CW;
-          nx[q] = i + lane < i1 && j < k ? A.V[(long long)j * n + c0 + i + lane] : make_double2(0.0, 0.0);
-        }
-      };
-      fetch(grp * per);
-      for (int i = grp * per; i < i1; i += 32) {
-#pragma unroll
-        for (int q = 0; q < kCpw; ++q) v[q] = nx[q];
-        fetch(i + 32);
-        const ffn2 wr = ff2_unpack(S.wr[i + lane]), wi = ff2_unpack(S.wi[i + lane]);
-#pragma unroll
-        for (int q = 0; q < kCpw; ++q)
-          if (cw + q * CW < k) {
-            const ffn2 p = ff2_split(v[q]);
-            d1[q] = ff2_fma_u(wr, p, d1[q]);
-            d2[q] = ff2_fma_u(wi, p, d2[q]);
-          }
-        if ((i & 96) == 96) {
-#pragma unroll
-          for (int q = 0; q < kCpw; ++q) {
-            d1[q] = ff2_norm(d1[q]);
-            d2[q] = ff2_norm(d2[q]);
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-  finish_pass<UPDATE, DOTS, NORM>(A, bidx, S, d1, d2, nrm);
-}
-
 template <bool UPDATE, bool DOTS, bool NORM, bool ROWS>
 __global__ void __launch_bounds__(kColThreads) k_col_pass(const __grid_constant__ ColArgs A, const int* gate,
                                                          const int* skip) {
@@ -773,6 +396,20 @@ void launch_col_pass(cudaStream_t st, const ColArgs& A, const int* gate, const i
 // Batched CGS2 over several handles (stab_jv_batch_orthogonalize): item i
 // owns the flat blocks [start[i], start[i+1]) (its own block count nb, so its
 // row ranges and reduction order are those of its single launch).
+__global__ void __launch_bounds__(kColThreads) k_cgs2_cluster(const CluArgs A, const int* gate) {
+  if (gate && *gate) return;
+  __shared__ CluShared C;
+  cgs2_cluster(A, blockIdx.x, C);
+  cluster_barrier();
+}
+
+template <int PASS>
+__global__ void __launch_bounds__(kColThreads) k_cgs2_clusters(const CluArgs A, const int* gate) {
+  if (gate && *gate) return;
+  __shared__ CluShared C;
+  cgs2_clusters<PASS>(A, blockIdx.x / kClu, blockIdx.x % kClu, C);
+}
+
 struct CgsItem {
   const double2* V;
   double2* w;
@@ -816,6 +453,31 @@ __device__ __forceinline__ int cgs_item(const int* __restrict__ start, int count
     else hi = mid - 1;
   }
   return lo;
+}
+
+__device__ __forceinline__ CluArgs clu_args(const CgsItem& it) {
+  return CluArgs{it.V, it.w, it.p1, it.p2, it.d_h, it.np, it.d_norm, it.counter, it.n, it.k, it.nb};
+}
+
+// one cluster per item
+__global__ void __launch_bounds__(kColThreads) k_cgs2_cluster_batch(const CgsItem* __restrict__ items) {
+  __shared__ CluShared C;
+  const CgsItem it = items[blockIdx.x / kCluOne];
+  if (it.gate && *it.gate) return;
+  cgs2_cluster(clu_args(it), blockIdx.x % kCluOne, C);
+  cluster_barrier();
+}
+
+// it.nb clusters per item
+template <int PASS>
+__global__ void __launch_bounds__(kColThreads) k_cgs2_clusters_batch(const CgsItem* __restrict__ items,
+                                                                     const int* __restrict__ start, int count) {
+  __shared__ CluShared C;
+  const int i = cgs_item(start, count, blockIdx.x);
+  const CgsItem it = items[i];
+  if (it.gate && *it.gate) return;
+  const unsigned b = blockIdx.x - (unsigned)__ldg(start + i);
+  cgs2_clusters<PASS>(clu_args(it), b / kClu, b % kClu, C);
 }
 
 template <int PASS, bool ROWS>
@@ -1087,6 +749,12 @@ int grid_n(long long n) {
 
 }  // namespace
 
+// Whether CGS2 of k vectors of n entries runs in clusters (gram_schmidt.cuh), and in one launch.
+static bool in_clusters(long long n, int k) { return k >= 1 && k <= kColMax && n < kCluMaxN; }
+bool kry_one_cluster(const StabHandle* h, long long n, int k) {
+  return in_clusters(n, k) && n <= kCluOneN && h->cluster_ok;
+}
+
 // completion counter of the Gram-Schmidt passes (zeroed at set-up, left at zero by every pass)
 static unsigned* col_counter(StabHandle* h) { return (unsigned*)(h->d_red + h->red_blocks + 16); }
 
@@ -1122,7 +790,22 @@ cudaError_t kry_cgs2(StabHandle* h, const double2* V, int k, long long n, double
   double* np = (double*)(p2 + (size_t)pb * (k > 0 ? k : 1));
   const int ts = phase_begin(h, STAB_PHASE_CGS2);
   cudaError_t e;
-  if (k > 0 && k <= kColMax) {
+  if (k > 0 && in_clusters(n, k)) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    const bool one = kry_one_cluster(h, n, k);
+    const int G = one ? 1 : clu_count(n, k);
+    cluster_config(cfg, attr, one ? kCluOne : kClu, (unsigned)G, h->stream);
+    const CluArgs A{V, w, p1, p2, d_h, np, d_norm, col_counter(h), n, k, G};
+    const int* gate = h->gate;
+    if (one) {
+      e = cudaLaunchKernelEx(&cfg, k_cgs2_cluster, A, gate);
+    } else {
+      e = cudaLaunchKernelEx(&cfg, k_cgs2_clusters<0>, A, gate);
+      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_cgs2_clusters<1>, A, gate);
+      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_cgs2_clusters<2>, A, gate);
+    }
+  } else if (k > 0 && k <= kColMax) {
     const int cb = col_blocks(n, k);
     unsigned* counter = col_counter(h);
     auto args = [&](int pass) { return cgs2_pass(pass, V, k, n, w, p1, d_h, np, d_norm, counter, cb); };
@@ -1272,7 +955,19 @@ cudaError_t kry_gemv32(StabHandle* h, const float2* V, int k, const int* kdev, l
 }
 
 // kernel attributes of this file, set for the current device at handle creation
-cudaError_t kry_init_attributes() {
+cudaError_t kry_init_attributes(StabHandle* h) {
+  // clusters of 16 CTAs are above the portable size of 8: allowed per kernel where the device has room
+  int clusters = 0;
+  for (const void* k : {(const void*)k_cgs2_cluster, (const void*)k_cgs2_cluster_batch})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  cluster_config(cfg, attr, kCluOne, 1, nullptr);
+  if (cudaOccupancyMaxActiveClusters(&clusters, k_cgs2_cluster, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    clusters = 0;
+  }
+  h->cluster_ok = clusters > 0;
   return cudaFuncSetAttribute(k_vq, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
@@ -1304,7 +999,7 @@ cudaError_t kry_cgs2_stream(cudaStream_t st, const double2* V, int k, long long 
 
 // Parameter image of a batched CGS2 (job i gated by J.gate) and its launches.
 cudaError_t cgs2_batch_plan(const std::vector<CgsJob>& jobs, BatchImage& im, CgsBatchPlan& plan) {
-  std::vector<CgsItem> items, cols[2];  // k > kColMax; k <= kColMax by columns, by rows
+  std::vector<CgsItem> items, cols[2], clus[2];  // k > kColMax; k <= kColMax by columns, by rows; one cluster, clusters
   std::vector<int> blocks, ones, col_bl[2];
   size_t sm = 0;
   for (const CgsJob& J : jobs) {
@@ -1323,6 +1018,12 @@ cudaError_t cgs2_batch_plan(const std::vector<CgsJob>& jobs, BatchImage& im, Cgs
     it.n = J.n;
     it.k = J.k;
     it.nb = J.k <= kColMax ? col_blocks(J.n, J.k) : cgs_blocks(J.n);
+    if (in_clusters(J.n, J.k)) {
+      const bool one = kry_one_cluster(J.h, J.n, J.k);
+      it.nb = one ? 1 : clu_count(J.n, J.k);
+      clus[one ? 0 : 1].push_back(it);
+      continue;
+    }
     if (J.k <= kColMax) {
       cols[by_rows(J.n)].push_back(it);
       col_bl[by_rows(J.n)].push_back(it.nb);
@@ -1333,6 +1034,11 @@ cudaError_t cgs2_batch_plan(const std::vector<CgsJob>& jobs, BatchImage& im, Cgs
     ones.push_back(1);
     sm = std::max(sm, (size_t)J.k * (sizeof(double2) + 2 * sizeof(ffn)));
   }
+  for (int r = 0; r < 2; ++r) {
+    std::vector<int> ctas;
+    for (const CgsItem& it : clus[r]) ctas.push_back((r == 0 ? kCluOne : kClu) * it.nb);
+    plan.U[r] = im.section(clus[r], ctas, kColThreads, 0);
+  }
   for (int r = 0; r < 2; ++r) plan.C[r] = im.section(cols[r], col_bl[r], kColThreads, 0);
   plan.S = im.section(items, blocks, kThreads, sm);
   plan.N = im.section(items, ones, 32, 0);
@@ -1341,6 +1047,25 @@ cudaError_t cgs2_batch_plan(const std::vector<CgsJob>& jobs, BatchImage& im, Cgs
 }
 
 cudaError_t cgs2_batch_launch(const CgsBatchPlan& plan, const unsigned char* d, cudaStream_t st) {
+  for (int r = 0; r < 2; ++r)
+    if (plan.U[r].count) {
+      const BatchSection& U = plan.U[r];
+      cudaLaunchConfig_t cfg;
+      cudaLaunchAttribute attr;
+      const int ctas = r == 0 ? kCluOne : kClu;
+      cluster_config(cfg, attr, ctas, (unsigned)(U.blocks / ctas), st);
+      const CgsItem* items = (const CgsItem*)(d + U.items);
+      const int* start = (const int*)(d + U.start);
+      cudaError_t e;
+      if (r == 0) {
+        e = cudaLaunchKernelEx(&cfg, k_cgs2_cluster_batch, items);
+      } else {
+        e = cudaLaunchKernelEx(&cfg, k_cgs2_clusters_batch<0>, items, start, U.count);
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_cgs2_clusters_batch<1>, items, start, U.count);
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_cgs2_clusters_batch<2>, items, start, U.count);
+      }
+      if (e != cudaSuccess) return e;
+    }
   auto pass = [&](auto by_col, auto by_row) {
     if (plan.C[0].count)
       by_col<<<plan.C[0].blocks, kColThreads, 0, st>>>((const CgsItem*)(d + plan.C[0].items),

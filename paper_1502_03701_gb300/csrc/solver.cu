@@ -15,6 +15,7 @@
 #include <cstring>
 #include <vector>
 
+#include "gram_schmidt.cuh"
 #include "hess_dev.cuh"
 #include "internal.cuh"
 
@@ -325,6 +326,34 @@ __global__ void __launch_bounds__(256) k_gm_step_scale(GmDev d, int j, double2* 
   }
 }
 
+// A whole orthogonalisation step of a small vector in one cluster: CGS2, then
+// CTA 0's first warp takes the Givens step while the other warps scale w.
+__global__ void __launch_bounds__(gs::kColThreads) k_gm_cgs2_step(gs::CluArgs A, GmDev d, int j) {
+  if (d.flags[0]) return;  // set by an earlier launch: the same for the whole cluster
+  __shared__ gs::CluShared C;
+  gs::cgs2_cluster(A, blockIdx.x, C);
+  gs::cluster_barrier();  // also: no CTA is still to read flags[0]
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    gm_step_body(d, j);
+    return;
+  }
+  const double s = 1.0 / C.norm;
+  const long long blk = 32LL * (gs::kColWarps / gs::col_warps(A.k));  // rows that a CTA takes at a time
+  const int t0 = blockIdx.x == 0 ? threadIdx.x - 32 : threadIdx.x, nt = blockIdx.x == 0 ? gs::kColThreads - 32 : gs::kColThreads;
+  for (long long r0 = blk * blockIdx.x; r0 < A.n; r0 += blk * gs::kCluOne)
+    for (long long i = r0 + t0; i < r0 + blk && i < A.n; i += nt) {
+      const double2 v = A.w[i];
+      A.w[i] = make_double2(v.x * s, v.y * s);
+    }
+}
+
+cudaError_t launch_cgs2_step(cudaStream_t st, const gs::CluArgs& A, const GmDev& d, int j) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  gs::cluster_config(cfg, attr, gs::kCluOne, 1, st);
+  return cudaLaunchKernelEx(&cfg, k_gm_cgs2_step, A, d, j);
+}
+
 // y = R^{-1} g over the jend columns of the cycle, by columns: y_i from the
 // diagonal, then every thread removes y_i's contribution from its rows.
 __device__ __forceinline__ void gm_solve_body(const GmDev& d) {
@@ -440,6 +469,8 @@ cudaGraphExec_t gm_graph(StabHandle* h, cd sigma, int eps_mode, const GmresWs& W
     slot = nullptr;
     slot_key.valid = false;
   }
+  if (h->cluster_ok)
+    ck(h, cudaFuncSetAttribute(k_gm_cgs2_step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "cluster size");
   if (!h->cap_stream) ck(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking), "capture stream");
   const stab_stats saved_stats = h->stats;
   cudaStream_t saved_stream = h->stream;
@@ -533,6 +564,11 @@ cudaGraphExec_t gm_graph(StabHandle* h, cd sigma, int eps_mode, const GmresWs& W
       }
       // tiny vectors: the fused four-kernel CGS2 (launch latency dominates); otherwise the
       // selective form, which reads the basis half as often
+      if (n < kSelectiveMinN && kry_one_cluster(h, n, j + 1)) {
+        h->gate = nullptr;
+        step(launch_cgs2_step(h->stream, gs::CluArgs{W.V, Vn, nullptr, nullptr, W.dh, nullptr, W.dnorm, nullptr, n, j + 1, 1}, D, j));
+        continue;
+      }
       if (n < kSelectiveMinN) step(kry_cgs2(h, W.V, j + 1, n, Vn, W.dh, W.dnorm, W.partial));
       else step(kry_dgks(h, W.V, j + 1, n, Vn, W.dh, W.dnorm, W.partial));
       h->gate = nullptr;

@@ -67,6 +67,7 @@ static void free_handle(stab_handle h) {
   dfree(h, h->d_coef_p);
   dfree(h, h->d_btab_f);
   dfree(h, h->d_tcoef);
+  if (h->pin_ortho) cudaFreeHost(h->pin_ortho);
   dfree(h, h->d_btab_low);
   for (int a = 0; a < 3; ++a) {
     dfree(h, h->ax[a].tab[0]);

@@ -122,6 +122,8 @@ struct PhaseTimer {
   long long dropped = 0;
 };
 
+constexpr int kPinOrtho = 256;  // coefficients that the pinned staging of stab_orthogonalize holds
+
 struct StabHandle {
   // problem
   int dim, nx, ny, nz, nv;
@@ -174,6 +176,7 @@ struct StabHandle {
   // statistics
   stab_stats stats;
   PhaseTimer timer;
+  double2* pin_ortho = nullptr;  // stab_orthogonalize: pinned norm and coefficients (allocated on first use)
   bool cluster_ok = false;  // the device schedules clusters of 16 CTAs (gram_schmidt.cuh)
   LineCfg line_cfg[3];  // per axis, from stab_autotune
   // graph capture of the GMRES cycle (solver.cu): while gate is set, the

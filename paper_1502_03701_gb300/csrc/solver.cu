@@ -820,14 +820,23 @@ extern "C" stab_status stab_orthogonalize(stab_handle hh, const void* V, int k, 
     const long long n = h->n;
     const size_t part = (size_t)kry_partial_elems(n, k);
     double2* ws = ensure(h, &h->d_ir, &h->ir_elems, part + 2 * (size_t)std::max(k, 1) + 2);
-    double2* dh = ws + part;
-    double* dn = (double*)(dh + 2 * std::max(k, 1));
+    // norm and coefficients side by side: one copy, through pinned memory
+    double* dn = (double*)(ws + part);
+    double2* dh = ws + part + 1;
+    if (!h->pin_ortho) {
+      void* p = nullptr;
+      ck(h, cudaHostAlloc(&p, (kPinOrtho + 1) * sizeof(double2), cudaHostAllocDefault), "pinned staging");
+      h->pin_ortho = (double2*)p;
+    }
     ck(h, kry_cgs2(h, (const double2*)V, k, n, (double2*)w, dh, dn, ws), "CGS2");
-    if (hcoef && k > 0) ck(h, cudaMemcpyAsync(hcoef, dh, sizeof(double2) * k, cudaMemcpyDeviceToHost, h->stream), "copy");
-    double nv = 0.0;
-    ck(h, cudaMemcpyAsync(&nv, dn, sizeof(double), cudaMemcpyDeviceToHost, h->stream), "copy");
+    const int back = hcoef ? std::min(k, kPinOrtho) : 0;
+    ck(h, cudaMemcpyAsync(h->pin_ortho, dn, sizeof(double2) * (1 + back), cudaMemcpyDeviceToHost, h->stream), "copy");
+    if (hcoef && k > back)
+      ck(h, cudaMemcpyAsync(hcoef + 2 * (size_t)back, dh + back, sizeof(double2) * (k - back), cudaMemcpyDeviceToHost,
+                            h->stream), "copy");
     ck(h, cudaStreamSynchronize(h->stream), "sync");
-    if (norm) *norm = nv;
+    if (back > 0) std::memcpy(hcoef, h->pin_ortho + 1, sizeof(double2) * back);
+    if (norm) *norm = h->pin_ortho[0].x;
     return STAB_OK;
   } catch (Fail& f) {
     return f.st;

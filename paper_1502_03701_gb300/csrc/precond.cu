@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "pairs.cuh"
 #include "pointwise.cuh"
 
 pw::Phys phys_of(const StabHandle* h);
@@ -379,22 +380,23 @@ __device__ __forceinline__ long long bt_dof(const BtApplyParams& P, unsigned til
   return (long long)a * P.npts + ((long long)z * P.ny + y) * P.nx + x;
 }
 
-// Rows per CTA and threads per row of the level products: G threads (a power
-// of two) share a row, G * m <= blockDim.
-__device__ __forceinline__ int bt_group(int m) {
+// Threads per row of the level products: G threads (a power of two) share a
+// row, G m <= threads of the CTA.
+constexpr int kBtRhsThreads = 256, kBtSweepThreads = 512;
+__host__ __device__ constexpr int bt_group(int m, int threads) {
   int G = 1;
-  while (G < 32 && 2 * G * m <= (int)blockDim.x) G *= 2;
+  while (G < 32 && 2 * G * m <= threads) G *= 2;
   return G;
 }
 
-// Shared-memory pitch (in complex values) of a staged level matrix: 16-byte
-// aligned rows, and the rows that half a warp reads together (16 / G of them, G
-// consecutive entries each) in different banks.
+// Shared-memory pitch (in complex values) of a staged level matrix: rows of 16
+// bytes times the row's threads apart from a multiple of all banks, so that the
+// 16-byte reads of eight neighbouring threads (a row's, or those of several rows)
+// meet all banks once.
 template <class R>
 __host__ __device__ constexpr int bt_pitch(int m, int G) {
   const int per = 128 / (int)sizeof(C2<R>);  // values per 32 banks
-  const int step = G < 2 ? 2 : G;
-  return (m + per - 1) / per * per + step;
+  return (m + per - 1) / per * per + (G < 8 ? G * 16 / (int)sizeof(C2<R>) : 0);
 }
 
 // Queue the copy of an m x m row-major matrix into shared memory (cp.async,
@@ -426,14 +428,60 @@ struct BtStage {
   }
 };
 
-// (M x)_row over this thread's entries g, g + G, ..., then over the row's G threads
+// A level's vector in shared memory.  FP32: the real parts and the imaginary
+// parts, each entry twice, so that two packed FMAs take a complex product:
+// (a.x, a.y) (b.x, b.x) and (a.x, a.y) (b.y, b.y), combined at the end.
 template <class R>
-__device__ __forceinline__ C2<R> bt_product(const C2<R>* Mrow, const C2<R>* x, int m, int g, int G, bool act) {
-  R sx = 0, sy = 0;
+struct BtVec;
+template <>
+struct BtVec<float> {
+  float4* re;  // entries 2 k, 2 k + 1
+  float4* im;
+  static __host__ __device__ constexpr size_t bytes(int m) { return (size_t)(m + 1) / 2 * 2 * sizeof(float4); }
+  __device__ __forceinline__ BtVec(void* p, int m) : re((float4*)p), im((float4*)p + (m + 1) / 2) {}
+  __device__ __forceinline__ void put(int r, C2<float> v) const {
+    ((float2*)re)[r] = make_float2(v.x, v.x);
+    ((float2*)im)[r] = make_float2(v.y, v.y);
+  }
+};
+template <>
+struct BtVec<double> {
+  C2<double>* v;
+  static __host__ __device__ constexpr size_t bytes(int m) { return (size_t)m * sizeof(C2<double>); }
+  __device__ __forceinline__ BtVec(void* p, int) : v((C2<double>*)p) {}
+  __device__ __forceinline__ void put(int r, C2<double> a) const { v[r] = a; }
+};
+
+// (M x)_row over this thread's 16-byte pieces g, g + G, ... of the row, then over the row's G threads
+__device__ __forceinline__ C2<float> bt_product(const C2<float>* Mrow, const BtVec<float>& x, int m, int g, int G,
+                                                bool act) {
+  float2 p = make_float2(0.0f, 0.0f), q = p;
+  if (act) {
+    const float4* M4 = (const float4*)Mrow;
+    const int half = m / 2;  // m is even
+#pragma unroll 4
+    for (int k = g; k < half; k += G) {
+      const float4 a = M4[k], br = x.re[k], bi = x.im[k];
+      p = v2_fma(make_float2(a.x, a.y), make_float2(br.x, br.y), p);
+      q = v2_fma(make_float2(a.x, a.y), make_float2(bi.x, bi.y), q);
+      p = v2_fma(make_float2(a.z, a.w), make_float2(br.z, br.w), p);
+      q = v2_fma(make_float2(a.z, a.w), make_float2(bi.z, bi.w), q);
+    }
+  }
+  float sx = p.x - q.y, sy = p.y + q.x;
+  for (int o = G >> 1; o > 0; o >>= 1) {
+    sx += __shfl_xor_sync(0xffffffffu, sx, o);
+    sy += __shfl_xor_sync(0xffffffffu, sy, o);
+  }
+  return C2<float>{sx, sy};
+}
+__device__ __forceinline__ C2<double> bt_product(const C2<double>* Mrow, const BtVec<double>& x, int m, int g, int G,
+                                                 bool act) {
+  double sx = 0, sy = 0;
   if (act) {
 #pragma unroll 4
     for (int k = g; k < m; k += G) {
-      const C2<R> a = Mrow[k], b = x[k];
+      const C2<double> a = Mrow[k], b = x.v[k];
       sx += a.x * b.x - a.y * b.y;
       sy += a.x * b.y + a.y * b.x;
     }
@@ -442,19 +490,29 @@ __device__ __forceinline__ C2<R> bt_product(const C2<R>* Mrow, const C2<R>* x, i
     sx += __shfl_xor_sync(0xffffffffu, sx, o);
     sy += __shfl_xor_sync(0xffffffffu, sy, o);
   }
-  return C2<R>{sx, sy};
+  return C2<double>{sx, sy};
 }
+
+// FP32 results to FP64 in integer arithmetic: the conversion instruction issues at 1/64 of the FP32 rate
+// (it takes zeros, subnormal numbers, infinities and NaN)
+__device__ __forceinline__ double bt_out(float s) {
+  const unsigned ex = (__float_as_uint(s) >> 23) & 0xFFu;
+  if (ex - 1u >= 254u) return (double)s;
+  return f2d_exact(s);
+}
+__device__ __forceinline__ double2 bt_out(C2<float> s) { return make_double2(bt_out(s.x), bt_out(s.y)); }
+__device__ __forceinline__ double2 bt_out(C2<double> s) { return make_double2(s.x, s.y); }
 
 // w_l = S_l^{-1} q_l for every level of every tile, into z (grid: tiles x levels).
 template <class R, bool Q32>
-__global__ void __launch_bounds__(256) k_bt_rhs(const __grid_constant__ BtApplyParams P) {
+__global__ void __launch_bounds__(kBtRhsThreads) k_bt_rhs(const __grid_constant__ BtApplyParams P) {
   if (P.gate && *P.gate) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int m = P.m, l = blockIdx.y;
-  const int G = bt_group(m), lg = __ffs(G) - 1, row = threadIdx.x >> lg, g = threadIdx.x & (G - 1);
+  const int G = bt_group(m, kBtRhsThreads), lg = __ffs(G) - 1, row = threadIdx.x >> lg, g = threadIdx.x & (G - 1);
   const int pitch = bt_pitch<R>(m, G);
   C2<R>* Ms = (C2<R>*)smraw;
-  C2<R>* t = Ms + (P.staged ? m * pitch : 0);
+  const BtVec<R> t(Ms + (P.staged ? m * pitch : 0), m);
   const long long tile = blockIdx.x, mm = (long long)m * m;
   const C2<R>* S = (const C2<R>*)P.F + (tile * P.nlev + l) * 3 * mm + mm;
   if (P.staged) {
@@ -463,76 +521,80 @@ __global__ void __launch_bounds__(256) k_bt_rhs(const __grid_constant__ BtApplyP
   }
   for (int r = threadIdx.x; r < m; r += blockDim.x) {
     const long long d = bt_dof(P, tile, l, r);
-    if (Q32) { const float2 v = P.q32[d]; t[r] = C2<R>{(R)v.x, (R)v.y}; }
-    else { const double2 v = P.q[d]; t[r] = C2<R>{(R)v.x, (R)v.y}; }
+    if (Q32) { const float2 v = P.q32[d]; t.put(r, C2<R>{(R)v.x, (R)v.y}); }
+    else { const double2 v = P.q[d]; t.put(r, C2<R>{(R)v.x, (R)v.y}); }
   }
   const bool act = row < m;
   double2* z = P.z + (act && g == 0 ? bt_dof(P, tile, l, row) : 0);
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   const C2<R>* Mr = P.staged ? Ms + row * pitch : S + (long long)row * m;
-  const C2<R> s = bt_product<R>(Mr, t, m, g, G, act);
-  if (act && g == 0) *z = make_double2((double)s.x, (double)s.y);
+  const C2<R> s = bt_product(Mr, t, m, g, G, act);
+  if (act && g == 0) *z = bt_out(s);
 }
 
 // The level recurrences of one tile (one CTA per tile), z holding w on entry:
 // forward y_l = w_l - P_l y_{l-1}, backward x_l = y_l - X_l x_{l+1}.  The chain is a
 // level's product, a shuffle sum and a barrier; the levels' matrices stream
 // through a ring of STAGES shared-memory buffers, STAGES - 1 levels ahead, and a
-// thread's right-hand sides one ring ahead in registers.  A row's unknowns of
-// consecutive levels are 2 nx apart, so their address is formed once (eight
-// integer divisions that used to run three times per level).  128 x 256 layer in
-// 8 x 64 tiles (64 tiles, 32 levels of 64 unknowns): 139 us before.
+// thread's right-hand sides one ring ahead in registers.  Shared-memory bandwidth
+// bounds it: matrix in, matrix out and the vector once per row.
 template <class R, int STAGES>
-__global__ void __launch_bounds__(256) k_bt_sweep(const __grid_constant__ BtApplyParams P) {
+__global__ void __launch_bounds__(kBtSweepThreads, STAGES == 5 ? 1 : 2) k_bt_sweep(const __grid_constant__ BtApplyParams P) {
   if (P.gate && *P.gate) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int m = P.m, nlev = P.nlev;
-  const int G = bt_group(m), lg = __ffs(G) - 1, row = threadIdx.x >> lg, g = threadIdx.x & (G - 1);
+  const int G = bt_group(m, kBtSweepThreads), lg = __ffs(G) - 1;
+  const int row = threadIdx.x >> lg, g = threadIdx.x & (G - 1);
   const int pitch = bt_pitch<R>(m, G);
   const bool act = row < m, lead = act && g == 0;
   const long long tile = blockIdx.x, mm = (long long)m * m;
   const C2<R>* Ft = (const C2<R>*)P.F + tile * nlev * 3 * mm;
   constexpr bool kStaged = STAGES > 0;
-  constexpr int kAhead = kStaged ? STAGES - 1 : 1;
+  constexpr int kRing = kStaged ? STAGES : 2, kAhead = kRing - 1;
   C2<R>* ring = (C2<R>*)smraw;
-  C2<R>* yp = ring + (size_t)STAGES * m * pitch;
-  C2<R>* yc = yp + m;
+  unsigned char* vec = smraw + (size_t)STAGES * m * pitch * sizeof(C2<R>);
+  BtVec<R> yp(vec, m), yc(vec + BtVec<R>::bytes(m), m);
   double2* z = P.z + (act ? bt_dof(P, tile, 0, row) : 0);
   const long long dz = 2LL * P.nx;
   const BtStage<R> stage(m, pitch);
   // one direction: level i of count is first + dir i, its matrix at M + 3 mm l
   auto sweep = [&](const C2<R>* M, int first, int dir, int count) {
-    double2 rhs[kAhead];
-    auto fetch = [&](int i) {
-      const int l = first + dir * i;
+    double2 rhs[kRing];
+    double2 *zin = z + first * dz, *zout = zin;
+    const C2<R>* Min = M + 3 * mm * first;
+    const C2<R>* Mrow = Min + (long long)(act ? row : 0) * m;  // unstaged: the row's matrix entries
+    int in = 0;
+    auto fetch = [&](int slot) {  // the next level
       if (kStaged) {
-        if (i < count) stage.copy(ring + (i % (kStaged ? STAGES : 1)) * m * pitch, pitch, M + 3 * mm * l, m);
+        if (in < count) stage.copy(ring + slot * m * pitch, pitch, Min, m);
         asm volatile("cp.async.commit_group;" ::: "memory");
+        Min += dir * 3 * mm;
       }
-      return lead && i < count ? z[l * dz] : make_double2(0.0, 0.0);
+      rhs[slot] = lead && in < count ? *zin : make_double2(0.0, 0.0);
+      zin += dir * dz;
+      ++in;
     };
 #pragma unroll
-    for (int d = 0; d < kAhead; ++d) rhs[d] = fetch(d);
-    for (int i0 = 0; i0 < count; i0 += kAhead) {
+    for (int d = 0; d < kAhead; ++d) fetch(d);
+    for (int i0 = 0; i0 < count; i0 += kRing) {
 #pragma unroll
-      for (int d = 0; d < kAhead; ++d) {
-        const int i = i0 + d;
-        if (i >= count) break;
+      for (int d = 0; d < kRing; ++d) {
+        if (i0 + d >= count) break;
         if (kStaged) asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
         __syncthreads();  // this level's matrix and the previous level's y; the previous buffer is free
-        const double2 w = rhs[d];
-        rhs[d] = fetch(i + kAhead);
-        const int l = first + dir * i;
-        const C2<R>* Mr = kStaged ? ring + ((size_t)(i % (kStaged ? STAGES : 1)) * m + row) * pitch
-                                  : M + 3 * mm * l + (long long)(act ? row : 0) * m;
-        const C2<R> s = bt_product<R>(Mr, yp, m, g, G, act);
+        fetch((d + kAhead) % kRing);
+        const C2<R> s = bt_product(kStaged ? ring + (d * m + row) * pitch : Mrow, yp, m, g, G, act);
+        Mrow += dir * 3 * mm;
         if (lead) {
-          const C2<R> y = {(R)w.x - s.x, (R)w.y - s.y};
-          yc[row] = y;
-          z[l * dz] = make_double2((double)y.x, (double)y.y);
+          const C2<R> y = {(R)rhs[d].x - s.x, (R)rhs[d].y - s.y};
+          yc.put(row, y);
+          *zout = bt_out(y);
         }
-        C2<R>* tmp = yp; yp = yc; yc = tmp;
+        zout += dir * dz;
+        const BtVec<R> tmp = yp;
+        yp = yc;
+        yc = tmp;
       }
     }
     if (kStaged) asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -541,49 +603,154 @@ __global__ void __launch_bounds__(256) k_bt_sweep(const __grid_constant__ BtAppl
   // forward: y_0 = w_0
   if (lead) {
     const double2 w = z[0];
-    yp[row] = C2<R>{(R)w.x, (R)w.y};
+    yp.put(row, C2<R>{(R)w.x, (R)w.y});
   }
   sweep(Ft, 1, 1, nlev - 1);
   // backward: x_{nlev-1} = y_{nlev-1} (in yp)
   sweep(Ft + 2 * mm, nlev - 2, -1, nlev - 1);
 }
 
+// The same for FP32 levels of at most kBtRegLevel unknowns: a thread's share of a
+// level's matrix (PC pieces of 16 bytes of one row) goes from global memory straight
+// into its registers, kBtDepth levels ahead, and only the level's vector passes
+// through shared memory.  Bound by the level chain (loads of the vector, products,
+// a sum in which the row's halves take one part each, barrier) at about 0.65 us a
+// level, a little above what HBM needs when 152 tiles run.  128 x 256 layer in
+// 8 x 64 tiles (64 tiles of 32 levels of 64 unknowns): 42 us, 71 us with the shared
+// ring above; with the first pass the apply takes 58 us, 164 us at one time (integer
+// divisions, matrices from global memory).  Three levels ahead measured the same,
+// two 2 us more.  Larger levels do not fit: their share of one level alone is half
+// of a thread's registers or more.
+constexpr int kBtRegLevel = 64, kBtDepth = 4;
+
+template <int G, int PC>
+__global__ void __launch_bounds__(kBtSweepThreads) k_bt_sweep_reg(const __grid_constant__ BtApplyParams P) {
+  if (P.gate && *P.gate) return;
+  __shared__ float4 ys[2][kBtRegLevel / 2];  // zero past the level's entries
+  const int m = P.m, nlev = P.nlev, half = m / 2;  // m is even
+  const int row = threadIdx.x / G, g = threadIdx.x % G;
+  // after the sum, the row's first thread holds the real and its G / 2-th one the imaginary part
+  const int im = g >= G / 2;
+  const bool act = row < m, lead = act && g % (G / 2) == 0;
+  const long long tile = blockIdx.x, mm = (long long)m * m;
+  // threads without a row, and pieces past the row's end, load something of the level and add nothing
+  const float2* Ft = (const float2*)P.F + tile * nlev * 3 * mm + (act ? (long long)row * m : 0);
+  int piece[PC];
+#pragma unroll
+  for (int q = 0; q < PC; ++q) piece[q] = g + q * G < half ? g + q * G : 0;
+  double* z = (double*)(P.z + bt_dof(P, tile, 0, act ? row : 0)) + im;
+  const long long dz = 4LL * P.nx;
+  int cur = 0;
+  if (threadIdx.x < kBtRegLevel) ys[threadIdx.x & 1][threadIdx.x >> 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  // one direction: level i of count is first + dir i, its matrix at M + 3 mm l
+  auto sweep = [&](const float2* M, int first, int dir, int count) {
+    if (count < 1) return;
+    float4 a[kBtDepth][PC];
+    double rhs[kBtDepth];
+    double *zin = z + first * dz, *zout = zin;
+    const float4* Min = (const float4*)(M + 3 * mm * first);
+    const long long dM = dir * 3 * mm / 2, dZ = dir * dz;
+    int left = count - 1;
+    auto fetch = [&](int slot) {  // the next level (past the end: the last one again)
+#pragma unroll
+      for (int q = 0; q < PC; ++q) a[slot][q] = __ldg(Min + piece[q]);
+      rhs[slot] = lead ? *zin : 0.0;
+      if (left > 0) {
+        Min += dM;
+        zin += dZ;
+      }
+      --left;
+    };
+#pragma unroll
+    for (int d = 0; d < kBtDepth; ++d) fetch(d);
+    for (int i0 = 0; i0 < count; i0 += kBtDepth) {
+#pragma unroll
+      for (int d = 0; d < kBtDepth; ++d) {
+        if (i0 + d >= count) break;
+        const float w = (float)rhs[d];
+        __syncthreads();  // the previous level's y
+        float sx = 0.0f, sy = 0.0f, tx = 0.0f, ty = 0.0f;
+#pragma unroll
+        for (int q = 0; q < PC; ++q) {
+          const float4 v = a[d][q], b = ys[cur][g + q * G];
+          sx = fmaf(v.x, b.x, sx);
+          sy = fmaf(v.x, b.y, sy);
+          tx = fmaf(v.y, b.y, tx);
+          ty = fmaf(v.y, b.x, ty);
+          sx = fmaf(v.z, b.z, sx);
+          sy = fmaf(v.z, b.w, sy);
+          tx = fmaf(v.w, b.w, tx);
+          ty = fmaf(v.w, b.z, ty);
+        }
+        fetch(d);
+        sx -= tx;
+        sy += ty;
+        float t = (im ? sy : sx) + __shfl_xor_sync(0xffffffffu, im ? sx : sy, G / 2);
+#pragma unroll
+        for (int o = G / 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        cur ^= 1;
+        const float y = w - t;
+        if (lead) {
+          ((float*)ys[cur])[2 * row + im] = y;
+          *zout = bt_out(y);
+        }
+        zout += dZ;
+      }
+    }
+    __syncthreads();
+  };
+  // forward: y_0 = w_0
+  __syncthreads();
+  if (lead) ((float*)ys[0])[2 * row + im] = (float)*z;
+  sweep(Ft, 1, 1, nlev - 1);
+  // backward: x_{nlev-1} = y_{nlev-1}
+  sweep(Ft + 2 * mm, nlev - 2, -1, nlev - 1);
+}
+
 constexpr size_t kBtSmem = 200 * 1024;
+
+template <class R>
+auto bt_sweep_kernel(int stages) -> void (*)(const BtApplyParams) {
+  return stages == 5 ? k_bt_sweep<R, 5> : stages == 3 ? k_bt_sweep<R, 3> : k_bt_sweep<R, 0>;
+}
 
 template <class R>
 cudaError_t launch_bt_apply(const BtApplyParams& B0, long long ntiles, cudaStream_t st) {
   BtApplyParams B = B0;
-  int G = 1;
-  while (G < 32 && 2 * G * B.m <= 256) G *= 2;
-  const size_t level = (size_t)B.m * bt_pitch<R>(B.m, G) * sizeof(C2<R>), vec = (size_t)B.m * sizeof(C2<R>);
+  const size_t vec = BtVec<R>::bytes(B.m);
+  auto level = [&](int threads) { return (size_t)B.m * bt_pitch<R>(B.m, bt_group(B.m, threads)) * sizeof(C2<R>); };
+  const size_t lr = level(kBtRhsThreads), ls = level(kBtSweepThreads);
   const dim3 grid((unsigned)ntiles, (unsigned)B.nlev);
   // a level per CTA, two CTAs per SM at least
-  B.staged = level + vec <= kBtSmem / 2;
-  const size_t rsm = (B.staged ? level : 0) + vec;
-  if (B.q32) k_bt_rhs<R, true><<<grid, 256, rsm, st>>>(B);
-  else k_bt_rhs<R, false><<<grid, 256, rsm, st>>>(B);
+  B.staged = lr + vec <= kBtSmem / 2;
+  const size_t rsm = (B.staged ? lr : 0) + vec;
+  if (B.q32) k_bt_rhs<R, true><<<grid, kBtRhsThreads, rsm, st>>>(B);
+  else k_bt_rhs<R, false><<<grid, kBtRhsThreads, rsm, st>>>(B);
+  if (sizeof(R) == 4 && B.m <= kBtRegLevel) {
+    const int G = bt_group(B.m, kBtSweepThreads);
+    auto kernel = G == 8 ? k_bt_sweep_reg<8, 4> : G == 16 ? k_bt_sweep_reg<16, 1> : k_bt_sweep_reg<32, 1>;
+    kernel<<<(unsigned)ntiles, kBtSweepThreads, 0, st>>>(B);
+    return cudaGetLastError();
+  }
   // ring: five buffers where every tile has an SM of its own, three where two tiles share one
-  const bool alone = ntiles <= 152;
-  auto sweep = [&](auto kernel, int stages) {
-    kernel<<<(unsigned)ntiles, 256, stages * level + 2 * vec, st>>>(B);
-  };
-  if (alone && 5 * level + 2 * vec <= kBtSmem) sweep(k_bt_sweep<R, 5>, 5);
-  else if (3 * level + 2 * vec <= kBtSmem) sweep(k_bt_sweep<R, 3>, 3);
-  else sweep(k_bt_sweep<R, 0>, 0);
+  const int stages = ntiles <= 152 && 5 * ls + 2 * vec <= kBtSmem ? 5 : 3 * ls + 2 * vec <= kBtSmem ? 3 : 0;
+  bt_sweep_kernel<R>(stages)<<<(unsigned)ntiles, kBtSweepThreads, stages * ls + 2 * vec, st>>>(B);
   return cudaGetLastError();
 }
 
 // shared-memory opt-in of the apply kernels (set at the build, never during a stream capture)
 template <class R>
 cudaError_t bt_attributes() {
-  const void* ks[5] = {(const void*)k_bt_rhs<R, true>, (const void*)k_bt_rhs<R, false>, (const void*)k_bt_sweep<R, 5>,
-                       (const void*)k_bt_sweep<R, 3>, (const void*)k_bt_sweep<R, 0>};
+  std::vector<const void*> ks = {(const void*)k_bt_rhs<R, true>, (const void*)k_bt_rhs<R, false>};
+  for (int stages : {0, 3, 5}) ks.push_back((const void*)bt_sweep_kernel<R>(stages));
   for (const void* k : ks) {
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBtSmem);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
+
+constexpr int kApplyThreads = 256;  // CTAs of the block-Jacobi apply
 
 struct ApplyParams {
   const double2* q;
@@ -593,12 +760,28 @@ struct ApplyParams {
   long long npts;
   const int* gate;  // when set and nonzero the launch does nothing (graph-captured GMRES after convergence)
   const float2* q32;  // FP32 input (GMRES with an FP32 basis) instead of q
+  FastDiv divntx, divnty, divpts, divtx, divty;
 };
 
-__device__ __forceinline__ long long tile_dof(const ApplyParams& P, long long tile, int r) {
-  const int tX = (int)(tile % P.ntx), tY = (int)((tile / P.ntx) % P.nty), tZ = (int)(tile / ((long long)P.ntx * P.nty));
-  const int var = r / P.ntpts, pp = r % P.ntpts;
-  const int px = pp % P.tx, py = (pp / P.tx) % P.ty, pz = pp / (P.tx * P.ty);
+void apply_divs(ApplyParams& P) {
+  P.divntx = make_fastdiv((unsigned)P.ntx);
+  P.divnty = make_fastdiv((unsigned)P.nty);
+  P.divpts = make_fastdiv((unsigned)P.ntpts);
+  P.divtx = make_fastdiv((unsigned)P.tx);
+  P.divty = make_fastdiv((unsigned)P.ty);
+}
+
+// row slices of the FP64 / FP32 apply: two rows per warp where that makes no more than four CTAs per SM
+// (four rows: one CTA or two per SM, latency of the loads in the open)
+int apply_row_slices(long long ntiles, int bsz) {
+  const int slices = (int)((4 * 152 + ntiles - 1) / ntiles);
+  return std::max(1, std::min(slices, bsz / 16));
+}
+
+__device__ __forceinline__ long long tile_dof(const ApplyParams& P, unsigned tile, unsigned r) {
+  const unsigned tYZ = fdiv(tile, P.divntx), tX = tile - tYZ * P.ntx, tZ = fdiv(tYZ, P.divnty), tY = tYZ - tZ * P.nty;
+  const unsigned var = fdiv(r, P.divpts), pp = r - var * P.ntpts;
+  const unsigned pyz = fdiv(pp, P.divtx), px = pp - pyz * P.tx, pz = fdiv(pyz, P.divty), py = pyz - pz * P.ty;
   return (long long)var * P.npts + ((long long)(tZ * P.tz + pz) * P.ny + (tY * P.ty + py)) * P.nx + tX * P.tx + px;
 }
 
@@ -658,8 +841,10 @@ __global__ void k_apply_cols(const ApplyParams P) {
 }
 
 // The same product for blocks of a multiple of four rows: each thread forms
-// four consecutive rows from one 16-byte load per column (four BF16 complex
-// entries), so a warp moves 512 bytes per load instruction.
+// four rows (16-byte loads), and the columns are split over as many groups of
+// threads as the CTA holds, added up through shared memory in group order.
+// 32 x 64 layer in 16 x 16 tiles (33 MB in BF16): 14.4 us; 142 us with all 1,024
+// columns in a row on eight threads of each CTA.
 template <bool Q32>
 __device__ __forceinline__ void apply_cols4_body(const ApplyParams& P, long long tile, unsigned slice, unsigned nslices) {
   extern __shared__ unsigned char smraw[];
@@ -678,11 +863,16 @@ __device__ __forceinline__ void apply_cols4_body(const ApplyParams& P, long long
     }
   }
   __syncthreads();
-  for (int r4 = q0 + threadIdx.x; r4 < q1; r4 += blockDim.x) {
+  // S threads for the slice's row quads, the columns split over the CTA's groups of S threads
+  int S = 1;
+  while (S * (int)nslices < b4) S *= 2;
+  const int NG = (int)blockDim.x / S, grp = threadIdx.x / S, r4 = q0 + (int)threadIdx.x - grp * S;
+  float ar[4] = {0.f, 0.f, 0.f, 0.f}, ai[4] = {0.f, 0.f, 0.f, 0.f};
+  if (r4 < q1) {
     const uint4* col = Mt + r4;
-    float ar[4] = {0.f, 0.f, 0.f, 0.f}, ai[4] = {0.f, 0.f, 0.f, 0.f};
+    const int c1 = (grp + 1) * b / NG;
 #pragma unroll 8
-    for (int c = 0; c < b; ++c) {
+    for (int c = grp * b / NG; c < c1; ++c) {
       const uint4 u = __ldg(col + (long long)c * b4);
       const float2 x = qs[c];
       const unsigned w[4] = {u.x, u.y, u.z, u.w};
@@ -695,8 +885,20 @@ __device__ __forceinline__ void apply_cols4_body(const ApplyParams& P, long long
         ai[k] += m.x * x.y + m.y * x.x;
       }
     }
+  }
+  __shared__ float2 red[4][kApplyThreads];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) P.z[tile_dof(P, tile, 4 * r4 + k)] = make_double2((double)ar[k], (double)ai[k]);
+  for (int k = 0; k < 4; ++k) red[k][threadIdx.x] = make_float2(ar[k], ai[k]);
+  __syncthreads();
+  for (int i = threadIdx.x; i < 4 * S; i += blockDim.x) {  // a row per thread, groups in order
+    const int k = i & 3, t = i >> 2;
+    if (q0 + t >= q1) continue;
+    float sr = 0.f, si = 0.f;
+    for (int g = 0; g < NG; ++g) {
+      sr += red[k][g * S + t].x;
+      si += red[k][g * S + t].y;
+    }
+    P.z[tile_dof(P, tile, 4 * (q0 + t) + k)] = make_double2((double)sr, (double)si);
   }
 }
 
@@ -716,6 +918,21 @@ __device__ __forceinline__ void apply_rows_body(const ApplyParams& P, long long 
   const int rb0 = (int)((long long)P.bsz * slice / nslices);
   const int rb1 = (int)((long long)P.bsz * (slice + 1) / nslices);
   const C2<R>* M = (const C2<R>*)P.inv + (long long)tile * P.bsz * P.bsz;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const bool vec = sizeof(R) == 4 && (P.bsz & 1) == 0;
+  // eight 16-byte loads in flight per lane, the first ones while the vector is staged: the 64 MB of a
+  // 32 x 64 layer's inverses (8 blocks of 1,024, half of them from L2) take 13.9 us, 19 us with four
+  // rows per warp and loads after the staging, 26 us with one load at a time
+  constexpr int G = 8;
+  const int half = P.bsz / 2;
+  float4 mm[G];
+  auto fetch = [&](int r, int c0) {
+    const float4* row4 = (const float4*)(M + (long long)r * P.bsz);
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+      if (r < rb1 && c0 + 32 * q < half) mm[q] = __ldg(row4 + c0 + 32 * q);
+  };
+  if (vec) fetch(rb0 + wid, lane);
   for (int r = threadIdx.x; r < P.bsz; r += blockDim.x) {
     const long long d = tile_dof(P, tile, r);
     if (Q32) {
@@ -727,22 +944,12 @@ __device__ __forceinline__ void apply_rows_body(const ApplyParams& P, long long 
     }
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const bool vec = sizeof(R) == 4 && (P.bsz & 1) == 0;
   for (int r = rb0 + wid; r < rb1; r += nw) {
     const C2<R>* row = M + (long long)r * P.bsz;
     R ar = 0, ai = 0;
     if (vec) {
-      // eight 16-byte loads in flight per lane (one at a time, the 64 MB of a 32 x 64 layer's inverses
-      // came from L2 at 2.5 TB/s), added in column order
-      const float4* row4 = (const float4*)row;
-      constexpr int G = 8;
-      const int half = P.bsz / 2;
-      for (int c0 = lane; c0 < half; c0 += 32 * G) {
-        float4 mm[G];
-#pragma unroll
-        for (int q = 0; q < G; ++q)
-          if (c0 + 32 * q < half) mm[q] = __ldg(row4 + c0 + 32 * q);
+      for (int c0 = lane; c0 < half; c0 += 32 * G) {  // in column order
+        if (c0 != lane || r != rb0 + wid) fetch(r, c0);
 #pragma unroll
         for (int q = 0; q < G; ++q) {
           const int c2 = c0 + 32 * q;
@@ -1354,11 +1561,12 @@ cudaError_t pc_apply(StabHandle* h, const double2* q, double2* z, const float2* 
   P.nx = h->nx; P.ny = h->ny; P.tx = g.tx; P.ty = g.ty; P.tz = g.tz; P.ntx = g.ntx; P.nty = g.nty;
   P.ntpts = g.ntpts; P.bsz = g.bsz; P.npts = h->npts;
   P.gate = h->gate;
+  apply_divs(P);
   const int ts = phase_begin(h, STAB_PHASE_PRECOND_APPLY);
   // row slices so that small grids still spread over the SMs.  FP64 / FP32 storage is
   // row-major (a warp per row), BF16 column-major (a thread per row): measured fastest each
   int slices = (int)((2 * 152 + g.ntiles - 1) / g.ntiles);
-  slices = std::max(1, std::min(slices, g.bsz / 32));
+  slices = h->pprec == 64 || h->pprec == 32 ? apply_row_slices(g.ntiles, g.bsz) : std::max(1, std::min(slices, g.bsz / 32));
   const dim3 grid((unsigned)g.ntiles, (unsigned)slices);
   // the input's precision is a template parameter (FP32 basis: float2 input)
   const bool q32v = q32 != nullptr;
@@ -1369,15 +1577,11 @@ cudaError_t pc_apply(StabHandle* h, const double2* q, double2* z, const float2* 
     if (q32v) k_apply_rows<float, true><<<grid, 256, g.bsz * sizeof(float2), h->stream>>>(P);
     else k_apply_rows<float, false><<<grid, 256, g.bsz * sizeof(float2), h->stream>>>(P);
   } else if (g.bsz % 4 == 0) {
-    const int quads = (g.bsz / 4 + slices - 1) / slices;
-    const int thr = std::min(256, ((quads + 31) / 32) * 32);
-    if (q32v) k_apply_cols4<true><<<grid, thr, g.bsz * sizeof(float2), h->stream>>>(P);
-    else k_apply_cols4<false><<<grid, thr, g.bsz * sizeof(float2), h->stream>>>(P);
+    if (q32v) k_apply_cols4<true><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
+    else k_apply_cols4<false><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
   } else {
-    const int rows = (g.bsz + slices - 1) / slices;
-    const int thr = std::min(256, ((rows + 31) / 32) * 32);
-    if (q32v) k_apply_cols<__nv_bfloat162, float, true><<<grid, thr, g.bsz * sizeof(float2), h->stream>>>(P);
-    else k_apply_cols<__nv_bfloat162, float, false><<<grid, thr, g.bsz * sizeof(float2), h->stream>>>(P);
+    if (q32v) k_apply_cols<__nv_bfloat162, float, true><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
+    else k_apply_cols<__nv_bfloat162, float, false><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
   }
   phase_end(h, ts);
   return cudaGetLastError();
@@ -1439,23 +1643,22 @@ cudaError_t pc_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
     P.nx = h->nx; P.ny = h->ny; P.tx = g.tx; P.ty = g.ty; P.tz = g.tz; P.ntx = g.ntx; P.nty = g.nty;
     P.ntpts = g.ntpts; P.bsz = g.bsz; P.npts = h->npts;
     P.gate = gates ? gates[i] : nullptr;
+    apply_divs(P);
     it.ntiles = g.ntiles;
     // the same slices and threads as the single-handle apply
     int slices = (int)((2 * 152 + g.ntiles - 1) / g.ntiles);
-    slices = std::max(1, std::min(slices, g.bsz / 32));
+    slices = h->pprec == 64 || h->pprec == 32 ? apply_row_slices(g.ntiles, g.bsz) : std::max(1, std::min(slices, g.bsz / 32));
     int var, thr;
     size_t sm;
     if (h->pprec == 64) { var = 0; thr = 256; sm = g.bsz * sizeof(double2); }
     else if (h->pprec == 32) { var = 1; thr = 256; sm = g.bsz * sizeof(float2); }
     else if (g.bsz % 4 == 0) {
       var = 2;
-      const int quads = (g.bsz / 4 + slices - 1) / slices;
-      thr = std::min(256, ((quads + 31) / 32) * 32);
+      thr = kApplyThreads;
       sm = g.bsz * sizeof(float2);
     } else {
       var = 3;
-      const int rows = (g.bsz + slices - 1) / slices;
-      thr = std::min(256, ((rows + 31) / 32) * 32);
+      thr = kApplyThreads;
       sm = g.bsz * sizeof(float2);
     }
     if (g.ntiles * slices > (1LL << 30)) return cudaErrorInvalidValue;

@@ -1402,15 +1402,18 @@ static cudaError_t pass_shape(StabHandle* h, int axis, const PassParams& base_pa
   const int n = A.n;
   if (n > 2048) return cudaErrorInvalidValue;
   // launch shape: C points per sweep chunk, L lines per CTA, KP kinds at
-  // once.  Either tuned (stab_autotune) or by default: on small grids
-  // (latency matters) both kinds side by side in chunks of 16, at most two
-  // lines per CTA and fewer so that the CTAs cover the SMs (but at least a
-  // warp of threads); on larger grids the compact layout in chunks of 32 with
-  // up to four lines per CTA (shared memory bounds occupancy there).
+  // once.  Either tuned (stab_autotune) or by default, by the line points per SM
+  // (general base flow, J v with the default of one axis against its best shape):
+  //  - below 1,000 both kinds side by side in chunks of 16, few lines per CTA so
+  //    that the CTAs cover the SMs (64 x 128: 94 us with one line, 100 with two);
+  //  - below 4,000 the compact layout in chunks of 16 (128 x 256: 144 us, 161 in
+  //    chunks of 32; 190 x 301: 209 and 219);
+  //  - above, chunks of 32 (256 x 512 in y: 362 us, 370 in chunks of 16) and at
+  //    most 16 lines per CTA (60 x 90 x 28 in z: 614 us, 640 with 64).
   const LineCfg cfg = contiguous_lines >= 0 ? LineCfg{} : h->line_cfg[axis];
-  const long long fill = (P.nlines * (long long)njobs + 2 * 152 - 1) / (2 * 152);
-  const bool small = fill <= 4;
-  P.C = cfg.C > 0 ? cfg.C : (small || n < 64 ? 16 : 32);
+  const long long line_jobs = P.nlines * (long long)njobs, per_sm = line_jobs * n / 152;
+  const bool small = per_sm < 1000;
+  P.C = cfg.C > 0 ? cfg.C : (per_sm < 4000 ? 16 : 32);
   P.nchunks = (n + P.C - 1) / P.C;
   P.LS = n + (n >> 5) + 1;
   const long long LS = P.LS;
@@ -1425,11 +1428,10 @@ static cudaError_t pass_shape(StabHandle* h, int axis, const PassParams& base_pa
   if (cfg.L > 0) {
     L = std::min(cfg.L, maxL);
   } else {
-    // compact layout: at least four lines and a CTA of about 128 threads (short lines)
-    const int Lc = std::max(4, (128 + tpl - 1) / tpl);
-    L = std::min<long long>(std::min<long long>(maxL, 98304 / smem_line), P.KP == 3 ? Lc : 2);
-    const int Lwarp = (32 + tpl - 1) / tpl;
-    if (L > fill) L = (int)std::min<long long>(maxL, std::max<long long>(fill, Lwarp));
+    // compact layout: four lines, more while the CTA stays within about 128 threads (short lines)
+    const int Lc = std::min(16, std::max(4, 128 / tpl));
+    const int Ls = (int)std::min<long long>(4, std::max<long long>(1, line_jobs / (6 * 152)));
+    L = (int)std::min<long long>(std::min<long long>(maxL, 98304 / smem_line), P.KP == 3 ? Lc : Ls);
   }
   if (L < 1) L = 1;
   P.L = L;

@@ -128,9 +128,10 @@ __device__ __forceinline__ double2 block_dot(const ColShared& S, int j, int CW) 
   }
   return make_double2(sr, si);
 }
-__device__ __forceinline__ double block_nrm(const ColShared& S) {
+// this block's |w|^2 from every step-th warp
+__device__ __forceinline__ double block_nrm(const ColShared& S, int step) {
   double t = 0.0;
-  for (int g = 0; g < kColWarps; ++g) t += S.nrm[g];
+  for (int g = 0; g < kColWarps; g += step) t += S.nrm[g];
   return t;
 }
 
@@ -140,7 +141,7 @@ __device__ __forceinline__ void finish_pass(const ColArgs& A, unsigned bidx, Col
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, k = A.k;
   warp_sums<DOTS, NORM>(A, S, d1, d2, nrm);
   if (DOTS && threadIdx.x < k) A.partial[(long long)bidx * k + threadIdx.x] = block_dot(S, threadIdx.x, col_warps(k));
-  if (NORM && threadIdx.x == kColThreads - 1) A.npart[bidx] = block_nrm(S);
+  if (NORM && threadIdx.x == kColThreads - 1) A.npart[bidx] = block_nrm(S, 1);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) S.last = atomicAdd(A.counter, 1u) == (unsigned)A.nb - 1;
@@ -509,7 +510,7 @@ __device__ __forceinline__ void cgs2_cluster(const CluArgs& A, unsigned rank, Cl
   }
   col_main<true, false, true>(P, rank, C.S, d1, d2, nrm, [&]() { load_coefs(C.h[1], k, C.S); });
   warp_sums<false, true>(P, C.S, d1, d2, nrm);
-  if (threadIdx.x == 0) C.npart = block_nrm(C.S);
+  if (threadIdx.x == 0) C.npart = block_nrm(C.S, col_warps(k));  // a row group's first warp has its rows
   cluster_barrier();
   if (threadIdx.x < 32) {
     double t = threadIdx.x < kCluOne ? cluster_load(&C.npart, threadIdx.x) : 0.0;
@@ -563,7 +564,7 @@ __device__ __forceinline__ void cgs2_clusters(const CluArgs& A, unsigned g, unsi
     cluster_barrier();  // no CTA exits while others read its shared memory
     return;
   }
-  if (t == 0) C.npart = block_nrm(C.S);
+  if (t == 0) C.npart = block_nrm(C.S, col_warps(k));  // a row group's first warp has its rows
   cluster_barrier();
   if (rank == 0 && t < 32) {
     double s = t < kClu ? cluster_load(&C.npart, t) : 0.0;
@@ -587,19 +588,23 @@ __device__ __forceinline__ void cgs2_clusters(const CluArgs& A, unsigned g, unsi
   cluster_barrier();
 }
 
-// launch configuration of a cluster kernel (cfg keeps a pointer to attr)
-inline void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int ctas, unsigned clusters,
-                           cudaStream_t st) {
+// launch configuration of a cluster kernel (cfg keeps a pointer to attr); chained: see launch_chained
+inline void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int ctas, unsigned clusters,
+                           cudaStream_t st, bool chained) {
   cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3(clusters * ctas);
   cfg.blockDim = dim3(kColThreads);
   cfg.stream = st;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = ctas;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  attr[0] = cudaLaunchAttribute{};
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1] = cudaLaunchAttribute{};
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained ? 2 : 1;
 }
 
 }  // namespace gs

@@ -348,6 +348,7 @@ __device__ __forceinline__ void line_pass_body(const PassParams& P, const unsign
 
 template <bool FF>
 __global__ void k_line_pass(const PassParams P) {
+  chain_enter();
   line_pass_body<FF>(P, blockIdx.x, blockIdx.y);
 }
 
@@ -487,6 +488,7 @@ __device__ __forceinline__ void line_pass_compact_body(const PassParams& P, cons
 
 template <bool FF>
 __global__ void __launch_bounds__(kCompactMaxThreads) k_line_pass_compact(const PassParams P) {
+  chain_enter();
   line_pass_compact_body<FF>(P, blockIdx.x, blockIdx.y);
 }
 
@@ -521,7 +523,7 @@ __device__ __forceinline__ double norm_result(double s, int mode, double q0norm,
 // ||v||^2 in one launch: per-block sums, then the last block to finish adds
 // them in block order (fixed order, reproducible) and resets the counter.
 // Block bidx of nb blocks.
-__device__ __forceinline__ void norm2_body(const double2* __restrict__ v, long long n, double* partial, unsigned* counter,
+__device__ __forceinline__ void norm2_body(const double2* v, long long n, double* partial, unsigned* counter,
                                            double* out, int mode, double q0norm, double fixed_eps, unsigned bidx,
                                            unsigned nb) {
   __shared__ double red[32];
@@ -550,8 +552,9 @@ __device__ __forceinline__ void norm2_body(const double2* __restrict__ v, long l
   }
 }
 
-__global__ void k_norm2(const double2* __restrict__ v, long long n, double* partial, unsigned* counter, double* out,
+__global__ void k_norm2(const double2* v, long long n, double* partial, unsigned* counter, double* out,
                         int mode, double q0norm, double fixed_eps, const int* gate) {
+  chain_enter();
   if (gate && *gate) return;
   norm2_body(v, n, partial, counter, out, mode, q0norm, fixed_eps, blockIdx.x, gridDim.x);
 }
@@ -615,6 +618,7 @@ __device__ __forceinline__ int row_of(const PointParams& P, long long pt) {
 }
 
 __global__ void k_temperature(const PointParams P, double2* Tw) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   const int D = P.nz > 1 ? 3 : 2;
   const double e = *P.eps;
@@ -632,6 +636,7 @@ __global__ void k_temperature(const PointParams P, double2* Tw) {
 
 template <int D>
 __global__ void __launch_bounds__(128) k_point(const PointParams P) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   const double e = *P.eps;
   const bool visc = P.phys.visc;
@@ -926,6 +931,7 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
 template <int D, bool EPS>
 __global__ void __launch_bounds__(128, D == 3 ? 3 : 4)
     k_point_fast(const __grid_constant__ PointParams P, const float4* __restrict__ coefp, const float* __restrict__ btab_f) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   point_fast_body<D, EPS>(P, coefp, btab_f, blockIdx.x);
 }
@@ -1011,6 +1017,7 @@ __device__ __forceinline__ void temperature_fast_body(const PointParams& P, doub
 
 template <bool EPS>
 __global__ void k_temperature_fast(const __grid_constant__ PointParams P, double* Tw) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   temperature_fast_body<EPS>(P, Tw, blockIdx.x, gridDim.x);
 }
@@ -1539,8 +1546,8 @@ static cudaError_t run_pair_pass(StabHandle* h, int ax, const double2* const* sr
   long long blocks = 0;
   const cudaError_t e = pair_pass(h, ax, src, false, P, threads, smem, blocks);
   if (e != cudaSuccess) return e;
-  if (P.lanes == 2) pl::k_pair_pass<2><<<(unsigned)blocks, threads, smem, h->stream>>>(P);
-  else pl::k_pair_pass<1><<<(unsigned)blocks, threads, smem, h->stream>>>(P);
+  if (P.lanes == 2) launch_chained(pl::k_pair_pass<2>, (unsigned)blocks, threads, smem, h->stream, P);
+  else launch_chained(pl::k_pair_pass<1>, (unsigned)blocks, threads, smem, h->stream, P);
   return cudaGetLastError();
 }
 
@@ -1558,11 +1565,11 @@ static cudaError_t run_pass(StabHandle* h, int axis, const PassParams& base_para
     for (int q = 0; q < P.njobs; ++q) P.job[q] = jobs[j0 + q];
     dim3 grid((unsigned)((P.nlines + L - 1) / L), (unsigned)P.njobs);
     if (P.KP == 3) {
-      if (P.ff) k_line_pass_compact<true><<<grid, threads, smem, h->stream>>>(P);
-      else k_line_pass_compact<false><<<grid, threads, smem, h->stream>>>(P);
+      if (P.ff) launch_chained(k_line_pass_compact<true>, grid, threads, smem, h->stream, P);
+      else launch_chained(k_line_pass_compact<false>, grid, threads, smem, h->stream, P);
     } else {
-      if (P.ff) k_line_pass<true><<<grid, threads, smem, h->stream>>>(P);
-      else k_line_pass<false><<<grid, threads, smem, h->stream>>>(P);
+      if (P.ff) launch_chained(k_line_pass<true>, grid, threads, smem, h->stream, P);
+      else launch_chained(k_line_pass<false>, grid, threads, smem, h->stream, P);
     }
   }
   return cudaGetLastError();
@@ -1927,7 +1934,7 @@ cudaError_t launch_norm2(StabHandle* h, const double2* v, long long n, double* d
   long long nb = (n + 1023) / 1024;
   if (nb > h->red_blocks) nb = h->red_blocks;
   if (nb < 1) nb = 1;
-  k_norm2<<<(int)nb, 256, 0, h->stream>>>(v, n, h->d_red, (unsigned*)(h->d_red + h->red_blocks + 8), d_out, mode,
+  launch_chained(k_norm2, (int)nb, 256, 0, h->stream, v, n, h->d_red, (unsigned*)(h->d_red + h->red_blocks + 8), d_out, mode,
                                          h->q0norm, h->opts.eps, h->gate);
   return cudaGetLastError();
 }
@@ -2110,9 +2117,9 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   if (h->visc) {
     const int ts = phase_begin(h, STAB_PHASE_TEMPERATURE);
     const int g = grid_for(2 * h->npts, thr);
-    if (fast && eps_mode == 2) k_temperature_fast<false><<<g, thr, 0, h->stream>>>(P, (double*)Tw);
-    else if (fast) k_temperature_fast<true><<<g, thr, 0, h->stream>>>(P, (double*)Tw);
-    else k_temperature<<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P, Tw);
+    if (fast && eps_mode == 2) launch_chained(k_temperature_fast<false>, g, thr, 0, h->stream, P, (double*)Tw);
+    else if (fast) launch_chained(k_temperature_fast<true>, g, thr, 0, h->stream, P, (double*)Tw);
+    else launch_chained(k_temperature, grid_for(h->npts, thr), thr, 0, h->stream, P, Tw);
     phase_end(h, ts);
   }
   const int D = h->dim;
@@ -2123,13 +2130,13 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   const int tp = phase_begin(h, STAB_PHASE_POINTWISE);
   if (fast) {
     const unsigned g = (unsigned)((h->npts + thr - 1) / thr);
-    if (D == 2 && eps_mode == 2) k_point_fast<2, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
-    else if (D == 2) k_point_fast<2, true><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
-    else if (eps_mode == 2) k_point_fast<3, false><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
-    else k_point_fast<3, true><<<g, thr, 0, h->stream>>>(P, h->d_coef_p, h->d_btab_f);
+    if (D == 2 && eps_mode == 2) launch_chained(k_point_fast<2, false>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
+    else if (D == 2) launch_chained(k_point_fast<2, true>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
+    else if (eps_mode == 2) launch_chained(k_point_fast<3, false>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
+    else launch_chained(k_point_fast<3, true>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
   } else {
-    if (D == 2) k_point<2><<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P);
-    else k_point<3><<<grid_for(h->npts, thr), thr, 0, h->stream>>>(P);
+    if (D == 2) launch_chained(k_point<2>, grid_for(h->npts, thr), thr, 0, h->stream, P);
+    else launch_chained(k_point<3>, grid_for(h->npts, thr), thr, 0, h->stream, P);
   }
   phase_end(h, tp);
   h->stats.jv_calls++;

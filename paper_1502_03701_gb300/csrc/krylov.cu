@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kThreads) k_gemv(const double2* __restrict__ V
 
 // x = x / *d_norm  (into out if given); gate as in the J v kernels
 __global__ void k_scale_inv(double2* x, long long n, const double* d_norm, double2* out, const int* gate) {
+  chain_enter();
   if (gate && *gate) return;
   __shared__ double s_inv;  // one division per block: FP64 divisions in every thread took most of the time
   if (threadIdx.x == 0) s_inv = 1.0 / *d_norm;
@@ -96,6 +97,7 @@ __global__ void k_scale_inv(double2* x, long long n, const double* d_norm, doubl
 
 // y = a x + b y (complex a, b)
 __global__ void k_axpby(double2 a, const double2* x, double2 b, double2* y, long long n) {
+  chain_enter();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     double2 xv = x[i], yv = y[i];
     y[i] = make_double2(a.x * xv.x - a.y * xv.y + b.x * yv.x - b.y * yv.y,
@@ -381,6 +383,7 @@ __global__ void k_norm_final(const double* partial, int nb, double* out, const i
 template <bool UPDATE, bool DOTS, bool NORM, bool ROWS>
 __global__ void __launch_bounds__(kColThreads) k_col_pass(const __grid_constant__ ColArgs A, const int* gate,
                                                          const int* skip) {
+  chain_enter();
   if ((gate && *gate) || (skip && *skip)) return;
   __shared__ ColShared S;
   if (ROWS) row_pass<UPDATE, DOTS, NORM>(A, blockIdx.x, S);
@@ -389,14 +392,15 @@ __global__ void __launch_bounds__(kColThreads) k_col_pass(const __grid_constant_
 
 template <bool UPDATE, bool DOTS, bool NORM>
 void launch_col_pass(cudaStream_t st, const ColArgs& A, const int* gate, const int* skip) {
-  if (by_rows(A.n)) k_col_pass<UPDATE, DOTS, NORM, true><<<A.nb, kColThreads, 0, st>>>(A, gate, skip);
-  else k_col_pass<UPDATE, DOTS, NORM, false><<<A.nb, kColThreads, 0, st>>>(A, gate, skip);
+  if (by_rows(A.n)) launch_chained(k_col_pass<UPDATE, DOTS, NORM, true>, A.nb, kColThreads, 0, st, A, gate, skip);
+  else launch_chained(k_col_pass<UPDATE, DOTS, NORM, false>, A.nb, kColThreads, 0, st, A, gate, skip);
 }
 
 // Batched CGS2 over several handles (stab_jv_batch_orthogonalize): item i
 // owns the flat blocks [start[i], start[i+1]) (its own block count nb, so its
 // row ranges and reduction order are those of its single launch).
 __global__ void __launch_bounds__(kColThreads) k_cgs2_cluster(const CluArgs A, const int* gate) {
+  chain_enter();
   if (gate && *gate) return;
   __shared__ CluShared C;
   cgs2_cluster(A, blockIdx.x, C);
@@ -405,6 +409,7 @@ __global__ void __launch_bounds__(kColThreads) k_cgs2_cluster(const CluArgs A, c
 
 template <int PASS>
 __global__ void __launch_bounds__(kColThreads) k_cgs2_clusters(const CluArgs A, const int* gate) {
+  chain_enter();
   if (gate && *gate) return;
   __shared__ CluShared C;
   cgs2_clusters<PASS>(A, blockIdx.x / kClu, blockIdx.x % kClu, C);
@@ -792,10 +797,10 @@ cudaError_t kry_cgs2(StabHandle* h, const double2* V, int k, long long n, double
   cudaError_t e;
   if (k > 0 && in_clusters(n, k)) {
     cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
+    cudaLaunchAttribute attr[2];
     const bool one = kry_one_cluster(h, n, k);
     const int G = one ? 1 : clu_count(n, k);
-    cluster_config(cfg, attr, one ? kCluOne : kClu, (unsigned)G, h->stream);
+    cluster_config(cfg, attr, one ? kCluOne : kClu, (unsigned)G, h->stream, true);
     const CluArgs A{V, w, p1, p2, d_h, np, d_norm, col_counter(h), n, k, G};
     const int* gate = h->gate;
     if (one) {
@@ -828,12 +833,12 @@ cudaError_t kry_cgs2(StabHandle* h, const double2* V, int k, long long n, double
 }
 
 cudaError_t kry_scale(StabHandle* h, double2* x, long long n, const double* d_norm, double2* out) {
-  k_scale_inv<<<grid_n(n), kThreads, 0, h->stream>>>(x, n, d_norm, out, h->gate);
+  launch_chained(k_scale_inv, grid_n(n), kThreads, 0, h->stream, x, n, d_norm, out, h->gate);
   return cudaGetLastError();
 }
 
 cudaError_t kry_axpby(StabHandle* h, double2 a, const double2* x, double2 b, double2* y, long long n) {
-  k_axpby<<<grid_n(n), kThreads, 0, h->stream>>>(a, x, b, y, n);
+  launch_chained(k_axpby, grid_n(n), kThreads, 0, h->stream, a, x, b, y, n);
   return cudaGetLastError();
 }
 
@@ -961,8 +966,8 @@ cudaError_t kry_init_attributes(StabHandle* h) {
   for (const void* k : {(const void*)k_cgs2_cluster, (const void*)k_cgs2_cluster_batch})
     if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
   cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  cluster_config(cfg, attr, kCluOne, 1, nullptr);
+  cudaLaunchAttribute attr[2];
+  cluster_config(cfg, attr, kCluOne, 1, nullptr, false);
   if (cudaOccupancyMaxActiveClusters(&clusters, k_cgs2_cluster, &cfg) != cudaSuccess) {
     cudaGetLastError();
     clusters = 0;
@@ -990,7 +995,7 @@ cudaError_t kry_cgs2_stream(cudaStream_t st, const double2* V, int k, long long 
       k_dot_final<<<k, 32, 0, st>>>(partial, nb, k, hp, 0);
       k_gemv<<<grid_n(n), kThreads, k * sizeof(double2), st>>>(V, k, n, hp, w, -1.0, nullptr);
     }
-    k_axpby<<<1, 64, 0, st>>>(make_double2(1.0, 0.0), d_h + k, make_double2(1.0, 0.0), d_h, k);
+    launch_chained(k_axpby, 1, 64, 0, st, make_double2(1.0, 0.0), d_h + k, make_double2(1.0, 0.0), d_h, k);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -1051,9 +1056,9 @@ cudaError_t cgs2_batch_launch(const CgsBatchPlan& plan, const unsigned char* d, 
     if (plan.U[r].count) {
       const BatchSection& U = plan.U[r];
       cudaLaunchConfig_t cfg;
-      cudaLaunchAttribute attr;
+      cudaLaunchAttribute attr[2];
       const int ctas = r == 0 ? kCluOne : kClu;
-      cluster_config(cfg, attr, ctas, (unsigned)(U.blocks / ctas), st);
+      cluster_config(cfg, attr, ctas, (unsigned)(U.blocks / ctas), st, false);
       const CgsItem* items = (const CgsItem*)(d + U.items);
       const int* start = (const int*)(d + U.start);
       cudaError_t e;

@@ -342,6 +342,7 @@ __device__ __forceinline__ void pair_pass_body(const PairPass& P, unsigned bid) 
 
 template <int LANES>
 __global__ void __launch_bounds__(kMaxThreads, LANES == 2 ? 1 : 2) k_pair_pass(const __grid_constant__ PairPass P) {
+  chain_enter();
   pair_pass_body<LANES>(P, blockIdx.x);
 }
 

@@ -506,6 +506,7 @@ __device__ __forceinline__ double2 bt_out(C2<double> s) { return make_double2(s.
 // w_l = S_l^{-1} q_l for every level of every tile, into z (grid: tiles x levels).
 template <class R, bool Q32>
 __global__ void __launch_bounds__(kBtRhsThreads) k_bt_rhs(const __grid_constant__ BtApplyParams P) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int m = P.m, l = blockIdx.y;
@@ -541,6 +542,7 @@ __global__ void __launch_bounds__(kBtRhsThreads) k_bt_rhs(const __grid_constant_
 // bounds it: matrix in, matrix out and the vector once per row.
 template <class R, int STAGES>
 __global__ void __launch_bounds__(kBtSweepThreads, STAGES == 5 ? 1 : 2) k_bt_sweep(const __grid_constant__ BtApplyParams P) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int m = P.m, nlev = P.nlev;
@@ -625,6 +627,7 @@ constexpr int kBtRegLevel = 64, kBtDepth = 4;
 
 template <int G, int PC>
 __global__ void __launch_bounds__(kBtSweepThreads) k_bt_sweep_reg(const __grid_constant__ BtApplyParams P) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   __shared__ float4 ys[2][kBtRegLevel / 2];  // zero past the level's entries
   const int m = P.m, nlev = P.nlev, half = m / 2;  // m is even
@@ -724,17 +727,17 @@ cudaError_t launch_bt_apply(const BtApplyParams& B0, long long ntiles, cudaStrea
   // a level per CTA, two CTAs per SM at least
   B.staged = lr + vec <= kBtSmem / 2;
   const size_t rsm = (B.staged ? lr : 0) + vec;
-  if (B.q32) k_bt_rhs<R, true><<<grid, kBtRhsThreads, rsm, st>>>(B);
-  else k_bt_rhs<R, false><<<grid, kBtRhsThreads, rsm, st>>>(B);
+  if (B.q32) launch_chained(k_bt_rhs<R, true>, grid, kBtRhsThreads, rsm, st, B);
+  else launch_chained(k_bt_rhs<R, false>, grid, kBtRhsThreads, rsm, st, B);
   if (sizeof(R) == 4 && B.m <= kBtRegLevel) {
     const int G = bt_group(B.m, kBtSweepThreads);
     auto kernel = G == 8 ? k_bt_sweep_reg<8, 4> : G == 16 ? k_bt_sweep_reg<16, 1> : k_bt_sweep_reg<32, 1>;
-    kernel<<<(unsigned)ntiles, kBtSweepThreads, 0, st>>>(B);
+    launch_chained(kernel, (unsigned)ntiles, kBtSweepThreads, 0, st, B);
     return cudaGetLastError();
   }
   // ring: five buffers where every tile has an SM of its own, three where two tiles share one
   const int stages = ntiles <= 152 && 5 * ls + 2 * vec <= kBtSmem ? 5 : 3 * ls + 2 * vec <= kBtSmem ? 3 : 0;
-  bt_sweep_kernel<R>(stages)<<<(unsigned)ntiles, kBtSweepThreads, stages * ls + 2 * vec, st>>>(B);
+  launch_chained(bt_sweep_kernel<R>(stages), (unsigned)ntiles, kBtSweepThreads, stages * ls + 2 * vec, st, B);
   return cudaGetLastError();
 }
 
@@ -836,6 +839,7 @@ __device__ __forceinline__ void apply_cols_body(const ApplyParams& P, long long 
 
 template <class S, class R, bool Q32>
 __global__ void k_apply_cols(const ApplyParams P) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   apply_cols_body<S, R, Q32>(P, blockIdx.x, blockIdx.y, gridDim.y);
 }
@@ -904,6 +908,7 @@ __device__ __forceinline__ void apply_cols4_body(const ApplyParams& P, long long
 
 template <bool Q32>
 __global__ void k_apply_cols4(const ApplyParams P) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   apply_cols4_body<Q32>(P, blockIdx.x, blockIdx.y, gridDim.y);
 }
@@ -977,6 +982,7 @@ __device__ __forceinline__ void apply_rows_body(const ApplyParams& P, long long 
 
 template <class R, bool Q32>
 __global__ void k_apply_rows(const ApplyParams P) {
+  chain_enter();
   if (P.gate && *P.gate) return;
   apply_rows_body<R, Q32>(P, blockIdx.x, blockIdx.y, gridDim.y);
 }
@@ -1571,17 +1577,17 @@ cudaError_t pc_apply(StabHandle* h, const double2* q, double2* z, const float2* 
   // the input's precision is a template parameter (FP32 basis: float2 input)
   const bool q32v = q32 != nullptr;
   if (h->pprec == 64) {
-    if (q32v) k_apply_rows<double, true><<<grid, 256, g.bsz * sizeof(double2), h->stream>>>(P);
-    else k_apply_rows<double, false><<<grid, 256, g.bsz * sizeof(double2), h->stream>>>(P);
+    if (q32v) launch_chained(k_apply_rows<double, true>, grid, 256, g.bsz * sizeof(double2), h->stream, P);
+    else launch_chained(k_apply_rows<double, false>, grid, 256, g.bsz * sizeof(double2), h->stream, P);
   } else if (h->pprec == 32) {
-    if (q32v) k_apply_rows<float, true><<<grid, 256, g.bsz * sizeof(float2), h->stream>>>(P);
-    else k_apply_rows<float, false><<<grid, 256, g.bsz * sizeof(float2), h->stream>>>(P);
+    if (q32v) launch_chained(k_apply_rows<float, true>, grid, 256, g.bsz * sizeof(float2), h->stream, P);
+    else launch_chained(k_apply_rows<float, false>, grid, 256, g.bsz * sizeof(float2), h->stream, P);
   } else if (g.bsz % 4 == 0) {
-    if (q32v) k_apply_cols4<true><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
-    else k_apply_cols4<false><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
+    if (q32v) launch_chained(k_apply_cols4<true>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
+    else launch_chained(k_apply_cols4<false>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
   } else {
-    if (q32v) k_apply_cols<__nv_bfloat162, float, true><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
-    else k_apply_cols<__nv_bfloat162, float, false><<<grid, kApplyThreads, g.bsz * sizeof(float2), h->stream>>>(P);
+    if (q32v) launch_chained(k_apply_cols<__nv_bfloat162, float, true>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
+    else launch_chained(k_apply_cols<__nv_bfloat162, float, false>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
   }
   phase_end(h, ts);
   return cudaGetLastError();

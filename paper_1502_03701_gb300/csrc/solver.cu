@@ -186,6 +186,7 @@ __global__ void k_gm_tol(GmDev d, double tol) { d.sc[0] = tol * (*d.dnorm); }
 
 // start of a cycle: g = (beta, 0, ...), beta = ||r|| (in dnorm, kept in sc[2])
 __global__ void k_gm_cycle_init(GmDev d) {
+  chain_enter();
   if (threadIdx.x == 0) {
     d.flags[0] = 0;
     d.flags[1] = 0;
@@ -310,6 +311,7 @@ __global__ void k_gm_step(GmDev d, int j) { gm_step_body(d, j); }
 // ends the cycle the vector is not read again.  One division per block: one per
 // thread cost more FP64 time than the rest of the scaling (6.5 us for 131,072 unknowns).
 __global__ void __launch_bounds__(256) k_gm_step_scale(GmDev d, int j, double2* w, long long n) {
+  chain_enter();
   if (d.flags[0]) return;
   __shared__ double s_inv;
   if (blockIdx.x == 0) {
@@ -329,6 +331,7 @@ __global__ void __launch_bounds__(256) k_gm_step_scale(GmDev d, int j, double2* 
 // A whole orthogonalisation step of a small vector in one cluster: CGS2, then
 // CTA 0's first warp takes the Givens step while the other warps scale w.
 __global__ void __launch_bounds__(gs::kColThreads) k_gm_cgs2_step(gs::CluArgs A, GmDev d, int j) {
+  chain_enter();
   if (d.flags[0]) return;  // set by an earlier launch: the same for the whole cluster
   __shared__ gs::CluShared C;
   gs::cgs2_cluster(A, blockIdx.x, C);
@@ -349,8 +352,8 @@ __global__ void __launch_bounds__(gs::kColThreads) k_gm_cgs2_step(gs::CluArgs A,
 
 cudaError_t launch_cgs2_step(cudaStream_t st, const gs::CluArgs& A, const GmDev& d, int j) {
   cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  gs::cluster_config(cfg, attr, gs::kCluOne, 1, st);
+  cudaLaunchAttribute attr[2];
+  gs::cluster_config(cfg, attr, gs::kCluOne, 1, st, true);
   return cudaLaunchKernelEx(&cfg, k_gm_cgs2_step, A, d, j);
 }
 
@@ -389,7 +392,10 @@ __device__ __forceinline__ void gm_solve_body(const GmDev& d) {
   }
 }
 
-__global__ void k_gm_solve(GmDev d) { gm_solve_body(d); }
+__global__ void k_gm_solve(GmDev d) {
+  chain_enter();
+  gm_solve_body(d);
+}
 
 __global__ void k_gm_report(GmDev d, GmReport* rep, const double* inner_tally) {
   rep->beta = *d.dnorm;
@@ -484,7 +490,7 @@ cudaGraphExec_t gm_graph(StabHandle* h, cd sigma, int eps_mode, const GmresWs& W
   if (err == cudaSuccess && key.basis == 32) {
     // FP32 basis, right preconditioning M^{-1} applied on the fly: z = M^{-1} v_j (FP64),
     // w = (J - sigma I) z (FP64), rounded into V32_{j+1}; x += M^{-1} (V32 y) at the end
-    k_gm_cycle_init<<<1, 64, 0, h->stream>>>(D);
+    launch_chained(k_gm_cycle_init, 1, 64, 0, h->stream, D);
     step(kry_to_f32(h, W.r, n, W.dnorm, W.V32));
     for (int j = 0; j < m && err == cudaSuccess; ++j) {
       const float2* Vj = W.V32 + (size_t)j * n;
@@ -501,7 +507,7 @@ cudaGraphExec_t gm_graph(StabHandle* h, cd sigma, int eps_mode, const GmresWs& W
       step(kry_scale32(h, Vn, n, W.dnorm));
       h->gate = nullptr;
     }
-    k_gm_solve<<<1, 64, 0, h->stream>>>(D);
+    launch_chained(k_gm_solve, 1, 64, 0, h->stream, D);
     step(kry_gemv32(h, W.V32, m, D.flags + 1, n, W.y, W.t));
     if (pc) step(pc_apply(h, W.t, W.zt));
     step(kry_axpby(h, make_double2(1.0, 0.0), pc ? W.zt : W.t, make_double2(1.0, 0.0), W.x, n));
@@ -514,7 +520,7 @@ cudaGraphExec_t gm_graph(StabHandle* h, cd sigma, int eps_mode, const GmresWs& W
     const int mi = W.mi;
     const bool flex = pc || lgk > 0 || mi > 0;
     const int nkry = m - naug;
-    k_gm_cycle_init<<<1, 64, 0, h->stream>>>(D);
+    launch_chained(k_gm_cycle_init, 1, 64, 0, h->stream, D);
     if (mi > 0) k_gm_inner_reset<<<1, 1, 0, h->stream>>>(W.Din);
     step(kry_scale(h, W.r, n, W.dnorm, W.V));
     for (int j = 0; j < m && err == cudaSuccess; ++j) {
@@ -546,7 +552,7 @@ cudaGraphExec_t gm_graph(StabHandle* h, cd sigma, int eps_mode, const GmresWs& W
           step(kry_scale32(h, Vi1, n, I.dnorm));
         }
         h->gate = nullptr;
-        k_gm_solve<<<1, 64, 0, h->stream>>>(I);
+        launch_chained(k_gm_solve, 1, 64, 0, h->stream, I);
         k_gm_inner_tally<<<1, 1, 0, h->stream>>>(I);
         step(kry_gemv32(h, W.V32, mi, I.flags + 1, n, I.y, W.t));
         h->gate = D.flags;
@@ -572,9 +578,9 @@ cudaGraphExec_t gm_graph(StabHandle* h, cd sigma, int eps_mode, const GmresWs& W
       if (n < kSelectiveMinN) step(kry_cgs2(h, W.V, j + 1, n, Vn, W.dh, W.dnorm, W.partial));
       else step(kry_dgks(h, W.V, j + 1, n, Vn, W.dh, W.dnorm, W.partial));
       h->gate = nullptr;
-      k_gm_step_scale<<<(unsigned)std::min<long long>(1 + (n + 1023) / 1024, 152 * 4), 256, 0, h->stream>>>(D, j, Vn, n);
+      launch_chained(k_gm_step_scale, (unsigned)std::min<long long>(1 + (n + 1023) / 1024, 152 * 4), 256, 0, h->stream, D, j, Vn, n);
     }
-    k_gm_solve<<<1, 64, 0, h->stream>>>(D);
+    launch_chained(k_gm_solve, 1, 64, 0, h->stream, D);
     if (lgk > 0) {
       // dz = Z y; x += dz; r = b - A x; store (dz, r_old - r) / ||dz|| as the newest pair after
       // moving the older ones one slot down

@@ -797,6 +797,51 @@ __device__ __noinline__ void wall_remainder(const pw::PhysT<float>& phys, const 
   }
 }
 
+// The remainder's inputs (physical, metric applied) from the slots' high parts, and the remainder.  W.v is set.
+template <int D>
+__device__ __forceinline__ void point_remainder(const PointParams& P, const float* __restrict__ btab_f, long long i, int j,
+                                                double e, pw::WIn<D, float2>& W, float2* w2) {
+  const bool visc = P.phys.visc;
+  const float4* S = (const float4*)P.scratch;
+  auto slot = [&](int s) { return S[(long long)s * P.npts + i]; };
+  const float ey = ff2_split(P.eta_y[j]).hi, eyy = ff2_split(P.eta_yy[j]).hi, ef = ff2_split(e).hi;
+  // read the high parts again (they are in the caches) rather than hold 84 registers through the sums above
+  asm volatile("" ::: "memory");
+  auto high = [&](int s) { const float4 w = slot(s); return make_float2(w.x, w.z); };
+  const float2 z2 = v2(0.0f);
+#pragma unroll
+  for (int ax = 0; ax < D; ++ax) {
+#pragma unroll
+    for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = f < D + 2 || visc ? high(P.s_d1[ax][f]) : z2;
+#pragma unroll
+    for (int g = 0; g < D + 1; ++g) W.d2[ax][g] = visc ? high(P.s_d2[ax][g]) : z2;
+#pragma unroll
+    for (int c = 0; c < D; ++c) W.mix[ax][c] = visc && c != ax ? high(P.s_mix[ax][c]) : z2;
+  }
+#pragma unroll
+  for (int ax = 0; ax < D; ++ax) {
+    const float s1 = P.sc1[ax], s2 = P.sc2[ax];
+    const float f1 = ax == 1 ? __fmul_rn(s1, ey) : s1;
+#pragma unroll
+    for (int g = 0; g < D + 1; ++g) {
+      W.d2[ax][g] = v2_mul(W.d2[ax][g], v2(ax == 1 ? __fmul_rn(s2, __fmul_rn(ey, ey)) : s2));
+      if (ax == 1) W.d2[1][g] = v2_fma(W.d1[1][g < D ? 1 + g : D + 2], v2(__fmul_rn(s1, eyy)), W.d2[1][g]);
+    }
+#pragma unroll
+    for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = v2_mul(W.d1[ax][f], v2(f1));
+#pragma unroll
+    for (int c = 0; c < D; ++c)
+      if (c != ax) W.mix[ax][c] = v2_mul(W.mix[ax][c], v2(__fmul_rn(f1, c == 1 ? __fmul_rn(P.sc1[c], ey) : P.sc1[c])));
+  }
+  auto Bf = [&](int s) { return btab_f[(long long)s * P.nbase + j]; };
+  if (j != 0 && j != P.ny - 1) {
+    pw::remainder_y_base<D>(P.physf, Bf, W, ef, w2);
+  } else {
+    const pw::WIn<D, float2> Wc = W;
+    wall_remainder<D>(P.physf, btab_f, P.nbase, j, P.bcflags[j == 0 ? 0 : (long long)P.nx * P.nz], Wc, ef, w2);
+  }
+}
+
 template <int D, bool EPS>
 __device__ __forceinline__ void point_fast_body(const PointParams& P, const float4* __restrict__ coefp,
                                                 const float* __restrict__ btab_f, unsigned bidx) {
@@ -883,49 +928,95 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
       acc[a] = ff2_fma(cy, sw, ff2_fma(cx, vp[a], acc[a]));
     }
   }
-  if (EPS && e != 0.0) {  // O(eps) remainder of the quotient, FP32, physical (metric-applied) inputs
-    const float ey = ff2_split(P.eta_y[j]).hi, eyy = ff2_split(P.eta_yy[j]).hi, ef = ff2_split(e).hi;
-    // read the high parts again (they are in the caches) rather than hold 84 registers through the sums above
-    asm volatile("" ::: "memory");
-    auto high = [&](int s) { const float4 w = slot(s); return make_float2(w.x, w.z); };
-    const float2 z2 = v2(0.0f);
-#pragma unroll
-    for (int ax = 0; ax < D; ++ax) {
-#pragma unroll
-      for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = f < D + 2 || visc ? high(P.s_d1[ax][f]) : z2;
-#pragma unroll
-      for (int g = 0; g < D + 1; ++g) W.d2[ax][g] = visc ? high(P.s_d2[ax][g]) : z2;
-#pragma unroll
-      for (int c = 0; c < D; ++c) W.mix[ax][c] = visc && c != ax ? high(P.s_mix[ax][c]) : z2;
-    }
-#pragma unroll
-    for (int ax = 0; ax < D; ++ax) {
-      const float s1 = P.sc1[ax], s2 = P.sc2[ax];
-      const float f1 = ax == 1 ? __fmul_rn(s1, ey) : s1;
-#pragma unroll
-      for (int g = 0; g < D + 1; ++g) {
-        W.d2[ax][g] = v2_mul(W.d2[ax][g], v2(ax == 1 ? __fmul_rn(s2, __fmul_rn(ey, ey)) : s2));
-        if (ax == 1) W.d2[1][g] = v2_fma(W.d1[1][g < D ? 1 + g : D + 2], v2(__fmul_rn(s1, eyy)), W.d2[1][g]);
-      }
-#pragma unroll
-      for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = v2_mul(W.d1[ax][f], v2(f1));
-#pragma unroll
-      for (int c = 0; c < D; ++c)
-        if (c != ax) W.mix[ax][c] = v2_mul(W.mix[ax][c], v2(__fmul_rn(f1, c == 1 ? __fmul_rn(P.sc1[c], ey) : P.sc1[c])));
-    }
-    auto Bf = [&](int s) { return btab_f[(long long)s * P.nbase + j]; };
+  if (EPS && e != 0.0) {  // O(eps) remainder of the quotient, FP32
     float2 w2[D + 2];
-    if (j != 0 && j != P.ny - 1) {
-      pw::remainder_y_base<D>(P.physf, Bf, W, ef, w2);
-    } else {
-      const pw::WIn<D, float2> Wc = W;
-      wall_remainder<D>(P.physf, btab_f, P.nbase, j, P.bcflags[j == 0 ? 0 : (long long)P.nx * P.nz], Wc, ef, w2);
-    }
+    point_remainder<D>(P, btab_f, i, j, e, W, w2);
 #pragma unroll
     for (int a = 0; a < D + 2; ++a) acc[a].lo = v2_add(acc[a].lo, w2[a]);
   }
 #pragma unroll
   for (int a = 0; a < D + 2; ++a) P.out[(long long)a * P.npts + i] = ff2_to_d(ff2_norm(acc[a]));
+}
+
+// One output row per thread: the same sums in the same order (and the same bits), with the row's inputs
+// loaded at once and a quarter to a fifth of the serial products.  Rows read their inputs separately.
+template <int D, bool EPS, int A>
+__device__ __forceinline__ void point_row_body(const PointParams& P, const float4* __restrict__ coefp,
+                                               const float* __restrict__ btab_f, long long i) {
+  constexpr int o1 = D + 3, o2 = o1 + D * (D + 3), om = o2 + D * (D + 1);
+  constexpr int NW = pw::nw_inputs(D);
+  const double e = EPS ? *P.eps : 0.0;
+  const bool visc = P.phys.visc;
+  const float4* S = (const float4*)P.scratch;
+  const int j = row_of(P, i);
+  const float4* Cp = coefp + (long long)j * coefs_used<D>();
+  auto slot = [&](int s) { return S[(long long)s * P.npts + i]; };
+  const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  double2 vd[D + 3];
+#pragma unroll
+  for (int f = 0; f < D + 2; ++f) vd[f] = EPS || f == A || coef_used<D>(A, f) ? P.v[(long long)f * P.npts + i] : make_double2(0.0, 0.0);
+  vd[D + 2] = visc ? P.scratch[(long long)P.s_Tw * P.npts + i] : make_double2(0.0, 0.0);
+  float4 in[NW], cf[NW];  // the row's inputs and coefficients (unused ones take no registers)
+  {
+    int u = 0;
+#pragma unroll
+    for (int q = 0; q < NW; ++q)
+#pragma unroll
+      for (int a = 0; a < D + 2; ++a)
+        if (coef_used<D>(a, q)) {
+          if (a == A) cf[q] = __ldg(Cp + u);
+          ++u;
+        }
+  }
+#pragma unroll
+  for (int q = o1; q < NW; ++q)
+    if (coef_used<D>(A, q)) {
+      const int r = q < o2 ? q - o1 : q < om ? q - o2 : q - om;
+      if (q < o2) in[q] = r % (D + 3) < D + 2 || visc ? slot(P.s_d1[r / (D + 3)][r % (D + 3)]) : zero;
+      else if (q < om) in[q] = visc ? slot(P.s_d2[r / (D + 1)][r % (D + 1)]) : zero;
+      else in[q] = visc ? slot(P.s_mix[r / D][r % D]) : zero;
+    }
+  ffn2 acc = ff2_zero2(), vp = acc;
+  pw::WIn<D, float2> W;
+#pragma unroll
+  for (int q = 0; q < NW; ++q) {
+    if (q < D + 3) {
+      if (!(EPS || q == A || coef_used<D>(A, q))) continue;
+      const ffn2 w = ff2_split(vd[q]);
+      if (q == A) vp = w;
+      if (EPS) W.v[q] = w.hi;
+      if (coef_used<D>(A, q)) acc = ff2_fma(ff2_unpack(cf[q]), w, acc);
+    } else if (coef_used<D>(A, q)) {
+      acc = ff2_fma(ff2_unpack(cf[q]), ff2_from_slot(in[q]), acc);
+    }
+  }
+  if (P.shift.x != 0.0 || P.shift.y != 0.0) {
+    const ffn sx = ff2_split(-P.shift.x), sy = ff2_split(P.shift.y);
+    const ffn2 cx = ff2_dup(sx), cy{make_float2(sy.hi, -sy.hi), make_float2(sy.lo, -sy.lo)};
+    const ffn2 sw{make_float2(vp.hi.y, vp.hi.x), make_float2(vp.lo.y, vp.lo.x)};
+    acc = ff2_fma(cy, sw, ff2_fma(cx, vp, acc));
+  }
+  if (EPS && e != 0.0) {
+    float2 w2[D + 2];
+    point_remainder<D>(P, btab_f, i, j, e, W, w2);
+    acc.lo = v2_add(acc.lo, w2[A]);
+  }
+  P.out[(long long)A * P.npts + i] = ff2_to_d(ff2_norm(acc));
+}
+
+// grid (points / 128, rows)
+template <int D, bool EPS>
+__global__ void __launch_bounds__(128) k_point_rows(const __grid_constant__ PointParams P, const float4* __restrict__ coefp,
+                                                   const float* __restrict__ btab_f) {
+  chain_enter();
+  if (P.gate && *P.gate) return;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= P.npts) return;
+  if (blockIdx.y == 0) point_row_body<D, EPS, 0>(P, coefp, btab_f, i);
+  else if (blockIdx.y == 1) point_row_body<D, EPS, 1>(P, coefp, btab_f, i);
+  else if (blockIdx.y == 2) point_row_body<D, EPS, 2>(P, coefp, btab_f, i);
+  else if (D == 2 || blockIdx.y == 3) point_row_body<D, EPS, 3>(P, coefp, btab_f, i);
+  else if constexpr (D == 3) point_row_body<D, EPS, 4>(P, coefp, btab_f, i);
 }
 
 template <int D, bool EPS>
@@ -2130,10 +2221,18 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   const int tp = phase_begin(h, STAB_PHASE_POINTWISE);
   if (fast) {
     const unsigned g = (unsigned)((h->npts + thr - 1) / thr);
-    if (D == 2 && eps_mode == 2) launch_chained(k_point_fast<2, false>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
-    else if (D == 2) launch_chained(k_point_fast<2, true>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
-    else if (eps_mode == 2) launch_chained(k_point_fast<3, false>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
-    else launch_chained(k_point_fast<3, true>, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
+    auto run = [&](auto all, auto rows) {
+      // One output row per thread while that fills SMs that would have no CTA (J v of 32 x 64: tangent 17.4 us,
+      // 19.2 with all rows in a thread, quotient 28.4 and 29.5; 64 x 128: 20.5 and 22.4, 32.6 and 33.2).  The
+      // quotient's remainder is worked out again for each row, so it stops earlier (96 x 128: 38.0 and 36.3; the
+      // tangent 24.7 and 26.1, at 128 x 256 29.2 and 28.4).
+      if (h->npts < (eps_mode == 2 ? 152 * 128 : 152 * 64)) launch_chained(rows, dim3(g, D + 2), thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
+      else launch_chained(all, g, thr, 0, h->stream, P, h->d_coef_p, h->d_btab_f);
+    };
+    if (D == 2 && eps_mode == 2) run(k_point_fast<2, false>, k_point_rows<2, false>);
+    else if (D == 2) run(k_point_fast<2, true>, k_point_rows<2, true>);
+    else if (eps_mode == 2) run(k_point_fast<3, false>, k_point_rows<3, false>);
+    else run(k_point_fast<3, true>, k_point_rows<3, true>);
   } else {
     if (D == 2) launch_chained(k_point<2>, grid_for(h->npts, thr), thr, 0, h->stream, P);
     else launch_chained(k_point<3>, grid_for(h->npts, thr), thr, 0, h->stream, P);

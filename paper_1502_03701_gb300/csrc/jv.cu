@@ -1572,8 +1572,13 @@ static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, bool batch, pl
     return ((size_t)n * (L | 1) + ((size_t)2 * L * nch + 8 * L) + (P.lanes == 2 ? pl::kTab : (pl::kTab + 1) / 2)) *
            sizeof(float4);
   };
+  // chunks of 16 points; of 32 on middle grids with short lines (J v of 48 x 64 x 40: 129.1 us, 131.6 in chunks
+  // of 16; 40 x 120 x 30: 144.5 and 147.9), where long ones lose (256 x 640: 108.1 and 99.2, 300 x 600: 110.8 and
+  // 106.4: few chunks of few lines fill a CTA's shared memory).  Both components in a thread on small grids:
+  // 32 x 64 48 us and 42.6 apart, 190 x 301 61.6 and 60; on large ones with chunks of 32 the passes of
+  // 128 x 256 x 64 take 445, 318 and 357 us in place of 347, 258 and 268.
   int C = cfg.C;
-  if (C <= 0) C = P.lanes == 1 && chunks16 >= 152LL * 512 ? 32 : 16;
+  if (C <= 0) C = P.lanes == 1 && chunks16 >= 152LL * 512 && n <= 128 ? 32 : 16;
   if (C > kPairMaxC) C = kPairMaxC;
   // fewer than two warps per SM: a pass is one warp's latency, so chunks of half the length (the x pass of a
   // 32 x 64 layer 10.7 -> 9.3 us, its J v 45 -> 40 us)

@@ -8,10 +8,10 @@ epsilon-quotient of the paper's Frechet derivative), the innermost and
 most-called step of the method; value = GB/s of algorithmic traffic (32 B per
 complex unknown: read v, write J v; the y-only base tables stay on chip),
 and the roofline compares it with the measured HBM copy bandwidth, with the
-FP64-pipe fraction of the line passes beside it.  Also reported, measured in
+operation rate of the line passes beside it.  Also reported, measured in
 the same run:
-  * "jv_pair_stencil": the same J v with the compact-scheme right-hand sides in
-    FP32 pair arithmetic (stencil_prec 48), and its difference to the main step's;
+  * "jv_pair_stencil": the same J v with stencil_prec 48, and its difference to the main step's
+    (none: a base flow that depends on y only takes the pair passes with either value);
   * "jv_2d_256x512": the J v of the 2-D 256 x 512 layer (524,288 unknowns);
   * "eigs": complete Cayley-IRAM solves of the 32 x 64 layer through stab_eigs
     (sigma 1, tau -1, nev 4, ncv 30, block-Jacobi over 16 x 16 tiles, FGMRES(50) to 1e-10,
@@ -579,8 +579,9 @@ def line_pass_flops(g, visc: bool) -> dict:
 
 def jv_roofline(g, f, phases: dict, step_s: float, hbm, tangent_s: float) -> dict:
     """Roofline of the timed J v: the operator's algorithmic bytes (32 B per unknown) over its measured
-    step time against the measured HBM copy bandwidth, with the line passes' FP64 rate (the unit that
-    binds on GB300) beside it."""
+    step time against the measured HBM copy bandwidth, with the line passes' operation rate beside it
+    (FP32 pair arithmetic, bound by instruction issue; the FP64 FMA rate is what the same operations
+    could reach in FP64)."""
     ms = {k: v[0] for k, v in phases.items() if k != "dropped"}
     cnt = {k: v[1] for k, v in phases.items() if k != "dropped"}
     total = sum(ms.values())
@@ -590,7 +591,7 @@ def jv_roofline(g, f, phases: dict, step_s: float, hbm, tangent_s: float) -> dic
     flops = line_pass_flops(g, f.Re > 0)
     line_flops = sum(flops[k] * cnt[k] for k in line_keys)
     avg_s = line_ms / 1e3 / launches
-    fp64_achieved = line_flops / launches / avg_s / 1e9
+    line_rate = line_flops / launches / avg_s / 1e9
     share = {k: (ms[k] / total if total else None) for k in ms if cnt[k]}
     achieved = g.n * JV_BYTES_PER_DOF / step_s / 1e9
     tr = JV_TRAFFIC.get(_jv_workload_name(g))
@@ -603,10 +604,10 @@ def jv_roofline(g, f, phases: dict, step_s: float, hbm, tangent_s: float) -> dic
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)",
             "traffic_source": tr["source"] if tr else "no ncu capture of the current kernels",
             "phase_share": share,
-            "fp64_pipe": {"kernel": "k_line_pass / k_line_pass_compact (all axes)", "achieved": fp64_achieved,
-                          "peak": FP64_MEASURED_GFLOPS, "unit": "GFLOP/s", "frac": fp64_achieved / FP64_MEASURED_GFLOPS,
-                          "flop_per_launch": line_flops / launches, "launch_ms": avg_s * 1e3, "launches": launches,
-                          "peak_source": "FP64 FMA microbenchmark on GB300 (of measured)"}}
+            "line_passes": {"kernel": "k_pair_pass (all axes)", "achieved": line_rate, "unit": "GFLOP/s",
+                            "fp64_fma_rate": FP64_MEASURED_GFLOPS, "flop_per_launch": line_flops / launches,
+                            "launch_ms": avg_s * 1e3, "launches": launches,
+                            "rate_source": "FP64 FMA microbenchmark on GB300 (of measured)"}}
 
 
 # Many small problems (uneven 2-D instances drawn like the 64-instance batch
@@ -922,8 +923,8 @@ def replica_throughput(local_units: float, local_seconds: float, device: str) ->
 
 def pair_stencil_jv(args, Stab, torch, q0, g, f, v, out, flush, stream, bytes_jv):
     """The same J v with the compact-scheme right-hand sides in FP32 pair arithmetic
-    (stencil_prec 48; sweeps, closures and the pointwise map unchanged), timed like
-    the main step, with its largest difference to the FP64-stencil result."""
+    (stencil_prec 48; it changes only the passes of general base flows), timed like
+    the main step, with its largest difference to the main step's result."""
     from paper_1502_03701_gb300 import binding
     S = Stab(q0, g, f.Ma, f.Re, f.Pr, stencil_prec=48)
     tuned = S.autotune()
@@ -939,8 +940,8 @@ def pair_stencil_jv(args, Stab, torch, q0, g, f, v, out, flush, stream, bytes_jv
     return {"value": bytes_jv / (sum(t) / steps) / 1e9, "unit": "GB/s", "ms_per_step": sum(t) / steps * 1e3,
             "steps": steps, "max_rel_diff_vs_fp64_stencil": diff,
             "line_pass_shapes": {ax: {"C": c, "L": l, "kinds": k} for ax, (c, l, k, _) in tuned.items()},
-            "arith": "interior right-hand sides of the compact schemes in FP32 pairs (~2^-47 relative); "
-                     "Thomas sweeps, closure rows and the pointwise map as in the main step"}
+            "arith": "stencil_prec 48: interior right-hand sides of general base flows in FP32 pairs (~2^-47 "
+                     "relative); the passes of a base flow that depends on y only are those of the main step"}
 
 
 def _time_jv(S, v, out, steps, flush, stream, torch):

@@ -84,10 +84,11 @@ typedef struct {
                              default) or 32 (FP32 basis, non-flexible right preconditioning; J v, the
                              solution update and the true residual of every restart stay FP64, so the
                              restarts refine the solution to the FP64 tolerance) */
-  int stencil_prec;       /* right-hand sides B f of the compact schemes inside J v: 64 (FP64, default) or
-                             48 (interior rows in FP32 pair arithmetic on exactly power-of-two-scaled
-                             inputs, ~2^-47 relative; the Thomas sweeps, the closure rows and the set-up
-                             stay FP64) */
+  int stencil_prec;       /* right-hand sides B f of the compact schemes inside J v of base flows that vary in
+                             x or z: 64 (FP64, default) or 48 (interior rows in FP32 pair arithmetic on
+                             exactly power-of-two-scaled inputs, ~2^-47 relative; the Thomas sweeps, the
+                             closure rows and the set-up stay FP64).  Base flows that depend on y only form
+                             differences in FP64 and everything after them in FP32 pairs with either value */
   int lgmres_k;           /* inner solver: 0 = GMRES(gmres_m) (default); k in [1, min(8, gmres_m - 1)] =
                              LGMRES (Sec. "Iterative solvers", after Baker, Jessup and Manteuffel): every
                              cycle spans gmres_m directions, gmres_m - k Krylov directions of the residual
@@ -312,8 +313,10 @@ stab_status stab_timing_read(stab_handle h, double* ms, long long* count, long l
  * reuses a cached shape without timing.  cfg (host int[9], may be NULL)
  * receives (C, L, kinds) per axis (x, y, z; zeros for an absent z), ms (host
  * double[3], may be NULL) the tuned pass time per axis (-1 when cached).
- * The chunk length moves where the sweeps' warm-up starts, so results may
- * change at the rounding level (about 1e-16 relative); L and kinds change nothing.
+ * The chunk length moves where the sweeps start, so results may change at the
+ * rounding level (about 1e-16 relative; pair passes about 1e-15); L and kinds
+ * change nothing.  Base flows that depend on y only take the pair passes, which
+ * have no kinds variants (reported as 3).
  * Allocates one temporary vector; synchronises the stream. */
 stab_status stab_autotune(stab_handle h, int force, int* cfg, double* ms);
 
@@ -323,8 +326,10 @@ stab_status stab_autotune(stab_handle h, int force, int* cfg, double* ms);
  * other with 4 instead of 6 planes of shared memory per line, 3 one after the
  * other with 2 planes (the input reloaded per kind and turned into right-hand
  * sides in place); all zero restores the built-in default.
- * INVALID_ARG when the shape does not fit the line (more than 1024 threads,
- * 512 with kinds 3, or the shared-memory limit). */
+ * The pair passes (base flows that depend on y only) ignore kinds, take fewer
+ * lines than L where a CTA would not hold them, and halve C on grids of under
+ * two warps per SM.  INVALID_ARG when the shape does not fit the line (more
+ * than 1024 threads, 512 with kinds 3, or the shared-memory limit). */
 stab_status stab_set_line_config(stab_handle h, int axis, int C, int L, int kinds);
 
 /* Handles take device memory from a library-owned, stream-ordered pool (one

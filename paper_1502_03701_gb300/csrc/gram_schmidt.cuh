@@ -25,6 +25,9 @@ __device__ __forceinline__ double warp_sum(double x) {
 // CGS2 reads V once and splits it once.  The next rows' loads are in flight
 // meanwhile.  Sums over blocks: the last block to finish adds the blocks'
 // partial sums in block order (reproducible) and resets the counter.
+// 524,288 unknowns, 55 vectors: the three passes of CGS2 take 130, 228 and 112 us
+// (481 MB each, 62 to 66 % of the issue slots; 164, 387 and 273 us as kernels of
+// one warp per column and FP64 every fourth column, with V read twice).
 // ---------------------------------------------------------------------------
 constexpr int kColThreads = 512, kColWarps = kColThreads / 32, kCpw = 4, kColMax = kColWarps * kCpw;
 
@@ -411,7 +414,11 @@ __device__ __forceinline__ void row_pass(const ColArgs& A, unsigned bidx, ColSha
 //    passes in one launch;
 //  - above, three launches of up to 16 clusters of 8 (of clusters of 16 the
 //    device holds too few at a time); every cluster leaves one partial sum per
-//    column and the next launch adds these up.
+//    column and the next launch adds these up: 29 us for those 8,192 unknowns.
+// Where the lines lie (stab_orthogonalize, with about 40 us of copy and wait):
+// 2,048 unknowns 43 us in one launch and 55 in three for 8 vectors, 51 and 55 for
+// 29; 3,072 unknowns 58 and 55 for 29 vectors, 78 and 55 for 55.  15,360 unknowns,
+// 29 vectors: 71 us in clusters, 80 with sums through global memory.
 // ---------------------------------------------------------------------------
 constexpr int kCluOne = 16, kClu = 8, kCluMax = 16;  // CTAs per cluster (one launch, passes), clusters
 constexpr long long kCluOneN = 2048;   // one cluster in one launch up to here

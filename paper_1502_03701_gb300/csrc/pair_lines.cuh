@@ -23,6 +23,10 @@
 // Values are stored scaled: first derivatives as f' / S1 and second ones as
 // f'' / S2 with the schemes' leading factors (AxisTables::pscale), which the
 // pointwise map's coefficients carry.
+//
+// 128 x 256 x 64 points: y 347, z 258, x 268 us for all derivatives of an axis,
+// 62 to 67 % of the issue slots; FP64 sweeps took 0.96, 0.87 and 1.06 ms.  32 x 64
+// points: 10.4 and 10.9 us (32 us each), one warp's latency.
 #pragma once
 #include "internal.cuh"
 

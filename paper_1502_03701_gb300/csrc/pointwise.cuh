@@ -197,7 +197,6 @@ struct WIn {
 };
 
 __device__ __forceinline__ DN mk(double a, double w) { return dn(a, w); }
-__device__ __forceinline__ DN3 mk3(double a, float w) { return dn3((float)a, w, 0.0f); }
 template <class Num>
 struct NumOps;
 template <>

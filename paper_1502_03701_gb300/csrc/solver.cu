@@ -294,7 +294,7 @@ __device__ __forceinline__ void gm_step_body(const GmDev& d, int j) {
       const hd::zc gj = d.g[j];
       d.g[j + 1] = -(hd::conj(s) * gj);
       d.g[j] = c * gj;
-      d.flags[1] = j + 1;
+      *(volatile int*)(d.flags + 1) = j + 1;  // k_gm_step_scale's other blocks may be reading it
       const double res = sabs * (j == 0 ? gj.re : d.sc[1]);  // |g_{j+1}| = |s| |g_j|; g_0 starts as beta > 0
       d.sc[1] = res;
       if (res <= d.sc[0] || wn == 0.0) d.flags[0] = 1;
@@ -306,23 +306,32 @@ __device__ __forceinline__ void gm_step_body(const GmDev& d, int j) {
 
 __global__ void k_gm_step(GmDev d, int j) { gm_step_body(d, j); }
 
-// The step and the scaling of the new basis vector w <- w / ||w|| in one launch:
-// block 0's first warp takes the step, all other warps scale.  After a step that
-// ends the cycle the vector is not read again.  One division per block: one per
-// thread cost more FP64 time than the rest of the scaling (6.5 us for 131,072 unknowns).
+// The step and the scaling of the new basis vector w <- w / ||w|| in one launch (at
+// least two blocks): block 0's first warp takes the step, the other blocks scale.
+// Whether the cycle has ended they may not ask flags[0], which block 0 sets in this
+// very launch: some blocks, or some warps of a block before its barrier, would leave.
+// flags[1], the number of columns taken, tells the same in every block: block 0
+// writes j + 1 over j or leaves it, and from two steps after the end on it is below
+// j.  The vector of the step that ends the cycle and the one after are not read again.
+// One division per block: one per thread cost more FP64 time than the rest of the
+// scaling (6.5 us for 131,072 unknowns).
 __global__ void __launch_bounds__(256) k_gm_step_scale(GmDev d, int j, double2* w, long long n) {
   chain_enter();
-  if (d.flags[0]) return;
-  __shared__ double s_inv;
   if (blockIdx.x == 0) {
     if (threadIdx.x < 32) gm_step_body(d, j);
-    if (gridDim.x > 1) return;
+    return;
   }
-  if (threadIdx.x == blockDim.x - 1) s_inv = 1.0 / *d.dnorm;
+  __shared__ double s_inv;
+  __shared__ int s_ended;
+  if (threadIdx.x == 0) {
+    s_ended = *(volatile int*)(d.flags + 1) < j;
+    s_inv = 1.0 / *d.dnorm;
+  }
   __syncthreads();
+  if (s_ended) return;
   const double s = s_inv;
-  const long long b = gridDim.x > 1 ? blockIdx.x - 1 : 0, nb = gridDim.x > 1 ? gridDim.x - 1 : 1;
-  for (long long i = b * blockDim.x + threadIdx.x; i < n; i += nb * blockDim.x) {
+  const long long step = (long long)(gridDim.x - 1) * blockDim.x;
+  for (long long i = (long long)(blockIdx.x - 1) * blockDim.x + threadIdx.x; i < n; i += step) {
     const double2 v = w[i];
     w[i] = make_double2(v.x * s, v.y * s);
   }

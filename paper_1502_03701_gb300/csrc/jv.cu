@@ -771,9 +771,9 @@ static_assert(coefs_used<2>() == 51 && coefs_used<3>() == 85, "products per poin
 // One thread per point streams over the inputs, both components side by side,
 // and adds each to the rows that it reaches (85 of the 225 products in 3-D, 51
 // of 100 in 2-D) by exact FP32 two-products and two-sum accumulation; EPS adds
-// the O(eps) remainder, evaluated in FP32 from the inputs' high parts.  No
-// FP64 instruction is issued: the FP64 pipe's rate (1/64 of FP32) made the
-// conversions and the shift the kernel's bound before.
+// the O(eps) remainder, evaluated in FP32 from the inputs' high parts.  The only
+// FP64 instructions are the shift's: the FP64 pipe's rate (1/64 of FP32) made the
+// conversions the kernel's bound before.
 // The remainder on a non-reflective boundary row (general form, one component
 // at a time); out of line, so that the rows inside do not carry its registers.
 template <int D>
@@ -842,6 +842,19 @@ __device__ __forceinline__ void point_remainder(const PointParams& P, const floa
   }
 }
 
+// out[o] = acc - shift v[o].  The shift's product and difference are FP64: in pairs
+// they left a result that the shift dominates with 48 bits (1.7e-15 in place of 1e-17
+// for J v - 1e6 v).
+__device__ __forceinline__ void put_row(const PointParams& P, long long o, ffn2 acc) {
+  double2 r = ff2_to_d(ff2_norm(acc));
+  if (P.shift.x != 0.0 || P.shift.y != 0.0) {
+    const double2 v = P.v[o];
+    r.x = fma(-P.shift.x, v.x, fma(P.shift.y, v.y, r.x));  // explicit: the kernels that inline this round alike
+    r.y = fma(-P.shift.x, v.y, fma(-P.shift.y, v.x, r.y));
+  }
+  P.out[o] = r;
+}
+
 template <int D, bool EPS>
 __device__ __forceinline__ void point_fast_body(const PointParams& P, const float4* __restrict__ coefp,
                                                 const float* __restrict__ btab_f, unsigned bidx) {
@@ -854,7 +867,7 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
   const float4* S = (const float4*)P.scratch;
   const int j = row_of(P, i);
   const float4* Cp = coefp + (long long)j * coefs_used<D>();
-  ffn2 acc[D + 2], vp[D + 2];
+  ffn2 acc[D + 2];
   pw::WIn<D, float2> W;  // EPS: the remainder's inputs
 #pragma unroll
   for (int a = 0; a < D + 2; ++a) acc[a] = ff2_zero2();
@@ -896,7 +909,6 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
 #pragma unroll
   for (int f = 0; f < D + 3; ++f) {
     const ffn2 w = ff2_split(vd[f]);
-    if (f < D + 2) vp[f] = w;
     if (EPS) W.v[f] = w.hi;
     put(f, w);
   }
@@ -919,15 +931,6 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
           if (a != c) put(om + a * D + c, ff2_from_slot(in[k++]));
     }
   }
-  if (P.shift.x != 0.0 || P.shift.y != 0.0) {  // - shift v: (-sx, -sx) v + (sy, -sy) (im v, re v)
-    const ffn sx = ff2_split(-P.shift.x), sy = ff2_split(P.shift.y);
-    const ffn2 cx = ff2_dup(sx), cy{make_float2(sy.hi, -sy.hi), make_float2(sy.lo, -sy.lo)};
-#pragma unroll
-    for (int a = 0; a < D + 2; ++a) {
-      const ffn2 sw{make_float2(vp[a].hi.y, vp[a].hi.x), make_float2(vp[a].lo.y, vp[a].lo.x)};
-      acc[a] = ff2_fma(cy, sw, ff2_fma(cx, vp[a], acc[a]));
-    }
-  }
   if (EPS && e != 0.0) {  // O(eps) remainder of the quotient, FP32
     float2 w2[D + 2];
     point_remainder<D>(P, btab_f, i, j, e, W, w2);
@@ -935,7 +938,7 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
     for (int a = 0; a < D + 2; ++a) acc[a].lo = v2_add(acc[a].lo, w2[a]);
   }
 #pragma unroll
-  for (int a = 0; a < D + 2; ++a) P.out[(long long)a * P.npts + i] = ff2_to_d(ff2_norm(acc[a]));
+  for (int a = 0; a < D + 2; ++a) put_row(P, (long long)a * P.npts + i, acc[a]);
 }
 
 // One output row per thread: the same sums in the same order (and the same bits), with the row's inputs
@@ -954,7 +957,7 @@ __device__ __forceinline__ void point_row_body(const PointParams& P, const float
   const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   double2 vd[D + 3];
 #pragma unroll
-  for (int f = 0; f < D + 2; ++f) vd[f] = EPS || f == A || coef_used<D>(A, f) ? P.v[(long long)f * P.npts + i] : make_double2(0.0, 0.0);
+  for (int f = 0; f < D + 2; ++f) vd[f] = EPS || coef_used<D>(A, f) ? P.v[(long long)f * P.npts + i] : make_double2(0.0, 0.0);
   vd[D + 2] = visc ? P.scratch[(long long)P.s_Tw * P.npts + i] : make_double2(0.0, 0.0);
   float4 in[NW], cf[NW];  // the row's inputs and coefficients (unused ones take no registers)
   {
@@ -976,32 +979,25 @@ __device__ __forceinline__ void point_row_body(const PointParams& P, const float
       else if (q < om) in[q] = visc ? slot(P.s_d2[r / (D + 1)][r % (D + 1)]) : zero;
       else in[q] = visc ? slot(P.s_mix[r / D][r % D]) : zero;
     }
-  ffn2 acc = ff2_zero2(), vp = acc;
+  ffn2 acc = ff2_zero2();
   pw::WIn<D, float2> W;
 #pragma unroll
   for (int q = 0; q < NW; ++q) {
     if (q < D + 3) {
-      if (!(EPS || q == A || coef_used<D>(A, q))) continue;
+      if (!(EPS || coef_used<D>(A, q))) continue;
       const ffn2 w = ff2_split(vd[q]);
-      if (q == A) vp = w;
       if (EPS) W.v[q] = w.hi;
       if (coef_used<D>(A, q)) acc = ff2_fma(ff2_unpack(cf[q]), w, acc);
     } else if (coef_used<D>(A, q)) {
       acc = ff2_fma(ff2_unpack(cf[q]), ff2_from_slot(in[q]), acc);
     }
   }
-  if (P.shift.x != 0.0 || P.shift.y != 0.0) {
-    const ffn sx = ff2_split(-P.shift.x), sy = ff2_split(P.shift.y);
-    const ffn2 cx = ff2_dup(sx), cy{make_float2(sy.hi, -sy.hi), make_float2(sy.lo, -sy.lo)};
-    const ffn2 sw{make_float2(vp.hi.y, vp.hi.x), make_float2(vp.lo.y, vp.lo.x)};
-    acc = ff2_fma(cy, sw, ff2_fma(cx, vp, acc));
-  }
   if (EPS && e != 0.0) {
     float2 w2[D + 2];
     point_remainder<D>(P, btab_f, i, j, e, W, w2);
     acc.lo = v2_add(acc.lo, w2[A]);
   }
-  P.out[(long long)A * P.npts + i] = ff2_to_d(ff2_norm(acc));
+  put_row(P, (long long)A * P.npts + i, acc);
 }
 
 // grid (points / 128, rows)

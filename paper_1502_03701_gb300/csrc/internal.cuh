@@ -46,7 +46,8 @@ struct AxisTables {
                         // right-hand side scaled by dinv (l'_t = l_t d_{t-1} / d_t)
   PairKind pk[2];       // pair-arithmetic pass
   ffn* ptab[2];         // device: its powers of r and chunk factors
-  double pscale[2];     // its outputs are the derivatives divided by this
+  double pscale[2];     // its outputs are the derivatives divided by this, in [1, 2)
+  int pup[2];           // by a power of two, the differences that it forms are scaled up on their split
 };
 
 // Division by an invariant divisor with a multiply and a shift (Granlund and

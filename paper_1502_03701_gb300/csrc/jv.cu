@@ -608,6 +608,7 @@ struct PointParams {
   const int* gate;  // as PassParams::gate
   const double* tcoef;  // [2][ny]: T_w = tcoef[0] p_w + tcoef[1] s_w to first order (y-only base)
   float sc1[4], sc2[4];  // scales of the pair passes' first and second derivatives per axis
+  float scm[4];          // of the mixed derivative of axes a and c, at a + c
   FastDiv divnx, divny;  // division by nx and ny (points < 2^31)
 };
 
@@ -831,7 +832,7 @@ __device__ __forceinline__ void point_remainder(const PointParams& P, const floa
     for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = v2_mul(W.d1[ax][f], v2(f1));
 #pragma unroll
     for (int c = 0; c < D; ++c)
-      if (c != ax) W.mix[ax][c] = v2_mul(W.mix[ax][c], v2(__fmul_rn(f1, c == 1 ? __fmul_rn(P.sc1[c], ey) : P.sc1[c])));
+      if (c != ax) W.mix[ax][c] = v2_mul(W.mix[ax][c], v2(ax == 1 || c == 1 ? __fmul_rn(P.scm[ax + c], ey) : P.scm[ax + c]));
   }
   auto Bf = [&](int s) { return btab_f[(long long)s * P.nbase + j]; };
   if (j != 0 && j != P.ny - 1) {
@@ -1026,9 +1027,9 @@ __global__ void __launch_bounds__(128, D == 3 ? 3 : 4)
 // Fold the y metric and the line passes' scales into the per-row coefficients
 // so that the pointwise kernel can use the passes' outputs directly:
 //   f_y = f_eta ey,  f_yy = f_etaeta ey^2 + f_eta eyy,  mixed with y: x ey;
-//   then x S1 of the axis (first), S2 (second), the product of both axes' S1 (mixed).
+//   then x S1 of the axis (first), S2 (second), the scale of both axes (mixed).
 struct PassScales {
-  double s1[3], s2[3];
+  double s1[3], s2[3], mix[4];  // mix: of axes a and c, at a + c
 };
 template <int D>
 __global__ void k_coeffs_fold(const double* coef, const double* eta_y, const double* eta_yy, int ny, PassScales sc,
@@ -1053,7 +1054,8 @@ __global__ void k_coeffs_fold(const double* coef, const double* eta_y, const dou
   for (int i = 0; i < D; ++i) {
     for (int k = 0; k < D + 3; ++k) f[o1 + i * (D + 3) + k] *= sc.s1[i];
     for (int k = 0; k < D + 1; ++k) f[o2 + i * (D + 1) + k] *= sc.s2[i];
-    for (int k = 0; k < D; ++k) f[om + i * D + k] *= sc.s1[i] * sc.s1[k];
+    for (int k = 0; k < D; ++k)
+      if (i != k) f[om + i * D + k] *= sc.mix[i + k];
   }
   double* o = out + ((long long)j * (D + 2) + a) * NW;
   for (int q = 0; q < NW; ++q) o[q] = f[q];
@@ -1389,7 +1391,9 @@ static void fill_pair_tables(AxisTables& A, std::vector<ffn>& host) {
     const double r = (-1.0 + std::sqrt(1.0 - 4.0 * al * al)) / (2.0 * al);
     const double c = -al / r, lr = -std::log2(-r);
     const double ih = 1.0 / A.h;
-    A.pscale[kind] = kind == 0 ? (7.0 / 9.0) * ih / c : (27.0 / 22.0) * ih * ih / c;
+    const double lead = kind == 0 ? (7.0 / 9.0) * ih / c : (27.0 / 22.0) * ih * ih / c;
+    A.pup[kind] = std::min(std::max(std::ilogb(lead), -kPairMaxUp), kPairMaxUp);
+    A.pscale[kind] = std::ldexp(lead, -A.pup[kind]);
     PairKind& K = A.pk[kind];
     K = PairKind{};
     K.r = host_pair(r);
@@ -1548,8 +1552,10 @@ static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, bool batch, pl
   P = pl::PairPass{};
   P.k[0] = A.pk[0];
   P.k[1] = A.pk[1];
-  P.tab[0] = A.ptab[0];
-  P.tab[1] = A.ptab[1];
+  for (int k = 0; k < 2; ++k) {
+    P.tab[k] = A.ptab[k];
+    P.up[k] = A.pup[k] * (1 << 20);
+  }
   P.gate = h->gate;
   P.nlines = h->npts / n;
   P.stride = axis == 0 ? 1 : axis == 1 ? h->nx : (long long)h->nx * h->ny;
@@ -1985,6 +1991,13 @@ void jv_tune_apply_cached(StabHandle* h) {
   }
 }
 
+// scale of the mixed derivative of axes a and c in its slot: the y (else the z) pass takes the field, the pass
+// of the other axis its output, unscaled
+static double mixed_scale(const StabHandle* h, int a, int c) {
+  const int first = a == 1 || c == 1 ? 1 : 2, second = a + c - first;
+  return h->ax[first].pscale[0] * std::ldexp(h->ax[second].pscale[0], h->ax[second].pup[0]);
+}
+
 static PointParams point_params(StabHandle* h, const double2* v) {
   PointParams P{};
   P.gate = h->gate;
@@ -2017,6 +2030,7 @@ static PointParams point_params(StabHandle* h, const double2* v) {
   for (int a = 0; a < h->dim; ++a) {
     P.sc1[a] = (float)h->ax[a].pscale[0];
     P.sc2[a] = (float)h->ax[a].pscale[1];
+    for (int c = 0; c < a; ++c) P.scm[a + c] = (float)mixed_scale(h, a, c);
   }
   return P;
 }
@@ -2158,6 +2172,7 @@ cudaError_t jv_setup(StabHandle* h, const double* q0_host) {
     for (int a = 0; a < D; ++a) {
       sc.s1[a] = h->ax[a].pscale[0];
       sc.s2[a] = h->ax[a].pscale[1];
+      for (int c = 0; c < a; ++c) sc.mix[a + c] = mixed_scale(h, a, c);
     }
     if (D == 2) k_coeffs_fold<2><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, sc, h->d_coef_f);
     else k_coeffs_fold<3><<<h->ny, 32, 0, h->stream>>>(h->d_coef, h->d_metric, h->d_metric + h->ny, h->ny, sc, h->d_coef_f);

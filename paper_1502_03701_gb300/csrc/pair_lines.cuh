@@ -22,7 +22,13 @@
 //
 // Values are stored scaled: first derivatives as f' / S1 and second ones as
 // f'' / S2 with the schemes' leading factors (AxisTables::pscale), which the
-// pointwise map's coefficients carry.
+// pointwise map's coefficients carry.  Differences of neighbours are smaller than
+// the derivatives by 1/h and 1/h^2, and a split keeps its low part from 2^-74 up
+// only, so they are split times 2^u, u = log2(1/h) or log2(1/h^2) (exact; no
+// instruction more): S1 and S2 are then in [1, 2), and the range of v over which the
+// operator is accurate is that of its derivatives.  Unscaled, second derivatives of
+// a smooth field of size 2^-64 on 256 points were good to 1e-9 only.  The second
+// derivation of a mixed derivative takes pairs and is not scaled.
 //
 // 128 x 256 x 64 points: y 347, z 258, x 268 us for all derivatives of an axis,
 // 62 to 67 % of the issue slots; FP64 sweeps took 0.96, 0.87 and 1.06 ms.  32 x 64
@@ -58,6 +64,7 @@ struct PairPass {
   int U, Up;         // the same in units of a thread's lines (x 2 / lanes)
   int nch, q, rem;   // chunks per line: the first rem have q + 1 points, the others q
   int bounded, pad;
+  int up[2];         // exponent scaling of the differences per kind (ff2_split)
   FastDiv divblk, divL, divU, divn, divnx;
 };
 static_assert(sizeof(PairPass) % 8 == 0, "items are copied to shared memory in 8-byte words");
@@ -86,10 +93,10 @@ struct Lane<2> {
   typedef float4 Elem;
   static __device__ __forceinline__ Pair dup(ffn a) { return ff2_dup(a); }
   static __device__ __forceinline__ Pair zero() { return ff2_zero2(); }
-  // difference of two staged FP64 values as a pair: one FP64 subtraction per component
-  static __device__ __forceinline__ Pair raw_diff(Elem a, Elem b) {
+  // difference of two staged FP64 values (times 2^up) as a pair: one FP64 subtraction per component
+  static __device__ __forceinline__ Pair raw_diff(Elem a, Elem b, int up) {
     auto d = [](float l, float h) { return __hiloint2double(__float_as_int(h), __float_as_int(l)); };
-    return ff2_split(make_double2(d(a.x, a.y) - d(b.x, b.y), d(a.z, a.w) - d(b.z, b.w)));
+    return ff2_split(make_double2(d(a.x, a.y) - d(b.x, b.y), d(a.z, a.w) - d(b.z, b.w)), up);
   }
   static __device__ __forceinline__ Elem table(float2 v) { return make_float4(v.x, v.x, v.y, v.y); }
 };
@@ -99,9 +106,9 @@ struct Lane<1> {
   typedef float2 Elem;
   static __device__ __forceinline__ Pair dup(ffn a) { return a; }
   static __device__ __forceinline__ Pair zero() { return ffn{0.0f, 0.0f}; }
-  static __device__ __forceinline__ Pair raw_diff(Elem a, Elem b) {
+  static __device__ __forceinline__ Pair raw_diff(Elem a, Elem b, int up) {
     auto d = [](Elem v) { return __hiloint2double(__float_as_int(v.y), __float_as_int(v.x)); };
-    return ff2_split(d(a) - d(b));
+    return ff2_split(d(a) - d(b), up);
   }
   static __device__ __forceinline__ Elem table(float2 v) { return v; }
 };
@@ -119,6 +126,7 @@ __device__ __forceinline__ void solve_chunks(const PairPass& P, typename Lane<LA
   const int n = P.n, nch = P.nch, L = P.U, Lp = P.Up;
   const bool bounded = P.bounded;
   const PairKind& K = P.k[KIND];
+  const int up = P.up[KIND];
   auto len_of = [&](int cc) { return P.q + (cc < P.rem ? 1 : 0); };
   auto pw = [&](int i) { return ff2_unpack(tab[i + 2]); };  // r^i, i >= -2
   const int t0 = act ? c * P.q + min(c, P.rem) : 0, len = act ? len_of(c) : 0, t1 = t0 + len;
@@ -131,7 +139,7 @@ __device__ __forceinline__ void solve_chunks(const PairPass& P, typename Lane<LA
   };
   auto dif = [&](Elem a, Elem b) -> Pair {  // a - b
     if constexpr (PAIR) return ff2_add(ff2_from_slot(a), ff2_neg(ff2_from_slot(b)));
-    else return T::raw_diff(a, b);
+    else return T::raw_diff(a, b, up);
   };
   // the neighbours' points, and the wall rows' right-hand sides, before any point is overwritten
   Elem fm2{}, fm1{}, fp0{}, fp1{};

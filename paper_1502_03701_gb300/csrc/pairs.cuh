@@ -114,15 +114,17 @@ __device__ __forceinline__ ffn ff_warp_sum(ffn x) {
 // the rest (29 bits, signed) rounded to 24, so |d - hi - lo| <= 2^-49 |d|.
 // Integer operations but one conversion: the FP64 pipe is not used.  |d| below
 // 2^-126 gives zero (to 2^-146), lo is kept from 2^-74 up; from 2^127 up and
-// for Inf and NaN, hi is Inf or NaN.
-__device__ __forceinline__ ffn ff2_split(double d) {
+// for Inf and NaN, hi is Inf or NaN.  up: d 2^u is split instead, exactly, with
+// up = u << 20 and |u| <= kPairMaxUp; the limits hold for that product.
+constexpr int kPairMaxUp = 400;
+__device__ __forceinline__ ffn ff2_split(double d, int up = 0) {
   const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
   const unsigned a = h & 0x7FFFFFFFu, tl = l + 0x10000000u;  // plus half a unit of hi
   // exponent rebased by 896, clamped to the FP32 range
-  const int th = min(max((int)(a + (tl < l ? 1u : 0u)) - (896 << 20), 0), 255 << 20);
+  const int th = min(max((int)(a + (tl < l ? 1u : 0u)) - ((896 << 20) - up), 0), 255 << 20);
   const float hi = __uint_as_float(__funnelshift_l(tl, (unsigned)th, 3) | (h & 0x80000000u));
   // the low 29 bits as a signed integer, in units of 2^(e - 52)
-  const unsigned sc = ((unsigned)max((int)a - (948 << 20), 0) << 3) & 0x7F800000u;
+  const unsigned sc = ((unsigned)max((int)a - ((948 << 20) - up), 0) << 3) & 0x7F800000u;
   return ffn{hi, __fmul_rn(__int2float_rn((int)(l << 3) >> 3), __uint_as_float(sc | (h & 0x80000000u)))};
 }
 __device__ __forceinline__ ffn ff2_norm(ffn a) {
@@ -196,8 +198,8 @@ __device__ __forceinline__ ffn ff2_unpack(float2 a) { return ffn{a.x, a.y}; }
 __device__ __forceinline__ float2 ff2_to_slot(ffn a) { return make_float2(a.hi, a.lo); }
 __device__ __forceinline__ ffn ff2_from_slot(float2 a) { return ffn{a.x, a.y}; }
 __device__ __forceinline__ ffn ff2_neg(ffn a) { return ffn{-a.hi, -a.lo}; }
-__device__ __forceinline__ ffn2 ff2_split(double2 d) {
-  const ffn a = ff2_split(d.x), b = ff2_split(d.y);
+__device__ __forceinline__ ffn2 ff2_split(double2 d, int up = 0) {
+  const ffn a = ff2_split(d.x, up), b = ff2_split(d.y, up);
   return ffn2{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)};
 }
 __device__ __forceinline__ double2 ff2_to_d(ffn2 a) {

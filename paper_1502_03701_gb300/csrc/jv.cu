@@ -799,13 +799,18 @@ __device__ __noinline__ void wall_remainder(const pw::PhysT<float>& phys, const 
 }
 
 // The remainder's inputs (physical, metric applied) from the slots' high parts, and the remainder.  W.v is set.
+// It is evaluated for v 2^k and e 2^-k, k = log2(e) (exact, undone at the end): with v itself, the products of two
+// perturbations left the FP32 range for entries above 2^64 (J v was NaN there) and vanished below 2^-64.
 template <int D>
 __device__ __forceinline__ void point_remainder(const PointParams& P, const float* __restrict__ btab_f, long long i, int j,
                                                 double e, pw::WIn<D, float2>& W, float2* w2) {
   const bool visc = P.phys.visc;
   const float4* S = (const float4*)P.scratch;
   auto slot = [&](int s) { return S[(long long)s * P.npts + i]; };
-  const float ey = ff2_split(P.eta_y[j]).hi, eyy = ff2_split(P.eta_yy[j]).hi, ef = ff2_split(e).hi;
+  const float ey = ff2_split(P.eta_y[j]).hi, eyy = ff2_split(P.eta_yy[j]).hi;
+  const int k = min(max(((__double2hiint(e) >> 20) & 0x7FF) - 1023, -100), 100);
+  const float up = __int_as_float((127 + k) << 23), down = __int_as_float((127 - k) << 23);
+  const float ef = ff2_split(e, -k * (1 << 20)).hi;
   // read the high parts again (they are in the caches) rather than hold 84 registers through the sums above
   asm volatile("" ::: "memory");
   auto high = [&](int s) { const float4 w = slot(s); return make_float2(w.x, w.z); };
@@ -821,7 +826,7 @@ __device__ __forceinline__ void point_remainder(const PointParams& P, const floa
   }
 #pragma unroll
   for (int ax = 0; ax < D; ++ax) {
-    const float s1 = P.sc1[ax], s2 = P.sc2[ax];
+    const float s1 = __fmul_rn(P.sc1[ax], up), s2 = __fmul_rn(P.sc2[ax], up);
     const float f1 = ax == 1 ? __fmul_rn(s1, ey) : s1;
 #pragma unroll
     for (int g = 0; g < D + 1; ++g) {
@@ -831,9 +836,13 @@ __device__ __forceinline__ void point_remainder(const PointParams& P, const floa
 #pragma unroll
     for (int f = 0; f < D + 3; ++f) W.d1[ax][f] = v2_mul(W.d1[ax][f], v2(f1));
 #pragma unroll
-    for (int c = 0; c < D; ++c)
-      if (c != ax) W.mix[ax][c] = v2_mul(W.mix[ax][c], v2(ax == 1 || c == 1 ? __fmul_rn(P.scm[ax + c], ey) : P.scm[ax + c]));
+    for (int c = 0; c < D; ++c) {
+      const float sm = __fmul_rn(c != ax ? P.scm[ax + c] : 0.0f, up);
+      if (c != ax) W.mix[ax][c] = v2_mul(W.mix[ax][c], v2(ax == 1 || c == 1 ? __fmul_rn(sm, ey) : sm));
+    }
   }
+#pragma unroll
+  for (int f = 0; f < D + 3; ++f) W.v[f] = v2_mul(W.v[f], v2(up));
   auto Bf = [&](int s) { return btab_f[(long long)s * P.nbase + j]; };
   if (j != 0 && j != P.ny - 1) {
     pw::remainder_y_base<D>(P.physf, Bf, W, ef, w2);
@@ -841,6 +850,8 @@ __device__ __forceinline__ void point_remainder(const PointParams& P, const floa
     const pw::WIn<D, float2> Wc = W;
     wall_remainder<D>(P.physf, btab_f, P.nbase, j, P.bcflags[j == 0 ? 0 : (long long)P.nx * P.nz], Wc, ef, w2);
   }
+#pragma unroll
+  for (int a = 0; a < D + 2; ++a) w2[a] = v2_mul(w2[a], v2(down));
 }
 
 // out[o] = acc - shift v[o].  The shift's product and difference are FP64: in pairs

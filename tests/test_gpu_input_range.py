@@ -30,7 +30,7 @@ def _waves(g):
     return np.stack(out).reshape(-1)
 
 
-@pytest.mark.parametrize("mode", [2], ids=["tangent"])
+@pytest.mark.parametrize("mode", [2, 0], ids=["tangent", "quotient"])
 @pytest.mark.parametrize("g", GRIDS, ids=[f"{g.nx}x{g.ny}x{g.nz}" for g in GRIDS])
 def test_scaled_input_gives_scaled_output(g, mode):
     import torch

@@ -320,6 +320,7 @@ __device__ __forceinline__ void row_pass(const ColArgs& A, unsigned bidx, ColSha
 #pragma unroll
   for (int q = 0; q < kCpw; ++q) d1[q] = d2[q] = ff2_zero2();
   double nrm = 0.0;
+  int rounds = 0;  // over all chunks: with few columns a warp has one or two rounds of each
   const long long rows = ((n + A.nb - 1) / A.nb + 31) / 32 * 32;
   const long long r0 = rows * bidx, r1 = r0 + rows < n ? r0 + rows : n;
   for (long long c0 = r0; c0 < r1; c0 += kColThreads) {
@@ -390,7 +391,7 @@ __device__ __forceinline__ void row_pass(const ColArgs& A, unsigned bidx, ColSha
             d1[q] = ff2_fma_u(wr, p, d1[q]);
             d2[q] = ff2_fma_u(wi, p, d2[q]);
           }
-        if ((i & 96) == 96) {
+        if ((++rounds & 3) == 0) {
 #pragma unroll
           for (int q = 0; q < kCpw; ++q) {
             d1[q] = ff2_norm(d1[q]);

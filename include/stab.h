@@ -308,8 +308,10 @@ stab_status stab_timing_read(stab_handle h, double* ms, long long* count, long l
  * the first and second derivatives side by side in 6 planes of shared memory
  * per line, or one after the other in 4 or 2)
  * with CUDA events on the handle's stream and keeps the fastest, in h and in a
- * process-wide cache keyed by device, line length, line count, job count and
- * boundary type; stab_create applies cached shapes to new handles.  force = 0
+ * process-wide cache keyed by device, line length, line count, job count,
+ * boundary type and kind of pass (FP64, FP64 with pair right-hand sides, pair
+ * passes of base flows that depend on y only); stab_create applies cached shapes
+ * to new handles.  force = 0
  * reuses a cached shape without timing.  cfg (host int[9], may be NULL)
  * receives (C, L, kinds) per axis (x, y, z; zeros for an absent z), ms (host
  * double[3], may be NULL) the tuned pass time per axis (-1 when cached).
@@ -340,7 +342,9 @@ stab_status stab_set_line_config(stab_handle h, int axis, int C, int L, int kind
 int stab_trim_memory(void);
 
 /* Write / read the process-wide tuning cache as text ("n nlines njobs
- * periodic C L kinds" per line; loaded entries apply to the current device).
+ * periodic C L kinds ff pair" per line, the last two 1 for entries of FP64 passes
+ * with pair right-hand sides and of pair passes and 0 where a line ends before
+ * them; loaded entries apply to the current device).
  * Return the number of entries, or -1 if the file cannot be opened. */
 int stab_autotune_save(const char* path);
 int stab_autotune_load(const char* path);

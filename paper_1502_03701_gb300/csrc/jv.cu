@@ -1826,17 +1826,18 @@ static cudaError_t run_derivatives(StabHandle* h, const double2* const* src, int
 // Autotuner of the line-pass launch shape (C, L) per axis: every admissible
 // candidate is timed with CUDA events on this handle's jobs, the fastest is
 // kept in the handle and in a process-wide cache keyed by device, line length,
-// line count, job count and boundary type.  C changes where the sweeps'
-// warm-up starts, so results may differ at the rounding level between shapes;
-// L does not change any result.
+// line count, job count, boundary type and kind of pass.  C changes where the
+// sweeps' warm-up starts, so results may differ at the rounding level between
+// shapes; L does not change any result.
 // ---------------------------------------------------------------------------
 namespace {
 struct TuneKey {
-  int dev, n, njobs, periodic, ff;
+  int dev, n, njobs, periodic, ff, pair;  // pair: the pair passes (one shape is not the other's best)
   long long nlines;
   bool operator<(const TuneKey& o) const {
     if (dev != o.dev) return dev < o.dev;
     if (ff != o.ff) return ff < o.ff;
+    if (pair != o.pair) return pair < o.pair;
     if (n != o.n) return n < o.n;
     if (nlines != o.nlines) return nlines < o.nlines;
     if (njobs != o.njobs) return njobs < o.njobs;
@@ -1847,6 +1848,9 @@ std::mutex g_tune_mu;
 std::map<TuneKey, LineCfg> g_tune;
 }  // namespace
 
+// whether J v takes the pair passes and the pointwise map of per-row coefficients
+static bool pair_path(const StabHandle* h) { return h->homog && h->d_coef && !h->force_dn_path; }
+
 static TuneKey tune_key(StabHandle* h, int ax, int njobs) {
   TuneKey k;
   cudaGetDevice(&k.dev);
@@ -1855,6 +1859,7 @@ static TuneKey tune_key(StabHandle* h, int ax, int njobs) {
   k.njobs = njobs;
   k.periodic = h->ax[ax].periodic;
   k.ff = h->stencil_ff;
+  k.pair = pair_path(h);
   return k;
 }
 
@@ -1889,7 +1894,7 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
     P.ff = h->stencil_ff;
     const int n = h->ax[ax].n;
     // with a y-only base flow the pair-arithmetic pass runs, which has no kinds variants
-    const bool fast = h->homog && h->d_coef && !h->force_dn_path;
+    const bool fast = pair_path(h);
     auto pass = [&]() { return fast ? run_pair_pass(h, ax, src) : run_pass(h, ax, P, jobs); };
     struct Candidate {
       LineCfg cfg;
@@ -1950,16 +1955,16 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
   return err;
 }
 
-// cache file: one line per entry, "n nlines njobs periodic C L kinds ff" (ff: pair
-// stencil; a line without it is an FP64-stencil entry); entries are applied to the
-// current device when loaded
+// cache file: one line per entry, "n nlines njobs periodic C L kinds ff pair" (ff: pair
+// right-hand sides, pair: pair passes; a line without them is an entry of the FP64
+// passes); entries are applied to the current device when loaded
 int jv_tune_save(const char* path) {
   FILE* f = std::fopen(path, "w");
   if (!f) return -1;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   for (const auto& kv : g_tune)
-    std::fprintf(f, "%d %lld %d %d %d %d %d %d\n", kv.first.n, kv.first.nlines, kv.first.njobs, kv.first.periodic,
-                 kv.second.C, kv.second.L, kv.second.kp, kv.first.ff);
+    std::fprintf(f, "%d %lld %d %d %d %d %d %d %d\n", kv.first.n, kv.first.nlines, kv.first.njobs, kv.first.periodic,
+                 kv.second.C, kv.second.L, kv.second.kp, kv.first.ff, kv.first.pair);
   std::fclose(f);
   return (int)g_tune.size();
 }
@@ -1975,11 +1980,12 @@ int jv_tune_load(const char* path) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   char line[256];
   while (std::fgets(line, sizeof line, f)) {
-    k.ff = 0;
-    const int got = std::sscanf(line, "%d %lld %d %d %d %d %d %d", &k.n, &k.nlines, &k.njobs, &k.periodic, &c.C, &c.L,
-                                &c.kp, &k.ff);
+    k.ff = k.pair = 0;
+    const int got = std::sscanf(line, "%d %lld %d %d %d %d %d %d %d", &k.n, &k.nlines, &k.njobs, &k.periodic, &c.C,
+                                &c.L, &c.kp, &k.ff, &k.pair);
     if (got < 7) continue;
-    if (c.C < 1 || c.L < 1 || c.kp < 1 || c.kp > 3 || k.n < 1 || (k.ff != 0 && k.ff != 1))
+    if (c.C < 1 || c.L < 1 || c.kp < 1 || c.kp > 3 || k.n < 1 || (k.ff != 0 && k.ff != 1) ||
+        (k.pair != 0 && k.pair != 1))
       continue;
     k.dev = dev;
     g_tune[k] = c;
@@ -2231,7 +2237,7 @@ cudaError_t jv_apply(StabHandle* h, const double2* v, double2* out, double2 shif
   P.shift = shift;
   double2* Tw = h->d_scratch + (long long)h->slots.Tw * h->npts;
   const int thr = 128;
-  const bool fast = h->homog && h->d_coef && !h->force_dn_path;
+  const bool fast = pair_path(h);
   if (h->visc) {
     const int ts = phase_begin(h, STAB_PHASE_TEMPERATURE);
     const int g = grid_for(2 * h->npts, thr);

@@ -1590,14 +1590,16 @@ static cudaError_t pair_shape(StabHandle* h, int axis, int njobs, bool batch, pl
   // 106.4: few chunks of few lines fill a CTA's shared memory).  Both components in a thread on small grids:
   // 32 x 64 48 us and 42.6 apart, 190 x 301 61.6 and 60; on large ones with chunks of 32 the passes of
   // 128 x 256 x 64 take 445, 318 and 357 us in place of 347, 258 and 268.
-  int C = cfg.C;
+  // A loaded shape can hold any positive C and L: chunks stay at 16 to 64 points (at least four points each,
+  // also halved: a wall's three rows lie in one chunk, the sweeps look two points ahead), CTAs at 32 lines.
+  int C = cfg.C > 0 ? std::max(cfg.C, 16) : 0;
   if (C <= 0) C = P.lanes == 1 && chunks16 >= 152LL * 512 && n <= 128 ? 32 : 16;
   if (C > kPairMaxC) C = kPairMaxC;
   // fewer than two warps per SM: a pass is one warp's latency, so chunks of half the length (the x pass of a
   // 32 x 64 layer 10.7 -> 9.3 us, its J v 45 -> 40 us)
   if (P.lanes == 1 && 2 * P.nlines * njobs * ((n + C - 1) / C) < 152LL * 64) C /= 2;
   const int nch = (n + C - 1) / C;
-  int L = cfg.L;
+  int L = std::min(cfg.L, 32);
   if (batch) {  // one launch for uneven instances: CTAs of about 128 threads for all of them
     L = std::max(1, 128 / (per * nch));
     while (L > 1 && smem_of(L, nch) > 48 * 1024) --L;

@@ -58,3 +58,22 @@ def test_file_of_the_older_format(orc, tmp_path):
         got = S.autotune(force=False)
         assert (got["y"] == (64, 2, 1, -1.0)) == taken and (got["x"] == (32, 3, 2, -1.0)) == taken
         S.close()
+
+
+@pytest.mark.parametrize("C,L", [(1, 1), (2, 7), (3, 100000), (7, 3), (1000, 2000000000)])
+def test_loaded_shapes_outside_the_tuned_ones(orc, C, L, tmp_path):
+    """Any positive C and L in the file: the pair passes keep chunks of four points or more."""
+    import torch
+    from paper_1502_03701_gb300 import Stab, binding
+    g, f = si.Grid(2, 9 + C % 5, 22 + 2 * (C % 7), 1, si.LX_04, -15, 15), si.Flow(0.4, 600.0)
+    path = str(tmp_path / "odd")
+    open(path, "w").write(f"{g.ny} {g.nx} 5 0 {C} {L} 3 0 1\n{g.nx} {g.ny} 7 1 {C} {L} 3 0 1\n")
+    assert binding.autotune_load(path) == 2
+    q0 = si.tanh_base_flow(g, f)
+    S = Stab(q0, g, f.Ma, f.Re, f.Pr, eps_mode=2)
+    v = si.random_complex(9, g.n)
+    out = torch.empty(g.n, dtype=torch.complex128, device="cuda")
+    S.apply_J(torch.from_numpy(v).cuda(), out)
+    ref = orc.core.jv(orc.Problem.from_inputs(g, f), q0, v, "tangent")
+    assert max_rel_err(out.cpu().numpy(), ref) < 2.8e-12
+    S.close()

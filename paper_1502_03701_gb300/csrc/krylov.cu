@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(kColThreads) k_col_pass(const __grid_constant_
 
 template <bool UPDATE, bool DOTS, bool NORM>
 void launch_col_pass(cudaStream_t st, const ColArgs& A, const int* gate, const int* skip) {
-  if (by_rows(A.n)) launch_chained(k_col_pass<UPDATE, DOTS, NORM, true>, A.nb, kColThreads, 0, st, A, gate, skip);
+  if (by_rows(A.n, A.k)) launch_chained(k_col_pass<UPDATE, DOTS, NORM, true>, A.nb, kColThreads, 0, st, A, gate, skip);
   else launch_chained(k_col_pass<UPDATE, DOTS, NORM, false>, A.nb, kColThreads, 0, st, A, gate, skip);
 }
 
@@ -1030,8 +1030,8 @@ cudaError_t cgs2_batch_plan(const std::vector<CgsJob>& jobs, BatchImage& im, Cgs
       continue;
     }
     if (J.k <= kColMax) {
-      cols[by_rows(J.n)].push_back(it);
-      col_bl[by_rows(J.n)].push_back(it.nb);
+      cols[by_rows(J.n, J.k)].push_back(it);
+      col_bl[by_rows(J.n, J.k)].push_back(it.nb);
       continue;
     }
     items.push_back(it);

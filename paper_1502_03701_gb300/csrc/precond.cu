@@ -753,7 +753,20 @@ cudaError_t bt_attributes() {
   return cudaSuccess;
 }
 
-constexpr int kApplyThreads = 256;  // CTAs of the block-Jacobi apply
+constexpr int kApplyThreads = 256;  // CTAs of the block-Jacobi apply, at most
+
+// Threads of the BF16 applies.  Four rows per thread and the columns split (blocks of a multiple of four rows): as
+// many as rows, twice that below four CTAs per SM (a power of two, 32 to 256), so that a thread keeps about eight
+// columns or more; every block of 256 rows or more takes 256.  Layer of 256 x 512 points, blocks of 4, 16, 32, 64 and
+// 128 rows: 88, 22, 19, 32 and 53 us; with 256 threads for all 478, 80, 41, 41 and 57.  One row per thread (other
+// sizes): threads for the slice's rows and no more (131,072 blocks of five rows 68 us, 155 with 256 threads).
+int apply_cols_threads(int bsz, int slices, long long ntiles) {
+  if (bsz % 4) return std::min(kApplyThreads, (((bsz + slices - 1) / slices + 31) / 32) * 32);
+  const int want = ntiles * slices < 4 * 152 ? 2 * bsz : bsz;
+  int t = 32;
+  while (t < kApplyThreads && t < want) t *= 2;
+  return t;
+}
 
 struct ApplyParams {
   const double2* q;
@@ -763,6 +776,7 @@ struct ApplyParams {
   long long npts;
   const int* gate;  // when set and nonzero the launch does nothing (graph-captured GMRES after convergence)
   const float2* q32;  // FP32 input (GMRES with an FP32 basis) instead of q
+  int threads;        // that share the columns of a BF16 block (a batch's CTAs may have more)
   FastDiv divntx, divnty, divpts, divtx, divty;
 };
 
@@ -870,23 +884,30 @@ __device__ __forceinline__ void apply_cols4_body(const ApplyParams& P, long long
   // S threads for the slice's row quads, the columns split over the CTA's groups of S threads
   int S = 1;
   while (S * (int)nslices < b4) S *= 2;
-  const int NG = (int)blockDim.x / S, grp = threadIdx.x / S, r4 = q0 + (int)threadIdx.x - grp * S;
+  const int NG = P.threads / S, grp = threadIdx.x / S, r4 = q0 + (int)threadIdx.x - grp * S;
   float ar[4] = {0.f, 0.f, 0.f, 0.f}, ai[4] = {0.f, 0.f, 0.f, 0.f};
-  if (r4 < q1) {
+  if (grp < NG && r4 < q1) {
     const uint4* col = Mt + r4;
     const int c1 = (grp + 1) * b / NG;
-#pragma unroll 8
-    for (int c = grp * b / NG; c < c1; ++c) {
-      const uint4 u = __ldg(col + (long long)c * b4);
-      const float2 x = qs[c];
-      const unsigned w[4] = {u.x, u.y, u.z, u.w};
+    constexpr int U = 4;  // columns in flight, also in the last step
+    for (int c = grp * b / NG; c < c1; c += U) {
+      uint4 u[U];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        __nv_bfloat162 e;
-        memcpy(&e, &w[k], sizeof(e));
-        const float2 m = __bfloat1622float2(e);
-        ar[k] += m.x * x.x - m.y * x.y;
-        ai[k] += m.x * x.y + m.y * x.x;
+      for (int q = 0; q < U; ++q)
+        if (c + q < c1) u[q] = __ldg(col + (long long)(c + q) * b4);
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (c + q >= c1) break;
+        const float2 x = qs[c + q];
+        const unsigned w[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          __nv_bfloat162 e;
+          memcpy(&e, &w[k], sizeof(e));
+          const float2 m = __bfloat1622float2(e);
+          ar[k] += m.x * x.x - m.y * x.y;
+          ai[k] += m.x * x.y + m.y * x.x;
+        }
       }
     }
   }
@@ -1573,6 +1594,7 @@ cudaError_t pc_apply(StabHandle* h, const double2* q, double2* z, const float2* 
   // row-major (a warp per row), BF16 column-major (a thread per row): measured fastest each
   int slices = (int)((2 * 152 + g.ntiles - 1) / g.ntiles);
   slices = h->pprec == 64 || h->pprec == 32 ? apply_row_slices(g.ntiles, g.bsz) : std::max(1, std::min(slices, g.bsz / 32));
+  P.threads = apply_cols_threads(g.bsz, slices, g.ntiles);
   const dim3 grid((unsigned)g.ntiles, (unsigned)slices);
   // the input's precision is a template parameter (FP32 basis: float2 input)
   const bool q32v = q32 != nullptr;
@@ -1583,11 +1605,11 @@ cudaError_t pc_apply(StabHandle* h, const double2* q, double2* z, const float2* 
     if (q32v) launch_chained(k_apply_rows<float, true>, grid, 256, g.bsz * sizeof(float2), h->stream, P);
     else launch_chained(k_apply_rows<float, false>, grid, 256, g.bsz * sizeof(float2), h->stream, P);
   } else if (g.bsz % 4 == 0) {
-    if (q32v) launch_chained(k_apply_cols4<true>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
-    else launch_chained(k_apply_cols4<false>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
+    if (q32v) launch_chained(k_apply_cols4<true>, grid, P.threads, g.bsz * sizeof(float2), h->stream, P);
+    else launch_chained(k_apply_cols4<false>, grid, P.threads, g.bsz * sizeof(float2), h->stream, P);
   } else {
-    if (q32v) launch_chained(k_apply_cols<__nv_bfloat162, float, true>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
-    else launch_chained(k_apply_cols<__nv_bfloat162, float, false>, grid, kApplyThreads, g.bsz * sizeof(float2), h->stream, P);
+    if (q32v) launch_chained(k_apply_cols<__nv_bfloat162, float, true>, grid, P.threads, g.bsz * sizeof(float2), h->stream, P);
+    else launch_chained(k_apply_cols<__nv_bfloat162, float, false>, grid, P.threads, g.bsz * sizeof(float2), h->stream, P);
   }
   phase_end(h, ts);
   return cudaGetLastError();
@@ -1654,17 +1676,18 @@ cudaError_t pc_batch_plan(const std::vector<StabHandle*>& hs, const double2* con
     // the same slices and threads as the single-handle apply
     int slices = (int)((2 * 152 + g.ntiles - 1) / g.ntiles);
     slices = h->pprec == 64 || h->pprec == 32 ? apply_row_slices(g.ntiles, g.bsz) : std::max(1, std::min(slices, g.bsz / 32));
+    P.threads = apply_cols_threads(g.bsz, slices, g.ntiles);
     int var, thr;
     size_t sm;
     if (h->pprec == 64) { var = 0; thr = 256; sm = g.bsz * sizeof(double2); }
     else if (h->pprec == 32) { var = 1; thr = 256; sm = g.bsz * sizeof(float2); }
     else if (g.bsz % 4 == 0) {
       var = 2;
-      thr = kApplyThreads;
+      thr = P.threads;
       sm = g.bsz * sizeof(float2);
     } else {
       var = 3;
-      thr = kApplyThreads;
+      thr = P.threads;
       sm = g.bsz * sizeof(float2);
     }
     if (g.ntiles * slices > (1LL << 30)) return cudaErrorInvalidValue;

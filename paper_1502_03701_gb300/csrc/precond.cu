@@ -486,11 +486,13 @@ __device__ __forceinline__ C2<double> bt_product(const C2<double>* Mrow, const B
       sy += a.x * b.y + a.y * b.x;
     }
   }
-  for (int o = G >> 1; o > 0; o >>= 1) {
-    sx += __shfl_xor_sync(0xffffffffu, sx, o);
-    sy += __shfl_xor_sync(0xffffffffu, sy, o);
-  }
-  return C2<double>{sx, sy};
+  // the row's halves sum one part each: the FP64 pipe takes every lane's addition, log2(G) in place of 2 log2(G)
+  if (G == 1) return C2<double>{sx, sy};
+  const bool im = g >= G / 2;
+  double t = (im ? sy : sx) + __shfl_xor_sync(0xffffffffu, im ? sx : sy, G / 2);
+  for (int o = G >> 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const double u = __shfl_xor_sync(0xffffffffu, t, G / 2);
+  return im ? C2<double>{u, t} : C2<double>{t, u};
 }
 
 // FP32 results to FP64 in integer arithmetic: the conversion instruction issues at 1/64 of the FP32 rate
@@ -546,7 +548,7 @@ __global__ void __launch_bounds__(kBtSweepThreads, STAGES == 5 ? 1 : 2) k_bt_swe
   if (P.gate && *P.gate) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int m = P.m, nlev = P.nlev;
-  const int G = bt_group(m, kBtSweepThreads), lg = __ffs(G) - 1;
+  const int G = bt_group(m, blockDim.x), lg = __ffs(G) - 1;
   const int row = threadIdx.x >> lg, g = threadIdx.x & (G - 1);
   const int pitch = bt_pitch<R>(m, G);
   const bool act = row < m, lead = act && g == 0;
@@ -722,7 +724,11 @@ cudaError_t launch_bt_apply(const BtApplyParams& B0, long long ntiles, cudaStrea
   BtApplyParams B = B0;
   const size_t vec = BtVec<R>::bytes(B.m);
   auto level = [&](int threads) { return (size_t)B.m * bt_pitch<R>(B.m, bt_group(B.m, threads)) * sizeof(C2<R>); };
-  const size_t lr = level(kBtRhsThreads), ls = level(kBtSweepThreads);
+  // FP64 tiles that share SMs are bound by the FP64 pipe, not by the level chain: half the threads spend half as
+  // many additions on a row's sum.  256 tiles of 64-unknown levels 1,282 us, 1,369 with 512 threads; 64 tiles 646
+  // and 598.
+  const int sweep = sizeof(R) == 8 && ntiles > 152 ? kBtSweepThreads / 2 : kBtSweepThreads;
+  const size_t lr = level(kBtRhsThreads), ls = level(sweep);
   const dim3 grid((unsigned)ntiles, (unsigned)B.nlev);
   // a level per CTA, two CTAs per SM at least
   B.staged = lr + vec <= kBtSmem / 2;
@@ -737,7 +743,7 @@ cudaError_t launch_bt_apply(const BtApplyParams& B0, long long ntiles, cudaStrea
   }
   // ring: five buffers where every tile has an SM of its own, three where two tiles share one
   const int stages = ntiles <= 152 && 5 * ls + 2 * vec <= kBtSmem ? 5 : 3 * ls + 2 * vec <= kBtSmem ? 3 : 0;
-  launch_chained(bt_sweep_kernel<R>(stages), (unsigned)ntiles, kBtSweepThreads, stages * ls + 2 * vec, st, B);
+  launch_chained(bt_sweep_kernel<R>(stages), (unsigned)ntiles, sweep, stages * ls + 2 * vec, st, B);
   return cudaGetLastError();
 }
 

@@ -299,6 +299,8 @@ struct stab_jv_batch_s {
   size_t d_cap = 0;
   void* h_buf = nullptr;  // pinned
   size_t h_cap = 0;
+  void* r_buf = nullptr;  // pinned: results that come back (batch_results)
+  size_t r_cap = 0;
   cudaEvent_t copied = nullptr;  // the last transfer out of h_buf has completed
   cudaEvent_t order = nullptr;   // orders the batch's stream against its handles' streams
   std::string err;
@@ -344,6 +346,7 @@ struct BatchImage {
 };
 
 cudaError_t batch_stage(stab_jv_batch_s* B, const BatchImage& im);
+cudaError_t batch_results(stab_jv_batch_s* B, size_t bytes);  // B->r_buf of that size (nothing in flight into it)
 
 // Planned batched phases: the sections of a parameter image (built once,
 // copied to the device once) and the launches that read them.  gates[i]

@@ -2291,6 +2291,17 @@ cudaError_t launch_norm2_stream(cudaStream_t st, const double2* v, long long n, 
 // (from a pinned staging buffer guarded by an event), and each phase is one
 // launch per kernel variant for all instances.
 // ---------------------------------------------------------------------------
+// Pinned memory for results, kept with the batch and grown on demand.
+cudaError_t batch_results(stab_jv_batch_s* B, size_t bytes) {
+  if (B->r_cap >= bytes) return cudaSuccess;
+  if (B->r_buf) cudaFreeHost(B->r_buf);
+  B->r_buf = nullptr;
+  B->r_cap = 0;
+  const cudaError_t e = cudaHostAlloc(&B->r_buf, bytes, cudaHostAllocDefault);
+  if (e == cudaSuccess) B->r_cap = bytes;
+  return e;
+}
+
 // Copy a parameter image to the batch's device buffer: through the pinned
 // staging buffer, once the previous transfer out of it has completed.
 cudaError_t batch_stage(stab_jv_batch_s* B, const BatchImage& im) {
@@ -2594,6 +2605,7 @@ extern "C" void stab_jv_batch_destroy(stab_jv_batch B) {
   cudaEventSynchronize(B->copied);
   if (B->d_buf) cudaFreeAsync(B->d_buf, B->stream);
   if (B->h_buf) cudaFreeHost(B->h_buf);
+  if (B->r_buf) cudaFreeHost(B->r_buf);
   cudaEventDestroy(B->copied);
   if (B->order) cudaEventDestroy(B->order);
   delete B;

@@ -854,13 +854,14 @@ __device__ __forceinline__ void point_remainder(const PointParams& P, const floa
   for (int a = 0; a < D + 2; ++a) w2[a] = v2_mul(w2[a], v2(down));
 }
 
-// out[o] = acc - shift v[o].  The shift's product and difference are FP64: in pairs
-// they left a result that the shift dominates with 48 bits (1.7e-15 in place of 1e-17
-// for J v - 1e6 v).
-__device__ __forceinline__ void put_row(const PointParams& P, long long o, ffn2 acc) {
+// out[o] = acc - shift v, in FP64: as pairs the product and the difference left a result that the shift
+// dominates with 48 bits (J v - 1e6 v 1.7e-15 off in place of 1e-17).  v = P.v[o] is read again, since kept from
+// the start it takes registers that the loads in flight need: in the tangent's kernel ahead of the last sums, in
+// the quotient's after the remainder (60 x 90 x 28 tangent 120.4 us, 124.9 read last; 128 x 256 x 64 quotient
+// 1,504 us, 1,535 read first).
+__device__ __forceinline__ void put_row(const PointParams& P, long long o, ffn2 acc, double2 v) {
   double2 r = ff2_to_d(ff2_norm(acc));
   if (P.shift.x != 0.0 || P.shift.y != 0.0) {
-    const double2 v = P.v[o];
     r.x = fma(-P.shift.x, v.x, fma(P.shift.y, v.y, r.x));  // explicit: the kernels that inline this round alike
     r.y = fma(-P.shift.x, v.y, fma(-P.shift.y, v.x, r.y));
   }
@@ -943,6 +944,10 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
           if (a != c) put(om + a * D + c, ff2_from_slot(in[k++]));
     }
   }
+  double2 vs[D + 2];
+  const bool shifted = P.shift.x != 0.0 || P.shift.y != 0.0;
+#pragma unroll
+  for (int a = 0; a < D + 2; ++a) vs[a] = !EPS && shifted ? P.v[(long long)a * P.npts + i] : make_double2(0.0, 0.0);
   if (EPS && e != 0.0) {  // O(eps) remainder of the quotient, FP32
     float2 w2[D + 2];
     point_remainder<D>(P, btab_f, i, j, e, W, w2);
@@ -950,7 +955,10 @@ __device__ __forceinline__ void point_fast_body(const PointParams& P, const floa
     for (int a = 0; a < D + 2; ++a) acc[a].lo = v2_add(acc[a].lo, w2[a]);
   }
 #pragma unroll
-  for (int a = 0; a < D + 2; ++a) put_row(P, (long long)a * P.npts + i, acc[a]);
+  for (int a = 0; a < D + 2; ++a) {
+    const long long o = (long long)a * P.npts + i;
+    put_row(P, o, acc[a], EPS ? P.v[o] : vs[a]);
+  }
 }
 
 // One output row per thread: the same sums in the same order (and the same bits), with the row's inputs
@@ -969,7 +977,7 @@ __device__ __forceinline__ void point_row_body(const PointParams& P, const float
   const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   double2 vd[D + 3];
 #pragma unroll
-  for (int f = 0; f < D + 2; ++f) vd[f] = EPS || coef_used<D>(A, f) ? P.v[(long long)f * P.npts + i] : make_double2(0.0, 0.0);
+  for (int f = 0; f < D + 2; ++f) vd[f] = EPS || f == A || coef_used<D>(A, f) ? P.v[(long long)f * P.npts + i] : make_double2(0.0, 0.0);
   vd[D + 2] = visc ? P.scratch[(long long)P.s_Tw * P.npts + i] : make_double2(0.0, 0.0);
   float4 in[NW], cf[NW];  // the row's inputs and coefficients (unused ones take no registers)
   {
@@ -1009,7 +1017,8 @@ __device__ __forceinline__ void point_row_body(const PointParams& P, const float
     point_remainder<D>(P, btab_f, i, j, e, W, w2);
     acc.lo = v2_add(acc.lo, w2[A]);
   }
-  put_row(P, (long long)A * P.npts + i, acc);
+  const long long o = (long long)A * P.npts + i;
+  put_row(P, o, acc, EPS ? P.v[o] : vd[A]);
 }
 
 // grid (points / 128, rows)

@@ -342,9 +342,9 @@ stab_status stab_set_line_config(stab_handle h, int axis, int C, int L, int kind
 int stab_trim_memory(void);
 
 /* Write / read the process-wide tuning cache as text ("n nlines njobs
- * periodic C L kinds ff pair" per line, the last two 1 for entries of FP64 passes
- * with pair right-hand sides and of pair passes and 0 where a line ends before
- * them; loaded entries apply to the current device).
+ * periodic C L kinds ff" per line, ff = 1 for pair right-hand sides, and a ninth
+ * column, 1, for entries of the pair passes; columns that a line does not have
+ * count as 0; loaded entries apply to the current device).
  * Return the number of entries, or -1 if the file cannot be opened. */
 int stab_autotune_save(const char* path);
 int stab_autotune_load(const char* path);

@@ -1966,16 +1966,17 @@ cudaError_t jv_autotune(StabHandle* h, int force, double* ms_out) {
   return err;
 }
 
-// cache file: one line per entry, "n nlines njobs periodic C L kinds ff pair" (ff: pair
-// right-hand sides, pair: pair passes; a line without them is an entry of the FP64
-// passes); entries are applied to the current device when loaded
+// cache file: one line per entry, "n nlines njobs periodic C L kinds ff [pair]" (ff: pair
+// right-hand sides; pair: 1, written for entries of the pair passes; a line without
+// them is an entry of the FP64 passes); entries are applied to the current device when
+// loaded
 int jv_tune_save(const char* path) {
   FILE* f = std::fopen(path, "w");
   if (!f) return -1;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   for (const auto& kv : g_tune)
-    std::fprintf(f, "%d %lld %d %d %d %d %d %d %d\n", kv.first.n, kv.first.nlines, kv.first.njobs, kv.first.periodic,
-                 kv.second.C, kv.second.L, kv.second.kp, kv.first.ff, kv.first.pair);
+    std::fprintf(f, "%d %lld %d %d %d %d %d %d%s\n", kv.first.n, kv.first.nlines, kv.first.njobs, kv.first.periodic,
+                 kv.second.C, kv.second.L, kv.second.kp, kv.first.ff, kv.first.pair ? " 1" : "");
   std::fclose(f);
   return (int)g_tune.size();
 }

@@ -81,14 +81,16 @@ typedef struct {
   int max_restarts;       /* IRAM restart limit, default 300 */
   unsigned long long seed;/* start vector seed when no v0 is given, default 0x5EED */
   int gmres_basis_prec;   /* GMRES Krylov basis and its orthogonalisation: 64 (FP64 flexible GMRES,
-                             default) or 32 (FP32 basis, non-flexible right preconditioning; J v, the
-                             solution update and the true residual of every restart stay FP64, so the
-                             restarts refine the solution to the FP64 tolerance) */
+                             default) or 32 (FP32 basis, non-flexible right preconditioning; J v of FP64
+                             vectors, the solution update and the true residual of every restart do not
+                             change, so the restarts refine the solution to the FP64 tolerance) */
   int stencil_prec;       /* right-hand sides B f of the compact schemes inside J v of base flows that vary in
                              x or z: 64 (FP64, default) or 48 (interior rows in FP32 pair arithmetic on
                              exactly power-of-two-scaled inputs, ~2^-47 relative; the Thomas sweeps, the
                              closure rows and the set-up stay FP64).  Base flows that depend on y only form
-                             differences in FP64 and everything after them in FP32 pairs with either value */
+                             differences and the shift's term in FP64 and everything else in FP32 pairs with
+                             either value: J v within 6e-15 of 64-bit evaluation (5e-16 for general base
+                             flows with 64) */
   int lgmres_k;           /* inner solver: 0 = GMRES(gmres_m) (default); k in [1, min(8, gmres_m - 1)] =
                              LGMRES (Sec. "Iterative solvers", after Baker, Jessup and Manteuffel): every
                              cycle spans gmres_m directions, gmres_m - k Krylov directions of the residual
@@ -105,7 +107,7 @@ typedef struct {
                              step of the FP64 flexible GMRES(gmres_m) takes as its direction z_j an inner
                              GMRES(k) approximation of (J - sigma I)^{-1} v_j with an FP32 Krylov basis and FP32
                              orthogonalisation, right preconditioned with the block-Jacobi inverses (opts.precond),
-                             run until its residual is below gmres_inner_tol ||v_j|| or k steps; J v stays FP64.
+                             run until its residual is below gmres_inner_tol ||v_j|| or k steps; J v does not change.
                              Needs gmres_basis_prec = 64 and lgmres_k = 0 (else STAB_ERR_UNSUPPORTED) */
   double gmres_inner_tol; /* relative tolerance of each inner solve, default 1e-3 */
 } stab_opts;

@@ -25,7 +25,7 @@ __device__ __forceinline__ double warp_sum(double x) {
 // CGS2 reads V once and splits it once.  The next rows' loads are in flight
 // meanwhile.  Sums over blocks: the last block to finish adds the blocks'
 // partial sums in block order (reproducible) and resets the counter.
-// 524,288 unknowns, 55 vectors: the three passes of CGS2 take 130, 228 and 112 us
+// 524,288 unknowns, 55 vectors: the three passes of CGS2 take 139, 226 and 108 us
 // (481 MB each, 62 to 66 % of the issue slots; 164, 387 and 273 us as kernels of
 // one warp per column and FP64 every fourth column, with V read twice).
 // ---------------------------------------------------------------------------

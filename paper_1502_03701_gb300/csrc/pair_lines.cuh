@@ -30,9 +30,9 @@
 // a smooth field of size 2^-64 on 256 points were good to 1e-9 only.  The second
 // derivation of a mixed derivative takes pairs and is not scaled.
 //
-// 128 x 256 x 64 points: y 347, z 258, x 268 us for all derivatives of an axis,
-// 62 to 67 % of the issue slots; FP64 sweeps took 0.96, 0.87 and 1.06 ms.  32 x 64
-// points: 10.4 and 10.9 us (32 us each), one warp's latency.
+// 128 x 256 x 64 points: y 257, z 267, x 346 us for all derivatives of an axis;
+// FP64 sweeps took 0.96, 0.87 and 1.06 ms.  60 x 90 x 28 points: 62 to 67 % of the
+// issue slots.  32 x 64 points: 10.5 and 8.7 us (32 us each), one warp's latency.
 #pragma once
 #include "internal.cuh"
 
